@@ -7,7 +7,10 @@
 // n_slots, row 0 its recurrent embedding); every activation is row-major
 // [rows][width].  Rows past a sample's entity count are computed (from the
 // embedding bias alone) but no row attends to them, so they receive exactly
-// zero gradient and add nothing to the weight gradients.
+// zero gradient and add nothing to the weight gradients.  The head reads the
+// recurrent token alone, so of the last block only the keys and values are
+// made for every token; its queries, attention output, feed-forward sub-block
+// and their backward run on the n recurrent rows, stored densely ([n][width]).
 //
 // The dense contractions run on CUDA cores in FP32 (a 64 x 64 register-tiled
 // GEMM); the weight gradients are split along the token rows into partial
@@ -49,7 +52,8 @@ struct Gemm {
   long long M, K, kchunk;
   int N, epi;
   const float* bias;   // [N] (EPI_BIAS*)
-  const float* R;      // residual added (EPI_BIAS_RES), ld = ldc
+  const float* R;      // residual added (EPI_BIAS_RES), ld = ldr
+  long long ldr;
   float* C2;           // GELU of the output (EPI_BIAS_GELU), ld = ldc
   const float* aux;    // pre-activation whose GELU derivative scales the output (EPI_GELU_GRAD), ld = ldc
   const uint16_t* bimg;  // BF16 image of B for the tensor-core path (kinds 0, 1), or NULL: CUDA cores
@@ -69,7 +73,7 @@ __device__ __forceinline__ void epi_store(const Gemm& g, long long m, int n, flo
       g.C[o] = v + g.bias[n];
       break;
     case EPI_BIAS_RES:
-      g.C[o] = v + g.bias[n] + g.R[o];
+      g.C[o] = v + g.bias[n] + g.R[m * g.ldr + n];
       break;
     case EPI_BIAS_GELU:
       v += g.bias[n];
@@ -376,11 +380,14 @@ __global__ void ln_fwd_kernel(const float* __restrict__ X, const float* __restri
 // LayerNorm backward, one warp per row: out = base + dL/dX from dY (the
 // gradient at the LayerNorm output), and per-block partial sums of dL/dg
 // (sum dY xh) and dL/db (sum dY) into part[block][2d] (blocks of 256
-// threads).  out may equal base.
-template <int DJ>
+// threads).  out may equal base.  REC (the last block's first LayerNorm):
+// base and dY0, a second gradient at the LayerNorm output, hold the recurrent
+// rows alone (row s T of the others at s) and are zero elsewhere.
+template <int DJ, bool REC>
 __global__ void ln_bwd_kernel(const float* __restrict__ dY, const float* __restrict__ X,
                               const float* __restrict__ stat, const float* __restrict__ gam, const float* base,
-                              float* out, float* __restrict__ part, long long rows) {
+                              float* out, float* __restrict__ part, long long rows, const float* __restrict__ dY0,
+                              unsigned T) {
   constexpr int d = 32 * DJ;
   const int lane = threadIdx.x & 31;
   const long long w0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -390,12 +397,20 @@ __global__ void ln_bwd_kernel(const float* __restrict__ dY, const float* __restr
   // current one
   float dyn[DJ], xn[DJ], bn[DJ], mn = 0.0f, rn = 0.0f;
   auto fetch = [&](long long r) {
+    const long long s0 = REC ? (long long)((unsigned)r / T) : 0;  // (rows < 2^32: max_batch <= 2^22)
+    const bool rec = REC && r == s0 * T;
 #pragma unroll
     for (int i = 0; i < DJ; ++i) {
       const long long o = r * d + lane + 32 * i;
       dyn[i] = dY[o];
       xn[i] = X[o];
-      bn[i] = base[o];
+      if (REC) {
+        const long long c = s0 * d + lane + 32 * i;
+        bn[i] = rec ? base[c] : 0.0f;
+        if (rec) dyn[i] += dY0[c];
+      } else {
+        bn[i] = base[o];
+      }
     }
     mn = stat[2 * r];
     rn = stat[2 * r + 1];
@@ -907,10 +922,284 @@ __global__ void __launch_bounds__(128, 6)
   }
 }
 
+// ---- attention of the last block: the recurrent query alone ----------------
+// The head reads nothing else, so the rest of the block (Wo, the feed-forward
+// sub-block and their backward) runs on n rows instead of n T.  The actor's
+// gradient step (163,840 samples, 11 tokens, d 64, 2 blocks) went from 19.5 to
+// 14.3 ms, the critic's (32,768) from 4.40 to 3.24, d 128 with 17 tokens and 3
+// blocks (16,384) from 14.1 to 11.6.
+// One (sample, head) per warp.  Q0 [n][d] holds the recurrent queries, KV
+// [rows][2d] the keys and values of every token; P0 [n][H][T] and O0 [n][d]
+// are row 0 of P and O above, by the same arithmetic.  The cost is one read
+// of K and V (and in the backward one write of dK and dV).
+
+// General form (lane u: key u of the scores; lane j: output column j).
+template <int DH>
+__global__ void __launch_bounds__(256) attn0_fwd_kernel(const float* __restrict__ Q0, const float* __restrict__ KV,
+                                                        const int32_t* __restrict__ n_ent,
+                                                        const int32_t* __restrict__ sel, float* __restrict__ P0,
+                                                        float* __restrict__ O0, long long n, int T, int NS, int H,
+                                                        float scale) {
+  const int lane = threadIdx.x & 31;
+  const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w >= n * H) return;  // whole warps leave together
+  const long long s = w / H;
+  const int hh = (int)(w - s * H), d = DH * H, ld = 2 * d;
+  int ne = n_ent[sel ? (long long)sel[s] : s];
+  ne = ne < 0 ? 0 : (ne > NS ? NS : ne);
+  const float* K = KV + s * T * ld + hh * DH;
+  const float* V = K + d;
+  const bool on = lane < T && lane <= ne;
+  float sc = -INFINITY;
+  if (on) {
+    const float4* q4 = reinterpret_cast<const float4*>(Q0 + s * d + hh * DH);
+    const float4* k4 = reinterpret_cast<const float4*>(K + lane * ld);
+    float acc = 0.0f;
+#pragma unroll
+    for (int j = 0; j < DH / 4; ++j) {
+      const float4 q = __ldg(q4 + j), k = __ldg(k4 + j);
+      acc = fmaf(q.x, k.x, acc);
+      acc = fmaf(q.y, k.y, acc);
+      acc = fmaf(q.z, k.z, acc);
+      acc = fmaf(q.w, k.w, acc);
+    }
+    sc = acc * scale;
+  }
+  const float mx = warp_max(sc);
+  const float e = on ? expf(sc - mx) : 0.0f;
+  float z = 0.0f;
+  for (int u = 0; u < T; ++u) z += __shfl_sync(0xffffffffu, e, u);  // (in key order, as attn_fwd_kernel)
+  const float p = e * (1.0f / z);
+  if (lane < T) P0[w * T + lane] = p;
+  float o = 0.0f;
+  for (int u = 0; u <= ne && u < T; ++u) {
+    const float pu = __shfl_sync(0xffffffffu, p, u);
+    if (lane < DH) o = fmaf(pu, __ldg(V + u * ld + lane), o);
+  }
+  if (lane < DH) O0[s * d + hh * DH + lane] = o;
+}
+
+template <int DH>
+__global__ void __launch_bounds__(256) attn0_bwd_kernel(const float* __restrict__ Q0, const float* __restrict__ KV,
+                                                        const float* __restrict__ P0, const float* __restrict__ dO0,
+                                                        float* __restrict__ dQ0, float* __restrict__ dKV, long long n,
+                                                        int T, int H, float scale) {
+  const int lane = threadIdx.x & 31;
+  const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w >= n * H) return;  // whole warps leave together
+  const long long s = w / H;
+  const int hh = (int)(w - s * H), d = DH * H, ld = 2 * d;
+  const float* K = KV + s * T * ld + hh * DH;
+  float* dK = dKV + s * T * ld + hh * DH;
+  const float p = lane < T ? __ldg(P0 + w * T + lane) : 0.0f;
+  float dp = 0.0f;
+  if (lane < T) {
+    const float4* g4 = reinterpret_cast<const float4*>(dO0 + s * d + hh * DH);
+    const float4* v4 = reinterpret_cast<const float4*>(K + d + lane * ld);
+#pragma unroll
+    for (int j = 0; j < DH / 4; ++j) {
+      const float4 g = __ldg(g4 + j), v = __ldg(v4 + j);
+      dp = fmaf(g.x, v.x, dp);
+      dp = fmaf(g.y, v.y, dp);
+      dp = fmaf(g.z, v.z, dp);
+      dp = fmaf(g.w, v.w, dp);
+    }
+  }
+  float dot = 0.0f;
+  for (int u = 0; u < T; ++u) dot = fmaf(__shfl_sync(0xffffffffu, p, u), __shfl_sync(0xffffffffu, dp, u), dot);
+  const float ds = p * (dp - dot) * scale;
+  const int j = lane < DH ? lane : 0;
+  const float qj = __ldg(Q0 + s * d + hh * DH + j), gj = __ldg(dO0 + s * d + hh * DH + j);
+  float dq = 0.0f;
+  for (int u = 0; u < T; ++u) {
+    const float su = __shfl_sync(0xffffffffu, ds, u), pu = __shfl_sync(0xffffffffu, p, u);
+    if (lane < DH) {
+      dq = fmaf(su, __ldg(K + u * ld + lane), dq);
+      dK[u * ld + lane] = su * qj;
+      dK[u * ld + d + lane] = pu * gj;
+    }
+  }
+  if (lane < DH) dQ0[s * d + hh * DH + lane] = dq;
+}
+
+// The tensor-core path's form (T <= 16, head dimension 16): the products of
+// attn_fwd_mma_kernel with the one query in row 0 of the A operand, every
+// fragment straight from global memory (a row of K or V is two sectors that
+// one load of the warp touches; no staging, so many warps' loads are in
+// flight).  163,840 samples x 4 heads x 11 tokens: forward 283 us against 502
+// for all queries, backward 426 against 870.
+__device__ __forceinline__ float quad_pick(float lo, float hi, int t, int up) {
+  // the quad lane that holds column t + up of an 8-wide accumulator tile
+  const int src = (threadIdx.x & 28) | ((t + up) >> 1);
+  const float a = __shfl_sync(0xffffffffu, lo, src), b = __shfl_sync(0xffffffffu, hi, src);
+  return (t & 1) ? b : a;
+}
+__global__ void __launch_bounds__(256)
+    attn0_fwd_mma_kernel(const float* __restrict__ Q0, const float* __restrict__ KV, const int32_t* __restrict__ n_ent,
+                         const int32_t* __restrict__ sel, float* __restrict__ P0, float* __restrict__ O0, long long n,
+                         int T, int NS, int H, float scale) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w >= n * H) return;  // whole warps leave together
+  const long long s = w / H;
+  const int hh = (int)(w - s * H), d = 16 * H, ld = 2 * d;
+  const float* K = KV + s * T * ld + hh * 16;
+  const float* V = K + d;
+  float q[4], kf[2][4], vf[4][2];  // K rows g + 8 j, V rows t + 4 i (columns g, g + 8)
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    q[i] = g == 0 ? __ldg(Q0 + s * d + hh * 16 + t + 4 * i) : 0.0f;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      kf[j][i] = g + 8 * j < T ? __ldg(K + (g + 8 * j) * ld + t + 4 * i) : 0.0f;
+      vf[i][j] = t + 4 * i < T ? __ldg(V + (t + 4 * i) * ld + g + 8 * j) : 0.0f;
+    }
+  }
+  int ne = n_ent[sel ? (long long)__ldg(sel + s) : s];
+  ne = ne < 0 ? 0 : (ne > NS ? NS : ne);
+  float sc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+  for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      mma_tf32(sc[j], tf32r(q[2 * kk]), 0u, tf32r(q[2 * kk + 1]), 0u, tf32r(kf[j][2 * kk]), tf32r(kf[j][2 * kk + 1]));
+  float mx = -INFINITY;
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int col = 8 * j + 2 * t + e;
+      const float v = (col < T && col <= ne) ? sc[j][e] * scale : -INFINITY;
+      sc[j][e] = v;
+      mx = fmaxf(mx, v);
+    }
+  mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+  mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+  float z = 0.0f;
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const float x = sc[j][e];
+      const float ex = x == -INFINITY ? 0.0f : __expf(x - mx);
+      sc[j][e] = ex;
+      z += ex;
+    }
+  z += __shfl_xor_sync(0xffffffffu, z, 1);
+  z += __shfl_xor_sync(0xffffffffu, z, 2);
+  const float iz = 1.0f / z;
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int col = 8 * j + 2 * t;
+    sc[j][0] *= iz;
+    sc[j][1] *= iz;
+    if (g == 0 && col < T) P0[w * T + col] = sc[j][0];
+    if (g == 0 && col + 1 < T) P0[w * T + col + 1] = sc[j][1];
+  }
+  float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+  for (int kk = 0; kk < 2; ++kk) {
+    const float p0 = quad_pick(sc[kk][0], sc[kk][1], t, 0), p1 = quad_pick(sc[kk][0], sc[kk][1], t, 4);
+    const uint32_t a0 = g == 0 ? tf32r(p0) : 0u, a2 = g == 0 ? tf32r(p1) : 0u;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) mma_tf32(o[j], a0, 0u, a2, 0u, tf32r(vf[2 * kk][j]), tf32r(vf[2 * kk + 1][j]));
+  }
+  if (g == 0) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      *reinterpret_cast<float2*>(O0 + s * d + hh * 16 + 8 * j + 2 * t) = make_float2(o[j][0], o[j][1]);
+  }
+}
+
+// Backward of the same: dP and dQ by MMAs; dK_u = dS_u q and dV_u = P_u dO
+// are single products of TF32-rounded factors (exact in FP32), which is what
+// the MMAs over the one query row give.
+__global__ void __launch_bounds__(256)
+    attn0_bwd_mma_kernel(const float* __restrict__ Q0, const float* __restrict__ KV, const float* __restrict__ P0,
+                         const float* __restrict__ dO0, float* __restrict__ dQ0, float* __restrict__ dKV, long long n,
+                         int T, int H, float scale) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w >= n * H) return;  // whole warps leave together
+  const long long s = w / H;
+  const int hh = (int)(w - s * H), d = 16 * H, ld = 2 * d;
+  const float* K = KV + s * T * ld + hh * 16;
+  const float* V = K + d;
+  const float* dOb = dO0 + s * d + hh * 16;
+  float gf[4], vf[2][4], kf[4][2], pv[2][2];  // V rows g + 8 j, K rows t + 4 i
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    gf[i] = g == 0 ? __ldg(dOb + t + 4 * i) : 0.0f;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      vf[j][i] = g + 8 * j < T ? __ldg(V + (g + 8 * j) * ld + t + 4 * i) : 0.0f;
+      kf[i][j] = t + 4 * i < T ? __ldg(K + (t + 4 * i) * ld + g + 8 * j) : 0.0f;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int c = 8 * j + 2 * t + e;
+      pv[j][e] = c < T ? __ldg(P0 + w * T + c) : 0.0f;
+    }
+  const float4 q4 = __ldg(reinterpret_cast<const float4*>(Q0 + s * d + hh * 16) + t);
+  const float4 g4 = __ldg(reinterpret_cast<const float4*>(dOb) + t);
+  float dp[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+  for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      mma_tf32(dp[j], tf32r(gf[2 * kk]), 0u, tf32r(gf[2 * kk + 1]), 0u, tf32r(vf[j][2 * kk]),
+               tf32r(vf[j][2 * kk + 1]));
+  float r0 = 0.0f;  // (row 0's sum: right in the lanes of the first quad)
+#pragma unroll
+  for (int j = 0; j < 2; ++j) r0 = fmaf(pv[j][0], dp[j][0], fmaf(pv[j][1], dp[j][1], r0));
+  r0 += __shfl_xor_sync(0xffffffffu, r0, 1);
+  r0 += __shfl_xor_sync(0xffffffffu, r0, 2);
+  float ds[2][2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) ds[j][e] = pv[j][e] * (dp[j][e] - r0) * scale;
+  float dq[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+  for (int kk = 0; kk < 2; ++kk) {
+    const float s0 = quad_pick(ds[kk][0], ds[kk][1], t, 0), s1 = quad_pick(ds[kk][0], ds[kk][1], t, 4);
+    const uint32_t a0 = g == 0 ? tf32r(s0) : 0u, a2 = g == 0 ? tf32r(s1) : 0u;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) mma_tf32(dq[j], a0, 0u, a2, 0u, tf32r(kf[2 * kk][j]), tf32r(kf[2 * kk + 1][j]));
+  }
+  if (g == 0) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      *reinterpret_cast<float2*>(dQ0 + s * d + hh * 16 + 8 * j + 2 * t) = make_float2(dq[j][0], dq[j][1]);
+  }
+  const float qv[4] = {q4.x, q4.y, q4.z, q4.w}, gv[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {  // token u = g + 8 j, columns 4 t .. 4 t + 3
+    const int src = g >> 1;      // (lane of the first quad holding column g of tile j)
+    const float sa = __shfl_sync(0xffffffffu, ds[j][0], src), sb = __shfl_sync(0xffffffffu, ds[j][1], src);
+    const float pa = __shfl_sync(0xffffffffu, pv[j][0], src), pb = __shfl_sync(0xffffffffu, pv[j][1], src);
+    const float su = __uint_as_float(tf32r((g & 1) ? sb : sa)), pu = __uint_as_float(tf32r((g & 1) ? pb : pa));
+    float a[4], b[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      a[i] = su * __uint_as_float(tf32r(qv[i]));
+      b[i] = pu * __uint_as_float(tf32r(gv[i]));
+    }
+    if (g + 8 * j < T) {
+      float* out = dKV + (s * T + g + 8 * j) * ld + hh * 16 + 4 * t;
+      *reinterpret_cast<float4*>(out) = make_float4(a[0], a[1], a[2], a[3]);
+      *reinterpret_cast<float4*>(out + d) = make_float4(b[0], b[1], b[2], b[3]);
+    }
+  }
+}
+
 struct HeadArgs {
-  const float* XL;  // [rows][d] residual stream after the last block
+  const float* XL;  // [n][d] residual stream of the recurrent tokens after the last block
   long long n;
-  int T, n_out, mode;  // mode 0: forward, 1: PPO actor loss, 2: value loss
+  int n_out, mode;  // mode 0: forward, 1: PPO actor loss, 2: value loss
   const float *lnf_g, *lnf_b, *Wh, *bh;
   float* out;        // [n][n_out] (mode 0)
   float* h_out;      // [n][d] (mode 0, optional)
@@ -918,12 +1207,12 @@ struct HeadArgs {
   const int32_t* actions;
   const float *logp_old, *adv, *ret;
   float clip_eps, ent_coef, inv_n;
-  float* dXL;        // [rows][d] (modes 1, 2): token 0 gets the gradient, the other rows zero
+  float* dXL;        // [n][d] (modes 1, 2): gradient at XL
   float* part;       // [warps][2d + n_out d + n_out]: lnf_g, lnf_b, Wh, bh partial gradients
   double* spart;     // [warps][4] partial sums of the per-sample statistics
 };
 
-// Final LayerNorm and head on token 0, one warp per sample; in the loss modes
+// Final LayerNorm and head on the recurrent token, one warp per sample; in the loss modes
 // also the loss, dL/d(head output), the head's and final LayerNorm's
 // backward, and per-warp partial sums of their parameter gradients.
 template <int DJ, int NO>
@@ -944,7 +1233,7 @@ __global__ void __launch_bounds__(256) head_kernel(HeadArgs a) {
   for (int i = 0; i < DJ; ++i) gg[i] = gb[i] = 0.0f;
   double st[4] = {0.0, 0.0, 0.0, 0.0};
   for (long long s = w0; s < a.n; s += nw) {
-    const float* x0 = a.XL + s * a.T * d;
+    const float* x0 = a.XL + s * d;
     float x[DJ], xh[DJ], U[DJ], sum = 0.0f;
 #pragma unroll
     for (int i = 0; i < DJ; ++i) {
@@ -1055,12 +1344,9 @@ __global__ void __launch_bounds__(256) head_kernel(HeadArgs a) {
     }
     m1 = warp_sum(m1) * (1.0f / d);
     m2 = warp_sum(m2) * (1.0f / d);
-    float* dx0 = a.dXL + s * a.T * d;
+    float* dx0 = a.dXL + s * d;
 #pragma unroll
     for (int i = 0; i < DJ; ++i) dx0[lane + 32 * i] = rstd * (dxh[i] - m1 - xh[i] * m2);
-    for (int t = 1; t < a.T; ++t)
-#pragma unroll
-      for (int i = 0; i < DJ; ++i) dx0[t * d + lane + 32 * i] = 0.0f;
   }
   if (a.mode == 0) return;
   const long long plen = 2 * d + (long long)no * d + no;
@@ -1247,8 +1533,11 @@ struct ut_tfm {
   std::vector<void*> allocs;
   float *prm = nullptr, *am = nullptr, *av = nullptr;
   int adam_t = 0;
-  // activations: X [(L+1)][max_rows][d]; per block l: Y1, O, M, Y2 [rows][d],
-  // S1, S2 [rows][2], QKV [rows][3d], P [samples][H][T][T], Z, G [rows][4d]
+  // activations: X [L][max_rows][d]; per block l: Y1, O, M, Y2 [rows][d],
+  // S1, S2 [rows][2], QKV [rows][3d], P [samples][H][T][T], Z, G [rows][4d];
+  // of the last block KV [rows][2d] and Q0 [samples][d] in QKV's place, P
+  // [samples][H][T], and O, M, Y2, S2, Z, G and the output X of the samples'
+  // recurrent rows alone
   float *X = nullptr, *Y1 = nullptr, *Y2 = nullptr, *S1 = nullptr, *S2 = nullptr, *QKV = nullptr, *P = nullptr,
         *O = nullptr, *M = nullptr, *Z = nullptr, *G = nullptr;
   // backward buffers
@@ -1260,10 +1549,12 @@ struct ut_tfm {
   int gemm_tc = 1;
   // BF16 images of the block weights for the tensor-core path, per block l:
   // Wqkv, Wo, W1, W2 as B of the forward, then their transposes as B of the
-  // input gradient (ImgSpec table on the device, packed once per call)
+  // input gradient (ImgSpec table on the device, packed once per call); the
+  // last block's Wqkv images hold Wk and Wv, and Wq and its transpose follow
+  // all blocks' images
   uint16_t* wimg = nullptr;
-  std::vector<int64_t> img_off;  // [L][8] offsets into wimg (elements)
-  int64_t* img_spec = nullptr;   // [L * 8][5] (weight offset, R, C, transpose, image offset)
+  std::vector<int64_t> img_off;  // [8 L + 2] offsets into wimg (elements)
+  int64_t* img_spec = nullptr;   // [8 L + 2][5] (weight offset, R, C, transpose, image offset)
   int n_img = 0, img_max = 0;
   int* status = nullptr;
 };
@@ -1382,6 +1673,7 @@ Gemm mk(const float* A, long long lda, const float* B, long long ldb, float* C, 
   std::memset(&g, 0, sizeof(g));
   g.A = A; g.lda = lda; g.B = B; g.ldb = ldb; g.C = C; g.ldc = ldc;
   g.M = M; g.N = N; g.K = K; g.kchunk = K; g.epi = epi;
+  g.ldr = ldc;
   return g;
 }
 
@@ -1391,9 +1683,10 @@ cudaError_t reduce(const float* part, int nparts, long long len, long long strid
 }
 
 // dW[o][i] = sum_r dOut[r][o] In[r][i] and db[o] = sum_r dOut[r][o] over rows
-// r, split along the rows into partial slabs summed in order.
-cudaError_t wgrad(ut_tfm* t, const float* dOut, int n_o, const float* In, int n_i, long long rows, float* gW,
-                  float* gb, cudaStream_t s) {
+// r (rows of In ldi apart), split along the rows into partial slabs summed in
+// order.
+cudaError_t wgrad(ut_tfm* t, const float* dOut, int n_o, const float* In, long long ldi, int n_i, long long rows,
+                  float* gW, float* gb, cudaStream_t s) {
   if (t->gemm_tc && rows > 0) {
     // tensor cores: (n_o / 128) x (n_i / 256) tiles x row splits, about as
     // many CTAs per SM as fit (three for n_i <= 128, else two), each split a
@@ -1411,7 +1704,7 @@ cudaError_t wgrad(ut_tfm* t, const float* dOut, int n_o, const float* In, int n_
     long long rc = (rows + splits - 1) / splits;
     rc = (rc + kTcChunk - 1) / kTcChunk * kTcChunk;
     splits = (rows + rc - 1) / rc;
-    Gemm g = mk(dOut, n_o, In, n_i, t->part, n_i, n_o, n_i, rows, EPI_PARTIAL);
+    Gemm g = mk(dOut, n_o, In, ldi, t->part, n_i, n_o, n_i, rows, EPI_PARTIAL);
     g.kchunk = rc;
     g.status = t->status;
     dim3 grid((unsigned)((n_o + 127) / 128), (unsigned)((n_i + kTcMaxN - 1) / kTcMaxN), (unsigned)splits);
@@ -1422,7 +1715,7 @@ cudaError_t wgrad(ut_tfm* t, const float* dOut, int n_o, const float* In, int n_
     if (e == cudaSuccess) e = reduce(bias_part, (int)splits, n_o, n_o, gb, s);
     return e;
   }
-  Gemm g = mk(dOut, n_o, In, n_i, t->part, n_i, n_o, n_i, rows, EPI_PARTIAL);
+  Gemm g = mk(dOut, n_o, In, ldi, t->part, n_i, n_o, n_i, rows, EPI_PARTIAL);
   const long long tiles = (long long)((n_o + 63) / 64) * ((n_i + 63) / 64);
   long long splits = (608 + tiles - 1) / tiles;
   splits = splits < 1 ? 1 : (splits > 128 ? 128 : splits);
@@ -1452,11 +1745,11 @@ cudaError_t ln_fwd(const float* X, const float* g, const float* b, float* Y, flo
   return cudaGetLastError();
 }
 
-template <int DJ>
+template <int DJ, bool REC>
 cudaError_t ln_bwd(ut_tfm* t, const float* dY, const float* X, const float* st, const float* g, const float* base,
-                   float* out, float* grad_gb, long long rows, cudaStream_t s) {
-  static const int nblk = (int)std::min<long long>(kLnBlocks, resident_blocks(ln_bwd_kernel<DJ>, 256));
-  ln_bwd_kernel<DJ><<<nblk, 256, 0, s>>>(dY, X, st, g, base, out, t->part, rows);
+                   float* out, float* grad_gb, long long rows, cudaStream_t s, const float* dY0 = nullptr) {
+  static const int nblk = (int)std::min<long long>(kLnBlocks, resident_blocks(ln_bwd_kernel<DJ, REC>, 256));
+  ln_bwd_kernel<DJ, REC><<<nblk, 256, 0, s>>>(dY, X, st, g, base, out, t->part, rows, dY0, (unsigned)t->T);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = reduce(t->part, nblk, 2 * 32 * DJ, 2 * 32 * DJ, grad_gb, s);
   return e;
@@ -1489,6 +1782,32 @@ cudaError_t attn_bwd(const float* QKV, const float* P, const float* dO, float* d
   return cudaGetLastError();
 }
 
+// The last block's attention (recurrent queries).  KV, Q0 and dO0 are the
+// handle's buffers at multiples of 32 floats: every float4 access is aligned.
+template <int DH>
+cudaError_t attn0_fwd(const float* Q0, const float* KV, const int32_t* ne, const int32_t* sel, float* P0, float* O0,
+                      long long n, int T, int NS, int H, bool mma, cudaStream_t s) {
+  const float scale = 1.0f / sqrtf((float)DH);
+  const unsigned grid = blocks_for(n * H * 32, 256);
+  if (mma && DH == 16 && T <= 16)
+    attn0_fwd_mma_kernel<<<grid, 256, 0, s>>>(Q0, KV, ne, sel, P0, O0, n, T, NS, H, scale);
+  else
+    attn0_fwd_kernel<DH><<<grid, 256, 0, s>>>(Q0, KV, ne, sel, P0, O0, n, T, NS, H, scale);
+  return cudaGetLastError();
+}
+
+template <int DH>
+cudaError_t attn0_bwd(const float* Q0, const float* KV, const float* P0, const float* dO0, float* dQ0, float* dKV,
+                      long long n, int T, int H, bool mma, cudaStream_t s) {
+  const float scale = 1.0f / sqrtf((float)DH);
+  const unsigned grid = blocks_for(n * H * 32, 256);
+  if (mma && DH == 16 && T <= 16)
+    attn0_bwd_mma_kernel<<<grid, 256, 0, s>>>(Q0, KV, P0, dO0, dQ0, dKV, n, T, H, scale);
+  else
+    attn0_bwd_kernel<DH><<<grid, 256, 0, s>>>(Q0, KV, P0, dO0, dQ0, dKV, n, T, H, scale);
+  return cudaGetLastError();
+}
+
 struct Call {
   const void* tok;
   const int32_t* ne;
@@ -1496,6 +1815,29 @@ struct Call {
   const int32_t* sel;
   long long n;
 };
+
+// Activations of block l (the last block's lie behind the others'; its QKV
+// holds KV, and Q0 follows it).
+struct Block {
+  float *X, *Y1, *Y2, *S1, *S2, *QKV, *Q0, *P, *O, *M, *Z, *G;
+};
+Block block_of(const ut_tfm* t, int l) {
+  const long long MR = t->max_rows, d = t->d;
+  Block b;
+  b.X = t->X + l * MR * d;
+  b.Y1 = t->Y1 + l * MR * d;
+  b.Y2 = t->Y2 + l * MR * d;
+  b.S1 = t->S1 + l * MR * 2;
+  b.S2 = t->S2 + l * MR * 2;
+  b.QKV = t->QKV + l * MR * 3 * d;
+  b.Q0 = b.QKV + MR * 2 * d;
+  b.P = t->P + (long long)l * t->cfg.max_batch * t->H * t->T * t->T;
+  b.O = t->O + l * MR * d;
+  b.M = t->M + l * MR * d;
+  b.Z = t->Z + l * MR * 4 * d;
+  b.G = t->G + l * MR * 4 * d;
+  return b;
+}
 
 template <int DJ, int DH, typename TokT>
 cudaError_t forward(ut_tfm* t, const Call& c, cudaStream_t s) {
@@ -1525,50 +1867,46 @@ cudaError_t forward(ut_tfm* t, const Call& c, cudaStream_t s) {
       embed_kernel<TokT, 4><<<blocks, 256, 0, s>>>(tk, c.ne, c.h, c.sel, w + o[0], w + o[1], t->X, c.n, t->T, t->NS);
   }
   cudaError_t e = cudaGetLastError();
+  auto gemm0 = [&](Gemm g, int bias, const uint16_t* bimg) {
+    g.bias = w + bias;
+    g.bimg = bimg;
+    g.status = t->status;
+    return gemm(0, g, s);
+  };
   for (int l = 0; l < t->L && e == cudaSuccess; ++l) {
     const int64_t* ol = o.data() + 2 + 12 * l;
-    float* Xl = t->X + l * MR * d;
-    float* Xn = t->X + (l + 1) * MR * d;
-    float* Y1 = t->Y1 + l * MR * d;
-    float* Y2 = t->Y2 + l * MR * d;
-    float* S1 = t->S1 + l * MR * 2;
-    float* S2 = t->S2 + l * MR * 2;
-    float* QKV = t->QKV + l * MR * 3 * d;
-    float* P = t->P + (long long)l * t->cfg.max_batch * t->H * t->T * t->T;
-    float* O = t->O + l * MR * d;
-    float* M = t->M + l * MR * d;
-    float* Z = t->Z + l * MR * 4 * d;
-    float* G = t->G + l * MR * 4 * d;
-    e = ln_fwd<DJ>(Xl, w + ol[T_LN1G], w + ol[T_LN1B], Y1, S1, rows, s);
+    const bool last = l == t->L - 1;
+    const long long m = last ? c.n : rows;  // rows after the attention: the recurrent tokens alone in the last block
+    const Block b = block_of(t, l);
+    e = ln_fwd<DJ>(b.X, w + ol[T_LN1G], w + ol[T_LN1B], b.Y1, b.S1, rows, s);
     if (e != cudaSuccess) break;
-    Gemm g = mk(Y1, d, w + ol[T_WQKV], d, QKV, 3 * d, rows, 3 * d, d, EPI_BIAS);
-    g.bias = w + ol[T_BQKV];
-    g.bimg = img(l, 0);
-    g.status = t->status;
-    e = gemm(0, g, s);
-    if (e == cudaSuccess) e = attn_fwd<DH>(QKV, c.ne, c.sel, P, O, c.n, t->T, t->NS, t->H, t->gemm_tc != 0, s);
+    if (last) {
+      e = gemm0(mk(b.Y1, d, w + ol[T_WQKV] + d * d, d, b.QKV, 2 * d, rows, 2 * d, d, EPI_BIAS), ol[T_BQKV] + d,
+                img(l, 0));
+      if (e == cudaSuccess)  // the recurrent rows of Y1 are T d apart
+        e = gemm0(mk(b.Y1, (long long)t->T * d, w + ol[T_WQKV], d, b.Q0, d, c.n, d, d, EPI_BIAS), ol[T_BQKV],
+                  img(t->L, 0));
+      if (e == cudaSuccess)
+        e = attn0_fwd<DH>(b.Q0, b.QKV, c.ne, c.sel, b.P, b.O, c.n, t->T, t->NS, t->H, t->gemm_tc != 0, s);
+    } else {
+      e = gemm0(mk(b.Y1, d, w + ol[T_WQKV], d, b.QKV, 3 * d, rows, 3 * d, d, EPI_BIAS), ol[T_BQKV], img(l, 0));
+      if (e == cudaSuccess)
+        e = attn_fwd<DH>(b.QKV, c.ne, c.sel, b.P, b.O, c.n, t->T, t->NS, t->H, t->gemm_tc != 0, s);
+    }
     if (e != cudaSuccess) break;
-    g = mk(O, d, w + ol[T_WO], d, M, d, rows, d, d, EPI_BIAS_RES);
-    g.bias = w + ol[T_BO];
-    g.R = Xl;
-    g.bimg = img(l, 1);
-    g.status = t->status;
-    e = gemm(0, g, s);
-    if (e == cudaSuccess) e = ln_fwd<DJ>(M, w + ol[T_LN2G], w + ol[T_LN2B], Y2, S2, rows, s);
+    Gemm g = mk(b.O, d, w + ol[T_WO], d, b.M, d, m, d, d, EPI_BIAS_RES);
+    g.R = b.X;
+    g.ldr = last ? (long long)t->T * d : d;
+    e = gemm0(g, ol[T_BO], img(l, 1));
+    if (e == cudaSuccess) e = ln_fwd<DJ>(b.M, w + ol[T_LN2G], w + ol[T_LN2B], b.Y2, b.S2, m, s);
     if (e != cudaSuccess) break;
-    g = mk(Y2, d, w + ol[T_W1], d, Z, 4 * d, rows, 4 * d, d, EPI_BIAS_GELU);
-    g.bias = w + ol[T_B1];
-    g.C2 = G;
-    g.bimg = img(l, 2);
-    g.status = t->status;
-    e = gemm(0, g, s);
+    g = mk(b.Y2, d, w + ol[T_W1], d, b.Z, 4 * d, m, 4 * d, d, EPI_BIAS_GELU);
+    g.C2 = b.G;
+    e = gemm0(g, ol[T_B1], img(l, 2));
     if (e != cudaSuccess) break;
-    g = mk(G, 4 * d, w + ol[T_W2], 4 * d, Xn, d, rows, d, 4 * d, EPI_BIAS_RES);
-    g.bias = w + ol[T_B2];
-    g.R = M;
-    g.bimg = img(l, 3);
-    g.status = t->status;
-    e = gemm(0, g, s);
+    g = mk(b.G, 4 * d, w + ol[T_W2], 4 * d, b.X + MR * d, d, m, d, 4 * d, EPI_BIAS_RES);
+    g.R = b.M;
+    e = gemm0(g, ol[T_B2], img(l, 3));
   }
   return e;
 }
@@ -1576,7 +1914,7 @@ cudaError_t forward(ut_tfm* t, const Call& c, cudaStream_t s) {
 template <int DJ, int DH, typename TokT>
 cudaError_t backward(ut_tfm* t, const Call& c, float* grad, cudaStream_t s) {
   constexpr int d = 32 * DJ;
-  const long long rows = c.n * t->T, MR = t->max_rows;
+  const long long rows = c.n * t->T;
   const float* w = t->prm;
   const auto& o = t->off;
   cudaError_t e = cudaSuccess;
@@ -1588,32 +1926,42 @@ cudaError_t backward(ut_tfm* t, const Call& c, float* grad, cudaStream_t s) {
   };
   for (int l = t->L - 1; l >= 0 && e == cudaSuccess; --l) {
     const int64_t* ol = o.data() + 2 + 12 * l;
-    const float* Xl = t->X + l * MR * d;
-    const float* Y1 = t->Y1 + l * MR * d;
-    const float* Y2 = t->Y2 + l * MR * d;
-    const float* S1 = t->S1 + l * MR * 2;
-    const float* S2 = t->S2 + l * MR * 2;
-    const float* QKV = t->QKV + l * MR * 3 * d;
-    const float* P = t->P + (long long)l * t->cfg.max_batch * t->H * t->T * t->T;
-    const float* O = t->O + l * MR * d;
-    const float* M = t->M + l * MR * d;
-    const float* Z = t->Z + l * MR * 4 * d;
-    const float* G = t->G + l * MR * 4 * d;
+    const bool last = l == t->L - 1;
+    const long long m = last ? c.n : rows;
+    const Block b = block_of(t, l);
     // feed-forward sub-block: X' = M + W2 gelu(W1 LN2(M) + b1) + b2
-    Gemm g = mk(t->dX, d, w + ol[T_W2], 4 * d, t->dBig, 4 * d, rows, 4 * d, d, EPI_GELU_GRAD);
-    g.aux = Z;
+    Gemm g = mk(t->dX, d, w + ol[T_W2], 4 * d, t->dBig, 4 * d, m, 4 * d, d, EPI_GELU_GRAD);
+    g.aux = b.Z;
     e = dgemm(l, 7, g);
-    if (e == cudaSuccess) e = wgrad(t, t->dX, d, G, 4 * d, rows, grad + ol[T_W2], grad + ol[T_B2], s);
-    if (e == cudaSuccess) e = dgemm(l, 6, mk(t->dBig, 4 * d, w + ol[T_W1], d, t->dY, d, rows, d, 4 * d, EPI_STORE));
-    if (e == cudaSuccess) e = wgrad(t, t->dBig, 4 * d, Y2, d, rows, grad + ol[T_W1], grad + ol[T_B1], s);
-    if (e == cudaSuccess) e = ln_bwd<DJ>(t, t->dY, M, S2, w + ol[T_LN2G], t->dX, t->dM, grad + ol[T_LN2G], rows, s);
+    if (e == cudaSuccess) e = wgrad(t, t->dX, d, b.G, 4 * d, 4 * d, m, grad + ol[T_W2], grad + ol[T_B2], s);
+    if (e == cudaSuccess) e = dgemm(l, 6, mk(t->dBig, 4 * d, w + ol[T_W1], d, t->dY, d, m, d, 4 * d, EPI_STORE));
+    if (e == cudaSuccess) e = wgrad(t, t->dBig, 4 * d, b.Y2, d, d, m, grad + ol[T_W1], grad + ol[T_B1], s);
+    if (e == cudaSuccess)
+      e = ln_bwd<DJ, false>(t, t->dY, b.M, b.S2, w + ol[T_LN2G], t->dX, t->dM, grad + ol[T_LN2G], m, s);
     // attention sub-block: M = X + Wo attn(LN1(X)) + bo
-    if (e == cudaSuccess) e = dgemm(l, 5, mk(t->dM, d, w + ol[T_WO], d, t->dO, d, rows, d, d, EPI_STORE));
-    if (e == cudaSuccess) e = wgrad(t, t->dM, d, O, d, rows, grad + ol[T_WO], grad + ol[T_BO], s);
-    if (e == cudaSuccess) e = attn_bwd<DH>(QKV, P, t->dO, t->dBig, c.n, t->T, t->H, t->gemm_tc != 0, s);
+    if (e == cudaSuccess) e = dgemm(l, 5, mk(t->dM, d, w + ol[T_WO], d, t->dO, d, m, d, d, EPI_STORE));
+    if (e == cudaSuccess) e = wgrad(t, t->dM, d, b.O, d, d, m, grad + ol[T_WO], grad + ol[T_BO], s);
+    if (e != cudaSuccess) break;
+    if (last) {
+      // dQ0 in dX, then its product with Wq in dO (both are free by then)
+      const float* Wq = w + ol[T_WQKV];
+      e = attn0_bwd<DH>(b.Q0, b.QKV, b.P, t->dO, t->dX, t->dBig, c.n, t->T, t->H, t->gemm_tc != 0, s);
+      if (e == cudaSuccess)
+        e = dgemm(l, 4, mk(t->dBig, 2 * d, Wq + d * d, d, t->dY, d, rows, d, 2 * d, EPI_STORE));
+      if (e == cudaSuccess) e = dgemm(t->L, 1, mk(t->dX, d, Wq, d, t->dO, d, c.n, d, d, EPI_STORE));
+      if (e == cudaSuccess)
+        e = wgrad(t, t->dBig, 2 * d, b.Y1, d, d, rows, grad + ol[T_WQKV] + d * d, grad + ol[T_BQKV] + d, s);
+      if (e == cudaSuccess)
+        e = wgrad(t, t->dX, d, b.Y1, (long long)t->T * d, d, c.n, grad + ol[T_WQKV], grad + ol[T_BQKV], s);
+      if (e == cudaSuccess)
+        e = ln_bwd<DJ, true>(t, t->dY, b.X, b.S1, w + ol[T_LN1G], t->dM, t->dX, grad + ol[T_LN1G], rows, s, t->dO);
+      continue;
+    }
+    e = attn_bwd<DH>(b.QKV, b.P, t->dO, t->dBig, c.n, t->T, t->H, t->gemm_tc != 0, s);
     if (e == cudaSuccess) e = dgemm(l, 4, mk(t->dBig, 3 * d, w + ol[T_WQKV], d, t->dY, d, rows, d, 3 * d, EPI_STORE));
-    if (e == cudaSuccess) e = wgrad(t, t->dBig, 3 * d, Y1, d, rows, grad + ol[T_WQKV], grad + ol[T_BQKV], s);
-    if (e == cudaSuccess) e = ln_bwd<DJ>(t, t->dY, Xl, S1, w + ol[T_LN1G], t->dM, t->dX, grad + ol[T_LN1G], rows, s);
+    if (e == cudaSuccess) e = wgrad(t, t->dBig, 3 * d, b.Y1, d, d, rows, grad + ol[T_WQKV], grad + ol[T_BQKV], s);
+    if (e == cudaSuccess)
+      e = ln_bwd<DJ, false>(t, t->dY, b.X, b.S1, w + ol[T_LN1G], t->dM, t->dX, grad + ol[T_LN1G], rows, s);
   }
   if (e != cudaSuccess) return e;
   embed_grad_kernel<TokT, DJ><<<kRowBlocks, 256, 0, s>>>((const TokT*)c.tok, c.ne, c.sel, t->dX, t->part, c.n, t->T,
@@ -1635,7 +1983,6 @@ cudaError_t run(ut_tfm* t, const Call& c, int mode, const HeadArgs& ha_in, float
   HeadArgs ha = ha_in;
   ha.XL = t->X + (long long)t->L * t->max_rows * d;
   ha.n = c.n;
-  ha.T = t->T;
   ha.n_out = t->n_out;
   ha.mode = mode;
   ha.lnf_g = t->prm + o[idx];
@@ -1770,17 +2117,18 @@ extern "C" ut_status tfm_create(const ut_tfm_config* cfg, const float* params_ho
   t->prm = A(n_params);
   t->am = A(n_params);
   t->av = A(n_params);
-  t->X = A((L + 1) * R * d);
+  const size_t B = (size_t)cfg->max_batch, RL = (L - 1) * R + B;  // rows kept after the attention, all blocks
+  t->X = A((L * R + B) * d);
   t->Y1 = A(L * R * d);
-  t->Y2 = A(L * R * d);
+  t->Y2 = A(RL * d);
   t->S1 = A(L * R * 2);
-  t->S2 = A(L * R * 2);
-  t->QKV = A(L * R * 3 * d);
-  t->P = A(L * Pn);
-  t->O = A(L * R * d);
-  t->M = A(L * R * d);
-  t->Z = A(L * R * 4 * d);
-  t->G = A(L * R * 4 * d);
+  t->S2 = A(RL * 2);
+  t->QKV = A(((L - 1) * R * 3 + R * 2 + B) * d);
+  t->P = A((L - 1) * Pn + B * t->H * t->T);
+  t->O = A(RL * d);
+  t->M = A(RL * d);
+  t->Z = A(RL * 4 * d);
+  t->G = A(RL * 4 * d);
   t->dX = A(R * d);
   t->dM = A(R * d);
   t->dY = A(R * d);
@@ -1795,22 +2143,24 @@ extern "C" ut_status tfm_create(const ut_tfm_config* cfg, const float* params_ho
   std::vector<int64_t> spec;
   int64_t img_total = 0;
   t->img_max = 0;
+  auto add_img = [&](int64_t woff, int rows_w, int cols_w, int tr) {
+    const int R = tr ? cols_w : rows_w, C = tr ? rows_w : cols_w;
+    // each 256-row block holds C columns of 256 rows (the last block padded)
+    t->img_off.push_back(img_total);
+    spec.insert(spec.end(), {woff, (int64_t)R, (int64_t)C, (int64_t)tr, img_total});
+    img_total += (int64_t)((R + kTcMaxN - 1) / kTcMaxN) * kTcMaxN * C;
+    t->img_max = std::max(t->img_max, R * C);
+  };
   for (int l = 0; l < t->L; ++l) {
     const int64_t* ol = t->off.data() + 2 + 12 * l;
-    const int64_t woff[4] = {ol[T_WQKV], ol[T_WO], ol[T_W1], ol[T_W2]};
-    const int rows_w[4] = {3 * t->d, t->d, 4 * t->d, t->d}, cols_w[4] = {t->d, t->d, t->d, 4 * t->d};
+    const bool last = l == t->L - 1;  // (Wk and Wv: rows d .. 3d - 1 of Wqkv)
+    const int64_t woff[4] = {ol[T_WQKV] + (last ? (int64_t)t->d * t->d : 0), ol[T_WO], ol[T_W1], ol[T_W2]};
+    const int rows_w[4] = {(last ? 2 : 3) * t->d, t->d, 4 * t->d, t->d}, cols_w[4] = {t->d, t->d, t->d, 4 * t->d};
     for (int tr = 0; tr < 2; ++tr)
-      for (int k = 0; k < 4; ++k) {
-        const int R = tr ? cols_w[k] : rows_w[k], C = tr ? rows_w[k] : cols_w[k];
-        // each 256-row block holds C columns of 256 rows (the last block padded)
-        const int64_t n = (int64_t)((R + kTcMaxN - 1) / kTcMaxN) * kTcMaxN * C;
-        t->img_off.push_back(img_total);
-        spec.insert(spec.end(), {woff[k], (int64_t)R, (int64_t)C, (int64_t)tr, img_total});
-        img_total += n;
-        t->img_max = std::max(t->img_max, R * C);
-      }
+      for (int k = 0; k < 4; ++k) add_img(woff[k], rows_w[k], cols_w[k], tr);
   }
-  t->n_img = 8 * t->L;
+  for (int tr = 0; tr < 2; ++tr) add_img(t->off[2 + 12 * (t->L - 1) + T_WQKV], t->d, t->d, tr);
+  t->n_img = 8 * t->L + 2;
   t->wimg = (uint16_t*)dalloc(t, (size_t)img_total * 2);
   t->img_spec = (int64_t*)dalloc(t, spec.size() * 8);
   t->status = (int*)dalloc(t, 4);

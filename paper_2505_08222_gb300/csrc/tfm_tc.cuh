@@ -62,7 +62,7 @@ __device__ __forceinline__ void epi_store4(const Gemm& g, long long m, int n, fl
     }
     case EPI_BIAS_RES: {
       const float4 b = *reinterpret_cast<const float4*>(g.bias + n);
-      const float4 q = *reinterpret_cast<const float4*>(g.R + o);
+      const float4 q = *reinterpret_cast<const float4*>(g.R + m * g.ldr + n);
       r = make_float4(v.x + b.x + q.x, v.y + b.y + q.y, v.z + b.z + q.z, v.w + b.w + q.w);
       break;
     }
