@@ -118,6 +118,7 @@ class Env:
         flags = (_abi.UT_FLAG_DEBUG if debug else 0) | (_abi.UT_FLAG_RING if ring else 0)
         self._cfg, self._keep = make_config(params, flags)
         self._stream = _stream_ptr(stream)
+        self._views = (None, None)  # step buffers' pointers and their views
         self._alloc = _TorchAllocator() if use_torch_allocator else None
         h = ctypes.c_void_p()
         rc = lib.env_create(ctypes.byref(self._cfg),
@@ -161,10 +162,23 @@ class Env:
             assert actions.numel() == self.NA
             ptr = ctypes.c_void_p(actions.data_ptr())
         out = _abi.StepOut()
-        _check(lib.env_step(self.h, ptr, ctypes.byref(out)), self.h, "env_step")
+        rc = lib.env_step(self.h, ptr, ctypes.byref(out))
+        if rc:
+            _check(rc, self.h, "env_step")
         return self._step_views(out)
 
     def _step_views(self, out) -> dict:
+        # A handle's step buffers stay where they are until it is destroyed
+        # (the logits appear once it has a policy), so their views are made on
+        # the first step: the eight of them cost about 70 us of host time, the
+        # small fleet's step 16 us of device time (87 us a step with views
+        # made each time, 15.5 us now).
+        key = bytes(out)
+        if self._views[0] != key:
+            self._views = (key, self._make_step_views(out))
+        return dict(self._views[1])
+
+    def _make_step_views(self, out) -> dict:
         return {
             "reward": device_view(out.reward, (self.E,)),
             "done": device_view(out.done, (self.E,), torch.int32),
