@@ -17,8 +17,17 @@ bool pf_variant_valid(int v, int P) {
 }
 
 int pf_default_variant(int P) {
-  // smallest 4-particles-per-thread block that covers P (variants 0..5)
-  for (int v = 0; v < 6; ++v)
+  // The smallest 4-particles-per-thread block that covers P, in its form with
+  // the most resident warps: those hide each other's barriers and loads, and
+  // the register caps cost no spills.  Filter launch over 100 M particles,
+  // before -> after: P = 64 2680 -> 1946 us, 128 1342 -> 928, 256 885 -> 778,
+  // 512 849 -> 688, 1000 1011 -> 823, 1024 935 -> 708, 1500 1481 -> 1137, 2048
+  // 1078 -> 815; over 64 filters the forms are equal (8.0-11.2 us).  They give the same bits.  Above 2048, 8 particles per
+  // thread are faster on large batches (4096: 1370 -> 1164 us) but round the
+  // estimate's sums in another order and lose on few filters (13.2 -> 17.2 us),
+  // so those stay with the autotuner.
+  constexpr int kBySize[] = {15, 16, 6, 7, 8, 5};
+  for (int v : kBySize)
     if (pf::kVariants[v].nt * 4 >= P) return v;
   return 5;
 }

@@ -13,7 +13,8 @@ struct Variant {
   const char* name;
 };
 
-// X(index, NT, PPT, MINB); the first six are the defaults for P <= 128 .. 4096.
+// X(index, NT, PPT, MINB, name).  Variants of one NT x PPT give the same bits
+// (MINB only caps the registers).
 #define UT_PF_VARIANTS_A(X)             \
   X(0, 32, 4, 16, "nt32x4")            \
   X(1, 64, 4, 16, "nt64x4")            \
@@ -30,7 +31,9 @@ struct Variant {
   X(11, 256, 8, 4, "nt256x8")          \
   X(12, 512, 8, 2, "nt512x8")          \
   X(13, 256, 8, 3, "nt256x8m3")        \
-  X(14, 128, 8, 6, "nt128x8m6")
+  X(14, 128, 8, 6, "nt128x8m6")        \
+  X(15, 32, 4, 32, "nt32x4m32")        \
+  X(16, 64, 4, 24, "nt64x4m24")
 
 #define UT_PF_ENTRY(i, nt, ppt, minb, name) {nt, ppt, minb, name},
 constexpr Variant kVariants[] = {UT_PF_VARIANTS_A(UT_PF_ENTRY) UT_PF_VARIANTS_B(UT_PF_ENTRY)};
