@@ -2,9 +2,8 @@
 // input-gradient pass, weight-gradient pass, Adam, feature recording.
 //
 // All three hidden layers run on the tensor cores (tcgen05.mma, BF16 x BF16 ->
-// FP32 in TMEM) with 128 rows per CTA: one thread per row in the epilogues of
-// the training / stand-alone forward, four per row in the environment step's
-// forward (fwd_env_kernel).  The first layer's inputs are FP32 features split into a BF16
+// FP32 in TMEM) with 128 rows per CTA, four threads per row in the epilogues.
+// The first layer's inputs are FP32 features split into a BF16
 // high part and a BF16 remainder that are multiplied by the same weights and
 // accumulated together: ranges of hundreds of metres keep ~1e-5 relative
 // precision instead of BF16's 4e-3, which matters for metre-level tracking.
@@ -23,8 +22,8 @@ namespace {
 constexpr int kT = 128;
 constexpr uint32_t TAG_BATCH = 14;
 constexpr float kMaxCorr = 3.0f;  // largest correction per step, in units of L
-constexpr size_t kFwdSmem = 65536 + 65536;
-constexpr size_t kWgradSmem = 32768 + 65536;
+constexpr size_t kImgA = (size_t)kT * HID * 2;  // one tile's operand image [HID / 8][128 rows][8] (64 KB)
+constexpr size_t kImgX = (size_t)kT * IN * 2;   // of the features (24 KB)
 
 // Derivative of erf-GELU for the backward pass: Phi(x) + x phi(x).  (The
 // forward passes evaluate GELU with gelu.cuh's form, within 5.4e-6 of the
@@ -40,12 +39,6 @@ __device__ __forceinline__ void store8(unsigned char* img, int row, int k0, int 
   p.z = bf16x2_bits(v[4], v[5]);
   p.w = bf16x2_bits(v[6], v[7]);
   *reinterpret_cast<uint4*>(img + tc::kmajor_offset(row, k0, rows)) = p;
-}
-
-__device__ __forceinline__ void copy_img(unsigned char* dst, const unsigned char* __restrict__ src, size_t bytes) {
-  const uint4* s = reinterpret_cast<const uint4*>(src);
-  uint4* t = reinterpret_cast<uint4*>(dst);
-  for (size_t i = threadIdx.x; i < bytes / 16; i += kT) t[i] = __ldg(s + i);
 }
 
 // Estimator features of filter f for its update at step g (reading C18):
@@ -81,128 +74,6 @@ __device__ __forceinline__ void ring_features(const EnvDev& d, int f, uint32_t g
   x[5 * kRing + 3] = vy / L;
 #pragma unroll
   for (int i = 5 * kRing + 4; i < IN; ++i) x[i] = 0.0f;
-}
-
-struct FwdArgs {
-  Net net;
-  const float* X;
-  const int32_t* rows;
-  int B;
-  float* out;
-  float* z;     // training: [3][B][256], else NULL
-  uint16_t* a;  // training: [3][B][256], else NULL
-  int* status;
-};
-
-__global__ void __launch_bounds__(kT, 1) fwd_kernel(FwdArgs p) {
-  extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* sA = smem;          // features hi | lo, then hidden activations [128 x 256]
-  unsigned char* sB = smem + 65536;  // one weight chunk [128 x K]
-  __shared__ __align__(8) uint64_t mbar;
-  __shared__ uint32_t tbase;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const long long b = (long long)blockIdx.x * kT + tid;
-  const long long n = (long long)p.B;
-  const bool valid = b < n;
-
-  if (warp == 0) {
-    tc::tmem_alloc(&tbase, 256);
-    tc::tmem_relinquish();
-  }
-  if (tid == 0) tc::mbar_init(&mbar, 1);
-
-  float x[IN];
-  {
-    const long long src = valid ? (p.rows ? (long long)p.rows[b] : b) : 0;
-#pragma unroll
-    for (int i = 0; i < IN; i += 4) {
-      float4 v = valid ? __ldg(reinterpret_cast<const float4*>(p.X + src * IN + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
-      x[i] = v.x; x[i + 1] = v.y; x[i + 2] = v.z; x[i + 3] = v.w;
-    }
-  }
-#pragma unroll
-  for (int c0 = 0; c0 < IN; c0 += 8) {
-    float hi[8], lo[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      hi[i] = bf_bits2f(f2bf_bits(x[c0 + i]));
-      lo[i] = x[c0 + i] - hi[i];
-    }
-    store8(sA, tid, c0, 128, hi);
-    store8(sA + 128 * IN * 2, tid, c0, 128, lo);
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = tbase;
-  const uint32_t lane = tmem + ((uint32_t)(warp * 32) << 16);
-  const uint32_t aA = tc::smem_addr(sA), aB = tc::smem_addr(sB);
-  uint32_t phase = 0;
-  bool ok = true;
-  const float* mst = p.net.master;
-
-  // layer 1: K = 96, both halves of the features, two N-halves of 128
-  {
-    const uint32_t a2[2] = {aA, aA + 128 * IN * 2};
-    for (int h = 0; h < 2; ++h) {
-      copy_img(sB, p.net.img + IMG_W1_OFF + (size_t)h * 128 * IN * 2, (size_t)128 * IN * 2);
-      ok &= tc::mma_group(tmem + 128 * h, a2, 2, aB, 128, IN, false, &mbar, phase);
-    }
-  }
-  float o0 = 0.0f, o1 = 0.0f;
-  for (int l = 0; l < 3; ++l) {
-    // epilogue of hidden layer l: z = acc + b, a = GELU(z) -> next A operand
-    const float* bias = mst + (l == 0 ? B1_OFF : (l == 1 ? B2_OFF : B3_OFF));
-#pragma unroll 1
-    for (int c0 = 0; c0 < HID; c0 += 16) {
-      float v[16];
-      tc::tmem_ld16(lane + c0, v);
-      float av[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        v[i] += __ldg(bias + c0 + i);
-        av[i] = v[i];
-      }
-#pragma unroll
-      for (int i = 0; i < 16; i += 2) gelu2(av[i], av[i + 1]);  // same GELU as the environment step
-      if (p.z && valid) {
-        float* zr = p.z + ((long long)l * p.B + b) * HID + c0;
-        uint16_t* ar = p.a + ((long long)l * p.B + b) * HID + c0;
-#pragma unroll
-        for (int i = 0; i < 16; i += 4) *reinterpret_cast<float4*>(zr + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-#pragma unroll
-        for (int i = 0; i < 16; i += 2)
-          *reinterpret_cast<uint32_t*>(ar + i) = bf16x2_bits(av[i], av[i + 1]);
-      }
-      if (l < 2) {
-        store8(sA, tid, c0, 128, av);
-        store8(sA, tid, c0 + 8, 128, av + 8);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          o0 = fmaf(__ldg(mst + W4_OFF + c0 + i), av[i], o0);
-          o1 = fmaf(__ldg(mst + W4_OFF + HID + c0 + i), av[i], o1);
-        }
-      }
-    }
-    if (l < 2) {
-      const size_t base = l == 0 ? IMG_W2_OFF : IMG_W3_OFF;
-      for (int h = 0; h < 2; ++h) {
-        copy_img(sB, p.net.img + base + (size_t)h * 128 * HID * 2, (size_t)128 * HID * 2);
-        ok &= tc::mma_group(tmem + 128 * h, &aA, 1, aB, 128, HID, false, &mbar, phase);
-      }
-    }
-  }
-  o0 += __ldg(mst + B4_OFF);
-  o1 += __ldg(mst + B4_OFF + 1);
-  if (valid && ok) {
-    p.out[b * OUT] = o0;
-    p.out[b * OUT + 1] = o1;
-  }
-  if (!ok && tid == 0) raise_status(p.status, 2);
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, 256);
 }
 
 // ---------------------------------------------------------------------------
@@ -429,158 +300,430 @@ __global__ void __launch_bounds__(kTE, 1) fwd_env_kernel(Net net, EnvDev d, int 
 }
 
 // ---------------------------------------------------------------------------
-// Input-gradient pass: dz3, dz2, dz1 (BF16, for the weight gradients), bias
-// gradients and the output layer's gradients; loss.
+// The network on feature rows: forward (est_forward), and in training also
+// the loss, the input-gradient pass and the sums that need no contraction.
+// One CTA of 512 threads per 128 rows, thread = row x one of 4 column parts,
+// weights as in fwd_env_kernel (the transposed W3 and W2 follow as stages
+// 6 .. 9).  Training keeps what the weight gradients contract as BF16 operand
+// images in HBM (features, a1, a2 and dz1 .. dz3 of each tile, written with
+// 16-byte stores, 512 contiguous bytes per warp); z2 and z3 stay in tensor
+// memory until their derivative is needed, z1 goes through HBM.
+//
+// 128 CTAs of a 16,384-row batch are one wave, so the pass is the latency of
+// one tile, 65 us; on one thread per row and kernel, with a five-step warp sum
+// for each of 1,280 columns, the forward took 86 us and the backward 185.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kT, 1) bwd_kernel(Net net, TrainBufs t, int* status) {
+constexpr int kTrainStages = 10;  // W1, W2, W3, W3^T, W2^T, two N-halves each
+
+__device__ __forceinline__ void train_stage(int s, size_t& off, uint32_t& bytes) {
+  if (s < kEnvStages) {
+    env_stage(s, off, bytes);
+  } else {
+    const int h = (s - kEnvStages) & 1;
+    off = (s < kEnvStages + 2 ? IMG_W3T_OFF : IMG_W2T_OFF) + (size_t)h * 128 * HID * 2;
+    bytes = (uint32_t)(128 * HID * 2);
+  }
+}
+
+// Column sums of v[16] over the warp's 32 rows: lane i returns column i % 16
+// (each exchange halves the columns a lane still carries: 16 shuffles instead
+// of five per column).
+__device__ __forceinline__ float colsum16(const float (&v)[16]) {
+  const int lane = threadIdx.x & 31;
+  float a[8], b[4], c[2];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    a[i] = ((lane & 8) ? v[i + 8] : v[i]) + __shfl_xor_sync(0xffffffffu, (lane & 8) ? v[i] : v[i + 8], 8);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    b[i] = ((lane & 4) ? a[i + 4] : a[i]) + __shfl_xor_sync(0xffffffffu, (lane & 4) ? a[i] : a[i + 4], 4);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    c[i] = ((lane & 2) ? b[i + 2] : b[i]) + __shfl_xor_sync(0xffffffffu, (lane & 2) ? b[i] : b[i + 2], 2);
+  const float d = ((lane & 1) ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, (lane & 1) ? c[0] : c[1], 1);
+  return d + __shfl_xor_sync(0xffffffffu, d, 16);
+}
+
+template <bool TRAIN>
+__global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __restrict__ X,
+                                                     const int32_t* __restrict__ rows, int B, float* __restrict__ out,
+                                                     TrainBufs t, int* status) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* sA = smem;
-  unsigned char* sB = smem + 65536;
+  unsigned char* sA = smem;          // features hi | lo, then the current A operand [128 x 256]
+  unsigned char* sW = smem + 65536;  // two weight slots
+  __shared__ __align__(8) uint64_t full[2];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tbase;
-  // per-warp sums, each entry written once by lane 0 of its warp and summed
-  // over the warps in order after the last barrier: dW4, db3, db2, db1, db4
-  __shared__ float s_red[kT / 32][NB_PART];
-  __shared__ double s_loss[kT / 32];
-  const int tid = threadIdx.x, warp = tid >> 5, lanei = tid & 31;
-  const long long b = (long long)blockIdx.x * kT + tid;
-  const bool valid = b < t.B;
-  const long long row = valid ? (t.rows ? (long long)t.rows[b] : b) : 0;
+  __shared__ float sOut[kParts][2][128];
+  __shared__ float s_red[TRAIN ? 4 : 1][TRAIN ? NB_PART : 1];  // column sums of each 32-row quarter
+  __shared__ double s_loss[4];
+  __shared__ int bad;
+  constexpr uint32_t kCols = TRAIN ? 512 : 256;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, row = tid & 127, part = tid >> 7, quarter = warp & 3;
+  const long long b = (long long)blockIdx.x * kT + row;
+  const bool valid = b < B;
+  const long long src = valid ? (rows ? (long long)rows[b] : b) : 0;
+
+  if (warp == 0) {
+    tc::tmem_alloc(&tbase, kCols);
+    tc::tmem_relinquish();
+  }
+  if (tid == 32) {
+    tc::mbar_init(&full[0], 1);
+    tc::mbar_init(&full[1], 1);
+    tc::mbar_init(&mbar, 1);
+    bad = 0;
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = tbase;
+  const uint32_t tl = tmem + ((uint32_t)quarter << 21);  // this warp's lane quarter
+  const uint32_t aA = tc::smem_addr(sA), aW = tc::smem_addr(sW);
+  constexpr int kStages = TRAIN ? kTrainStages : kEnvStages;
+  auto fetch = [&](int st) {  // thread 0: stage st into slot st % 2
+    size_t off;
+    uint32_t bytes;
+    train_stage(st, off, bytes);
+    tc::mbar_expect_tx(&full[st & 1], bytes);
+    tc::bulk_g2s(sW + (st & 1) * kEnvSlot, net.img + off, bytes, &full[st & 1]);
+  };
+  if (tid == 0) {
+    fetch(0);
+    fetch(1);
+  }
+  // features of this row, columns 24 part .. + 23, as BF16 high and low parts
+  {
+    float x[24];
+#pragma unroll
+    for (int i = 0; i < 24; i += 4) {
+      const float4 v = valid ? __ldg(reinterpret_cast<const float4*>(X + src * IN + part * 24 + i))
+                             : make_float4(0.f, 0.f, 0.f, 0.f);
+      x[i] = v.x; x[i + 1] = v.y; x[i + 2] = v.z; x[i + 3] = v.w;
+    }
+#pragma unroll
+    for (int k = 0; k < 24; k += 8) {
+      const int c0 = part * 24 + k;
+      float hi[8], lo[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        hi[i] = bf_bits2f(f2bf_bits(x[k + i]));
+        lo[i] = x[k + i] - hi[i];
+      }
+      store8(sA, row, c0, 128, hi);
+      store8(sA + 128 * IN * 2, row, c0, 128, lo);
+      if (TRAIN) store8(t.x_img + (size_t)blockIdx.x * kImgX, row, c0, 128, hi);
+    }
+  }
+
+  bool ok = true;
+  uint32_t mphase = 0;
+  int stage = 0;
   const float* mst = net.master;
+  // D[128 x 256] at column `col` = A (sA; the hi and lo features of layer 1)
+  // times the next two stages' weights; every thread calls it
+  auto product = [&](uint32_t col, int K, int n_a) {
+    tc::fence_async_smem();
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (tid == 0) {
+      const uint32_t idesc = tc::idesc_bf16(128, 128);
+      for (int h = 0; h < 2; ++h) {
+        ok &= tc::mbar_wait(&full[(stage + h) & 1], (uint32_t)(((stage + h) >> 1) & 1), kEnvPolls);
+        const uint32_t bB = aW + (uint32_t)(((stage + h) & 1) * kEnvSlot);
+        bool acc = false;
+        for (int j = 0; j < n_a; ++j) {
+          const uint32_t a0 = aA + (uint32_t)(j * 128 * IN * 2);
+          for (int k = 0; k < K / 16; ++k) {
+            const uint64_t ad = tc::smem_desc(a0 + k * 2 * 128 * 16, 128 * 16, 128);
+            const uint64_t bd = tc::smem_desc(bB + k * 2 * 128 * 16, 128 * 16, 128);
+            tc::mma_bf16(tmem + col + 128 * h, ad, bd, idesc, acc ? 1u : 0u);
+            acc = true;
+          }
+        }
+      }
+      tc::mma_commit(&mbar);
+    }
+    ok &= tc::mbar_wait(&mbar, mphase, kEnvPolls);
+    mphase ^= 1u;
+    tc::fence_after_sync();
+    stage += 2;
+    if (tid == 0 && stage < kStages) {  // both slots are free again
+      fetch(stage);
+      fetch(stage + 1);
+    }
+  };
+  const int c_lo = part * (HID / kParts), c_hi = c_lo + HID / kParts;
+  constexpr uint32_t kZ2 = TRAIN ? 256 : 0;  // column of layer 2's accumulator (layers 1 and 3: 0)
+  float o0 = 0.0f, o1 = 0.0f;
+  for (int l = 0; l < 3; ++l) {
+    const uint32_t col = l == 1 ? kZ2 : 0u;
+    product(col, l == 0 ? IN : HID, l == 0 ? 2 : 1);
+    const float* bias = mst + (l == 0 ? B1_OFF : (l == 1 ? B2_OFF : B3_OFF));
+#pragma unroll 1
+    for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+      float v[16];
+      tc::tmem_ld16(tl + col + c0, v);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] += __ldg(bias + c0 + i);
+      if (TRAIN && l == 0) {
+        float4* zr = reinterpret_cast<float4*>(t.z + b * HID + c0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) zr[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+      }
+#pragma unroll
+      for (int i = 0; i < 16; i += 2) gelu2(v[i], v[i + 1]);  // erf-GELU, packed pairs
+      if (l < 2) {
+        store8(sA, row, c0, 128, v);
+        store8(sA, row, c0 + 8, 128, v + 8);
+        if (TRAIN) {
+          unsigned char* img = t.a_img + ((size_t)l * gridDim.x + blockIdx.x) * kImgA;
+          store8(img, row, c0, 128, v);
+          store8(img, row, c0 + 8, 128, v + 8);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          o0 = fmaf(__ldg(mst + W4_OFF + c0 + i), v[i], o0);
+          o1 = fmaf(__ldg(mst + W4_OFF + HID + c0 + i), v[i], o1);
+        }
+      }
+    }
+  }
+  sOut[part][0][row] = o0;
+  sOut[part][1][row] = o1;
+  __syncthreads();
+  o0 = __ldg(mst + B4_OFF);
+  o1 = __ldg(mst + B4_OFF + 1);
+#pragma unroll
+  for (int k = 0; k < kParts; ++k) {
+    o0 += sOut[k][0][row];
+    o1 += sOut[k][1][row];
+  }
+  if constexpr (TRAIN) {
+    // output layer: dL/dout / B; loss per row: sum over the two outputs of
+    // e^2 / 2 (Huber with delta > 0: quadratic inside |e| <= delta, linear
+    // outside).  The row's four threads hold the same values.
+    float d0 = 0.0f, d1 = 0.0f;
+    double se = 0.0;
+    if (valid) {
+      const float e[2] = {o0 - t.Y[src * OUT], o1 - t.Y[src * OUT + 1]};
+      float g[2];
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const float ae = fabsf(e[c]);
+        if (t.huber > 0.0f && ae > t.huber) {
+          g[c] = copysignf(t.huber, e[c]);
+          se += (double)t.huber * ((double)ae - 0.5 * t.huber);
+        } else {
+          g[c] = e[c];
+          se += 0.5 * (double)e[c] * e[c];
+        }
+      }
+      d0 = g[0] / (float)B;
+      d1 = g[1] / (float)B;
+    }
+    float* red = s_red[quarter];  // dW4, db3, db2, db1, db4
+    if (part == 0) {
+      se = warp_sum_d(se);
+      const float r0 = warp_sum(d0), r1 = warp_sum(d1);
+      if (lane == 0) {
+        s_loss[quarter] = se;
+        red[5 * HID] = r0;
+        red[5 * HID + 1] = r1;
+      }
+    }
+    // dz3 = (W4^T dout) GELU'(z3), then dz2 and dz1 through the transposed
+    // weights; each is the next product's A operand and an operand image of
+    // the weight gradients
+    for (int l = 2; l >= 0; --l) {
+      if (l < 2) product(0, HID, 1);
+      const float* bias = mst + (l == 0 ? B1_OFF : (l == 1 ? B2_OFF : B3_OFF));
+      unsigned char* img = t.dz_img + ((size_t)l * gridDim.x + blockIdx.x) * kImgA;
+#pragma unroll 1
+      for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+        float v[16], z[16];
+        if (l == 0) {
+          const float4* zr = reinterpret_cast<const float4*>(t.z + b * HID + c0);  // (this thread's own stores)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 q = zr[i];
+            z[4 * i] = q.x; z[4 * i + 1] = q.y; z[4 * i + 2] = q.z; z[4 * i + 3] = q.w;
+          }
+        } else {
+          tc::tmem_ld16(tl + (l == 1 ? kZ2 : 0u) + c0, z);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) z[i] += __ldg(bias + c0 + i);
+        }
+        if (l == 2) {
+          float a[16], a1[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) a[i] = z[i];
+#pragma unroll
+          for (int i = 0; i < 16; i += 2) gelu2(a[i], a[i + 1]);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            a1[i] = d1 * a[i];
+            a[i] = d0 * a[i];
+            v[i] = d0 * __ldg(mst + W4_OFF + c0 + i) + d1 * __ldg(mst + W4_OFF + HID + c0 + i);
+          }
+          const float w0 = colsum16(a), w1 = colsum16(a1);
+          if (lane < 16) {
+            red[c0 + lane] = w0;
+            red[HID + c0 + lane] = w1;
+          }
+        } else {
+          tc::tmem_ld16(tl + c0, v);
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = valid ? v[i] * gelu_grad(z[i]) : 0.0f;
+        const float sb = colsum16(v);
+        if (lane < 16) red[(4 - l) * HID + c0 + lane] = sb;
+        store8(img, row, c0, 128, v);
+        store8(img, row, c0 + 8, 128, v + 8);
+        if (l > 0) {
+          store8(sA, row, c0, 128, v);
+          store8(sA, row, c0 + 8, 128, v + 8);
+        }
+      }
+    }
+    __syncthreads();
+    // the CTA's partial sums: the four quarters' values added in order
+    float* pb = t.part_b + (long long)blockIdx.x * NB_PART;
+    for (int i = tid; i < NB_PART; i += kTE) pb[i] = ((s_red[0][i] + s_red[1][i]) + s_red[2][i]) + s_red[3][i];
+    if (tid == 0) t.part_loss[blockIdx.x] = ((s_loss[0] + s_loss[1]) + s_loss[2]) + s_loss[3];
+  }
+  if (!ok) atomicExch(&bad, 1);
+  __syncthreads();
+  if (!TRAIN && part == 0 && valid && bad == 0) {
+    out[b * OUT] = o0;
+    out[b * OUT + 1] = o1;
+  }
+  if (bad && tid == 0) {
+    // no copy may still be landing in shared memory when the CTA exits
+    for (int st = kStages - 2; st < kStages; ++st)
+      tc::mbar_wait(&full[st & 1], (uint32_t)((st >> 1) & 1), kEnvPolls);
+    raise_status(status, 2);
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, kCols);
+}
+
+// ---------------------------------------------------------------------------
+// Weight gradients dW_l = dz_l^T a_{l-1} summed over the batch: M = 128 output
+// features (one half), N = input features, K = the rows.  An operand image of
+// mlp_kernel [feature / 8][row][8] is also the MN-major form of its transpose
+// (descriptor: 8-row groups 128 B apart in K, 8-feature groups 128 * 16 B
+// apart in M / N), so a tile's two images go from HBM to the tensor core by
+// bulk copies, two tiles in flight, with no thread touching them (16,384 rows:
+// 14.5 us, against 77 when each CTA transposed its operands element by
+// element).  The
+// CTA's range of tiles accumulates in TMEM and is written to the split's slab,
+// summed over the splits in order by grad_reduce_kernel.  grid = (batch
+// splits, output half, layer).
+// ---------------------------------------------------------------------------
+constexpr size_t kWgradStage = kImgA / 2 + kImgA;  // half of dz's features, all of a's
+constexpr size_t kWgradSmem = 2 * kWgradStage;
+
+__global__ void __launch_bounds__(kT, 1) wgrad_kernel(TrainBufs t, int* status) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t full[2];
+  __shared__ __align__(8) uint64_t done[2];
+  __shared__ uint32_t tbase;
+  __shared__ int bad;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int layer = blockIdx.z, half = blockIdx.y;
+  const int n_in = layer == 0 ? IN : HID;
+  const int n_tiles = (t.B + kT - 1) / kT;
+  const int per = (n_tiles + gridDim.x - 1) / gridDim.x;
+  const int begin = blockIdx.x * per, n = min(n_tiles, begin + per) - begin;  // n <= 0: no rows left for this split
 
   if (warp == 0) {
     tc::tmem_alloc(&tbase, 256);
     tc::tmem_relinquish();
   }
-  if (tid == 0) tc::mbar_init(&mbar, 1);
+  if (tid == 0) {
+    for (int k = 0; k < 2; ++k) {
+      tc::mbar_init(&full[k], 1);
+      tc::mbar_init(&done[k], 1);
+    }
+    bad = 0;
+  }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tbase;
-  const uint32_t lane = tmem + ((uint32_t)(warp * 32) << 16);
-  const uint32_t aA = tc::smem_addr(sA), aB = tc::smem_addr(sB);
-  uint32_t phase = 0;
-  bool ok = true;
-  float* s_dW4 = s_red[warp];
-  float* s_db3 = s_dW4 + 2 * HID;
-  float* s_db2 = s_db3 + HID;
-  float* s_db1 = s_db2 + HID;
-  float* s_db4 = s_db1 + HID;
-
-  // output layer: dL/dout = (out - y) / B
-  // loss per row: sum over the two outputs of e^2 / 2 (Huber with delta > 0:
-  // quadratic inside |e| <= delta, linear outside); gradient / B
-  float d0 = 0.0f, d1 = 0.0f;
-  double se = 0.0;
-  if (valid) {
-    const float e[2] = {t.out[b * OUT] - t.Y[row * OUT], t.out[b * OUT + 1] - t.Y[row * OUT + 1]};
-    float g[2];
-    for (int c = 0; c < 2; ++c) {
-      const float ae = fabsf(e[c]);
-      if (t.huber > 0.0f && ae > t.huber) {
-        g[c] = copysignf(t.huber, e[c]);
-        se += (double)t.huber * ((double)ae - 0.5 * t.huber);
-      } else {
-        g[c] = e[c];
-        se += 0.5 * (double)e[c] * e[c];
+  if (tid == 0 && n > 0) {
+    const uint32_t bytes_b = (uint32_t)(kT * n_in * 2);
+    auto fetch = [&](int c) {
+      const size_t tile = (size_t)begin + c;
+      unsigned char* dst = smem + (c & 1) * kWgradStage;
+      const unsigned char* dz = t.dz_img + ((size_t)layer * n_tiles + tile) * kImgA + half * (kImgA / 2);
+      const unsigned char* a =
+          layer == 0 ? t.x_img + tile * kImgX : t.a_img + ((size_t)(layer - 1) * n_tiles + tile) * kImgA;
+      tc::mbar_expect_tx(&full[c & 1], (uint32_t)(kImgA / 2) + bytes_b);
+      tc::bulk_g2s(dst, dz, (uint32_t)(kImgA / 2), &full[c & 1]);
+      tc::bulk_g2s(dst + kImgA / 2, a, bytes_b, &full[c & 1]);
+    };
+    const uint32_t idesc = tc::idesc_bf16(128, (uint32_t)n_in) | (1u << 15) | (1u << 16);  // both MN-major
+    bool ok = true;
+    int fetched = min(n, 2);
+    for (int c = 0; c < fetched; ++c) fetch(c);
+    for (int c = 0; c < n && ok; ++c) {
+      ok = tc::mbar_wait(&full[c & 1], (uint32_t)((c >> 1) & 1), kEnvPolls);
+      if (!ok) break;
+      const uint32_t aa = tc::smem_addr(smem + (c & 1) * kWgradStage), bb = aa + (uint32_t)(kImgA / 2);
+      for (int j = 0; j < kT / 16; ++j) {
+        const uint64_t ad = tc::smem_desc(aa + j * 256, 128, kT * 16);
+        const uint64_t bd = tc::smem_desc(bb + j * 256, 128, kT * 16);
+        tc::mma_bf16(tmem, ad, bd, idesc, (c > 0 || j > 0) ? 1u : 0u);
+      }
+      tc::mma_commit(&done[c & 1]);
+      if (c + 1 < n) {  // refill the other stage once its MMAs (tile c - 1) are through
+        if (c >= 1 && fetched < n) {
+          ok = tc::mbar_wait(&done[(c - 1) & 1], (uint32_t)(((c - 1) >> 1) & 1), kEnvPolls);
+          if (ok) fetch(fetched++);
+        }
       }
     }
-    d0 = g[0] / (float)t.B;
-    d1 = g[1] / (float)t.B;
-  }
-  se = warp_sum_d(se);
-  if (lanei == 0) s_loss[warp] = se;
-  {
-    const float r0 = warp_sum(d0), r1 = warp_sum(d1);
-    if (lanei == 0) {
-      s_db4[0] = r0;
-      s_db4[1] = r1;
-    }
-  }
-  // dz3 = (W4^T dout) * GELU'(z3); dW4 += dout a3^T
-#pragma unroll 1
-  for (int c0 = 0; c0 < HID; c0 += 16) {
-    float dz[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const int k = c0 + i;
-      const float z = valid ? t.z[((long long)2 * t.B + b) * HID + k] : 0.0f;
-      const float a = valid ? gelu1(z) : 0.0f;  // the forward's GELU
-      const float w0 = warp_sum(d0 * a), w1 = warp_sum(d1 * a);
-      if (lanei == 0) {
-        s_dW4[k] = w0;
-        s_dW4[HID + k] = w1;
-      }
-      const float da = d0 * __ldg(mst + W4_OFF + k) + d1 * __ldg(mst + W4_OFF + HID + k);
-      dz[i] = valid ? da * gelu_grad(z) : 0.0f;
-      const float sdz = warp_sum(dz[i]);
-      if (lanei == 0) s_db3[k] = sdz;
-    }
-    if (valid) {
-      uint16_t* dr = t.dz + ((long long)2 * t.B + b) * HID + c0;
-#pragma unroll
-      for (int i = 0; i < 16; i += 2)
-        *reinterpret_cast<uint32_t*>(dr + i) = bf16x2_bits(dz[i], dz[i + 1]);
-    }
-    store8(sA, tid, c0, 128, dz);
-    store8(sA, tid, c0 + 8, 128, dz + 8);
-  }
-  // dz2, dz1 through the transposed weights on the tensor cores
-  for (int l = 1; l >= 0; --l) {
-    const size_t base = l == 1 ? IMG_W3T_OFF : IMG_W2T_OFF;
-    for (int h = 0; h < 2; ++h) {
-      copy_img(sB, net.img + base + (size_t)h * 128 * HID * 2, (size_t)128 * HID * 2);
-      ok &= tc::mma_group(tmem + 128 * h, &aA, 1, aB, 128, HID, false, &mbar, phase);
-    }
-    float* s_db = l == 1 ? s_db2 : s_db1;
-#pragma unroll 1
-    for (int c0 = 0; c0 < HID; c0 += 16) {
-      float v[16];
-      tc::tmem_ld16(lane + c0, v);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const float z = valid ? t.z[((long long)l * t.B + b) * HID + c0 + i] : 0.0f;
-        v[i] = valid ? v[i] * gelu_grad(z) : 0.0f;
-        const float s = warp_sum(v[i]);
-        if (lanei == 0) s_db[c0 + i] = s;
-      }
-      if (valid) {
-        uint16_t* dr = t.dz + ((long long)l * t.B + b) * HID + c0;
-#pragma unroll
-        for (int i = 0; i < 16; i += 2)
-          *reinterpret_cast<uint32_t*>(dr + i) = bf16x2_bits(v[i], v[i + 1]);
-      }
-      if (l == 1) {
-        store8(sA, tid, c0, 128, v);
-        store8(sA, tid, c0 + 8, 128, v + 8);
-      }
+    if (ok) ok = tc::mbar_wait(&done[(n - 1) & 1], (uint32_t)(((n - 1) >> 1) & 1), kEnvPolls);
+    if (!ok) {  // no copy may still be landing when the CTA exits
+      bad = 1;
+      for (int c = max(0, fetched - 2); c < fetched; ++c)
+        tc::mbar_wait(&full[c & 1], (uint32_t)((c >> 1) & 1), kEnvPolls);
+      raise_status(status, 2);
     }
   }
   tc::fence_before_sync();
   __syncthreads();
-  // the CTA's partial sums: the four warps' values added in warp order
-  float* pb = t.part_b + (long long)blockIdx.x * NB_PART;
-  for (int i = tid; i < NB_PART; i += kT) {
-    float acc = s_red[0][i];
+  tc::fence_after_sync();
+  if (!bad) {
+    // this split's slab: dW1 [256][96], then dW2 and dW3 [256][256]
+    const long long w_off = layer == 0 ? 0 : (long long)HID * IN + (long long)(layer - 1) * HID * HID;
+    float* pw = t.part_w + (long long)blockIdx.x * NW_PART + w_off + (long long)(half * 128 + tid) * n_in;
+    const uint32_t lane = tmem + ((uint32_t)(warp * 32) << 16);
+    for (int c0 = 0; c0 < n_in; c0 += 16) {
+      float v[16];
+      if (n > 0) {
+        tc::tmem_ld16(lane + c0, v);
+      } else {
 #pragma unroll
-    for (int w = 1; w < kT / 32; ++w) acc += s_red[w][i];
-    pb[i] = acc;
-  }
-  if (tid == 0) {
-    double acc = s_loss[0];
+        for (int i = 0; i < 16; ++i) v[i] = 0.0f;
+      }
 #pragma unroll
-    for (int w = 1; w < kT / 32; ++w) acc += s_loss[w];
-    t.part_loss[blockIdx.x] = acc;
+      for (int i = 0; i < 16; i += 4)
+        *reinterpret_cast<float4*>(pw + c0 + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    }
   }
-  if (!ok && tid == 0) raise_status(status, 2);
+  tc::fence_before_sync();
+  __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tmem, 256);
 }
 
-// grad[dst(i)] = sum over p of part[p][i], i < len: block x sums entries
-// 32x .. 32x+31, thread row g the parts p = g (mod 32) in increasing p, then
-// the 32 row sums in order of g (a fixed association: deterministic).  dst
-// maps a slab position to its canonical parameter offset: `which` 0 for the
-// bias / output-layer slab, 1 for the hidden weight slab.
+// Canonical parameter offset of a slab position: `which` 0 for the bias /
+// output-layer slab, 1 for the hidden weight slab.
 __device__ __forceinline__ long long part_dst(int which, long long i) {
   if (which == 0) {
     if (i < 2 * HID) return W4_OFF + i;
@@ -594,127 +737,60 @@ __device__ __forceinline__ long long part_dst(int which, long long i) {
   return W3_OFF + (i - (long long)HID * IN - (long long)HID * HID);
 }
 
-__global__ void __launch_bounds__(1024) part_reduce_kernel(const float* __restrict__ part, int nparts, long long len,
-                                                           int which, float* __restrict__ grad) {
-  __shared__ float red[32][33];
-  const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
-  const long long i = (long long)blockIdx.x * 32 + c;
-  float s = 0.0f;
-  if (i < len)
-    for (int p = g; p < nparts; p += 32) s += part[(long long)p * len + i];
-  red[g][c] = s;
-  __syncthreads();
-  if (g == 0 && i < len) {
-    float acc = 0.0f;
-#pragma unroll
-    for (int k = 0; k < 32; ++k) acc += red[k][c];
-    grad[part_dst(which, i)] = acc;
-  }
-}
+// Gradient and loss from the partial slabs, every sum in a fixed order.
+// Blocks 0 .. kRedW - 1: four hidden weights per thread, over the splits in
+// order (the slabs' tensors start at multiples of 4, so a thread's four stay
+// in one tensor; 4 us for all three kinds, 34 as three kernels).  The next
+// kRedB: 32 entries of the bias slab each, thread
+// row g the parts p = g (mod 8), then the 8 row sums in order.  The last: the
+// loss, parts p = i (mod 256), then warp and block sums.
+constexpr int kRedW = (int)((NW_PART / 4 + 255) / 256), kRedB = (NB_PART + 31) / 32;
 
-// Batch loss = (sum of the CTA partials, in order of p mod 256, then the 256
-// sums in order) / B.
-__global__ void __launch_bounds__(256) loss_reduce_kernel(const double* __restrict__ part, int nparts, int B,
-                                                          double* __restrict__ loss) {
-  __shared__ double red[256];
+__global__ void __launch_bounds__(256) grad_reduce_kernel(TrainBufs t, int splits, int n_cta) {
+  const int tid = threadIdx.x;
+  if (blockIdx.x < kRedW) {
+    const long long i = ((long long)blockIdx.x * 256 + tid) * 4;
+    if (i >= NW_PART) return;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+    for (int p = 0; p < splits; ++p) {
+      const float4 v = *reinterpret_cast<const float4*>(t.part_w + (long long)p * NW_PART + i);
+      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+    float* g = t.grad + part_dst(1, i);
+    g[0] = s.x; g[1] = s.y; g[2] = s.z; g[3] = s.w;
+    return;
+  }
+  if (blockIdx.x < kRedW + kRedB) {
+    __shared__ float red[8][33];
+    const int c = tid & 31, g = tid >> 5, i = ((int)blockIdx.x - kRedW) * 32 + c;
+    float s = 0.0f;
+    if (i < NB_PART) {
+#pragma unroll 8
+      for (int p = g; p < n_cta; p += 8) s += t.part_b[(long long)p * NB_PART + i];
+    }
+    red[g][c] = s;
+    __syncthreads();
+    if (g == 0 && i < NB_PART) {
+      float acc = 0.0f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) acc += red[k][c];
+      t.grad[part_dst(0, i)] = acc;
+    }
+    return;
+  }
+  __shared__ double sl[8];
   double s = 0.0;
-  for (int p = threadIdx.x; p < nparts; p += 256) s += part[p];
-  red[threadIdx.x] = s;
+  for (int p = tid; p < n_cta; p += 256) s += t.part_loss[p];
+  s = warp_sum_d(s);
+  if ((tid & 31) == 0) sl[tid >> 5] = s;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     double acc = 0.0;
-    for (int k = 0; k < 256; ++k) acc += red[k];
-    *loss = acc / B;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Weight gradients dW_l = dz_l^T a_{l-1} summed over the batch, on the tensor
-// cores: M = 128 output features (one half), N = input features, K = 128
-// batch rows per MMA group, accumulated in TMEM over the CTA's batch range
-// and written to the split's partial slab (summed over the splits in a fixed
-// order by part_reduce_kernel).  The transposed operands are written
-// element-wise into K-major images.  grid = (batch splits, output half, layer).
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kT, 2) wgrad_kernel(TrainBufs t, int* status) {
-  extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* sA = smem;          // dz^T [128 x 128]
-  unsigned char* sB = smem + 32768;  // a^T [N_in x 128]
-  __shared__ __align__(8) uint64_t mbar;
-  __shared__ uint32_t tbase;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int layer = blockIdx.z, half = blockIdx.y;
-  const int n_in = layer == 0 ? IN : HID;
-  const int n_chunks = (t.B + kT - 1) / kT;
-  const int per = (n_chunks + gridDim.x - 1) / gridDim.x;
-  const int c_begin = blockIdx.x * per, c_end = min(n_chunks, c_begin + per);
-
-  if (warp == 0) {
-    tc::tmem_alloc(&tbase, 256);
-    tc::tmem_relinquish();
-  }
-  if (tid == 0) tc::mbar_init(&mbar, 1);
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = tbase;
-  const uint32_t aA = tc::smem_addr(sA), aB = tc::smem_addr(sB);
-  uint32_t phase = 0;
-  bool ok = true;
-  uint16_t* sAh = reinterpret_cast<uint16_t*>(sA);
-  uint16_t* sBh = reinterpret_cast<uint16_t*>(sB);
-  for (int c = c_begin; c < c_end; ++c) {
-    const long long b = (long long)c * kT + tid;
-    const bool valid = b < t.B;
-    // dz^T: element (o, b) of the [128 x 128] operand
-    const uint16_t* dzr = t.dz + ((long long)layer * t.B + b) * HID + half * 128;
-#pragma unroll 4
-    for (int o = 0; o < 128; o += 8) {
-      uint4 v = valid ? *reinterpret_cast<const uint4*>(dzr + o) : make_uint4(0, 0, 0, 0);
-      const uint16_t* e = reinterpret_cast<const uint16_t*>(&v);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) sAh[tc::kmajor_offset(o + i, tid, 128) / 2] = e[i];
-    }
-    // a^T: element (i, b) of the [n_in x 128] operand (layer 0: the features)
-    if (layer == 0) {
-      const long long row = valid ? (t.rows ? (long long)t.rows[b] : b) : 0;
-      for (int i = 0; i < IN; ++i)
-        sBh[tc::kmajor_offset(i, tid, IN) / 2] = valid ? f2bf_bits(t.X[row * IN + i]) : (uint16_t)0;
-    } else {
-      const uint16_t* ar = t.a + ((long long)(layer - 1) * t.B + b) * HID;
-#pragma unroll 4
-      for (int i = 0; i < HID; i += 8) {
-        uint4 v = valid ? *reinterpret_cast<const uint4*>(ar + i) : make_uint4(0, 0, 0, 0);
-        const uint16_t* e = reinterpret_cast<const uint16_t*>(&v);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) sBh[tc::kmajor_offset(i + j, tid, HID) / 2] = e[j];
-      }
-    }
-    ok &= tc::mma_group(tmem, &aA, 1, aB, n_in, kT, c > c_begin, &mbar, phase);
+    for (int k = 0; k < 8; ++k) acc += sl[k];
+    *t.loss = acc / t.B;
   }
-  if (c_end <= c_begin) {  // per = ceil(chunks / splits) can leave the last splits without rows: zero slab
-    const int o = warp * 32 + (tid & 31);
-    const long long w_off = layer == 0 ? 0 : (long long)HID * IN + (long long)(layer - 1) * HID * HID;
-    float* pw = t.part_w + (long long)blockIdx.x * NW_PART + w_off;
-    for (int c = 0; c < n_in; ++c) pw[(long long)(half * 128 + o) * n_in + c] = 0.0f;
-  }
-  if (c_end > c_begin && ok) {
-    const int o = warp * 32 + (tid & 31);
-    // this split's slab: dW1 [256][96], then dW2 and dW3 [256][256]
-    const long long w_off = layer == 0 ? 0 : (long long)HID * IN + (long long)(layer - 1) * HID * HID;
-    float* pw = t.part_w + (long long)blockIdx.x * NW_PART + w_off;
-    const uint32_t lane = tmem + ((uint32_t)(warp * 32) << 16);
-    for (int c0 = 0; c0 < n_in; c0 += 16) {
-      float v[16];
-      tc::tmem_ld16(lane + c0, v);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) pw[(long long)(half * 128 + o) * n_in + c0 + i] = v[i];
-    }
-  }
-  if (!ok && tid == 0) raise_status(status, 2);
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, 256);
 }
 
 // Image position of weight element (layer, out, in) in the forward operand
@@ -780,22 +856,12 @@ __global__ void record_kernel(EnvDev d, float* feat, float* label) {
 
 }  // namespace
 
-cudaError_t launch_forward(const Net& net, const float* X, const int32_t* rows, int B, float* out, float* z,
-                           uint16_t* a, cudaStream_t s) {
+cudaError_t launch_forward(const Net& net, const float* X, int B, float* out, cudaStream_t s) {
   static std::atomic<unsigned long long> ready{0};
-  cudaError_t e = smem_optin(fwd_kernel, kFwdSmem, ready);
+  cudaError_t e = smem_optin(mlp_kernel<false>, kEnvSmem, ready);
   if (e != cudaSuccess) return e;
   if (B <= 0) return cudaSuccess;
-  FwdArgs p;
-  memset(&p, 0, sizeof(p));
-  p.net = net;
-  p.X = X;
-  p.rows = rows;
-  p.B = B;
-  p.out = out;
-  p.z = z;
-  p.a = a;
-  fwd_kernel<<<(B + kT - 1) / kT, kT, kFwdSmem, s>>>(p);
+  mlp_kernel<false><<<(B + kT - 1) / kT, kTE, kEnvSmem, s>>>(net, X, nullptr, B, out, TrainBufs{}, nullptr);
   return cudaGetLastError();
 }
 
@@ -815,24 +881,21 @@ cudaError_t launch_record(const EnvDev& d, float* feat, float* label, cudaStream
   return cudaGetLastError();
 }
 
-cudaError_t launch_backward(const Net& net, const TrainBufs& t, cudaStream_t s) {
-  static std::atomic<unsigned long long> ready_b{0}, ready_w{0};
-  cudaError_t e = smem_optin(bwd_kernel, kFwdSmem, ready_b);
+cudaError_t launch_loss_grad(const Net& net, const TrainBufs& t, cudaStream_t s) {
+  static std::atomic<unsigned long long> ready_m{0}, ready_w{0};
+  cudaError_t e = smem_optin(mlp_kernel<true>, kEnvSmem, ready_m);
   if (e == cudaSuccess) e = smem_optin(wgrad_kernel, kWgradSmem, ready_w);
   if (e != cudaSuccess) return e;
   if (t.B <= 0) return cudaSuccess;
-  const int n_chunks = (t.B + kT - 1) / kT;
-  bwd_kernel<<<n_chunks, kT, kFwdSmem, s>>>(net, t, nullptr);
+  const int n_cta = (t.B + kT - 1) / kT;
+  mlp_kernel<true><<<n_cta, kTE, kEnvSmem, s>>>(net, t.X, t.rows, t.B, nullptr, t, nullptr);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int splits = n_chunks < kWgradSplits ? n_chunks : kWgradSplits;
+  const int splits = n_cta < kWgradSplits ? n_cta : kWgradSplits;
   wgrad_kernel<<<dim3(splits, 2, 3), kT, kWgradSmem, s>>>(t, nullptr);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  // fixed-order sums of the partial slabs into the gradient and the loss
-  part_reduce_kernel<<<(NB_PART + 31) / 32, 1024, 0, s>>>(t.part_b, n_chunks, NB_PART, 0, t.grad);
-  part_reduce_kernel<<<(unsigned)((NW_PART + 31) / 32), 1024, 0, s>>>(t.part_w, splits, NW_PART, 1, t.grad);
-  loss_reduce_kernel<<<1, 256, 0, s>>>(t.part_loss, n_chunks, t.B, t.loss);
+  grad_reduce_kernel<<<kRedW + kRedB + 1, 256, 0, s>>>(t, splits, n_cta);
   return cudaGetLastError();
 }
 

@@ -54,31 +54,33 @@ struct Net {
   const float* master;       // FP32 parameters, canonical order (biases, W4)
 };
 
-// Training buffers for one batch of B rows.
+// Training buffers for one batch of B rows (tiles = ceil(B / 128)).  An
+// operand image holds 128 rows as [feature / 8][row][8] BF16.
 struct TrainBufs {
-  const float* X;        // [n_rows][96] features
-  const float* Y;        // [n_rows][2] labels
-  const int32_t* rows;   // [B] dataset rows of the batch (NULL: rows 0..B-1)
-  float* z;              // [3][B][256] pre-activations
-  uint16_t* a;           // [3][B][256] BF16 activations (GELU(z))
-  float* out;            // [B][2]
-  uint16_t* dz;          // [3][B][256] BF16 gradients w.r.t. z
-  float* grad;           // [NPARAM] FP32 gradient
-  double* loss;          // [1] loss of the batch
+  const float* X;         // [n_rows][96] features
+  const float* Y;         // [n_rows][2] labels
+  const int32_t* rows;    // [B] dataset rows of the batch (NULL: rows 0..B-1)
+  float* z;               // [tiles * 128][256] pre-activations of layer 1
+  unsigned char* x_img;   // [tiles] images of the features' BF16 high part
+  unsigned char* a_img;   // [2][tiles] images of GELU(z1), GELU(z2)
+  unsigned char* dz_img;  // [3][tiles] images of the gradients w.r.t. z
+  float* grad;            // [NPARAM] FP32 gradient (every entry written)
+  double* loss;           // [1] loss of the batch
   // fixed-order partial sums (no atomics: the gradient is deterministic)
-  float* part_b;         // [ceil(B/128)][NB_PART] per-CTA dW4, db3, db2, db1, db4
-  double* part_loss;     // [ceil(B/128)] per-CTA loss sums
-  float* part_w;         // [kWgradSplits][NW_PART] per-split dW1, dW2, dW3
-  float huber;           // 0: squared error; > 0: Huber threshold (label units)
+  float* part_b;          // [tiles][NB_PART] per-CTA dW4, db3, db2, db1, db4
+  double* part_loss;      // [tiles] per-CTA loss sums
+  float* part_w;          // [kWgradSplits][NW_PART] per-split dW1, dW2, dW3
+  float huber;            // 0: squared error; > 0: Huber threshold (label units)
   int B;
 };
 
-cudaError_t launch_forward(const Net& net, const float* X, const int32_t* rows, int B, float* out, float* z,
-                           uint16_t* a, cudaStream_t s);
+// Outputs [B][2] of the features X [B][96].
+cudaError_t launch_forward(const Net& net, const float* X, int B, float* out, cudaStream_t s);
+// Loss and gradient of one batch (t.loss, t.grad).
+cudaError_t launch_loss_grad(const Net& net, const TrainBufs& t, cudaStream_t s);
 cudaError_t launch_forward_env(const Net& net, const EnvDev& d, int stale, uint32_t test_wait_polls,
                                cudaStream_t s);
 cudaError_t launch_record(const EnvDev& d, float* feat, float* label, cudaStream_t s);
-cudaError_t launch_backward(const Net& net, const TrainBufs& t, cudaStream_t s);
 cudaError_t launch_adam(float* master, float* m, float* v, const float* grad, int step, float lr, float beta1,
                         float beta2, float eps, unsigned char* img, cudaStream_t s);
 cudaError_t launch_pack(const float* master, unsigned char* img, cudaStream_t s);

@@ -22,9 +22,9 @@ struct EstimatorState {
   // training buffers (sized for batch_cap rows)
   int batch_cap = 0;
   float* z = nullptr;
-  uint16_t* a = nullptr;
-  uint16_t* dz = nullptr;
-  float* out = nullptr;
+  unsigned char* x_img = nullptr;
+  unsigned char* a_img = nullptr;
+  unsigned char* dz_img = nullptr;
   int32_t* rows = nullptr;
   double* loss = nullptr;
   // fixed-order partial sums of the backward pass
@@ -262,18 +262,26 @@ ut_status est_alloc_weights(ut_env* h) {
 ut_status est_alloc_batch(ut_env* h, int B) {
   EstimatorState* es = est_state(h);
   if (es->batch_cap >= B) return UT_OK;
-  // earlier (smaller) buffers stay owned by the handle until destroy
-  es->z = (float*)env_alloc(h, (size_t)3 * B * est::HID * 4);
-  es->a = (uint16_t*)env_alloc(h, (size_t)3 * B * est::HID * 2);
-  es->dz = (uint16_t*)env_alloc(h, (size_t)3 * B * est::HID * 2);
-  es->out = (float*)env_alloc(h, (size_t)B * 2 * 4);
-  es->rows = (int32_t*)env_alloc(h, (size_t)B * 4);
-  const size_t n_cta = ((size_t)B + 127) / 128;
-  es->part_b = (float*)env_alloc(h, n_cta * est::NB_PART * 4);
-  es->part_loss = (double*)env_alloc(h, n_cta * 8);
+  // earlier (smaller) buffers stay owned by the handle until destroy, and in
+  // use until every new one is there
+  const size_t n_cta = ((size_t)B + 127) / 128, img = (size_t)128 * est::HID * 2;
+  float* z = (float*)env_alloc(h, n_cta * 128 * est::HID * 4);
+  unsigned char* x_img = (unsigned char*)env_alloc(h, n_cta * 128 * est::IN * 2);
+  unsigned char* a_img = (unsigned char*)env_alloc(h, 2 * n_cta * img);
+  unsigned char* dz_img = (unsigned char*)env_alloc(h, 3 * n_cta * img);
+  int32_t* rows = (int32_t*)env_alloc(h, (size_t)B * 4);
+  float* part_b = (float*)env_alloc(h, n_cta * est::NB_PART * 4);
+  double* part_loss = (double*)env_alloc(h, n_cta * 8);
   if (!es->part_w) es->part_w = (float*)env_alloc(h, (size_t)est::kWgradSplits * est::NW_PART * 4);
-  if (!es->z || !es->a || !es->dz || !es->out || !es->rows || !es->part_b || !es->part_loss || !es->part_w)
+  if (!z || !x_img || !a_img || !dz_img || !rows || !part_b || !part_loss || !es->part_w)
     return est_fail(h, UT_ERR_NOMEM, "estimator: batch allocation failed");
+  es->z = z;
+  es->x_img = x_img;
+  es->a_img = a_img;
+  es->dz_img = dz_img;
+  es->rows = rows;
+  es->part_b = part_b;
+  es->part_loss = part_loss;
   es->batch_cap = B;
   return UT_OK;
 }
@@ -285,30 +293,26 @@ est::Net est_net(ut_env* h) {
   return n;
 }
 
-// Forward + backward of one batch into es->grad (cleared first) and es->loss.
-cudaError_t est_grad_batch(ut_env* h, const float* X, const float* Y, const int32_t* rows, int B, float huber) {
+// Loss and gradient of one batch into es->loss and grad.
+cudaError_t est_grad_batch(ut_env* h, const float* X, const float* Y, const int32_t* rows, int B, float huber,
+                           float* grad) {
   EstimatorState* es = h->est;
-  cudaStream_t s = h->stream;
-  cudaError_t e = cudaMemsetAsync(es->grad, 0, est::NPARAM * 4, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(es->loss, 0, 8, s);
-  if (e == cudaSuccess) e = est::launch_forward(est_net(h), X, rows, B, es->out, es->z, es->a, s);
-  if (e != cudaSuccess) return e;
   est::TrainBufs t;
   t.X = X;
   t.Y = Y;
   t.rows = rows;
   t.z = es->z;
-  t.a = es->a;
-  t.out = es->out;
-  t.dz = es->dz;
-  t.grad = es->grad;
+  t.x_img = es->x_img;
+  t.a_img = es->a_img;
+  t.dz_img = es->dz_img;
+  t.grad = grad;
   t.loss = es->loss;
   t.part_b = es->part_b;
   t.part_loss = es->part_loss;
   t.part_w = es->part_w;
   t.huber = huber;
   t.B = B;
-  return est::launch_backward(est_net(h), t, s);
+  return est::launch_loss_grad(est_net(h), t, h->stream);
 }
 
 }  // namespace
@@ -362,7 +366,7 @@ extern "C" ut_status est_forward(ut_env* h, const float* X_dev, float* out_dev, 
   if (!h || n_rows < 0 || n_rows > 0x7fffffff || (n_rows && (!X_dev || !out_dev))) return UT_ERR_INVALID;
   if (!h->est || !h->est->weights_set) return est_fail(h, UT_ERR_STATE, "est_forward: no weights");
   if (reinterpret_cast<uintptr_t>(X_dev) & 15) return est_fail(h, UT_ERR_INVALID, "est_forward: X not 16-byte aligned");
-  cudaError_t e = est::launch_forward(est_net(h), X_dev, nullptr, (int)n_rows, out_dev, nullptr, nullptr, h->stream);
+  cudaError_t e = est::launch_forward(est_net(h), X_dev, (int)n_rows, out_dev, h->stream);
   return e == cudaSuccess ? UT_OK : est_fail(h, UT_ERR_CUDA, cudaGetErrorString(e));
 }
 
@@ -389,9 +393,7 @@ extern "C" ut_status est_loss_grad(ut_env* h, const float* X_dev, const float* Y
     if (er != cudaSuccess) return est_fail(h, UT_ERR_CUDA, cudaGetErrorString(er));
     rows = h->est->rows;
   }
-  cudaError_t e = est_grad_batch(h, X_dev, Y_dev, rows, B, huber_delta);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(grad_dev, h->est->grad, est::NPARAM * 4, cudaMemcpyDeviceToDevice, h->stream);
+  cudaError_t e = est_grad_batch(h, X_dev, Y_dev, rows, B, huber_delta, grad_dev);
   double loss = 0.0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&loss, h->est->loss, 8, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -434,7 +436,7 @@ extern "C" ut_status est_train(ut_env* h, const float* X_dev, const float* Y_dev
       e = est::launch_batch_rows(es->rows, B, n_rows, cfg->seed, (uint32_t)s, h->stream);
       rows = es->rows;
     }
-    if (e == cudaSuccess) e = est_grad_batch(h, X_dev, Y_dev, rows, B, cfg->huber_delta);
+    if (e == cudaSuccess) e = est_grad_batch(h, X_dev, Y_dev, rows, B, cfg->huber_delta, es->grad);
     // cosine decay of the learning rate over the run (reading C18)
     const double frac = cfg->steps > 1 ? (double)s / (double)(cfg->steps - 1) : 0.0;
     const float lr = cfg->cosine ? (float)(cfg->lr * 0.5 * (1.0 + std::cos(3.141592653589793 * frac))) : cfg->lr;
