@@ -27,6 +27,7 @@
 #include "common.cuh"
 #include "tc.cuh"
 #include "tfm.cuh"
+#include "warp_sums.cuh"
 
 namespace ut {
 namespace tfm {
@@ -1601,6 +1602,7 @@ bool valid_config(const ut_tfm_config* c) {
 }
 
 #include "tfm_tc.cuh"
+#include "tfm_ffn.cuh"
 
 // Every BF16 weight image of the handle: grid (elements, image).
 __global__ void pack_images_kernel(const float* __restrict__ prm, const int64_t* __restrict__ spec,
@@ -1839,6 +1841,27 @@ Block block_of(const ut_tfm* t, int l) {
   return b;
 }
 
+// Arguments of block l's feed-forward sub-block (tfm_ffn.cuh).
+FfnArgs ffn_args(const ut_tfm* t, int l, const float* M, float* out, long long rows) {
+  const int64_t* ol = t->off.data() + 2 + 12 * l;
+  const int64_t* im = t->img_off.data() + 8 * l;
+  FfnArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.M = M;
+  a.out = out;
+  a.gain = t->prm + ol[T_LN2G];
+  a.off = t->prm + ol[T_LN2B];
+  a.b1 = t->prm + ol[T_B1];
+  a.b2 = t->prm + ol[T_B2];
+  a.w1 = t->wimg + im[2];
+  a.w2 = t->wimg + im[3];
+  a.w1t = t->wimg + im[6];
+  a.w2t = t->wimg + im[7];
+  a.rows = rows;
+  a.status = t->status;
+  return a;
+}
+
 template <int DJ, int DH, typename TokT>
 cudaError_t forward(ut_tfm* t, const Call& c, cudaStream_t s) {
   constexpr int d = 32 * DJ;
@@ -1898,6 +1921,10 @@ cudaError_t forward(ut_tfm* t, const Call& c, cudaStream_t s) {
     g.R = b.X;
     g.ldr = last ? (long long)t->T * d : d;
     e = gemm0(g, ol[T_BO], img(l, 1));
+    if (t->gemm_tc && d == kFfD) {
+      if (e == cudaSuccess) e = ffn_fwd(ffn_args(t, l, b.M, b.X + MR * d, m), s);
+      continue;
+    }
     if (e == cudaSuccess) e = ln_fwd<DJ>(b.M, w + ol[T_LN2G], w + ol[T_LN2B], b.Y2, b.S2, m, s);
     if (e != cudaSuccess) break;
     g = mk(b.Y2, d, w + ol[T_W1], d, b.Z, 4 * d, m, 4 * d, d, EPI_BIAS_GELU);
@@ -1930,14 +1957,28 @@ cudaError_t backward(ut_tfm* t, const Call& c, float* grad, cudaStream_t s) {
     const long long m = last ? c.n : rows;
     const Block b = block_of(t, l);
     // feed-forward sub-block: X' = M + W2 gelu(W1 LN2(M) + b1) + b2
-    Gemm g = mk(t->dX, d, w + ol[T_W2], 4 * d, t->dBig, 4 * d, m, 4 * d, d, EPI_GELU_GRAD);
-    g.aux = b.Z;
-    e = dgemm(l, 7, g);
-    if (e == cudaSuccess) e = wgrad(t, t->dX, d, b.G, 4 * d, 4 * d, m, grad + ol[T_W2], grad + ol[T_B2], s);
-    if (e == cudaSuccess) e = dgemm(l, 6, mk(t->dBig, 4 * d, w + ol[T_W1], d, t->dY, d, m, d, 4 * d, EPI_STORE));
-    if (e == cudaSuccess) e = wgrad(t, t->dBig, 4 * d, b.Y2, d, d, m, grad + ol[T_W1], grad + ol[T_B1], s);
-    if (e == cudaSuccess)
-      e = ln_bwd<DJ, false>(t, t->dY, b.M, b.S2, w + ol[T_LN2G], t->dX, t->dM, grad + ol[T_LN2G], m, s);
+    if (t->gemm_tc && d == kFfD) {
+      FfnArgs a = ffn_args(t, l, b.M, t->dM, m);
+      a.dX = t->dX;
+      a.slab = t->part;
+      a.vec = t->part + 152ll * kFfSlab;
+      int ctas = 0;
+      e = ffn_bwd(a, &ctas, s);
+      if (e == cudaSuccess) e = reduce(a.slab, ctas, kFfH * kFfD, kFfSlab, grad + ol[T_W1], s);
+      if (e == cudaSuccess) e = reduce(a.slab + kFfH * kFfD, ctas, kFfH * kFfD, kFfSlab, grad + ol[T_W2], s);
+      if (e == cudaSuccess) e = reduce(a.vec, ctas, kFfH, kFfVec, grad + ol[T_B1], s);
+      if (e == cudaSuccess) e = reduce(a.vec + kFfH, ctas, kFfD, kFfVec, grad + ol[T_B2], s);
+      if (e == cudaSuccess) e = reduce(a.vec + kFfH + kFfD, ctas, 2 * kFfD, kFfVec, grad + ol[T_LN2G], s);
+    } else {
+      Gemm g = mk(t->dX, d, w + ol[T_W2], 4 * d, t->dBig, 4 * d, m, 4 * d, d, EPI_GELU_GRAD);
+      g.aux = b.Z;
+      e = dgemm(l, 7, g);
+      if (e == cudaSuccess) e = wgrad(t, t->dX, d, b.G, 4 * d, 4 * d, m, grad + ol[T_W2], grad + ol[T_B2], s);
+      if (e == cudaSuccess) e = dgemm(l, 6, mk(t->dBig, 4 * d, w + ol[T_W1], d, t->dY, d, m, d, 4 * d, EPI_STORE));
+      if (e == cudaSuccess) e = wgrad(t, t->dBig, 4 * d, b.Y2, d, d, m, grad + ol[T_W1], grad + ol[T_B1], s);
+      if (e == cudaSuccess)
+        e = ln_bwd<DJ, false>(t, t->dY, b.M, b.S2, w + ol[T_LN2G], t->dX, t->dM, grad + ol[T_LN2G], m, s);
+    }
     // attention sub-block: M = X + Wo attn(LN1(X)) + bo
     if (e == cudaSuccess) e = dgemm(l, 5, mk(t->dM, d, w + ol[T_WO], d, t->dO, d, m, d, d, EPI_STORE));
     if (e == cudaSuccess) e = wgrad(t, t->dM, d, b.O, d, d, m, grad + ol[T_WO], grad + ol[T_BO], s);
