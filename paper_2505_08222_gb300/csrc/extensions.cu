@@ -43,6 +43,10 @@ struct PolicyState {
   uint16_t* h = nullptr;
   float* logits = nullptr;
   int32_t* n_ent = nullptr;
+  // two-kernel form of large batches: the step's workspace, and the pool of
+  // policy_forward's, one per call (calls on several streams may overlap)
+  void* ws = nullptr;
+  cudaMemPool_t pool = nullptr;
 };
 
 namespace ut {
@@ -76,6 +80,7 @@ static PolicyDev policy_dev(ut_env* h) {
   p.sample = 1;
   p.status = h->d.status;
   p.test_wait_polls = h->test_wait_polls;
+  if (ps->ws) policy_ws_set(p, ps->d, ps->ws);
   return p;
 }
 
@@ -109,6 +114,7 @@ ut_status extension_create(ut_env* h) {
 }
 
 void extension_destroy(ut_env* h) {
+  if (h->policy && h->policy->pool) cudaMemPoolDestroy(h->policy->pool);
   delete h->policy;
   h->policy = nullptr;
   delete h->est;
@@ -125,7 +131,11 @@ cudaError_t extension_policy_actions(ut_env* h, cudaStream_t s) {
   return launch_policy(policy_dev(h), h->policy->d, s);
 }
 
-int extension_policy_kernels(ut_env*) { return 1; }
+int extension_policy_kernels(ut_env* h) {
+  if (!h->policy || !h->policy->ws) return 1;
+  const long long chunk = policy_chunk(h->policy->d, h->NA, 128 / (1 + h->d.NS));
+  return 2 * (int)((h->NA + chunk - 1) / chunk);
+}
 cudaError_t extension_estimate_impl(ut_env* h, cudaStream_t s);
 cudaError_t extension_estimate(ut_env* h, cudaStream_t s) { return extension_estimate_impl(h, s); }
 const float* extension_logits(ut_env* h) { return h->policy ? h->policy->logits : nullptr; }
@@ -166,6 +176,8 @@ extern "C" ut_status env_set_policy(ut_env* h, const float* params_host, int64_t
     ps->emb = emb_d;
     ps->head = head_d;
     ps->wimg = wimg;
+    // (without a workspace the step keeps the one-kernel form)
+    if (policy_split(ps->d, h->NA, 1 + h->d.NS)) ps->ws = env_alloc(h, policy_ws_bytes(ps->d, h->NA, 1 + h->d.NS));
   }
   cudaError_t e = cudaMemcpyAsync(ps->wimg, img.data(), img.size(), cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(ps->vec, vec.data(), vec.size() * 4, cudaMemcpyHostToDevice, h->stream);
@@ -179,6 +191,34 @@ extern "C" ut_status env_set_policy(ut_env* h, const float* params_host, int64_t
   }
   h->policy_ready = true;
   return UT_OK;
+}
+
+// Workspace of one policy_forward call, stream-ordered from the handle's own
+// pool (which keeps up to 64 MB between calls and goes with the handle): NULL
+// where the one-kernel form is the faster one, in a stream capture, and when
+// there is no memory for it.
+static void* forward_ws(ut_env* h, const PolicyDev& p, cudaStream_t s) {
+  PolicyState* ps = h->policy;
+  if (!policy_split(ps->d, p.NA, p.R)) return nullptr;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  void* ws = nullptr;
+  bool ok = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  if (ok && !ps->pool) {
+    cudaMemPoolProps props;
+    std::memset(&props, 0, sizeof(props));
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = h->device;
+    uint64_t keep = 64ull << 20;
+    ok = cudaMemPoolCreate(&ps->pool, &props) == cudaSuccess &&
+         cudaMemPoolSetAttribute(ps->pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess;
+  }
+  if (ok) ok = cudaMallocFromPoolAsync(&ws, policy_ws_bytes(ps->d, p.NA, p.R), ps->pool, s) == cudaSuccess;
+  if (!ok) {
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  return ws;
 }
 
 extern "C" ut_status policy_forward(ut_env* h, const uint16_t* tokens_dev, const int32_t* n_ent_dev, uint16_t* h_dev,
@@ -199,6 +239,7 @@ extern "C" ut_status policy_forward(ut_env* h, const uint16_t* tokens_dev, const
     return UT_ERR_INVALID;
   }
   PolicyDev p = policy_dev(h);
+  p.ws_x = nullptr;
   p.NA = n_agents;
   p.NS = n_slots;
   p.R = 1 + n_slots;
@@ -211,7 +252,14 @@ extern "C" ut_status policy_forward(ut_env* h, const uint16_t* tokens_dev, const
   p.sample = actions_dev ? 1 : 0;
   p.counters = nullptr;
   p.step = step;
-  cudaError_t e = launch_policy(p, h->policy->d, (cudaStream_t)cuda_stream);
+  const cudaStream_t s = (cudaStream_t)cuda_stream;
+  void* ws = forward_ws(h, p, s);
+  if (ws) policy_ws_set(p, h->policy->d, ws);
+  cudaError_t e = launch_policy(p, h->policy->d, s);
+  if (ws) {
+    const cudaError_t ef = cudaFreeAsync(ws, s);
+    if (e == cudaSuccess) e = ef;
+  }
   if (e != cudaSuccess) {
     h->err = std::string("policy_forward: ") + cudaGetErrorString(e);
     return UT_ERR_CUDA;

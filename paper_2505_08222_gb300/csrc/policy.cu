@@ -33,6 +33,14 @@
 // layout (tc.cuh); each weight image is one contiguous bulk copy, streamed
 // through a three-slot shared-memory ring by the bulk-copy engine while the
 // CUDA cores work on the previous stage.
+//
+// The head reads the recurrent token alone, so behind the last block's
+// attention only one row in R matters.  Large batches run two kernels: kBody
+// stops there and hands each agent's attention output (BF16, the next
+// operand) and residual stream (FP32) of the recurrent row to kTail, which
+// takes the last block's Wo and FFN and the head for 128 agents per tile.
+// Small ones run kWhole, one kernel.  The arithmetic of a row is the same:
+// the results are equal bit for bit (policy_split says where the line lies).
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -177,11 +185,14 @@ __device__ __forceinline__ void stage_image(int s, size_t& off, uint32_t& bytes)
 }
 
 // Loader state, meaningful in thread 0 (the only thread that issues copies
-// and MMAs): stage `next` is the next image to fetch; slot s % kSlots may be
-// refilled once the MMA that read stage s - kSlots has completed.
+// and MMAs): stage `next` is the next image to fetch (stages count from the
+// kernel's first image, `base`); slot s % kSlots may be refilled once the MMA
+// that read stage s - kSlots has completed.
 struct Loader {
-  int next, done, total;
+  int next, done, total, base;
 };
+
+enum { kWhole = 0, kBody = 1, kTail = 2 };
 
 template <int D>
 __device__ __forceinline__ void pump(Loader& ld, const unsigned char* __restrict__ wimg, unsigned char* ring,
@@ -189,7 +200,7 @@ __device__ __forceinline__ void pump(Loader& ld, const unsigned char* __restrict
   while (ld.next < ld.total && ld.next < ld.done + kSlots) {
     size_t off;
     uint32_t bytes;
-    stage_image<D>(ld.next, off, bytes);
+    stage_image<D>(ld.base + ld.next, off, bytes);
     const int slot = ld.next % kSlots;
     tc::mbar_expect_tx(&full[slot], bytes);
     tc::bulk_g2s(ring + slot * Geo<D>::SLOT, wimg + off, bytes, &full[slot]);
@@ -749,7 +760,7 @@ __device__ __forceinline__ void attend_warp(uint32_t aQ, uint32_t aK, uint32_t a
     }
 }
 
-template <int D>
+template <int D, int MODE>
 __global__ void __launch_bounds__(Geo<D>::THREADS, D == 64 ? 2 : 1) policy_fwd_kernel(PolicyDev p) {
   pdl_wait();  // (dependents launch as this grid's CTAs exit: no early trigger in a many-wave kernel)
   using G = Geo<D>;
@@ -776,15 +787,18 @@ __global__ void __launch_bounds__(Geo<D>::THREADS, D == 64 ? 2 : 1) policy_fwd_k
   // row layout: agents of at most 16 tokens contiguous (slot * R + tok);
   // longer ones split: entity rows slot * NS + (tok - 1), then the recurrent
   // rows (tok 0) at NS * apt + slot; rows past those are padding (slot >= apt)
-  const bool split = p.R > 16;
+  // (kTail: the recurrent rows of 128 agents)
+  const bool split = MODE != kTail && p.R > 16;
   const int rb = p.NS * p.apt;
-  const int slot = split ? (row < rb ? row / p.NS : row - rb) : row / p.R;
-  const int tok = split ? (row < rb ? 1 + row - slot * p.NS : 0) : row - slot * p.R;
-  const long long ag = (long long)blockIdx.x * p.apt + slot;
-  const bool agent_ok = slot < p.apt && ag < p.NA;
-  const int n_tok = agent_ok ? 1 + min(max(p.n_ent[ag], 0), p.NS) : 0;
+  const int apt = MODE == kTail ? 128 : p.apt;
+  const int slot = MODE == kTail ? row : (split ? (row < rb ? row / p.NS : row - rb) : row / p.R);
+  const int tok = MODE == kTail ? 0 : (split ? (row < rb ? 1 + row - slot * p.NS : 0) : row - slot * p.R);
+  const long long ag = (long long)blockIdx.x * apt + slot;
+  // (an agent whose body tile gave up a wait has nothing to go on)
+  const bool agent_ok = slot < apt && ag < p.NA && (MODE != kTail || p.ws_ok[ag / p.apt] != 0);
+  const int n_tok = MODE == kTail ? (agent_ok ? 1 : 0) : (agent_ok ? 1 + min(max(p.n_ent[ag], 0), p.NS) : 0);
   const bool row_ok = tok < n_tok;
-  if (tid < p.apt) {
+  if (MODE != kTail && tid < p.apt) {
     const long long a2 = (long long)blockIdx.x * p.apt + tid;
     s_nent[tid] = a2 < p.NA ? min(max(p.n_ent[a2], 0), p.NS) : 0;
   }
@@ -817,7 +831,10 @@ __global__ void __launch_bounds__(Geo<D>::THREADS, D == 64 ? 2 : 1) policy_fwd_k
   }
   const uint32_t tl = tmem + ((uint32_t)(warp & 3) << 21);  // this warp's lane quarter (lane 32 (w % 4))
   const uint32_t aA = tc::smem_addr(sA), aH = tc::smem_addr(sH), aRing = tc::smem_addr(ring);
-  Loader ld{0, 0, p.L * G::NSTG};
+  constexpr int kAtt = 3;  // a layer's images before Wo
+  const int first = MODE == kTail ? (p.L - 1) * G::NSTG + kAtt : 0;
+  const int images = MODE == kBody ? (p.L - 1) * G::NSTG + kAtt : p.L * G::NSTG - first;
+  Loader ld{0, 0, images, first};
   if (tid == 0) pump<D>(ld, p.wimg, ring, full);
   uint32_t mphase = 0, phases = 0;  // bit k: parity of bar[k]
   bool ok = true;  // every bounded wait of this thread succeeded
@@ -865,11 +882,22 @@ __global__ void __launch_bounds__(Geo<D>::THREADS, D == 64 ? 2 : 1) policy_fwd_k
     for (int i = tid; i < G::VEC / 4; i += kThreads) cp_async16(dst + 4 * i, src + 4 * i);
     cp_async_commit();
   };
-  prefetch_vec(0);
+  prefetch_vec(MODE == kTail ? p.L - 1 : 0);
 
   // ---- token rows ----------------------------------------------------------
   float x[COLS];
-  if (row_ok && tok == 0) {
+  if (MODE == kTail && row_ok) {  // residual stream and attention output of the agent's recurrent row
+    const float4* xs = reinterpret_cast<const float4*>(p.ws_x + ag * D + c_lo);
+#pragma unroll
+    for (int c = 0; c < COLS; c += 4) {
+      const float4 v = xs[c / 4];
+      x[c] = v.x; x[c + 1] = v.y; x[c + 2] = v.z; x[c + 3] = v.w;
+    }
+#pragma unroll
+    for (int c = 0; c < COLS; c += 8)
+      *reinterpret_cast<uint4*>(sA + tc::kmajor_offset(row, c_lo + c, 128)) =
+          *reinterpret_cast<const uint4*>(p.ws_o + ag * D + c_lo + c);
+  } else if (MODE != kTail && row_ok && tok == 0) {
     const uint16_t* hp = p.h + ag * D + c_lo;
 #pragma unroll
     for (int c0 = 0; c0 < COLS; c0 += 16) {
@@ -878,7 +906,7 @@ __global__ void __launch_bounds__(Geo<D>::THREADS, D == 64 ? 2 : 1) policy_fwd_k
 #pragma unroll
       for (int i = 0; i < 16; ++i) x[c0 + i] = v[i];
     }
-  } else if (row_ok) {
+  } else if (MODE != kTail && row_ok) {
     const uint4 t4 = *reinterpret_cast<const uint4*>(p.tokens + (ag * p.NS + (tok - 1)) * 8);
     const float t[8] = {bf_lo(t4.x), bf_hi(t4.x), bf_lo(t4.y), bf_hi(t4.y),
                         bf_lo(t4.z), bf_hi(t4.z), bf_lo(t4.w), bf_hi(t4.w)};
@@ -900,11 +928,16 @@ __global__ void __launch_bounds__(Geo<D>::THREADS, D == 64 ? 2 : 1) policy_fwd_k
   } else {
 #pragma unroll
     for (int c = 0; c < COLS; ++c) x[c] = 0.0f;
+    if (MODE == kTail) {  // padding rows of the operand
+#pragma unroll
+      for (int c = 0; c < COLS; c += 8)
+        *reinterpret_cast<uint4*>(sA + tc::kmajor_offset(row, c_lo + c, 128)) = make_uint4(0u, 0u, 0u, 0u);
+    }
   }
 
   // Every thread runs every stage (the barriers stay uniform); a wait that
   // gave up only marks the result invalid.
-  for (int l = 0; l < p.L; ++l) {
+  for (int l = MODE == kTail ? p.L - 1 : 0; l < p.L; ++l) {
     float* vec = sVec + (l & 1) * G::VEC;  // double-buffered: the previous layer may still read its copy
     cp_async_wait_all();
     const float *ln1g = vec, *ln1b = vec + D, *bq = vec + 2 * D, *bk = vec + 3 * D, *bv = vec + 4 * D;
@@ -913,6 +946,7 @@ __global__ void __launch_bounds__(Geo<D>::THREADS, D == 64 ? 2 : 1) policy_fwd_k
     // ---- attention sub-block: the LayerNorm output in TMEM is the A
     // operand of Q, K and V (three MMA groups, each drained as it completes
     // while the later ones run) ----
+    if constexpr (MODE != kTail) {
     ln_part_to_tmem<D>(x, ln1g, ln1b, tl + G::COL_A + (uint32_t)(c_lo / 2), sStat, row, part);  // (publishes `vec`)
     publish();
     if (tid == 0) {
@@ -984,6 +1018,10 @@ __global__ void __launch_bounds__(Geo<D>::THREADS, D == 64 ? 2 : 1) policy_fwd_k
       }
     }
     if (l + 1 < p.L) prefetch_vec(l + 1);  // (buffer (l + 1) & 1 was last read in layer l - 1)
+    if constexpr (MODE == kBody) {
+      if (l == p.L - 1) break;
+    }
+    }
     publish();
     if (tid == 0) {
       wait_images(1);
@@ -1140,7 +1178,19 @@ __global__ void __launch_bounds__(Geo<D>::THREADS, D == 64 ? 2 : 1) policy_fwd_k
   // argmax with the lowest index among equal maxima).
   float* sY = reinterpret_cast<float*>(smem + G::KV_OFF);  // [apt][D]
   if (!ok) atomicExch(&bad, 1);
-  {
+  if constexpr (MODE == kBody) {  // hand the recurrent rows over
+    __syncthreads();  // every head's O is in sA
+    if (bad == 0 && agent_ok && tok == 0) {
+      float4* xs = reinterpret_cast<float4*>(p.ws_x + ag * D + c_lo);
+#pragma unroll
+      for (int c = 0; c < COLS; c += 4) xs[c / 4] = make_float4(x[c], x[c + 1], x[c + 2], x[c + 3]);
+#pragma unroll
+      for (int c = 0; c < COLS; c += 8)
+        *reinterpret_cast<uint4*>(p.ws_o + ag * D + c_lo + c) =
+            *reinterpret_cast<const uint4*>(sA + tc::kmajor_offset(row, c_lo + c, 128));
+    }
+    if (tid == 0) p.ws_ok[blockIdx.x] = bad == 0;
+  } else {
     float mean, inv;
     ln_part_stats<D>(x, sStat, row, part, mean, inv);
     if (agent_ok && tok == 0) {
@@ -1160,60 +1210,85 @@ __global__ void __launch_bounds__(Geo<D>::THREADS, D == 64 ? 2 : 1) policy_fwd_k
   }
   __syncthreads();
   const bool good = bad == 0;
+  // (kTail: four agents per warp at a time, for their independent chains)
+  constexpr int AG = MODE == kTail ? 4 : 1, NW = kThreads / 32;
 #pragma unroll 1
-  for (int sl = warp; sl < p.apt && good; sl += kThreads / 32) {
+  for (int sl = warp; MODE != kBody && sl < apt && good; sl += AG * NW) {
     const int lane = tid & 31, n_act = p.n_act;
-    const long long a2 = (long long)blockIdx.x * p.apt + sl;
-    if (a2 < p.NA) {  // (warp-uniform)
-      float y[D / 32];
+    long long a2[AG];
+    bool on[AG];  // (warp-uniform)
+    float y[AG][D / 32], mine[AG];  // mine: lane j's logit of action j
 #pragma unroll
-      for (int i = 0; i < D / 32; ++i) y[i] = sY[sl * D + lane + 32 * i];
-      float mine = 0.0f;  // lane j: logit of action j
-      for (int j0 = 0; j0 < n_act; j0 += 8) {
-        float acc[8];
+    for (int k = 0; k < AG; ++k) {
+      const int s2 = sl + k * NW;
+      a2[k] = (long long)blockIdx.x * apt + s2;
+      on[k] = s2 < apt && a2[k] < p.NA && (MODE != kTail || p.ws_ok[a2[k] / p.apt] != 0);
+      mine[k] = 0.0f;
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-          acc[jj] = 0.0f;
-          if (j0 + jj < n_act) {
-            const float* w = p.head_w + (size_t)(j0 + jj) * D + lane;
+      for (int i = 0; i < D / 32; ++i) y[k][i] = on[k] ? sY[s2 * D + lane + 32 * i] : 0.0f;
+    }
+    for (int j0 = 0; j0 < n_act; j0 += 8) {
+      float acc[AG][8];
 #pragma unroll
-            for (int i = 0; i < D / 32; ++i) acc[jj] = fmaf(__ldg(w + 32 * i), y[i], acc[jj]);
+      for (int jj = 0; jj < 8; ++jj) {
+#pragma unroll
+        for (int k = 0; k < AG; ++k) acc[k][jj] = 0.0f;
+        if (j0 + jj < n_act) {
+          const float* w = p.head_w + (size_t)(j0 + jj) * D + lane;
+#pragma unroll
+          for (int i = 0; i < D / 32; ++i) {
+            const float wi = __ldg(w + 32 * i);
+#pragma unroll
+            for (int k = 0; k < AG; ++k) acc[k][jj] = fmaf(wi, y[k][i], acc[k][jj]);
           }
         }
+      }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
+      for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-          for (int jj = 0; jj < 8; ++jj) acc[jj] += __shfl_xor_sync(0xffffffffu, acc[jj], o);
+        for (int k = 0; k < AG; ++k)
+#pragma unroll
+          for (int jj = 0; jj < 8; ++jj) acc[k][jj] += __shfl_xor_sync(0xffffffffu, acc[k][jj], o);
+#pragma unroll
+      for (int k = 0; k < AG; ++k)
 #pragma unroll
         for (int jj = 0; jj < 8; ++jj)
-          if (lane == j0 + jj) mine = acc[jj];
-      }
-      if (lane < n_act) {
-        mine += __ldg(p.head_b + lane);
-        p.logits[a2 * n_act + lane] = mine;
-      }
-      if (p.sample) {
-        float z = -INFINITY;
-        int arg = lane;
-        if (lane < n_act) {
+          if (lane == j0 + jj) mine[k] = acc[k][jj];
+    }
+    float z[AG];
+    int arg[AG];
+#pragma unroll
+    for (int k = 0; k < AG; ++k) {
+      z[k] = -INFINITY;
+      arg[k] = lane;
+      if (lane < n_act && on[k]) {
+        mine[k] += __ldg(p.head_b + lane);
+        p.logits[a2[k] * n_act + lane] = mine[k];
+        if (p.sample) {
           const uint32_t g = p.counters ? p.counters[0] + 1u : p.step;
-          const Rand4 r = philox(p.gid_agent + (uint32_t)a2, (uint32_t)(lane >> 2), g, TAG_GUMBEL, p.seed);
+          const Rand4 r = philox(p.gid_agent + (uint32_t)a2[k], (uint32_t)(lane >> 2), g, TAG_GUMBEL, p.seed);
           const int q = lane & 3;
           const uint32_t u = q == 0 ? r.x[0] : (q == 1 ? r.x[1] : (q == 2 ? r.x[2] : r.x[3]));
-          z = mine - logf(-logf(unif_mid(u)));
-          if (!(z == z)) z = -INFINITY;  // a NaN never wins
+          z[k] = mine[k] - logf(-logf(unif_mid(u)));
+          if (!(z[k] == z[k])) z[k] = -INFINITY;  // a NaN never wins
         }
+      }
+    }
+    if (p.sample) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const float oz = __shfl_xor_sync(0xffffffffu, z, o);
-          const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
-          if (oz > z || (oz == z && oa < arg)) {
-            z = oz;
-            arg = oa;
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < AG; ++k) {
+          const float oz = __shfl_xor_sync(0xffffffffu, z[k], o);
+          const int oa = __shfl_xor_sync(0xffffffffu, arg[k], o);
+          if (oz > z[k] || (oz == z[k] && oa < arg[k])) {
+            z[k] = oz;
+            arg[k] = oa;
           }
         }
-        if (lane == 0) p.actions[a2] = arg;
-      }
+#pragma unroll
+      for (int k = 0; k < AG; ++k)
+        if (lane == 0 && on[k]) p.actions[a2[k]] = arg[k];
     }
   }
 
@@ -1229,24 +1304,41 @@ __global__ void __launch_bounds__(Geo<D>::THREADS, D == 64 ? 2 : 1) policy_fwd_k
   if (warp == 0) tc::tmem_dealloc(tmem, G::TMEM_COLS);
 }
 
+template <int D, int MODE>
+cudaError_t launch_mode(const PolicyDev& p, cudaStream_t s) {
+  static std::atomic<unsigned long long> ready{0};
+  const cudaError_t e = smem_optin(policy_fwd_kernel<D, MODE>, Geo<D>::SMEM, ready);
+  if (e != cudaSuccess) return e;
+  const int apt = MODE == kTail ? 128 : p.apt;
+  const long long tiles = (p.NA + apt - 1) / apt;
+  return launch_pdl(policy_fwd_kernel<D, MODE>, dim3((unsigned)tiles), dim3(Geo<D>::THREADS), Geo<D>::SMEM, s, p);
+}
+
 template <int D>
 cudaError_t launch_policy_t(const PolicyDev& p, cudaStream_t s) {
-  static std::atomic<unsigned long long> ready{0};
-  {
-    const cudaError_t e = smem_optin(policy_fwd_kernel<D>, Geo<D>::SMEM, ready);
-    if (e != cudaSuccess) return e;
-  }
   // (a lane per action; the row layouts need R = 1 + NS and R apt <= 128)
   if (p.n_act < 1 || p.n_act > 32 || p.NS < 1 || p.NS > 16 || p.R != 1 + p.NS || p.apt < 1 || p.apt > 64 ||
       p.R * p.apt > 128)
     return cudaErrorInvalidValue;
-  const long long tiles = (p.NA + p.apt - 1) / p.apt;
-  if (tiles > 0) {
-    const cudaError_t e =
-        launch_pdl(policy_fwd_kernel<D>, dim3((unsigned)tiles), dim3(Geo<D>::THREADS), Geo<D>::SMEM, s, p);
-    if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
+  if (p.NA > 0 && !p.ws_x) e = launch_mode<D, kWhole>(p, s);
+  if (p.NA > 0 && p.ws_x) {
+    // body and tail over chunks of agents that share the workspace, in order
+    const long long chunk = policy_chunk(D, p.NA, p.apt);
+    for (long long a = 0; a < p.NA && e == cudaSuccess; a += chunk) {
+      PolicyDev q = p;
+      q.NA = p.NA - a < chunk ? p.NA - a : chunk;
+      q.tokens += a * p.NS * 8;
+      q.n_ent += a;
+      q.h += a * D;
+      q.logits += a * p.n_act;
+      if (q.actions) q.actions += a;
+      q.gid_agent += (uint32_t)a;
+      e = launch_mode<D, kBody>(q, s);
+      if (e == cudaSuccess) e = launch_mode<D, kTail>(q, s);
+    }
   }
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // Host-side packing of one [N x K] block (rows of a row-major matrix with
@@ -1318,6 +1410,37 @@ void policy_pack(int d, int L, int n_act, const float* prm, std::vector<unsigned
     std::memcpy(v + 12 * D, b2, D * 4);
   }
   head.assign(q, q + 2 * D + (size_t)n_act * D + n_act);  // lnf_g, lnf_b, Wh, bh
+}
+
+// Agents per body / tail pair: at most 3 (d = 128) or 2 (d = 64) waves of
+// tails, in whole body tiles; the workspace stays below 46 MB.
+long long policy_chunk(int d, long long NA, int apt) {
+  const long long most = (d == 64 ? 2 * 304 : 3 * 152) * 128 / apt * apt;
+  return NA < most ? NA : most;
+}
+
+// The tail adds the latency of a second kernel (about 22 us) and saves the last
+// block's Wo and FFN of all but its own tiles: even at three waves of tiles,
+// better beyond.  One kernel -> two, at 3, 4 and 12 waves: d = 64, L = 2, 11
+// tokens 115 -> 112, 152 -> 138, 441 -> 377 us; d = 128, L = 3, 17 tokens 178
+// -> 175, 236 -> 221, 704 -> 588; d = 128, L = 1 77 -> 72, 102 -> 85, 303 ->
+// 214.  131,072 agents of 17 tokens, d = 128, L = 3: 7.20 -> 5.94 ms.
+bool policy_split(int d, long long NA, int R) {
+  const long long tiles = (NA + 128 / R - 1) / (128 / R);
+  return tiles > 3 * (d == 64 ? 304 : 152);
+}
+
+size_t policy_ws_bytes(int d, long long NA, int R) {
+  const int apt = 128 / R;
+  const long long n = policy_chunk(d, NA, apt);
+  return (size_t)n * d * 6 + (size_t)((n + apt - 1) / apt) * 4;
+}
+
+void policy_ws_set(PolicyDev& p, int d, void* ws) {
+  const long long n = policy_chunk(d, p.NA, p.apt);
+  p.ws_x = static_cast<float*>(ws);
+  p.ws_o = reinterpret_cast<uint16_t*>(p.ws_x + n * d);
+  p.ws_ok = reinterpret_cast<int*>(p.ws_o + n * d);
 }
 
 cudaError_t launch_policy(const PolicyDev& p, int d, cudaStream_t s) {

@@ -37,6 +37,13 @@ struct PolicyDev {
   // barrier that nothing signals, for this many polls, and take the
   // timed-out path (status 2) before it issues any copy or MMA
   uint32_t test_wait_polls;
+  // Workspace of the two-kernel form (policy_ws_set), or NULL: one kernel.
+  // The recurrent rows after the last block's attention: residual stream
+  // [chunk][d], attention output [chunk][d] BF16; whether each body tile
+  // succeeded [tiles of a chunk].
+  float* ws_x;
+  uint16_t* ws_o;
+  int* ws_ok;
 };
 
 int64_t policy_param_count(int d, int L, int n_act);
@@ -45,5 +52,13 @@ size_t policy_layer_bytes(int d);
 void policy_pack(int d, int L, int n_act, const float* prm, std::vector<unsigned char>& img, std::vector<float>& vec,
                  std::vector<float>& emb, std::vector<float>& head);
 cudaError_t launch_policy(const PolicyDev& p, int d, cudaStream_t s);
+
+// The two-kernel form: whether it is the faster one for NA agents of R tokens,
+// its chunk of agents, the bytes of its workspace, and the workspace's use by
+// a launch.  Launches that may overlap need workspaces of their own.
+bool policy_split(int d, long long NA, int R);
+long long policy_chunk(int d, long long NA, int apt);
+size_t policy_ws_bytes(int d, long long NA, int R);
+void policy_ws_set(PolicyDev& p, int d, void* ws);
 
 }  // namespace ut
