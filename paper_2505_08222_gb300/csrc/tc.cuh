@@ -38,6 +38,12 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
   return d;
 }
 
+// The descriptor of the same operand `bytes` further on (a multiple of 16; the
+// 14-bit address field holds every shared-memory address): one add, where
+// building each K step's descriptors anew cost the issuing thread about 120
+// cycles per MMA.
+__device__ __forceinline__ uint64_t desc_advance(uint64_t d, uint32_t bytes) { return d + (bytes >> 4); }
+
 // Instruction descriptor of kind::f16 with BF16 A and B, FP32 accumulator,
 // both operands K-major, shape M x N (x K = 16).
 __host__ __device__ constexpr uint32_t idesc_bf16(uint32_t M, uint32_t N) {

@@ -382,8 +382,8 @@ __global__ void ln_fwd_kernel(const float* __restrict__ X, const float* __restri
 // gradient at the LayerNorm output), and per-block partial sums of dL/dg
 // (sum dY xh) and dL/db (sum dY) into part[block][2d] (blocks of 256
 // threads).  out may equal base.  REC (the last block's first LayerNorm):
-// base and dY0, a second gradient at the LayerNorm output, hold the recurrent
-// rows alone (row s T of the others at s) and are zero elsewhere.
+// row s T takes its gradient from dY0 at s instead of dY; base holds the
+// recurrent rows alone in the same way and is zero elsewhere.
 template <int DJ, bool REC>
 __global__ void ln_bwd_kernel(const float* __restrict__ dY, const float* __restrict__ X,
                               const float* __restrict__ stat, const float* __restrict__ gam, const float* base,
@@ -408,7 +408,7 @@ __global__ void ln_bwd_kernel(const float* __restrict__ dY, const float* __restr
       if (REC) {
         const long long c = s0 * d + lane + 32 * i;
         bn[i] = rec ? base[c] : 0.0f;
-        if (rec) dyn[i] += dY0[c];
+        if (rec) dyn[i] = dY0[c];
       } else {
         bn[i] = base[o];
       }
@@ -930,7 +930,8 @@ __global__ void __launch_bounds__(128, 6)
 // 14.3 ms, the critic's (32,768) from 4.40 to 3.24, d 128 with 17 tokens and 3
 // blocks (16,384) from 14.1 to 11.6.
 // One (sample, head) per warp.  Q0 [n][d] holds the recurrent queries, KV
-// [rows][2d] the keys and values of every token; P0 [n][H][T] and O0 [n][d]
+// [rows][2d] the keys and values of every token; dKV [rows][2d] and D0 [n][3d]
+// (dQ, dK, dV of the recurrent rows) are their gradients; P0 [n][H][T] and O0 [n][d]
 // are row 0 of P and O above, by the same arithmetic.  The cost is one read
 // of K and V (and in the backward one write of dK and dV).
 
@@ -983,7 +984,7 @@ __global__ void __launch_bounds__(256) attn0_fwd_kernel(const float* __restrict_
 template <int DH>
 __global__ void __launch_bounds__(256) attn0_bwd_kernel(const float* __restrict__ Q0, const float* __restrict__ KV,
                                                         const float* __restrict__ P0, const float* __restrict__ dO0,
-                                                        float* __restrict__ dQ0, float* __restrict__ dKV, long long n,
+                                                        float* __restrict__ D0, float* __restrict__ dKV, long long n,
                                                         int T, int H, float scale) {
   const int lane = threadIdx.x & 31;
   const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1018,9 +1019,13 @@ __global__ void __launch_bounds__(256) attn0_bwd_kernel(const float* __restrict_
       dq = fmaf(su, __ldg(K + u * ld + lane), dq);
       dK[u * ld + lane] = su * qj;
       dK[u * ld + d + lane] = pu * gj;
+      if (u == 0) {
+        D0[s * 3 * d + d + hh * DH + lane] = su * qj;
+        D0[s * 3 * d + 2 * d + hh * DH + lane] = pu * gj;
+      }
     }
   }
-  if (lane < DH) dQ0[s * d + hh * DH + lane] = dq;
+  if (lane < DH) D0[s * 3 * d + hh * DH + lane] = dq;
 }
 
 // The tensor-core path's form (T <= 16, head dimension 16): the products of
@@ -1117,7 +1122,7 @@ __global__ void __launch_bounds__(256)
 // the MMAs over the one query row give.
 __global__ void __launch_bounds__(256)
     attn0_bwd_mma_kernel(const float* __restrict__ Q0, const float* __restrict__ KV, const float* __restrict__ P0,
-                         const float* __restrict__ dO0, float* __restrict__ dQ0, float* __restrict__ dKV, long long n,
+                         const float* __restrict__ dO0, float* __restrict__ D0, float* __restrict__ dKV, long long n,
                          int T, int H, float scale) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1174,7 +1179,7 @@ __global__ void __launch_bounds__(256)
   if (g == 0) {
 #pragma unroll
     for (int j = 0; j < 2; ++j)
-      *reinterpret_cast<float2*>(dQ0 + s * d + hh * 16 + 8 * j + 2 * t) = make_float2(dq[j][0], dq[j][1]);
+      *reinterpret_cast<float2*>(D0 + s * 3 * d + hh * 16 + 8 * j + 2 * t) = make_float2(dq[j][0], dq[j][1]);
   }
   const float qv[4] = {q4.x, q4.y, q4.z, q4.w}, gv[4] = {g4.x, g4.y, g4.z, g4.w};
 #pragma unroll
@@ -1191,6 +1196,11 @@ __global__ void __launch_bounds__(256)
     }
     if (g + 8 * j < T) {
       float* out = dKV + (s * T + g + 8 * j) * ld + hh * 16 + 4 * t;
+      *reinterpret_cast<float4*>(out) = make_float4(a[0], a[1], a[2], a[3]);
+      *reinterpret_cast<float4*>(out + d) = make_float4(b[0], b[1], b[2], b[3]);
+    }
+    if (g == 0 && j == 0) {
+      float* out = D0 + s * 3 * d + d + hh * 16 + 4 * t;
       *reinterpret_cast<float4*>(out) = make_float4(a[0], a[1], a[2], a[3]);
       *reinterpret_cast<float4*>(out + d) = make_float4(b[0], b[1], b[2], b[3]);
     }
@@ -1551,11 +1561,11 @@ struct ut_tfm {
   // BF16 images of the block weights for the tensor-core path, per block l:
   // Wqkv, Wo, W1, W2 as B of the forward, then their transposes as B of the
   // input gradient (ImgSpec table on the device, packed once per call); the
-  // last block's Wqkv images hold Wk and Wv, and Wq and its transpose follow
-  // all blocks' images
+  // last block's Wqkv images hold Wk and Wv; Wq and its transpose, then the
+  // whole Wqkv and its transpose, follow all blocks' images
   uint16_t* wimg = nullptr;
-  std::vector<int64_t> img_off;  // [8 L + 2] offsets into wimg (elements)
-  int64_t* img_spec = nullptr;   // [8 L + 2][5] (weight offset, R, C, transpose, image offset)
+  std::vector<int64_t> img_off;  // [8 L + 4] offsets into wimg (elements)
+  int64_t* img_spec = nullptr;   // [8 L + 4][5] (weight offset, R, C, transpose, image offset)
   int n_img = 0, img_max = 0;
   int* status = nullptr;
 };
@@ -1603,6 +1613,7 @@ bool valid_config(const ut_tfm_config* c) {
 
 #include "tfm_tc.cuh"
 #include "tfm_ffn.cuh"
+#include "tfm_qkv.cuh"
 
 // Every BF16 weight image of the handle: grid (elements, image).
 __global__ void pack_images_kernel(const float* __restrict__ prm, const int64_t* __restrict__ spec,
@@ -1685,10 +1696,10 @@ cudaError_t reduce(const float* part, int nparts, long long len, long long strid
 }
 
 // dW[o][i] = sum_r dOut[r][o] In[r][i] and db[o] = sum_r dOut[r][o] over rows
-// r (rows of In ldi apart), split along the rows into partial slabs summed in
-// order.
-cudaError_t wgrad(ut_tfm* t, const float* dOut, int n_o, const float* In, long long ldi, int n_i, long long rows,
-                  float* gW, float* gb, cudaStream_t s) {
+// r (rows of dOut ldo and of In ldi apart), split along the rows into partial
+// slabs summed in order.
+cudaError_t wgrad(ut_tfm* t, const float* dOut, long long ldo, int n_o, const float* In, long long ldi, int n_i,
+                  long long rows, float* gW, float* gb, cudaStream_t s) {
   if (t->gemm_tc && rows > 0) {
     // tensor cores: (n_o / 128) x (n_i / 256) tiles x row splits, about as
     // many CTAs per SM as fit (three for n_i <= 128, else two), each split a
@@ -1706,7 +1717,7 @@ cudaError_t wgrad(ut_tfm* t, const float* dOut, int n_o, const float* In, long l
     long long rc = (rows + splits - 1) / splits;
     rc = (rc + kTcChunk - 1) / kTcChunk * kTcChunk;
     splits = (rows + rc - 1) / rc;
-    Gemm g = mk(dOut, n_o, In, ldi, t->part, n_i, n_o, n_i, rows, EPI_PARTIAL);
+    Gemm g = mk(dOut, ldo, In, ldi, t->part, n_i, n_o, n_i, rows, EPI_PARTIAL);
     g.kchunk = rc;
     g.status = t->status;
     dim3 grid((unsigned)((n_o + 127) / 128), (unsigned)((n_i + kTcMaxN - 1) / kTcMaxN), (unsigned)splits);
@@ -1717,7 +1728,7 @@ cudaError_t wgrad(ut_tfm* t, const float* dOut, int n_o, const float* In, long l
     if (e == cudaSuccess) e = reduce(bias_part, (int)splits, n_o, n_o, gb, s);
     return e;
   }
-  Gemm g = mk(dOut, n_o, In, ldi, t->part, n_i, n_o, n_i, rows, EPI_PARTIAL);
+  Gemm g = mk(dOut, ldo, In, ldi, t->part, n_i, n_o, n_i, rows, EPI_PARTIAL);
   const long long tiles = (long long)((n_o + 63) / 64) * ((n_i + 63) / 64);
   long long splits = (608 + tiles - 1) / tiles;
   splits = splits < 1 ? 1 : (splits > 128 ? 128 : splits);
@@ -1732,7 +1743,7 @@ cudaError_t wgrad(ut_tfm* t, const float* dOut, int n_o, const float* In, long l
   if (e != cudaSuccess) return e;
   long long nblk = (rows + 63) / 64;
   nblk = nblk < 1 ? 1 : (nblk > 256 ? 256 : nblk);
-  colsum_kernel<<<dim3((unsigned)((n_o + 31) / 32), (unsigned)nblk), 256, 0, s>>>(dOut, n_o, rows, n_o, t->part);
+  colsum_kernel<<<dim3((unsigned)((n_o + 31) / 32), (unsigned)nblk), 256, 0, s>>>(dOut, ldo, rows, n_o, t->part);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = reduce(t->part, (int)nblk, n_o, n_o, gb, s);
   return e;
@@ -1799,14 +1810,14 @@ cudaError_t attn0_fwd(const float* Q0, const float* KV, const int32_t* ne, const
 }
 
 template <int DH>
-cudaError_t attn0_bwd(const float* Q0, const float* KV, const float* P0, const float* dO0, float* dQ0, float* dKV,
+cudaError_t attn0_bwd(const float* Q0, const float* KV, const float* P0, const float* dO0, float* D0, float* dKV,
                       long long n, int T, int H, bool mma, cudaStream_t s) {
   const float scale = 1.0f / sqrtf((float)DH);
   const unsigned grid = blocks_for(n * H * 32, 256);
   if (mma && DH == 16 && T <= 16)
-    attn0_bwd_mma_kernel<<<grid, 256, 0, s>>>(Q0, KV, P0, dO0, dQ0, dKV, n, T, H, scale);
+    attn0_bwd_mma_kernel<<<grid, 256, 0, s>>>(Q0, KV, P0, dO0, D0, dKV, n, T, H, scale);
   else
-    attn0_bwd_kernel<DH><<<grid, 256, 0, s>>>(Q0, KV, P0, dO0, dQ0, dKV, n, T, H, scale);
+    attn0_bwd_kernel<DH><<<grid, 256, 0, s>>>(Q0, KV, P0, dO0, D0, dKV, n, T, H, scale);
   return cudaGetLastError();
 }
 
@@ -1862,6 +1873,24 @@ FfnArgs ffn_args(const ut_tfm* t, int l, const float* M, float* out, long long r
   return a;
 }
 
+// Arguments of block l's LayerNorm and Q, K, V (tfm_qkv.cuh), last block's form
+// included.
+QkvArgs qkv_args(const ut_tfm* t, int l, const Block& b, long long rows) {
+  const int64_t* ol = t->off.data() + 2 + 12 * l;
+  QkvArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.X = b.X;
+  a.gain = t->prm + ol[T_LN1G];
+  a.off = t->prm + ol[T_LN1B];
+  a.bias = t->prm + ol[T_BQKV];
+  a.qkv = b.QKV;
+  a.q0 = b.Q0;
+  a.rows = rows;
+  a.T = l == t->L - 1 ? t->T : 0;
+  a.status = t->status;
+  return a;
+}
+
 template <int DJ, int DH, typename TokT>
 cudaError_t forward(ut_tfm* t, const Call& c, cudaStream_t s) {
   constexpr int d = 32 * DJ;
@@ -1901,18 +1930,28 @@ cudaError_t forward(ut_tfm* t, const Call& c, cudaStream_t s) {
     const bool last = l == t->L - 1;
     const long long m = last ? c.n : rows;  // rows after the attention: the recurrent tokens alone in the last block
     const Block b = block_of(t, l);
-    e = ln_fwd<DJ>(b.X, w + ol[T_LN1G], w + ol[T_LN1B], b.Y1, b.S1, rows, s);
+    const bool fused = t->gemm_tc && d == kFfD;
+    if (fused) {
+      QkvArgs a = qkv_args(t, l, b, rows);
+      a.w = last ? img(t->L, 2) : img(l, 0);
+      e = qkv_fwd(a, s);
+    } else {
+      e = ln_fwd<DJ>(b.X, w + ol[T_LN1G], w + ol[T_LN1B], b.Y1, b.S1, rows, s);
+    }
     if (e != cudaSuccess) break;
     if (last) {
+      if (!fused) {
       e = gemm0(mk(b.Y1, d, w + ol[T_WQKV] + d * d, d, b.QKV, 2 * d, rows, 2 * d, d, EPI_BIAS), ol[T_BQKV] + d,
                 img(l, 0));
       if (e == cudaSuccess)  // the recurrent rows of Y1 are T d apart
         e = gemm0(mk(b.Y1, (long long)t->T * d, w + ol[T_WQKV], d, b.Q0, d, c.n, d, d, EPI_BIAS), ol[T_BQKV],
                   img(t->L, 0));
+      }
       if (e == cudaSuccess)
         e = attn0_fwd<DH>(b.Q0, b.QKV, c.ne, c.sel, b.P, b.O, c.n, t->T, t->NS, t->H, t->gemm_tc != 0, s);
     } else {
-      e = gemm0(mk(b.Y1, d, w + ol[T_WQKV], d, b.QKV, 3 * d, rows, 3 * d, d, EPI_BIAS), ol[T_BQKV], img(l, 0));
+      if (!fused)
+        e = gemm0(mk(b.Y1, d, w + ol[T_WQKV], d, b.QKV, 3 * d, rows, 3 * d, d, EPI_BIAS), ol[T_BQKV], img(l, 0));
       if (e == cudaSuccess)
         e = attn_fwd<DH>(b.QKV, c.ne, c.sel, b.P, b.O, c.n, t->T, t->NS, t->H, t->gemm_tc != 0, s);
     }
@@ -1921,7 +1960,7 @@ cudaError_t forward(ut_tfm* t, const Call& c, cudaStream_t s) {
     g.R = b.X;
     g.ldr = last ? (long long)t->T * d : d;
     e = gemm0(g, ol[T_BO], img(l, 1));
-    if (t->gemm_tc && d == kFfD) {
+    if (fused) {
       if (e == cudaSuccess) e = ffn_fwd(ffn_args(t, l, b.M, b.X + MR * d, m), s);
       continue;
     }
@@ -1973,34 +2012,57 @@ cudaError_t backward(ut_tfm* t, const Call& c, float* grad, cudaStream_t s) {
       Gemm g = mk(t->dX, d, w + ol[T_W2], 4 * d, t->dBig, 4 * d, m, 4 * d, d, EPI_GELU_GRAD);
       g.aux = b.Z;
       e = dgemm(l, 7, g);
-      if (e == cudaSuccess) e = wgrad(t, t->dX, d, b.G, 4 * d, 4 * d, m, grad + ol[T_W2], grad + ol[T_B2], s);
+      if (e == cudaSuccess) e = wgrad(t, t->dX, d, d, b.G, 4 * d, 4 * d, m, grad + ol[T_W2], grad + ol[T_B2], s);
       if (e == cudaSuccess) e = dgemm(l, 6, mk(t->dBig, 4 * d, w + ol[T_W1], d, t->dY, d, m, d, 4 * d, EPI_STORE));
-      if (e == cudaSuccess) e = wgrad(t, t->dBig, 4 * d, b.Y2, d, d, m, grad + ol[T_W1], grad + ol[T_B1], s);
+      if (e == cudaSuccess) e = wgrad(t, t->dBig, 4 * d, 4 * d, b.Y2, d, d, m, grad + ol[T_W1], grad + ol[T_B1], s);
       if (e == cudaSuccess)
         e = ln_bwd<DJ, false>(t, t->dY, b.M, b.S2, w + ol[T_LN2G], t->dX, t->dM, grad + ol[T_LN2G], m, s);
     }
     // attention sub-block: M = X + Wo attn(LN1(X)) + bo
     if (e == cudaSuccess) e = dgemm(l, 5, mk(t->dM, d, w + ol[T_WO], d, t->dO, d, m, d, d, EPI_STORE));
-    if (e == cudaSuccess) e = wgrad(t, t->dM, d, b.O, d, d, m, grad + ol[T_WO], grad + ol[T_BO], s);
+    if (e == cudaSuccess) e = wgrad(t, t->dM, d, d, b.O, d, d, m, grad + ol[T_WO], grad + ol[T_BO], s);
     if (e != cudaSuccess) break;
+    const bool fused = t->gemm_tc && d == kFfD;
+    float* D0 = t->dBig + rows * 2 * d;  // behind dKV: [n][3d] of the 2d n T floats that are left (T >= 2)
+    if (fused) {
+      if (last)
+        e = attn0_bwd<DH>(b.Q0, b.QKV, b.P, t->dO, D0, t->dBig, c.n, t->T, t->H, true, s);
+      else
+        e = attn_bwd<DH>(b.QKV, b.P, t->dO, t->dBig, c.n, t->T, t->H, true, s);
+      QkvArgs a = qkv_args(t, l, b, rows);
+      a.w = t->wimg + t->img_off[last ? 8 * t->L + 3 : 8 * l + 4];
+      a.dqkv = t->dBig;
+      a.dq0 = D0;
+      a.base = t->dM;
+      a.out = t->dX;
+      a.slab = t->part;
+      a.vec = t->part + (long long)kQkvCtas * kQkvSlab;
+      int ctas = 0;
+      if (e == cudaSuccess) e = qkv_bwd(a, &ctas, s);
+      if (e == cudaSuccess) e = reduce(a.slab, ctas, kQkvSlab, kQkvSlab, grad + ol[T_WQKV], s);
+      if (e == cudaSuccess) e = reduce(a.vec, ctas, kQkvN, kQkvVec, grad + ol[T_BQKV], s);
+      if (e == cudaSuccess) e = reduce(a.vec + kQkvN, ctas, 2 * kFfD, kQkvVec, grad + ol[T_LN1G], s);
+      continue;
+    }
     if (last) {
-      // dQ0 in dX, then its product with Wq in dO (both are free by then)
+      // the recurrent rows' input gradient is a product of its own, over dQ,
+      // dK and dV in one sum as in the other blocks
       const float* Wq = w + ol[T_WQKV];
-      e = attn0_bwd<DH>(b.Q0, b.QKV, b.P, t->dO, t->dX, t->dBig, c.n, t->T, t->H, t->gemm_tc != 0, s);
+      e = attn0_bwd<DH>(b.Q0, b.QKV, b.P, t->dO, D0, t->dBig, c.n, t->T, t->H, t->gemm_tc != 0, s);
       if (e == cudaSuccess)
         e = dgemm(l, 4, mk(t->dBig, 2 * d, Wq + d * d, d, t->dY, d, rows, d, 2 * d, EPI_STORE));
-      if (e == cudaSuccess) e = dgemm(t->L, 1, mk(t->dX, d, Wq, d, t->dO, d, c.n, d, d, EPI_STORE));
+      if (e == cudaSuccess) e = dgemm(t->L, 3, mk(D0, 3 * d, Wq, d, t->dO, d, c.n, d, 3 * d, EPI_STORE));
       if (e == cudaSuccess)
-        e = wgrad(t, t->dBig, 2 * d, b.Y1, d, d, rows, grad + ol[T_WQKV] + d * d, grad + ol[T_BQKV] + d, s);
+        e = wgrad(t, t->dBig, 2 * d, 2 * d, b.Y1, d, d, rows, grad + ol[T_WQKV] + d * d, grad + ol[T_BQKV] + d, s);
       if (e == cudaSuccess)
-        e = wgrad(t, t->dX, d, b.Y1, (long long)t->T * d, d, c.n, grad + ol[T_WQKV], grad + ol[T_BQKV], s);
+        e = wgrad(t, D0, 3 * d, d, b.Y1, (long long)t->T * d, d, c.n, grad + ol[T_WQKV], grad + ol[T_BQKV], s);
       if (e == cudaSuccess)
         e = ln_bwd<DJ, true>(t, t->dY, b.X, b.S1, w + ol[T_LN1G], t->dM, t->dX, grad + ol[T_LN1G], rows, s, t->dO);
       continue;
     }
     e = attn_bwd<DH>(b.QKV, b.P, t->dO, t->dBig, c.n, t->T, t->H, t->gemm_tc != 0, s);
     if (e == cudaSuccess) e = dgemm(l, 4, mk(t->dBig, 3 * d, w + ol[T_WQKV], d, t->dY, d, rows, d, 3 * d, EPI_STORE));
-    if (e == cudaSuccess) e = wgrad(t, t->dBig, 3 * d, b.Y1, d, d, rows, grad + ol[T_WQKV], grad + ol[T_BQKV], s);
+    if (e == cudaSuccess) e = wgrad(t, t->dBig, 3 * d, 3 * d, b.Y1, d, d, rows, grad + ol[T_WQKV], grad + ol[T_BQKV], s);
     if (e == cudaSuccess)
       e = ln_bwd<DJ, false>(t, t->dY, b.X, b.S1, w + ol[T_LN1G], t->dM, t->dX, grad + ol[T_LN1G], rows, s);
   }
@@ -2200,8 +2262,9 @@ extern "C" ut_status tfm_create(const ut_tfm_config* cfg, const float* params_ho
     for (int tr = 0; tr < 2; ++tr)
       for (int k = 0; k < 4; ++k) add_img(woff[k], rows_w[k], cols_w[k], tr);
   }
-  for (int tr = 0; tr < 2; ++tr) add_img(t->off[2 + 12 * (t->L - 1) + T_WQKV], t->d, t->d, tr);
-  t->n_img = 8 * t->L + 2;
+  for (int n : {1, 3})
+    for (int tr = 0; tr < 2; ++tr) add_img(t->off[2 + 12 * (t->L - 1) + T_WQKV], n * t->d, t->d, tr);
+  t->n_img = 8 * t->L + 4;
   t->wimg = (uint16_t*)dalloc(t, (size_t)img_total * 2);
   t->img_spec = (int64_t*)dalloc(t, spec.size() * 8);
   t->status = (int*)dalloc(t, 4);

@@ -14,8 +14,8 @@
 // gradients accumulate in tensor memory over all of a CTA's tiles.  What
 // bounds both is the CUDA cores' work per hidden value (erf, and in the
 // backward the exponential of its derivative) and the chain of stages within a
-// tile.  1.97 M rows (163,840 samples' two blocks): forward 0.93 ms, backward
-// 1.68 ms; the actor's gradient step 14.3 -> 10.4 ms, the critic's (32,768
+// tile.  1.97 M rows (163,840 samples' two blocks): forward 0.78 ms, backward
+// 1.46 ms; the actor's gradient step 14.3 -> 10.4 ms, the critic's (32,768
 // samples) 3.24 -> 2.33.  It also serves small calls: 5 launches and 5
 // reductions become 1 and 5.
 //
@@ -33,8 +33,13 @@
 constexpr int kFfD = 64, kFfH = 256;                 // width, hidden width
 constexpr size_t kFfW = (size_t)kFfD * kFfH * 2;     // one weight image (32 KB)
 constexpr size_t kFfA = (size_t)128 * 64 * 2;        // operand tile of 64 features (16 KB)
-constexpr size_t kFfFwdSmem = 2 * kFfW + 3 * kFfA;   // W1, W2; Y2, two G chunks: two CTAs per SM
-constexpr size_t kFfBwdSmem = 3 * kFfW + 2 * kFfA + 4 * kFfA + 128 * 64 * 4;  // 224 KB, one CTA per SM
+// Tiles written a row per warp have their 8-feature groups 2048 + 32 bytes
+// apart: the four groups of a store fall into different banks.  (Not in the
+// forward here, where 112 KB is the most that two CTAs per SM can have.)
+constexpr uint32_t kRowGrp = 2048 + 32;
+constexpr size_t kRowA = 8 * (size_t)kRowGrp;
+constexpr size_t kFfFwdSmem = 2 * kFfW + 3 * kFfA;  // W1, W2; Y2, two G chunks
+constexpr size_t kFfBwdSmem = 3 * kFfW + 2 * kRowA + 4 * kFfA + 128 * 64 * 4;  // 224 KB, one CTA per SM
 constexpr int kFfSlab = 2 * kFfD * kFfH;             // per-CTA partials: dW1 [256][64], dW2 [64][256]
 constexpr int kFfVec = kFfH + 3 * kFfD;              // and db1, db2, d(ln2 gain), d(ln2 offset)
 constexpr uint32_t kMnMajorA = 1u << 15, kMnMajorB = 1u << 16;  // instruction descriptor: transposed operands
@@ -52,21 +57,25 @@ struct FfnArgs {
   int* status;
 };
 
-// D[128 x 64] (+)= A[128 x 64] B[64 x 64]^T, both K-major; B's rows `b_rows`
-// apart in its image.
-__device__ __forceinline__ void ffn_mma(uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t b_rows, bool accumulate) {
+// D[128 x 64] (+)= A[128 x 64] B[64 x 64]^T, both K-major; A's 8-feature groups
+// `a_grp` bytes apart, B's image `b_rows` rows high.
+__device__ __forceinline__ void ffn_mma(uint32_t d_tmem, uint32_t a, uint32_t a_grp, uint32_t b, uint32_t b_rows,
+                                        bool accumulate) {
   constexpr uint32_t idesc = tc::idesc_bf16(128, 64);
+  const uint64_t ad = tc::smem_desc(a, a_grp, 128), bd = tc::smem_desc(b, b_rows * 16, 128);
 #pragma unroll
   for (int j = 0; j < 4; ++j)
-    tc::mma_bf16(d_tmem, tc::smem_desc(a + j * 2 * 128 * 16, 128 * 16, 128),
-                 tc::smem_desc(b + j * 2 * b_rows * 16, b_rows * 16, 128), idesc, (accumulate || j > 0) ? 1u : 0u);
+    tc::mma_bf16(d_tmem, tc::desc_advance(ad, j * 2 * a_grp), tc::desc_advance(bd, j * 2 * b_rows * 16), idesc,
+                 (accumulate || j > 0) ? 1u : 0u);
 }
-// D[128 x 64] (+)= A^T B over the tile's 128 token rows: A 128 features, B 64.
+// D[128 x 64] (+)= A^T B over the tile's 128 token rows: A 128 features (groups
+// 2048 bytes apart), B 64 (kRowGrp).
 __device__ __forceinline__ void ffn_mma_rows(uint32_t d_tmem, uint32_t a, uint32_t b, bool accumulate) {
   constexpr uint32_t idesc = tc::idesc_bf16(128, 64) | kMnMajorA | kMnMajorB;
+  const uint64_t ad = tc::smem_desc(a, 128, 128 * 16), bd = tc::smem_desc(b, 128, kRowGrp);
 #pragma unroll
   for (int j = 0; j < 8; ++j)
-    tc::mma_bf16(d_tmem, tc::smem_desc(a + j * 256, 128, 128 * 16), tc::smem_desc(b + j * 256, 128, 128 * 16), idesc,
+    tc::mma_bf16(d_tmem, tc::desc_advance(ad, j * 256), tc::desc_advance(bd, j * 256), idesc,
                  (accumulate || j > 0) ? 1u : 0u);
 }
 __device__ __forceinline__ void ffn_publish() {
@@ -75,8 +84,67 @@ __device__ __forceinline__ void ffn_publish() {
   __syncthreads();
   tc::fence_after_sync();
 }
-__device__ __forceinline__ void st_bf(unsigned char* img, int row, int c, float v) {
-  *reinterpret_cast<uint16_t*>(img + tc::kmajor_offset(row, c, 128)) = f2bf_bits(v);
+// Rows `row` and `row` + 1 of a tile from lanes that hold one column of each
+// (column c0 + lane): neighbouring lanes trade, so that each stores two columns
+// of one row.
+__device__ __forceinline__ void st_bf_rows(unsigned char* img, uint32_t grp, int row, int c0, float va, float vb) {
+  const int odd = threadIdx.x & 1, c = c0 + (threadIdx.x & 30);
+  const float got = __shfl_xor_sync(0xffffffffu, odd ? va : vb, 1);
+  *reinterpret_cast<uint32_t*>(img + (c >> 3) * grp + (row + odd) * 16 + (c & 7) * 2) =
+      odd ? pack_bf2(got, vb) : pack_bf2(va, got);
+}
+// LayerNorm of N rows on the warp, lane: columns `lane` and `lane` + 32 of each
+// (the arithmetic of ln_fwd_kernel): x becomes (x - mean) rstd, rs the rstd.
+template <int N>
+__device__ __forceinline__ void rows_normalise(float (&x)[N][2], float (&rs)[N]) {
+  float v[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) v[i] = x[i][0] + x[i][1];
+  const float mean = row_sums(v) * (1.0f / 64);
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const float m = row_get<N>(mean, i);
+    x[i][0] -= m;
+    x[i][1] -= m;
+    v[i] = 0.0f;
+    v[i] += x[i][0] * x[i][0];
+    v[i] += x[i][1] * x[i][1];
+  }
+  const float rstd = 1.0f / sqrtf(row_sums(v) * (1.0f / 64) + 1e-5f);
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    rs[i] = row_get<N>(rstd, i);
+    x[i][0] *= rs[i];
+    x[i][1] *= rs[i];
+  }
+}
+// LayerNorm backward of N rows (the arithmetic of ln_bwd_kernel): y the
+// gradient at the LayerNorm output, xh and rs from rows_normalise; y becomes
+// the residual's gradient res plus the gradient at its input (one rounding), pg
+// and pb gather the gain's and offset's.
+template <int N>
+__device__ __forceinline__ void rows_ln_bwd(float (&y)[N][2], const float (*xh)[2], const float* rs,
+                                            const float (*res)[2], float g0, float g1, float (&pg)[2],
+                                            float (&pb)[2]) {
+  float s1[N], s2[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    pg[0] = fmaf(y[i][0], xh[i][0], pg[0]);
+    pg[1] = fmaf(y[i][1], xh[i][1], pg[1]);
+    pb[0] += y[i][0];
+    pb[1] += y[i][1];
+    y[i][0] *= g0;
+    y[i][1] *= g1;
+    s1[i] = y[i][0] + y[i][1];
+    s2[i] = fmaf(y[i][1], xh[i][1], y[i][0] * xh[i][0]);
+  }
+  const float t1 = row_sums(s1) * (1.0f / 64), t2 = row_sums(s2) * (1.0f / 64);
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const float m1 = row_get<N>(t1, i), m2 = row_get<N>(t2, i);
+    y[i][0] = fmaf(rs[i], y[i][0] - m1 - xh[i][0] * m2, res[i][0]);
+    y[i][1] = fmaf(rs[i], y[i][1] - m1 - xh[i][1] * m2, res[i][1]);
+  }
 }
 __device__ __forceinline__ void st8_bf(unsigned char* img, int row, int c, const float* v) {
   *reinterpret_cast<uint4*>(img + tc::kmajor_offset(row, c, 128)) =
@@ -99,8 +167,8 @@ struct Bar {
 // a 64-wide hidden chunk.  The MMAs of chunk c + 1's pre-activations and of
 // chunk c - 1's output product run during chunk c's GELU.
 __global__ void __launch_bounds__(256, 2) ffn_fwd_kernel(FfnArgs a) {
-  extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* sW1 = smem;
+  extern __shared__ __align__(128) unsigned char sm_tile[];  // (a wider alignment would cost the second CTA)
+  unsigned char* sW1 = sm_tile;
   unsigned char* sW2 = sW1 + kFfW;
   unsigned char* sY = sW2 + kFfW;
   unsigned char* sG = sY + kFfA;               // two chunks
@@ -139,20 +207,21 @@ __global__ void __launch_bounds__(256, 2) ffn_fwd_kernel(FfnArgs a) {
       x[i][0] = in ? __ldg(a.M + (r0 + i) * 64 + lane) : 0.0f;
       x[i][1] = in ? __ldg(a.M + (r0 + i) * 64 + lane + 32) : 0.0f;
     }
+    {
+      float y[16][2], rs[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const float mean = warp_sum(x[i][0] + x[i][1]) * (1.0f / 64);
-      float v = 0.0f;
-      v += (x[i][0] - mean) * (x[i][0] - mean);
-      v += (x[i][1] - mean) * (x[i][1] - mean);
-      const float rstd = 1.0f / sqrtf(warp_sum(v) * (1.0f / 64) + 1e-5f);
-      st_bf(sY, warp * 16 + i, lane, (x[i][0] - mean) * rstd * g0 + f0);
-      st_bf(sY, warp * 16 + i, lane + 32, (x[i][1] - mean) * rstd * g1 + f1);
+      for (int i = 0; i < 16; ++i) y[i][0] = x[i][0], y[i][1] = x[i][1];
+      rows_normalise(y, rs);
+#pragma unroll
+      for (int i = 0; i < 16; i += 2) {
+        st_bf_rows(sY, 2048, warp * 16 + i, 0, y[i][0] * g0 + f0, y[i + 1][0] * g0 + f0);
+        st_bf_rows(sY, 2048, warp * 16 + i, 32, y[i][1] * g1 + f1, y[i + 1][1] * g1 + f1);
+      }
     }
     ffn_publish();
     if (tid == 0) {
       if (first) ok &= tc::mbar_wait(&bars[4], 0u, kTcPolls);
-      ffn_mma(tmem, aY, aW1, kFfH, false);
+      ffn_mma(tmem, aY, 2048, aW1, kFfH, false);
       tc::mma_commit(&bars[0]);
     }
 #pragma unroll 1
@@ -161,7 +230,7 @@ __global__ void __launch_bounds__(256, 2) ffn_fwd_kernel(FfnArgs a) {
       if (c >= 2) ok &= (c & 1) ? o1.wait() : o0.wait();  // chunk c - 2's output product has read G buffer c & 1
       tc::fence_after_sync();
       if (tid == 0 && c < 3) {
-        ffn_mma(tmem + 64 * ((c + 1) & 1), aY, aW1 + (c + 1) * 64 * 16, kFfH, false);
+        ffn_mma(tmem + 64 * ((c + 1) & 1), aY, 2048, aW1 + (c + 1) * 64 * 16, kFfH, false);
         tc::mma_commit(&bars[(c + 1) & 1]);
       }
       unsigned char* g = sG + (c & 1) * kFfA;
@@ -180,7 +249,7 @@ __global__ void __launch_bounds__(256, 2) ffn_fwd_kernel(FfnArgs a) {
       for (int j = 0; j < 32; j += 8) st8_bf(g, row, half * 32 + j, v + j);
       ffn_publish();
       if (tid == 0) {
-        ffn_mma(tmem + kOut, aG + (c & 1) * (uint32_t)kFfA, aW2 + c * 8 * 64 * 16, kFfD, c > 0);
+        ffn_mma(tmem + kOut, aG + (c & 1) * (uint32_t)kFfA, 2048, aW2 + c * 8 * 64 * 16, kFfD, c > 0);
         tc::mma_commit(&bars[2 + (c & 1)]);
       }
     }
@@ -225,13 +294,13 @@ __global__ void __launch_bounds__(256, 2) ffn_fwd_kernel(FfnArgs a) {
 // GELU and its derivative with a thread per row and quarter of a 64-wide
 // hidden chunk.
 __global__ void __launch_bounds__(512, 1) ffn_bwd_kernel(FfnArgs a) {
-  extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* sW1 = smem;               // W1: pre-activations
+  extern __shared__ __align__(128) unsigned char sm_tile[];
+  unsigned char* sW1 = sm_tile;            // W1: pre-activations
   unsigned char* sW2t = sW1 + kFfW;        // W2^T: gradient at the GELU output
   unsigned char* sW1t = sW2t + kFfW;       // W1^T: gradient at the LayerNorm output
   unsigned char* sY = sW1t + kFfW;         // LayerNorm output
-  unsigned char* sD = sY + kFfA;           // dX'
-  unsigned char* sG = sD + kFfA;           // GELU outputs of a 128-wide hidden pair of chunks
+  unsigned char* sD = sY + kRowA;          // dX'
+  unsigned char* sG = sD + kRowA;          // GELU outputs of a 128-wide hidden pair of chunks
   unsigned char* sZ = sG + 2 * kFfA;       // gradients at its pre-activations
   float* sE = reinterpret_cast<float*>(sZ + 2 * kFfA);  // staging [128][64]
   __shared__ __align__(8) uint64_t bars[4];  // chunk products, pair products, output product, weights
@@ -260,7 +329,7 @@ __global__ void __launch_bounds__(512, 1) ffn_bwd_kernel(FfnArgs a) {
   }
   Bar chunk{&bars[0], 0}, pair{&bars[1], 0}, dy_bar{&bars[2], 0};
   const float g0 = a.gain[lane], g1 = a.gain[lane + 32], f0 = a.off[lane], f1 = a.off[lane + 32];
-  float pg0 = 0.0f, pg1 = 0.0f, pb0 = 0.0f, pb1 = 0.0f, pd0 = 0.0f, pd1 = 0.0f;  // LN gain, offset; db2
+  float pg[2] = {0.0f, 0.0f}, pb[2] = {0.0f, 0.0f}, pd0 = 0.0f, pd1 = 0.0f;  // LN gain, offset; db2
   float pz[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // db1 of hidden 64 c + 16 part + lane % 16 over this warp's rows
   const long long tiles = (a.rows + 127) / 128;
   bool ok = true, first = true;
@@ -281,30 +350,28 @@ __global__ void __launch_bounds__(512, 1) ffn_bwd_kernel(FfnArgs a) {
     const long long r0 = mt * 128 + warp * 8;
     float xh[8][2], dx[8][2], rs[8];  // normalised rows, dX', 1 / std
 #pragma unroll
+    for (int i = 0; i < 8; ++i) xh[i][0] = xn[i][0], xh[i][1] = xn[i][1];
+    rows_normalise(xh, rs);
+#pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const float x0 = xn[i][0], x1 = xn[i][1];
-      const float mean = warp_sum(x0 + x1) * (1.0f / 64);
-      float v = 0.0f;
-      v += (x0 - mean) * (x0 - mean);
-      v += (x1 - mean) * (x1 - mean);
-      rs[i] = 1.0f / sqrtf(warp_sum(v) * (1.0f / 64) + 1e-5f);
-      xh[i][0] = (x0 - mean) * rs[i];
-      xh[i][1] = (x1 - mean) * rs[i];
       dx[i][0] = dn[i][0];
       dx[i][1] = dn[i][1];
       pd0 += dx[i][0];
       pd1 += dx[i][1];
+    }
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
       const int r = warp * 8 + i;
-      st_bf(sY, r, lane, xh[i][0] * g0 + f0);
-      st_bf(sY, r, lane + 32, xh[i][1] * g1 + f1);
-      st_bf(sD, r, lane, dx[i][0]);
-      st_bf(sD, r, lane + 32, dx[i][1]);
+      st_bf_rows(sY, kRowGrp, r, 0, xh[i][0] * g0 + f0, xh[i + 1][0] * g0 + f0);
+      st_bf_rows(sY, kRowGrp, r, 32, xh[i][1] * g1 + f1, xh[i + 1][1] * g1 + f1);
+      st_bf_rows(sD, kRowGrp, r, 0, dx[i][0], dx[i + 1][0]);
+      st_bf_rows(sD, kRowGrp, r, 32, dx[i][1], dx[i + 1][1]);
     }
     ffn_publish();
     if (tid == 0) {
       if (first) ok &= tc::mbar_wait(&bars[3], 0u, kTcPolls);
-      ffn_mma(tmem + kPre, aY, aW1, kFfH, false);
-      ffn_mma(tmem + kGrad, aD, aW2t, kFfH, false);
+      ffn_mma(tmem + kPre, aY, kRowGrp, aW1, kFfH, false);
+      ffn_mma(tmem + kGrad, aD, kRowGrp, aW2t, kFfH, false);
       tc::mma_commit(&bars[0]);
     }
 #pragma unroll 1
@@ -320,8 +387,8 @@ __global__ void __launch_bounds__(512, 1) ffn_bwd_kernel(FfnArgs a) {
         __syncthreads();
         tc::fence_after_sync();
         if (tid == 0) {
-          ffn_mma(tmem + kPre, aY, aW1 + (c + 1) * 64 * 16, kFfH, false);
-          ffn_mma(tmem + kGrad, aD, aW2t + (c + 1) * 64 * 16, kFfH, false);
+          ffn_mma(tmem + kPre, aY, kRowGrp, aW1 + (c + 1) * 64 * 16, kFfH, false);
+          ffn_mma(tmem + kGrad, aD, kRowGrp, aW2t + (c + 1) * 64 * 16, kFfH, false);
           tc::mma_commit(&bars[0]);
         }
       }
@@ -351,7 +418,7 @@ __global__ void __launch_bounds__(512, 1) ffn_bwd_kernel(FfnArgs a) {
         if (k == c) pz[k] += s;
       ffn_publish();
       if (tid == 0) {
-        ffn_mma(tmem + kDy, aZ + (c & 1) * 8 * 2048, aW1t + c * 8 * 64 * 16, kFfD, c > 0);
+        ffn_mma(tmem + kDy, aZ + (c & 1) * 8 * 2048, 2048, aW1t + c * 8 * 64 * 16, kFfD, c > 0);
         if (c & 1) {
           ffn_mma_rows(tmem + kW1 + (c >> 1) * 64, aZ, aY, !first);
           ffn_mma_rows(tmem + kW2 + (c >> 1) * 64, aG, aD, !first);
@@ -375,25 +442,20 @@ __global__ void __launch_bounds__(512, 1) ffn_bwd_kernel(FfnArgs a) {
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
+    {
+      float y[8][2];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int r = warp * 8 + i;
-      const float y0 = sE[epi_pos(r, lane >> 2) + (lane & 3)], y1 = sE[epi_pos(r, 8 + (lane >> 2)) + (lane & 3)];
-      const float q0 = y0 * g0, q1 = y1 * g1;
-      pg0 = fmaf(y0, xh[i][0], pg0);
-      pg1 = fmaf(y1, xh[i][1], pg1);
-      pb0 += y0;
-      pb1 += y1;
-      float m1 = 0.0f, m2 = 0.0f;
-      m1 += q0;
-      m2 = fmaf(q0, xh[i][0], m2);
-      m1 += q1;
-      m2 = fmaf(q1, xh[i][1], m2);
-      m1 = warp_sum(m1) * (1.0f / 64);
-      m2 = warp_sum(m2) * (1.0f / 64);
-      if (r0 + i < a.rows) {
-        a.out[(r0 + i) * 64 + lane] = dx[i][0] + rs[i] * (q0 - m1 - xh[i][0] * m2);
-        a.out[(r0 + i) * 64 + lane + 32] = dx[i][1] + rs[i] * (q1 - m1 - xh[i][1] * m2);
+      for (int i = 0; i < 8; ++i) {
+        y[i][0] = sE[epi_pos(warp * 8 + i, lane >> 2) + (lane & 3)];
+        y[i][1] = sE[epi_pos(warp * 8 + i, 8 + (lane >> 2)) + (lane & 3)];
+      }
+      rows_ln_bwd(y, xh, rs, dx, g0, g1, pg, pb);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if (r0 + i < a.rows) {
+          a.out[(r0 + i) * 64 + lane] = y[i][0];
+          a.out[(r0 + i) * 64 + lane + 32] = y[i][1];
+        }
       }
     }
     // (the next tile's LayerNorm writes sY and sD, whose MMAs are done; sE is
@@ -431,10 +493,10 @@ __global__ void __launch_bounds__(512, 1) ffn_bwd_kernel(FfnArgs a) {
     float* l = s_l + warp * 192;
     l[lane] = pd0;
     l[lane + 32] = pd1;
-    l[64 + lane] = pg0;
-    l[96 + lane] = pg1;
-    l[128 + lane] = pb0;
-    l[160 + lane] = pb1;
+    l[64 + lane] = pg[0];
+    l[96 + lane] = pg[1];
+    l[128 + lane] = pb[0];
+    l[160 + lane] = pb[1];
     __syncthreads();
     float* vec = a.vec + (long long)blockIdx.x * kFfVec;
     if (tid < kFfH) {
