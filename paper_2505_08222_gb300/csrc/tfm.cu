@@ -286,10 +286,23 @@ __global__ void __launch_bounds__(256) sgemm128_kernel(Gemm g) {
   }
 }
 
+// The entity tokens of one sample, 4 slots per register: lane i of v[j] holds
+// feature i % 8 of slot 4 j + i / 8 (one coalesced load for 4 tokens), zero for
+// slots past the sample's ne entities.  A feature then comes by one shuffle.
+constexpr int kTokRegs = (UT_MAX_AGENTS + UT_MAX_TARGETS + 3) / 4;
+template <typename TokT>
+__device__ __forceinline__ void load_tokens(const TokT* __restrict__ tok, long long bs, int NS, int ne, int lane,
+                                            float (&v)[kTokRegs]) {
+#pragma unroll
+  for (int j = 0; j < kTokRegs; ++j)
+    v[j] = 4 * j + (lane >> 3) < ne ? (float)tok[(bs * NS + 4 * j) * 8 + lane] : 0.0f;
+}
+
 // Embedding of the entity tokens; token 0 of each sample is its recurrent
-// embedding.  Warps loop over token rows (lane: outputs lane + 32 i, its
-// rows of W and its biases held in registers; a row's 8 token features read
-// once).
+// embedding.  Warps loop over samples (lane: outputs lane + 32 i, its rows of W
+// and its biases held in registers).  Bound by its writes; a warp per token row,
+// with a 64-bit division and eight scalar loads per row, took 265 us for
+// 163,840 samples of 11 tokens, this 92.
 template <typename TokT, int DJ>
 __global__ void __launch_bounds__(256) embed_kernel(const TokT* __restrict__ tok, const int32_t* __restrict__ n_ent,
                                                     const float* __restrict__ h, const int32_t* __restrict__ sel,
@@ -306,32 +319,28 @@ __global__ void __launch_bounds__(256) embed_kernel(const TokT* __restrict__ tok
 #pragma unroll
     for (int k = 0; k < 8; ++k) wr[i][k] = W[(lane + 32 * i) * 8 + k];
   }
-  for (long long row = w0; row < n * T; row += nw) {
-    const long long s = row / T;
-    const int t = (int)(row - s * T);
+  for (long long s = w0; s < n; s += nw) {
     const long long bs = sel ? (long long)sel[s] : s;
-    float* x = X + row * d;
-    if (t == 0) {
-#pragma unroll
-      for (int i = 0; i < DJ; ++i) x[lane + 32 * i] = h[bs * d + lane + 32 * i];
-      continue;
-    }
     int ne = n_ent[bs];
     ne = ne < 0 ? 0 : (ne > NS ? NS : ne);
-    float q[8];
+    float v[kTokRegs];
+    load_tokens(tok, bs, NS, ne, lane, v);
+    float* x = X + s * T * d + lane;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) q[k] = 0.0f;
-    if (t <= ne) {
-      const TokT* qt = tok + (bs * NS + (t - 1)) * 8;
+    for (int i = 0; i < DJ; ++i) x[32 * i] = h[bs * d + lane + 32 * i];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) q[k] = (float)qt[k];
-    }
+    for (int t = 0; t < 4 * kTokRegs; ++t) {
+      if (t >= NS) break;  // (warp-uniform)
+      float q[8];
 #pragma unroll
-    for (int i = 0; i < DJ; ++i) {
-      float acc = br[i];
+      for (int k = 0; k < 8; ++k) q[k] = __shfl_sync(0xffffffffu, v[t / 4], 8 * (t & 3) + k);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) acc = fmaf(wr[i][k], q[k], acc);
-      x[lane + 32 * i] = acc;
+      for (int i = 0; i < DJ; ++i) {
+        float acc = br[i];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc = fmaf(wr[i][k], q[k], acc);
+        x[(t + 1) * d + 32 * i] = acc;
+      }
     }
   }
 }
@@ -1223,9 +1232,16 @@ struct HeadArgs {
   double* spart;     // [warps][4] partial sums of the per-sample statistics
 };
 
-// Final LayerNorm and head on the recurrent token, one warp per sample; in the loss modes
-// also the loss, dL/d(head output), the head's and final LayerNorm's
-// backward, and per-warp partial sums of their parameter gradients.
+// Final LayerNorm and head on the recurrent token, one warp per sample; in the
+// loss modes also the loss, dL/d(head output), the head's and final
+// LayerNorm's backward, and per-warp partial sums of their parameter
+// gradients.  NO: a compile-time bound of n_out, so that the outputs' dot
+// products and exponentials are independent chains.  A sample's row, its index
+// and then the values gathered by it are loaded during the previous sample.
+// The statistics are summed in double: each lane keeps one sample's terms and
+// all 32 are added at once (the FP64 pipe takes a warp instruction for 16
+// cycles).  163,840 samples, 7 outputs: 146 us (583 with
+// neither).
 template <int DJ, int NO>
 __global__ void __launch_bounds__(256) head_kernel(HeadArgs a) {
   constexpr int d = 32 * DJ;
@@ -1233,7 +1249,7 @@ __global__ void __launch_bounds__(256) head_kernel(HeadArgs a) {
   const long long w0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
   const int no = a.n_out;
-  float gW[NO][DJ], gB[NO], gg[DJ], gb[DJ];
+  float gW[NO][DJ], gB[NO], gg[DJ], gb[DJ], lg[DJ], lb[DJ];
 #pragma unroll
   for (int o = 0; o < NO; ++o) {
     gB[o] = 0.0f;
@@ -1241,16 +1257,53 @@ __global__ void __launch_bounds__(256) head_kernel(HeadArgs a) {
     for (int i = 0; i < DJ; ++i) gW[o][i] = 0.0f;
   }
 #pragma unroll
-  for (int i = 0; i < DJ; ++i) gg[i] = gb[i] = 0.0f;
+  for (int i = 0; i < DJ; ++i) {
+    gg[i] = gb[i] = 0.0f;
+    lg[i] = a.lnf_g[lane + 32 * i];
+    lb[i] = a.lnf_b[lane + 32 * i];
+  }
   double st[4] = {0.0, 0.0, 0.0, 0.0};
-  for (long long s = w0; s < a.n; s += nw) {
-    const float* x0 = a.XL + s * d;
+  float keep[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  auto flush = [&]() {
+    st[0] += a.mode == 2 ? (double)keep[0] * keep[0] : (double)keep[0];
+#pragma unroll
+    for (int k = 1; k < 4; ++k) st[k] += (double)keep[k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) keep[k] = 0.0f;
+  };
+  float xn[DJ], f0 = 0.0f, f1 = 0.0f;  // next sample: row; logp_old and advantage, or return
+  int an = 0;                          // and its action
+  long long bn = 0;                    // and its batch row
+  auto fetch_row = [&](long long s) {
+#pragma unroll
+    for (int i = 0; i < DJ; ++i) xn[i] = a.XL[s * d + lane + 32 * i];
+    bn = a.mode != 0 && a.sel ? (long long)a.sel[s] : s;
+  };
+  auto fetch_batch = [&]() {
+    if (a.mode == 1) {
+      an = a.actions[bn];
+      f0 = a.logp_old[bn];
+      f1 = a.adv[bn];
+    } else if (a.mode == 2) {
+      f0 = a.ret[bn];
+    }
+  };
+  if (w0 < a.n) {
+    fetch_row(w0);
+    fetch_batch();
+  }
+  int it = 0;
+  for (long long s = w0; s < a.n; s += nw, ++it) {
+    const bool more = s + nw < a.n;
+    const float lo = f0, A = f1;
+    const int act = an;
     float x[DJ], xh[DJ], U[DJ], sum = 0.0f;
 #pragma unroll
     for (int i = 0; i < DJ; ++i) {
-      x[i] = x0[lane + 32 * i];
+      x[i] = xn[i];
       sum += x[i];
     }
+    if (more) fetch_row(s + nw);
     const float mean = warp_sum(sum) * (1.0f / d);
     float v = 0.0f;
 #pragma unroll
@@ -1258,21 +1311,24 @@ __global__ void __launch_bounds__(256) head_kernel(HeadArgs a) {
     const float rstd = 1.0f / sqrtf(warp_sum(v) * (1.0f / d) + 1e-5f);
 #pragma unroll
     for (int i = 0; i < DJ; ++i) {
-      const int j = lane + 32 * i;
       xh[i] = (x[i] - mean) * rstd;
-      U[i] = xh[i] * a.lnf_g[j] + a.lnf_b[j];
+      U[i] = xh[i] * lg[i] + lb[i];
     }
     float z[NO];
 #pragma unroll
     for (int o = 0; o < NO; ++o) {
       z[o] = 0.0f;
-      if (o < no) {
-        float acc = 0.0f;
 #pragma unroll
-        for (int i = 0; i < DJ; ++i) acc = fmaf(a.Wh[o * d + lane + 32 * i], U[i], acc);
-        z[o] = warp_sum(acc) + a.bh[o];
-      }
+      for (int i = 0; i < DJ; ++i) z[o] = fmaf(o < no ? __ldg(a.Wh + o * d + lane + 32 * i) : 0.0f, U[i], z[o]);
     }
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1)
+#pragma unroll
+      for (int o = 0; o < NO; ++o) z[o] += __shfl_xor_sync(0xffffffffu, z[o], k);
+#pragma unroll
+    for (int o = 0; o < NO; ++o)
+      if (o < no) z[o] += __ldg(a.bh + o);
+    if (more) fetch_batch();
     if (a.mode == 0) {
       if (lane < no) {
 #pragma unroll
@@ -1284,15 +1340,14 @@ __global__ void __launch_bounds__(256) head_kernel(HeadArgs a) {
         for (int i = 0; i < DJ; ++i) a.h_out[s * d + lane + 32 * i] = x[i];
       continue;
     }
-    const long long bs = a.sel ? (long long)a.sel[s] : s;
-    float dz[NO];
+    float dz[NO], stat[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     if (a.mode == 2) {
-      const float e = z[0] - a.ret[bs];
+      const float e = z[0] - lo;
 #pragma unroll
       for (int o = 0; o < NO; ++o) dz[o] = 0.0f;
       dz[0] = 2.0f * e * a.inv_n;
-      st[0] += (double)e * e;
-      st[1] += (double)z[0];
+      stat[0] = e;
+      stat[1] = z[0];
     } else {
       float mx = -INFINITY;
 #pragma unroll
@@ -1303,16 +1358,17 @@ __global__ void __launch_bounds__(256) head_kernel(HeadArgs a) {
       for (int o = 0; o < NO; ++o)
         if (o < no) zs += expf(z[o] - mx);
       const float lse = mx + logf(zs);
-      const int act = a.actions[bs];
-      float ent = 0.0f, lpa = 0.0f;
+      float ent = 0.0f, lpa = 0.0f, p[NO];
 #pragma unroll
-      for (int o = 0; o < NO; ++o)
+      for (int o = 0; o < NO; ++o) {
+        p[o] = 0.0f;
         if (o < no) {
           const float lp = z[o] - lse;
-          ent -= expf(lp) * lp;
+          p[o] = expf(lp);
+          ent -= p[o] * lp;
           if (o == act) lpa = lp;
         }
-      const float A = a.adv[bs], lo = a.logp_old[bs];
+      }
       const float r = expf(lpa - lo);
       const float rc = fminf(fmaxf(r, 1.0f - a.clip_eps), 1.0f + a.clip_eps);
       const float s1 = r * A, s2 = rc * A;
@@ -1321,33 +1377,36 @@ __global__ void __launch_bounds__(256) head_kernel(HeadArgs a) {
       for (int o = 0; o < NO; ++o) {
         dz[o] = 0.0f;
         if (o < no) {
-          const float lp = z[o] - lse, p = expf(lp);
-          dz[o] = (gl * ((o == act ? 1.0f : 0.0f) - p) + a.ent_coef * p * (lp + ent)) * a.inv_n;
+          const float lp = z[o] - lse;
+          dz[o] = (gl * ((o == act ? 1.0f : 0.0f) - p[o]) + a.ent_coef * p[o] * (lp + ent)) * a.inv_n;
         }
       }
-      st[0] += (double)(-fminf(s1, s2) - a.ent_coef * ent);
-      st[1] += (double)ent;
-      st[2] += fabsf(r - 1.0f) > a.clip_eps ? 1.0 : 0.0;
-      st[3] += (double)(lo - lpa);
+      stat[0] = -fminf(s1, s2) - a.ent_coef * ent;
+      stat[1] = ent;
+      stat[2] = fabsf(r - 1.0f) > a.clip_eps ? 1.0f : 0.0f;
+      stat[3] = lo - lpa;
     }
+    if (lane == (it & 31)) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) keep[k] = stat[k];
+    }
+    if ((it & 31) == 31) flush();
     float dU[DJ];
 #pragma unroll
     for (int i = 0; i < DJ; ++i) dU[i] = 0.0f;
 #pragma unroll
-    for (int o = 0; o < NO; ++o)
-      if (o < no) {
-        gB[o] += dz[o];
+    for (int o = 0; o < NO; ++o) {
+      gB[o] += dz[o];
 #pragma unroll
-        for (int i = 0; i < DJ; ++i) {
-          gW[o][i] = fmaf(dz[o], U[i], gW[o][i]);
-          dU[i] = fmaf(a.Wh[o * d + lane + 32 * i], dz[o], dU[i]);
-        }
+      for (int i = 0; i < DJ; ++i) {
+        gW[o][i] = fmaf(dz[o], U[i], gW[o][i]);
+        dU[i] = fmaf(o < no ? __ldg(a.Wh + o * d + lane + 32 * i) : 0.0f, dz[o], dU[i]);
       }
+    }
     float dxh[DJ], m1 = 0.0f, m2 = 0.0f;
 #pragma unroll
     for (int i = 0; i < DJ; ++i) {
-      const int j = lane + 32 * i;
-      dxh[i] = dU[i] * a.lnf_g[j];
+      dxh[i] = dU[i] * lg[i];
       gg[i] = fmaf(dU[i], xh[i], gg[i]);
       gb[i] += dU[i];
       m1 += dxh[i];
@@ -1360,6 +1419,9 @@ __global__ void __launch_bounds__(256) head_kernel(HeadArgs a) {
     for (int i = 0; i < DJ; ++i) dx0[lane + 32 * i] = rstd * (dxh[i] - m1 - xh[i] * m2);
   }
   if (a.mode == 0) return;
+  flush();
+#pragma unroll
+  for (int k = 0; k < 4; ++k) st[k] = warp_sum_d(st[k]);
   const long long plen = 2 * d + (long long)no * d + no;
   float* pp = a.part + w0 * plen;
 #pragma unroll
@@ -1380,7 +1442,8 @@ __global__ void __launch_bounds__(256) head_kernel(HeadArgs a) {
 
 // Embedding weight gradients, one warp per sample: per-warp partial sums of
 // dW_emb[j][k] = sum dX[row][j] tok[row][k] and db_emb[j] over the sample's
-// entity rows, into part[warp][9d] (W_emb then b_emb).
+// entity rows, into part[warp][9d] (W_emb then b_emb).  163,840 samples of 10
+// entities, d = 64: 163 us (315 with a token's loads waited for one by one).
 template <typename TokT, int DJ>
 __global__ void __launch_bounds__(256) embed_grad_kernel(const TokT* __restrict__ tok,
                                                          const int32_t* __restrict__ n_ent,
@@ -1398,23 +1461,40 @@ __global__ void __launch_bounds__(256) embed_grad_kernel(const TokT* __restrict_
 #pragma unroll
     for (int k = 0; k < 8; ++k) gW[i][k] = 0.0f;
   }
+  long long bn = 0;  // batch row and entities of the next sample, in flight during the current one
+  int nn = 0;
+  if (w0 < n) {
+    bn = sel ? (long long)sel[w0] : w0;
+    nn = n_ent[bn];
+  }
   for (long long s = w0; s < n; s += nw) {
-    const long long bs = sel ? (long long)sel[s] : s;
-    int ne = n_ent[bs];
-    ne = ne < 0 ? 0 : (ne > NS ? NS : ne);
-    for (int t = 1; t <= ne; ++t) {
-      const TokT* q = tok + (bs * NS + (t - 1)) * 8;
-      float tk[8];
+    const long long bs = bn;
+    const int ne = nn < 0 ? 0 : (nn > NS ? NS : nn);
+    float v[kTokRegs];
+    load_tokens(tok, bs, NS, ne, lane, v);
+    if (s + nw < n) bn = sel ? (long long)sel[s + nw] : s + nw;
+    const float* g0 = dX + (s * T + 1) * d + lane;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) tk[k] = (float)q[k];
+    for (int j = 0; j < kTokRegs; ++j) {
+      if (4 * j >= ne) break;  // (warp-uniform)
+      float g[4][DJ];  // four tokens' gradients at a time
 #pragma unroll
-      for (int i = 0; i < DJ; ++i) {
-        const float g = dX[(s * T + t) * d + lane + 32 * i];
-        gb[i] += g;
+      for (int t = 0; t < 4; ++t)
 #pragma unroll
-        for (int k = 0; k < 8; ++k) gW[i][k] = fmaf(g, tk[k], gW[i][k]);
+        for (int i = 0; i < DJ; ++i) g[t][i] = 4 * j + t < ne ? g0[(4 * j + t) * d + 32 * i] : 0.0f;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+#pragma unroll
+        for (int i = 0; i < DJ; ++i) gb[i] += g[t][i];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const float q = __shfl_sync(0xffffffffu, v[j], 8 * t + k);
+#pragma unroll
+          for (int i = 0; i < DJ; ++i) gW[i][k] = fmaf(g[t][i], q, gW[i][k]);
+        }
       }
     }
+    if (s + nw < n) nn = n_ent[bn];
   }
   float* pp = part + w0 * 9 * d;
 #pragma unroll
@@ -1907,7 +1987,7 @@ cudaError_t forward(ut_tfm* t, const Call& c, cudaStream_t s) {
     return t->gemm_tc ? t->wimg + t->img_off[8 * l + which] : nullptr;
   };
   {
-    const unsigned blocks = (unsigned)std::min<long long>((rows + 7) / 8, 152LL * 16);
+    const unsigned blocks = (unsigned)std::min<long long>((c.n + 7) / 8, 152LL * 8);
     const TokT* tk = (const TokT*)c.tok;
     if (d == 32)
       embed_kernel<TokT, 1><<<blocks, 256, 0, s>>>(tk, c.ne, c.h, c.sel, w + o[0], w + o[1], t->X, c.n, t->T, t->NS);
@@ -2099,6 +2179,8 @@ cudaError_t run(ut_tfm* t, const Call& c, int mode, const HeadArgs& ha_in, float
   ha.spart = t->spart;
   if (t->n_out == 1)
     head_kernel<DJ, 1><<<kRowBlocks, 256, 0, s>>>(ha);
+  else if (t->n_out <= 8)
+    head_kernel<DJ, 8><<<kRowBlocks, 256, 0, s>>>(ha);
   else
     head_kernel<DJ, 16><<<kRowBlocks, 256, 0, s>>>(ha);
   e = cudaGetLastError();
