@@ -25,6 +25,7 @@
 
 #include "../../include/utrack.h"
 #include "common.cuh"
+#include "f32x2.cuh"
 #include "tc.cuh"
 #include "tfm.cuh"
 #include "warp_sums.cuh"
@@ -468,171 +469,235 @@ __global__ void ln_bwd_kernel(const float* __restrict__ dY, const float* __restr
   }
 }
 
-// Attention work items: pair q = s * H + head.  A warp takes hp = 2 pairs
-// when 2T <= 32 (lanes 0..T-1 the first, T..2T-1 the second), else one.
-__host__ __device__ __forceinline__ int attn_pairs_per_warp(int T) { return 2 * T <= 32 ? 2 : 1; }
-constexpr int kAttnStage = 32;  // staged rows per warp: hp * T <= 32
+// FP32 attention (the CUDA-core path, and on the tensor-core path heads other
+// than 16 wide or samples of 17 tokens).  A block of 128 threads takes
+// 128 / T consecutive (sample, head) items q = s * H + head, a thread per query
+// token (119 of 128 threads busy at T = 17; a warp per item kept 17 of 32
+// lanes).  Rows are staged in shared memory by 16-byte loads; P goes through
+// it too, so that a block's P, one contiguous range, is read and written whole.
+// The products run on packed FP32 pairs: two keys of a score at once (staged
+// interleaved), two columns of an output at once, so each sum keeps its order.
+// Bound by issue and shared-memory loads: 131,072 items of 17 x 16 forward 274 us
+// (534 before), backward 524 (809).
+constexpr int kAttnThreads = 128;
+__host__ __device__ __forceinline__ int attn_items(int T) { return kAttnThreads / T; }
+constexpr size_t kAttnSmemMax = 112 * 1024;  // above attn_bwd_smem for every T and head width
+// Shared-memory floats: rows staged as they are, and key pairs (T rounded up
+// to even per item).
+__host__ __device__ __forceinline__ int attn_rows(int T) { return attn_items(T) * T; }
+__host__ __device__ __forceinline__ int attn_pair_rows(int T) { return attn_items(T) * ((T + 1) / 2 * 2); }
+inline size_t attn_fwd_smem(int T, int DH) {
+  const int kv = attn_rows(T) * DH + attn_pair_rows(T) * DH, p = attn_rows(T) * T;
+  return (size_t)(kv > p ? kv : p) * 4;
+}
+inline size_t attn_bwd_smem(int T, int DH) {
+  return ((size_t)3 * attn_rows(T) * DH + (size_t)attn_pair_rows(T) * DH + 2 * (size_t)attn_rows(T) * T + 4) * 4;
+}
 
-// Self-attention, lane (slot, t) = query token t of pair q0 + slot:
-// P[s][head][t][u] (zero for masked keys u > n_ent) and O = P V.  The warp
-// first copies its pairs' K and V rows to shared memory.  4 warps per block.
+// Column j of key u in the interleaved layout of an item's rows.
 template <int DH>
-__global__ void __launch_bounds__(128) attn_fwd_kernel(const float* __restrict__ QKV,
-                                                       const int32_t* __restrict__ n_ent,
-                                                       const int32_t* __restrict__ sel, float* __restrict__ P,
-                                                       float* __restrict__ O, long long n, int T, int NS, int H,
-                                                       float scale) {
-  __shared__ float sk[4][kAttnStage * DH];
-  __shared__ float sv[4][kAttnStage * DH];
-  const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-  const int hp = attn_pairs_per_warp(T);
-  const long long q0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * hp;
-  const long long nq = n * H;
-  if (q0 >= nq) return;  // whole warps leave together
-  const int d = DH * H, ld = 3 * d;
-  for (int i = lane; i < hp * T * DH; i += 32) {
-    const int slot = i / (T * DH), r = i - slot * T * DH, u = r / DH, j = r - u * DH;
-    const long long q = q0 + slot;
-    if (q < nq) {
-      const long long s = q / H;
-      const float* base = QKV + s * T * ld + (q - s * H) * DH;
-      sk[wl][i] = base[u * ld + d + j];
-      sv[wl][i] = base[u * ld + 2 * d + j];
+__device__ __forceinline__ int pair_pos(int u, int j) {
+  return (u >> 1) * 2 * DH + 2 * j + (u & 1);
+}
+
+// acc[u] = sum_j x[j] K[u][j] over the keys of an item (pairs), j in order.
+template <int DH>
+__device__ __forceinline__ void attn_dots(const float (&x)[DH], const float* pairs, int T, float (&acc)[kMaxT + 1]) {
+#pragma unroll
+  for (int u = 0; u < kMaxT; u += 2) {
+    acc[u] = acc[u + 1] = 0.0f;
+    if (u < T) {
+      const float4* k4 = reinterpret_cast<const float4*>(pairs + (u >> 1) * 2 * DH);
+      unsigned long long s = 0ull;
+#pragma unroll
+      for (int j = 0; j < DH; j += 2) {
+        const float4 k = k4[j / 2];  // (u, j), (u + 1, j), (u, j + 1), (u + 1, j + 1)
+        s = f2fma(f2pk(x[j], x[j]), f2pk(k.x, k.y), s);
+        s = f2fma(f2pk(x[j + 1], x[j + 1]), f2pk(k.z, k.w), s);
+      }
+      f2upk(s, acc[u], acc[u + 1]);
     }
   }
-  __syncwarp();
-  const int slot = lane / T, t = lane - slot * T;
-  const long long q = q0 + slot;
-  if (slot >= hp || q >= nq) return;
-  const long long s = q / H;
+}
+
+// o[j] += p row[j] on pairs of columns.
+template <int DH>
+__device__ __forceinline__ void attn_axpy(float p, const float* row, unsigned long long (&o)[DH / 2]) {
+  const float4* r4 = reinterpret_cast<const float4*>(row);
+  const unsigned long long pp = f2pk(p, p);
+#pragma unroll
+  for (int j = 0; j < DH / 4; ++j) {
+    const float4 v = r4[j];
+    o[2 * j] = f2fma(pp, f2pk(v.x, v.y), o[2 * j]);
+    o[2 * j + 1] = f2fma(pp, f2pk(v.z, v.w), o[2 * j + 1]);
+  }
+}
+
+template <int DH>
+__device__ __forceinline__ void attn_store(float* dst, const unsigned long long (&o)[DH / 2]) {
+#pragma unroll
+  for (int j = 0; j < DH / 4; ++j) {
+    float4 v;
+    f2upk(o[2 * j], v.x, v.y);
+    f2upk(o[2 * j + 1], v.z, v.w);
+    reinterpret_cast<float4*>(dst)[j] = v;
+  }
+}
+
+// P[s][head][t][u] (zero for masked keys u > n_ent) and O = P V.
+template <int DH>
+__global__ void __launch_bounds__(kAttnThreads) attn_fwd_kernel(const float* __restrict__ QKV,
+                                                                const int32_t* __restrict__ n_ent,
+                                                                const int32_t* __restrict__ sel, float* __restrict__ P,
+                                                                float* __restrict__ O, long long n, int T, int NS,
+                                                                int H, float scale) {
+  extern __shared__ __align__(16) float sm_attn[];
+  const int tid = threadIdx.x, ipb = attn_items(T), Tp = (T + 1) / 2 * 2;
+  float* sV = sm_attn;                       // [items][T][DH]
+  float* sK = sV + attn_rows(T) * DH;        // [items][Tp / 2][DH][2]
+  const long long q0 = (long long)blockIdx.x * ipb, nq = n * H;
+  const int items = (int)(nq - q0 < ipb ? nq - q0 : ipb);
+  const int d = DH * H, ld = 3 * d;
+  for (int i = tid; i < items * T * (DH / 4); i += kAttnThreads) {
+    const int r = i / (DH / 4), c = i - r * (DH / 4), it = r / T, u = r - it * T;
+    const long long q = q0 + it, s = q / H;
+    const float* src = QKV + (s * T + u) * ld + d + (q - s * H) * DH + 4 * c;
+    const float4 k = __ldg(reinterpret_cast<const float4*>(src));
+    float* dst = sK + it * Tp * DH;
+    dst[pair_pos<DH>(u, 4 * c)] = k.x;
+    dst[pair_pos<DH>(u, 4 * c + 1)] = k.y;
+    dst[pair_pos<DH>(u, 4 * c + 2)] = k.z;
+    dst[pair_pos<DH>(u, 4 * c + 3)] = k.w;
+    reinterpret_cast<float4*>(sV)[i] = __ldg(reinterpret_cast<const float4*>(src + d));
+  }
+  const int it = tid / T, t = tid - it * T;
+  const bool on = it < items;
+  const long long q = q0 + (on ? it : 0), s = q / H;
   const int hh = (int)(q - s * H);
   int ne = n_ent[sel ? (long long)sel[s] : s];
   ne = ne < 0 ? 0 : (ne > NS ? NS : ne);
-  const float* base = QKV + s * T * ld + hh * DH;
-  const float* K = sk[wl] + slot * T * DH;
-  const float* V = sv[wl] + slot * T * DH;
   float qv[DH];
 #pragma unroll
-  for (int j = 0; j < DH; ++j) qv[j] = base[t * ld + j];
-  float sc[kMaxT];
-  float mx = -INFINITY;
+  for (int j = 0; j < DH; j += 4) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(QKV + (s * T + (on ? t : 0)) * ld + hh * DH + j));
+    qv[j] = v.x; qv[j + 1] = v.y; qv[j + 2] = v.z; qv[j + 3] = v.w;
+  }
+  __syncthreads();
+  float sc[kMaxT + 1];
+  if (on) {
+    attn_dots<DH>(qv, sK + it * Tp * DH, T, sc);
+    float mx = -INFINITY;
 #pragma unroll
-  for (int u = 0; u < kMaxT; ++u) {
-    sc[u] = -INFINITY;
-    if (u < T && u <= ne) {
-      float acc = 0.0f;
-#pragma unroll
-      for (int j = 0; j < DH; ++j) acc = fmaf(qv[j], K[u * DH + j], acc);
-      sc[u] = acc * scale;
+    for (int u = 0; u < kMaxT; ++u) {
+      sc[u] = u < T && u <= ne ? sc[u] * scale : -INFINITY;
       mx = fmaxf(mx, sc[u]);
     }
-  }
-  float z = 0.0f;
+    float z = 0.0f;
 #pragma unroll
-  for (int u = 0; u < kMaxT; ++u) {
-    const float e = (u < T && u <= ne) ? expf(sc[u] - mx) : 0.0f;
-    sc[u] = e;
-    z += e;
-  }
-  const float iz = 1.0f / z;
-  float o[DH];
-#pragma unroll
-  for (int j = 0; j < DH; ++j) o[j] = 0.0f;
-  float* Pr = P + ((s * H + hh) * T + t) * T;
-#pragma unroll
-  for (int u = 0; u < kMaxT; ++u) {
-    if (u < T) {
-      const float p = sc[u] * iz;
-      Pr[u] = p;
-      if (u <= ne) {
-#pragma unroll
-        for (int j = 0; j < DH; ++j) o[j] = fmaf(p, V[u * DH + j], o[j]);
-      }
+    for (int u = 0; u < kMaxT; ++u) {
+      const float e = (u < T && u <= ne) ? expf(sc[u] - mx) : 0.0f;
+      sc[u] = e;
+      z += e;
     }
-  }
+    const float iz = 1.0f / z;
+    unsigned long long o[DH / 2];
 #pragma unroll
-  for (int j = 0; j < DH; ++j) O[(s * T + t) * d + hh * DH + j] = o[j];
+    for (int j = 0; j < DH / 2; ++j) o[j] = 0ull;
+#pragma unroll
+    for (int u = 0; u < kMaxT; ++u) {
+      sc[u] *= iz;
+      if (u < T && u <= ne) attn_axpy<DH>(sc[u], sV + (it * T + u) * DH, o);
+    }
+    attn_store<DH>(O + (s * T + t) * d + hh * DH, o);
+  }
+  __syncthreads();
+  if (on) {
+#pragma unroll
+    for (int u = 0; u < kMaxT; ++u)
+      if (u < T) sm_attn[tid * T + u] = sc[u];
+  }
+  __syncthreads();
+  float* Pb = P + q0 * T * T;
+  for (int i = tid; i < items * T * T; i += kAttnThreads) Pb[i] = sm_attn[i];
 }
 
-// Attention backward of one (sample, head) per warp (4 warps per block): from
-// dO and the stored P, dS = P (dP - rowsum(P dP)) scale with dP = dO V^T;
-// lane t writes dQ_t, then lane u writes dK_u = sum_t dS_tu Q_t and
-// dV_u = sum_t P_tu dO_t.  Q, K, V and dO rows are staged in shared memory.
+// Attention backward: from dO and the stored P, dS = P (dP - rowsum(P dP))
+// scale with dP = dO V^T; the thread of query t writes dQ_t, then the thread of
+// key u writes dK_u = sum_t dS_tu Q_t and dV_u = sum_t P_tu dO_t.
 template <int DH>
-__global__ void __launch_bounds__(128) attn_bwd_kernel(const float* __restrict__ QKV, const float* __restrict__ P,
-                                                       const float* __restrict__ dO, float* __restrict__ dQKV,
-                                                       long long n, int T, int H, float scale) {
-  __shared__ float sq[4][kMaxT * DH];
-  __shared__ float sk[4][kMaxT * DH];
-  __shared__ float sv[4][kMaxT * DH];
-  __shared__ float sg[4][kMaxT * DH];
-  __shared__ float sdS[4][kMaxT * kMaxT];
-  __shared__ float sP[4][kMaxT * kMaxT];
-  const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-  const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= n * H) return;  // whole warps leave together
-  const long long s = w / H;
-  const int hh = (int)(w - s * H);
+__global__ void __launch_bounds__(kAttnThreads) attn_bwd_kernel(const float* __restrict__ QKV,
+                                                                const float* __restrict__ P,
+                                                                const float* __restrict__ dO,
+                                                                float* __restrict__ dQKV, long long n, int T, int H,
+                                                                float scale) {
+  extern __shared__ __align__(16) float sm_attn[];
+  const int tid = threadIdx.x, ipb = attn_items(T), Tp = (T + 1) / 2 * 2, R = attn_rows(T);
+  float* sQ = sm_attn;                     // [items][T][DH]
+  float* sK = sQ + R * DH;
+  float* sG = sK + R * DH;                 // dO
+  float* sV = sG + R * DH;                 // [items][Tp / 2][DH][2]
+  float* sP = sV + attn_pair_rows(T) * DH; // [items][T][T]
+  float* sS = sP + R * T;                  // dS
+  const long long q0 = (long long)blockIdx.x * ipb, nq = n * H;
+  const int items = (int)(nq - q0 < ipb ? nq - q0 : ipb);
   const int d = DH * H, ld = 3 * d;
-  const float* base = QKV + s * T * ld + hh * DH;
-  const float* dOb = dO + s * T * d + hh * DH;
-  float* out = dQKV + s * T * ld + hh * DH;
-  const float* Pb = P + (s * H + hh) * T * T;
-  for (int i = lane; i < T * DH; i += 32) {
-    const int u = i / DH, j = i - u * DH;
-    sq[wl][i] = base[u * ld + j];
-    sk[wl][i] = base[u * ld + d + j];
-    sv[wl][i] = base[u * ld + 2 * d + j];
-    sg[wl][i] = dOb[u * d + j];
+  for (int i = tid; i < items * T * (DH / 4); i += kAttnThreads) {
+    const int r = i / (DH / 4), c = i - r * (DH / 4), it = r / T, u = r - it * T;
+    const long long q = q0 + it, s = q / H;
+    const long long hc = (q - s * H) * DH + 4 * c;
+    const float* src = QKV + (s * T + u) * ld + hc;
+    reinterpret_cast<float4*>(sQ)[i] = __ldg(reinterpret_cast<const float4*>(src));
+    reinterpret_cast<float4*>(sK)[i] = __ldg(reinterpret_cast<const float4*>(src + d));
+    reinterpret_cast<float4*>(sG)[i] = __ldg(reinterpret_cast<const float4*>(dO + (s * T + u) * d + hc));
+    const float4 v = __ldg(reinterpret_cast<const float4*>(src + 2 * d));
+    float* dst = sV + it * Tp * DH;
+    dst[pair_pos<DH>(u, 4 * c)] = v.x;
+    dst[pair_pos<DH>(u, 4 * c + 1)] = v.y;
+    dst[pair_pos<DH>(u, 4 * c + 2)] = v.z;
+    dst[pair_pos<DH>(u, 4 * c + 3)] = v.w;
   }
-  for (int i = lane; i < T * T; i += 32) sP[wl][i] = Pb[i];
-  __syncwarp();
-  if (lane < T) {
-    float dp[kMaxT], dot = 0.0f;
+  for (int i = tid; i < items * T * T; i += kAttnThreads) sP[i] = __ldg(P + q0 * T * T + i);
+  __syncthreads();
+  const int it = tid / T, t = tid - it * T;
+  const bool on = it < items;
+  const long long q = q0 + (on ? it : 0), s = q / H;
+  float* out = dQKV + (s * T + t) * ld + (q - s * H) * DH;
+  unsigned long long o[DH / 2];
+  if (on) {
+    float g[DH], dp[kMaxT + 1];
+#pragma unroll
+    for (int j = 0; j < DH; j += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(sG + tid * DH + j);
+      g[j] = v.x; g[j + 1] = v.y; g[j + 2] = v.z; g[j + 3] = v.w;
+    }
+    attn_dots<DH>(g, sV + it * Tp * DH, T, dp);
+    float dot = 0.0f;
+#pragma unroll
+    for (int u = 0; u < kMaxT; ++u)
+      if (u < T) dot = fmaf(sP[tid * T + u], dp[u], dot);
+#pragma unroll
+    for (int j = 0; j < DH / 2; ++j) o[j] = 0ull;
 #pragma unroll
     for (int u = 0; u < kMaxT; ++u) {
-      dp[u] = 0.0f;
       if (u < T) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int j = 0; j < DH; ++j) acc = fmaf(sg[wl][lane * DH + j], sv[wl][u * DH + j], acc);
-        dp[u] = acc;
-        dot = fmaf(sP[wl][lane * T + u], acc, dot);
+        const float ds = sP[tid * T + u] * (dp[u] - dot) * scale;
+        sS[tid * T + u] = ds;
+        attn_axpy<DH>(ds, sK + (it * T + u) * DH, o);
       }
     }
-    float dq[DH];
-#pragma unroll
-    for (int j = 0; j < DH; ++j) dq[j] = 0.0f;
-#pragma unroll
-    for (int u = 0; u < kMaxT; ++u) {
-      if (u < T) {
-        const float ds = sP[wl][lane * T + u] * (dp[u] - dot) * scale;
-        sdS[wl][lane * T + u] = ds;
-#pragma unroll
-        for (int j = 0; j < DH; ++j) dq[j] = fmaf(ds, sk[wl][u * DH + j], dq[j]);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < DH; ++j) out[lane * ld + j] = dq[j];
+    attn_store<DH>(out, o);
   }
-  __syncwarp();
-  if (lane < T) {
-    float dk[DH], dv[DH];
+  __syncthreads();
+  if (on) {
+    unsigned long long dv[DH / 2];
 #pragma unroll
-    for (int j = 0; j < DH; ++j) dk[j] = dv[j] = 0.0f;
-    for (int t = 0; t < T; ++t) {
-      const float ds = sdS[wl][t * T + lane], p = sP[wl][t * T + lane];
-#pragma unroll
-      for (int j = 0; j < DH; ++j) {
-        dk[j] = fmaf(ds, sq[wl][t * DH + j], dk[j]);
-        dv[j] = fmaf(p, sg[wl][t * DH + j], dv[j]);
-      }
+    for (int j = 0; j < DH / 2; ++j) o[j] = dv[j] = 0ull;
+    for (int r = it * T; r < it * T + T; ++r) {
+      attn_axpy<DH>(sS[r * T + t], sQ + r * DH, o);
+      attn_axpy<DH>(sP[r * T + t], sG + r * DH, dv);
     }
-#pragma unroll
-    for (int j = 0; j < DH; ++j) {
-      out[lane * ld + d + j] = dk[j];
-      out[lane * ld + 2 * d + j] = dv[j];
-    }
+    attn_store<DH>(out + d, o);
+    attn_store<DH>(out + 2 * d, dv);
   }
 }
 
@@ -1857,9 +1922,11 @@ cudaError_t attn_fwd(const float* QKV, const int32_t* ne, const int32_t* sel, fl
     attn_fwd_mma_kernel<<<(unsigned)grid, 128, 0, s>>>(QKV, ne, sel, P, O, n, T, NS, H, 1.0f / sqrtf((float)DH));
     return cudaGetLastError();
   }
-  const long long warps = (n * H + attn_pairs_per_warp(T) - 1) / attn_pairs_per_warp(T);
-  attn_fwd_kernel<DH><<<blocks_for(warps * 32, 128), 128, 0, s>>>(QKV, ne, sel, P, O, n, T, NS, H,
-                                                                   1.0f / sqrtf((float)DH));
+  static std::atomic<unsigned long long> ready{0};
+  const cudaError_t e = smem_optin(attn_fwd_kernel<DH>, kAttnSmemMax, ready);
+  if (e != cudaSuccess) return e;
+  attn_fwd_kernel<DH><<<blocks_for(n * H, attn_items(T)), kAttnThreads, attn_fwd_smem(T, DH), s>>>(
+      QKV, ne, sel, P, O, n, T, NS, H, 1.0f / sqrtf((float)DH));
   return cudaGetLastError();
 }
 
@@ -1870,8 +1937,13 @@ cudaError_t attn_bwd(const float* QKV, const float* P, const float* dO, float* d
   if (mma && DH == 16 && T <= 16 && ((uintptr_t)QKV & 15) == 0 && ((uintptr_t)dO & 15) == 0)
     attn_bwd_mma_kernel<<<(unsigned)att_grid(attn_bwd_mma_kernel, n * H), 128, 0, s>>>(QKV, P, dO, dQKV, n, T, H,
                                                                                        1.0f / sqrtf((float)DH));
-  else
-    attn_bwd_kernel<DH><<<blocks_for(n * H * 32, 128), 128, 0, s>>>(QKV, P, dO, dQKV, n, T, H, 1.0f / sqrtf((float)DH));
+  else {
+    static std::atomic<unsigned long long> ready{0};
+    const cudaError_t e = smem_optin(attn_bwd_kernel<DH>, kAttnSmemMax, ready);
+    if (e != cudaSuccess) return e;
+    attn_bwd_kernel<DH><<<blocks_for(n * H, attn_items(T)), kAttnThreads, attn_bwd_smem(T, DH), s>>>(
+        QKV, P, dO, dQKV, n, T, H, 1.0f / sqrtf((float)DH));
+  }
   return cudaGetLastError();
 }
 
