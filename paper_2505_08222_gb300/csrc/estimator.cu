@@ -42,6 +42,23 @@ __device__ __forceinline__ void store8(unsigned char* img, int row, int k0, int 
   *reinterpret_cast<uint4*>(img + tc::kmajor_offset(row, k0, rows)) = p;
 }
 
+// 24 consecutive features of a row from column c0 (a multiple of 8) on, as BF16
+// high parts and remainders in two operand images.
+__device__ __forceinline__ void store_features(unsigned char* hi_img, unsigned char* lo_img, int row, int c0,
+                                               const float (&x)[24]) {
+#pragma unroll
+  for (int k = 0; k < 24; k += 8) {
+    float hi[8], lo[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      hi[i] = bf_bits2f(f2bf_bits(x[k + i]));
+      lo[i] = x[k + i] - hi[i];
+    }
+    store8(hi_img, row, c0 + k, 128, hi);
+    store8(lo_img, row, c0 + k, 128, lo);
+  }
+}
+
 // Estimator features of filter f for its update at step g (reading C18):
 // in the local frame of the filter's current estimate e1 (units of L), each
 // of the 16 most recent pings, newest first, as [(q - e1) / L, range
@@ -49,38 +66,57 @@ __device__ __forceinline__ void store8(unsigned char* img, int row, int k0, int 
 // of the estimate (e1 - e2) / L and its smoothed motion v / L (the velocity
 // EMA including this update's e1 - e2); zero padded to 96.  The network's
 // output is the correction (x - e1) / L.
+// Columns LO .. LO + N - 1 of them.  STEP: the sum of squares with the step's
+// own roundings (its low bits decide BF16 roundings, so the order is fixed here
+// and not left to the compiler).
+template <int LO, bool STEP, int N>
 __device__ __forceinline__ void ring_features(const EnvDev& d, int f, uint32_t g, float e1x, float e1y, float e2x,
-                                              float e2y, float vx, float vy, float (&x)[IN]) {
+                                              float e2y, float vx, float vy, float (&x)[N]) {
   const int it = d.filt_target[f];
   const float dz = UT_IN_BOUNDS(it >= 0 && it < d.NT, d.status) ? d.tz[it] : 0.0f;  // target depth; senders at the surface
   const float L = d.est_scale;
   const int head = d.ring_head[f], cnt = d.ring_count[f];
   const float4* ring = reinterpret_cast<const float4*>(d.ring) + (long long)f * kRing;
 #pragma unroll
+  for (int i = 0; i < N; ++i) x[i] = 0.0f;
+#pragma unroll
   for (int s = 0; s < kRing; ++s) {
+    if (5 * s + 4 < LO || 5 * s >= LO + N) continue;  // (compile time: none of its columns wanted)
     float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
     const bool on = s < cnt;
     if (on) e = ring[(head - 1 - s) & (kRing - 1)];
     const float dx = e.x - e1x, dy = e.y - e1y;
-    const float rho = sqrtf(dx * dx + dy * dy + dz * dz);
-    x[5 * s + 0] = on ? dx / L : 0.0f;
-    x[5 * s + 1] = on ? dy / L : 0.0f;
-    x[5 * s + 2] = on ? (e.z - rho) / L : 0.0f;
-    x[5 * s + 3] = on ? ((float)g - e.w) / 16.0f : 0.0f;
-    x[5 * s + 4] = on ? 1.0f : 0.0f;
-  }
-  x[5 * kRing] = (e1x - e2x) / L;
-  x[5 * kRing + 1] = (e1y - e2y) / L;
-  x[5 * kRing + 2] = vx / L;
-  x[5 * kRing + 3] = vy / L;
+    const float rho = sqrtf(STEP ? __fadd_rn(fmaf(dx, dx, dy * dy), __fmul_rn(dz, dz)) : dx * dx + dy * dy + dz * dz);
+    const float v[5] = {on ? dx / L : 0.0f, on ? dy / L : 0.0f, on ? (e.z - rho) / L : 0.0f,
+                        on ? ((float)g - e.w) / 16.0f : 0.0f, on ? 1.0f : 0.0f};
 #pragma unroll
-  for (int i = 5 * kRing + 4; i < IN; ++i) x[i] = 0.0f;
+    for (int k = 0; k < 5; ++k)
+      if (5 * s + k >= LO && 5 * s + k < LO + N) x[5 * s + k - LO] = v[k];
+  }
+  const float m[4] = {(e1x - e2x) / L, (e1y - e2y) / L, vx / L, vy / L};
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (5 * kRing + k >= LO && 5 * kRing + k < LO + N) x[5 * kRing + k - LO] = m[k];
+}
+
+// acc[128 x 128] (+)= A[128 x 16 ksteps] B[128 x 16 ksteps]^T, issued by the
+// calling thread (both images 128 rows high).
+__device__ __forceinline__ void issue_mma(uint32_t d_tmem, uint32_t a, uint32_t b, int ksteps, bool accumulate) {
+  constexpr uint32_t idesc = tc::idesc_bf16(128, 128);
+  uint64_t ad = tc::smem_desc(a, 128 * 16, 128), bd = tc::smem_desc(b, 128 * 16, 128);
+#pragma unroll 2
+  for (int k = 0; k < ksteps; ++k) {
+    tc::mma_bf16(d_tmem, ad, bd, idesc, (accumulate || k > 0) ? 1u : 0u);
+    ad = tc::desc_advance(ad, 2 * 128 * 16);
+    bd = tc::desc_advance(bd, 2 * 128 * 16);
+  }
 }
 
 // ---------------------------------------------------------------------------
 // Estimator step in the environment (learned form): one CTA of 512 threads
-// per 128 filters, thread = filter row x one of 4 column parts.  Part 0
-// builds the row's features; the hidden-layer epilogues (bias, erf-GELU of
+// per 128 filters, thread = filter row x one of 4 column parts.  Each part
+// builds its 24 of the row's features (one thread per row built all 96: 13 k of
+// a tile's 48 k cycles; 102,400 filters 144 -> 124 us); the hidden-layer epilogues (bias, erf-GELU of
 // gelu.cuh in packed pairs, BF16 operand) split
 // the 256 hidden units 4 ways; the weight images (N-halves
 // of W1, W2, W3) stream through two shared-memory slots by the bulk-copy
@@ -160,32 +196,33 @@ __global__ void __launch_bounds__(kTE, 1) fwd_env_kernel(Net net, EnvDev d, int 
     fetch(1);
   }
 
-  // features of this row (part 0) -> A operand as BF16 high and low parts
-  float x[IN];
+  // this part's features of the row -> A operand as BF16 high and low parts
   float e1x = 0.0f, e1y = 0.0f, vnx = 0.0f, vny = 0.0f;
-  if (part == 0) {
+  bool fresh = false;  // (part 0) a ping received this step
+  {
+    float x[24];
     if (valid) {
       e1x = d.estx[f];
       e1y = d.esty[f];
       const float e2x = d.prev_estx[f], e2y = d.prev_esty[f];
       vnx = fmaf(kVelKeep, d.velx[f], (1.0f - kVelKeep) * (e1x - e2x));
       vny = fmaf(kVelKeep, d.vely[f], (1.0f - kVelKeep) * (e1y - e2y));
-      ring_features(d, (int)f, d.counters[0] + 1u, e1x, e1y, e2x, e2y, vnx, vny, x);
+      const uint32_t g = d.counters[0] + 1u;
+      if (part == 0) {
+        ring_features<0, true>(d, (int)f, g, e1x, e1y, e2x, e2y, vnx, vny, x);
+        fresh = x[3] == 0.0f && x[4] == 1.0f;
+      } else if (part == 1) {
+        ring_features<24, true>(d, (int)f, g, e1x, e1y, e2x, e2y, vnx, vny, x);
+      } else if (part == 2) {
+        ring_features<48, true>(d, (int)f, g, e1x, e1y, e2x, e2y, vnx, vny, x);
+      } else {
+        ring_features<72, true>(d, (int)f, g, e1x, e1y, e2x, e2y, vnx, vny, x);
+      }
     } else {
 #pragma unroll
-      for (int i = 0; i < IN; ++i) x[i] = 0.0f;
+      for (int i = 0; i < 24; ++i) x[i] = 0.0f;
     }
-#pragma unroll
-    for (int c0 = 0; c0 < IN; c0 += 8) {
-      float hi[8], lo[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        hi[i] = bf_bits2f(f2bf_bits(x[c0 + i]));
-        lo[i] = x[c0 + i] - hi[i];
-      }
-      store8(sA, row, c0, 128, hi);
-      store8(sA + 128 * IN * 2, row, c0, 128, lo);
-    }
+    store_features(sA, sA + 128 * IN * 2, row, part * 24, x);
   }
 
   bool ok = true;
@@ -200,22 +237,11 @@ __global__ void __launch_bounds__(kTE, 1) fwd_env_kernel(Net net, EnvDev d, int 
     __syncthreads();
     tc::fence_after_sync();
     if (tid == 0) {
-      const int K = l == 0 ? IN : HID;
-      const uint32_t idesc = tc::idesc_bf16(128, 128);
       for (int h = 0; h < 2; ++h) {
         ok &= tc::mbar_wait(&full[(stage + h) & 1], (uint32_t)(((stage + h) >> 1) & 1), kEnvPolls);
         const uint32_t bB = aW + (uint32_t)(((stage + h) & 1) * kEnvSlot);
-        const int nA = l == 0 ? 2 : 1;
-        bool acc = false;
-        for (int j = 0; j < nA; ++j) {
-          const uint32_t a0 = aA + (uint32_t)(j * 128 * IN * 2);
-          for (int k = 0; k < K / 16; ++k) {
-            const uint64_t ad = tc::smem_desc(a0 + k * 2 * 128 * 16, 128 * 16, 128);
-            const uint64_t bd = tc::smem_desc(bB + k * 2 * 128 * 16, 128 * 16, 128);
-            tc::mma_bf16(tmem + 128 * h, ad, bd, idesc, acc ? 1u : 0u);
-            acc = true;
-          }
-        }
+        issue_mma(tmem + 128 * h, aA, bB, (l == 0 ? IN : HID) / 16, false);
+        if (l == 0) issue_mma(tmem + 128 * h, aA + (uint32_t)(128 * IN * 2), bB, IN / 16, true);
       }
       tc::mma_commit(&mbar);
     }
@@ -230,20 +256,26 @@ __global__ void __launch_bounds__(kTE, 1) fwd_env_kernel(Net net, EnvDev d, int 
     // epilogue of hidden layer l on this thread's 64 hidden units
     const float* bias = mst + (l == 0 ? B1_OFF : (l == 1 ? B2_OFF : B3_OFF));
 #pragma unroll 1
-    for (int c0 = part * (HID / kParts); c0 < (part + 1) * (HID / kParts); c0 += 16) {
-      float v[16];
-      tc::tmem_ld16(tl + c0, v);
-      float av[16];
+    for (int c0 = part * (HID / kParts); c0 < (part + 1) * (HID / kParts); c0 += 32) {
+      float av[32];
+      tc::tmem_ld32(tl + c0, av);
+      const float4* b4 = reinterpret_cast<const float4*>(bias + c0);  // (every layer's biases start at a multiple of 4)
 #pragma unroll
-      for (int i = 0; i < 16; ++i) av[i] = v[i] + __ldg(bias + c0 + i);
+      for (int i = 0; i < 8; ++i) {
+        const float4 b = __ldg(b4 + i);
+        av[4 * i] += b.x;
+        av[4 * i + 1] += b.y;
+        av[4 * i + 2] += b.z;
+        av[4 * i + 3] += b.w;
+      }
 #pragma unroll
-      for (int i = 0; i < 16; i += 2) gelu2(av[i], av[i + 1]);  // erf-GELU, packed pairs
+      for (int i = 0; i < 32; i += 2) gelu2(av[i], av[i + 1]);  // erf-GELU, packed pairs
       if (l < 2) {
-        store8(sA, row, c0, 128, av);
-        store8(sA, row, c0 + 8, 128, av + 8);
+#pragma unroll
+        for (int i = 0; i < 32; i += 8) store8(sA, row, c0 + i, 128, av + i);
       } else {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
+        for (int i = 0; i < 32; ++i) {
           o0 = fmaf(__ldg(mst + W4_OFF + c0 + i), av[i], o0);
           o1 = fmaf(__ldg(mst + W4_OFF + HID + c0 + i), av[i], o1);
         }
@@ -269,13 +301,12 @@ __global__ void __launch_bounds__(kTE, 1) fwd_env_kernel(Net net, EnvDev d, int 
     // by the mode applies: hold the estimate (stale inputs cannot drive the
     // closed loop away), apply the network all the same, or coast by the
     // estimate's smoothed motion v (constant velocity).
-    const bool fresh = x[3] == 0.0f && x[4] == 1.0f;
     const float lim = (fresh || stale == 1) ? kMaxCorr : 0.0f;
     float c0 = isfinite(o0) ? fminf(fmaxf(o0, -lim), lim) : 0.0f;
     float c1 = isfinite(o1) ? fminf(fmaxf(o1, -lim), lim) : 0.0f;
     if (!fresh && stale == 2) {
-      c0 = fminf(fmaxf(x[5 * kRing + 2], -kMaxCorr), kMaxCorr);
-      c1 = fminf(fmaxf(x[5 * kRing + 3], -kMaxCorr), kMaxCorr);
+      c0 = fminf(fmaxf(vnx / d.est_scale, -kMaxCorr), kMaxCorr);
+      c1 = fminf(fmaxf(vny / d.est_scale, -kMaxCorr), kMaxCorr);
     }
     const float ex = e1x + d.est_scale * c0, ey = e1y + d.est_scale * c1;
     d.prev2_estx[f] = d.prev_estx[f];
@@ -336,7 +367,7 @@ __global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __res
   __shared__ __align__(8) uint64_t full[2];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tbase;
-  __shared__ float sOut[kParts][2][128];
+  __shared__ float sOut[2][128];
   __shared__ float s_red[TRAIN ? 4 : 1][TRAIN ? NB_PART : 1];  // column sums of each 32-row quarter
   __shared__ double s_loss[4];
   __shared__ int bad;
@@ -383,18 +414,10 @@ __global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __res
                              : make_float4(0.f, 0.f, 0.f, 0.f);
       x[i] = v.x; x[i + 1] = v.y; x[i + 2] = v.z; x[i + 3] = v.w;
     }
+    store_features(sA, sA + 128 * IN * 2, row, part * 24, x);
+    if (TRAIN) {
 #pragma unroll
-    for (int k = 0; k < 24; k += 8) {
-      const int c0 = part * 24 + k;
-      float hi[8], lo[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        hi[i] = bf_bits2f(f2bf_bits(x[k + i]));
-        lo[i] = x[k + i] - hi[i];
-      }
-      store8(sA, row, c0, 128, hi);
-      store8(sA + 128 * IN * 2, row, c0, 128, lo);
-      if (TRAIN) store8(t.x_img + (size_t)blockIdx.x * kImgX, row, c0, 128, hi);
+      for (int k = 0; k < 24; k += 8) store8(t.x_img + (size_t)blockIdx.x * kImgX, row, part * 24 + k, 128, x + k);
     }
   }
 
@@ -410,20 +433,11 @@ __global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __res
     __syncthreads();
     tc::fence_after_sync();
     if (tid == 0) {
-      const uint32_t idesc = tc::idesc_bf16(128, 128);
       for (int h = 0; h < 2; ++h) {
         ok &= tc::mbar_wait(&full[(stage + h) & 1], (uint32_t)(((stage + h) >> 1) & 1), kEnvPolls);
         const uint32_t bB = aW + (uint32_t)(((stage + h) & 1) * kEnvSlot);
-        bool acc = false;
-        for (int j = 0; j < n_a; ++j) {
-          const uint32_t a0 = aA + (uint32_t)(j * 128 * IN * 2);
-          for (int k = 0; k < K / 16; ++k) {
-            const uint64_t ad = tc::smem_desc(a0 + k * 2 * 128 * 16, 128 * 16, 128);
-            const uint64_t bd = tc::smem_desc(bB + k * 2 * 128 * 16, 128 * 16, 128);
-            tc::mma_bf16(tmem + col + 128 * h, ad, bd, idesc, acc ? 1u : 0u);
-            acc = true;
-          }
-        }
+        issue_mma(tmem + col + 128 * h, aA, bB, K / 16, false);
+        if (n_a == 2) issue_mma(tmem + col + 128 * h, aA + (uint32_t)(128 * IN * 2), bB, K / 16, true);
       }
       tc::mma_commit(&mbar);
     }
@@ -438,11 +452,10 @@ __global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __res
   };
   const int c_lo = part * (HID / kParts), c_hi = c_lo + HID / kParts;
   constexpr uint32_t kZ2 = TRAIN ? 256 : 0;  // column of layer 2's accumulator (layers 1 and 3: 0)
-  float o0 = 0.0f, o1 = 0.0f;
-  for (int l = 0; l < 3; ++l) {
+  for (int l = 0; l < 2; ++l) {
     const uint32_t col = l == 1 ? kZ2 : 0u;
     product(col, l == 0 ? IN : HID, l == 0 ? 2 : 1);
-    const float* bias = mst + (l == 0 ? B1_OFF : (l == 1 ? B2_OFF : B3_OFF));
+    const float* bias = mst + (l == 0 ? B1_OFF : B2_OFF);
 #pragma unroll 1
     for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
       float v[16];
@@ -456,32 +469,50 @@ __global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __res
       }
 #pragma unroll
       for (int i = 0; i < 16; i += 2) gelu2(v[i], v[i + 1]);  // erf-GELU, packed pairs
-      if (l < 2) {
-        store8(sA, row, c0, 128, v);
-        store8(sA, row, c0 + 8, 128, v + 8);
-        if (TRAIN) {
-          unsigned char* img = t.a_img + ((size_t)l * gridDim.x + blockIdx.x) * kImgA;
-          store8(img, row, c0, 128, v);
-          store8(img, row, c0 + 8, 128, v + 8);
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          o0 = fmaf(__ldg(mst + W4_OFF + c0 + i), v[i], o0);
-          o1 = fmaf(__ldg(mst + W4_OFF + HID + c0 + i), v[i], o1);
-        }
+      store8(sA, row, c0, 128, v);
+      store8(sA, row, c0 + 8, 128, v + 8);
+      if (TRAIN) {
+        unsigned char* img = t.a_img + ((size_t)l * gridDim.x + blockIdx.x) * kImgA;
+        store8(img, row, c0, 128, v);
+        store8(img, row, c0 + 8, 128, v + 8);
       }
     }
   }
-  sOut[part][0][row] = o0;
-  sOut[part][1][row] = o1;
-  __syncthreads();
-  o0 = __ldg(mst + B4_OFF);
-  o1 = __ldg(mst + B4_OFF + 1);
+  // layer 3, and the output layer's two sums over the hidden units in order:
+  // the four parts take their turns (their errors feed the BF16 gradients, and
+  // a small batch shows another order)
+  product(0, HID, 1);
+  float o0 = 0.0f, o1 = 0.0f;
+  {
+    float a3[HID / kParts];
 #pragma unroll
-  for (int k = 0; k < kParts; ++k) {
-    o0 += sOut[k][0][row];
-    o1 += sOut[k][1][row];
+    for (int k = 0; k < HID / kParts; k += 32) {
+      float v[32];
+      tc::tmem_ld32(tl + c_lo + k, v);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) a3[k + i] = v[i] + __ldg(mst + B3_OFF + c_lo + k + i);
+    }
+#pragma unroll
+    for (int i = 0; i < HID / kParts; i += 2) gelu2(a3[i], a3[i + 1]);
+#pragma unroll 1
+    for (int turn = 0; turn < kParts; ++turn) {
+      if (part == turn) {  // (warp-uniform)
+        if (turn > 0) {
+          o0 = sOut[0][row];
+          o1 = sOut[1][row];
+        }
+#pragma unroll
+        for (int i = 0; i < HID / kParts; ++i) {
+          o0 = fmaf(__ldg(mst + W4_OFF + c_lo + i), a3[i], o0);
+          o1 = fmaf(__ldg(mst + W4_OFF + HID + c_lo + i), a3[i], o1);
+        }
+        sOut[0][row] = o0;
+        sOut[1][row] = o1;
+      }
+      __syncthreads();
+    }
+    o0 = sOut[0][row] + __ldg(mst + B4_OFF);
+    o1 = sOut[1][row] + __ldg(mst + B4_OFF + 1);
   }
   if constexpr (TRAIN) {
     // output layer: dL/dout / B; loss per row: sum over the two outputs of
@@ -657,11 +688,11 @@ __global__ void __launch_bounds__(kT, 1) wgrad_kernel(TrainBufs t, int* status) 
       ok = tc::mbar_wait(&full[c & 1], (uint32_t)((c >> 1) & 1), kEnvPolls);
       if (!ok) break;
       const uint32_t aa = tc::smem_addr(smem + (c & 1) * kWgradStage), bb = aa + (uint32_t)(kImgA / 2);
-      for (int j = 0; j < kT / 16; ++j) {
-        const uint64_t ad = tc::smem_desc(aa + j * 256, 128, kT * 16);
-        const uint64_t bd = tc::smem_desc(bb + j * 256, 128, kT * 16);
-        tc::mma_bf16(tmem, ad, bd, idesc, (c > 0 || j > 0) ? 1u : 0u);
-      }
+      const uint64_t ad = tc::smem_desc(aa, 128, kT * 16), bd = tc::smem_desc(bb, 128, kT * 16);
+#pragma unroll
+      for (int j = 0; j < kT / 16; ++j)
+        tc::mma_bf16(tmem, tc::desc_advance(ad, j * 256), tc::desc_advance(bd, j * 256), idesc,
+                     (c > 0 || j > 0) ? 1u : 0u);
       tc::mma_commit(&done[c & 1]);
       if (c + 1 < n) {  // refill the other stage once its MMAs (tile c - 1) are through
         if (c >= 1 && fetched < n) {
@@ -827,7 +858,7 @@ __global__ void record_kernel(EnvDev d, float* feat, float* label) {
   // after the step: the update's inputs are the estimate history
   const float e1x = d.prev_estx[f], e1y = d.prev_esty[f];
   float x[IN];
-  ring_features(d, f, d.counters[0], e1x, e1y, d.prev2_estx[f], d.prev2_esty[f], d.velx[f], d.vely[f], x);
+  ring_features<0, false>(d, f, d.counters[0], e1x, e1y, d.prev2_estx[f], d.prev2_esty[f], d.velx[f], d.vely[f], x);
 #pragma unroll
   for (int i = 0; i < IN; i += 4)
     *reinterpret_cast<float4*>(feat + (long long)f * IN + i) = make_float4(x[i], x[i + 1], x[i + 2], x[i + 3]);
