@@ -79,6 +79,25 @@ struct EnvDev {
   int32_t* dbg_idx;
 };
 
+// What a step's environment stage and its filters hand each other: measurement
+// lists [F][AM], per-filter headers [F], tracking errors [F].  The handle's own
+// buffers (read from the kernel's arguments where they are used: held in
+// registers they made the filter kernel spill), or copies in shared memory
+// (persistent rollout).
+struct HandleLists {
+  const EnvDev& d;
+  __device__ float4* meas() const { return d.meas; }
+  __device__ float4* hdr() const { return d.meas_hdr; }
+  __device__ float* err() const { return d.err; }
+};
+struct StepLists {
+  float4 *meas_p, *hdr_p;
+  float* err_p;
+  __device__ float4* meas() const { return meas_p; }
+  __device__ float4* hdr() const { return hdr_p; }
+  __device__ float* err() const { return err_p; }
+};
+
 // Launchers (env_kernels.cu, pf_kernel.cu).
 cudaError_t launch_reset(const EnvDev& d, cudaStream_t s);
 cudaError_t launch_step_env(const EnvDev& d, const int32_t* act_in, cudaStream_t s);

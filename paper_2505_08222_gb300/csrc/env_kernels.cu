@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) step_env_kernel(EnvDev d,
   const int e = blockIdx.x * kWarpsPerBlock + wid;
   __shared__ EnvWarpSmem sw[kWarpsPerBlock];
   if (e >= d.E) return;  // warp-uniform
-  step_env_warp(d, e, act_in, d.counters[0] + 1u, sw[wid]);
+  step_env_warp(d, HandleLists{d}, e, act_in, d.counters[0] + 1u, sw[wid]);
 }
 
 // -------------------------------------------------------------------------

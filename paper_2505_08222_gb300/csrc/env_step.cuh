@@ -27,8 +27,9 @@ struct StepMetrics {
 // pings, communication and per-filter measurement lists (Sec. III-A.2).
 // Called by the whole warp that owns environment e, at global step g.
 // -------------------------------------------------------------------------
-__device__ __forceinline__ void step_env_warp(const EnvDev& d, int e, const int32_t* __restrict__ act_in, uint32_t g,
-                                              EnvWarpSmem& w) {
+template <typename Lists>
+__device__ __forceinline__ void step_env_warp(const EnvDev& d, const Lists& lists, int e,
+                                              const int32_t* __restrict__ act_in, uint32_t g, EnvWarpSmem& w) {
   const int lane = threadIdx.x & 31;
   const int a0 = d.agent_off[e], A = d.agent_off[e + 1] - a0;
   const int t0 = d.target_off[e], T = d.target_off[e + 1] - t0;
@@ -155,7 +156,7 @@ __device__ __forceinline__ void step_env_warp(const EnvDev& d, int e, const int3
     for (int b = 0; b < A; ++b) {
       if ((d.shared_filter || w.recv[a * kMaxAgents + b]) && w.valid[b * T + k]) {
         const float qx = w.ax[b], qy = w.ay[b], r = w.rng[b * T + k];
-        if (UT_IN_BOUNDS(n < d.AM, d.status)) d.meas[(long long)f * d.AM + n] = make_float4(qx, qy, 0.0f, r);
+        if (UT_IN_BOUNDS(n < d.AM, d.status)) lists.meas()[(long long)f * d.AM + n] = make_float4(qx, qy, 0.0f, r);
         ++n;
         if (d.ring_on) {
           reinterpret_cast<float4*>(d.ring)[(long long)f * kRing + head] = make_float4(qx, qy, r, (float)g);
@@ -166,7 +167,7 @@ __device__ __forceinline__ void step_env_warp(const EnvDev& d, int e, const int3
     }
     d.meas_n[f] = n;
     // per-filter header read by the filter step (no dependent loads there)
-    d.meas_hdr[f] = make_float4(w.tx[k], w.ty[k], w.tz[k] * w.tz[k], (float)n);
+    lists.hdr()[f] = make_float4(w.tx[k], w.ty[k], w.tz[k] * w.tz[k], (float)n);
     if (d.ring_on) {
       d.ring_head[f] = head;
       d.ring_count[f] = cnt;
@@ -182,6 +183,61 @@ __device__ __forceinline__ float tracking_reward(float err, float emin, float em
   const float t = (err - emin) / (emax - emin);
   if (t >= 1.0f) return 0.0f;
   return expf(-2.0f * t / (1.0f - t));
+}
+
+// What a step's reward takes from the positions: the follow reward of target
+// `lane` (Eq. 2; 0 with the tracking reward) and the crash flag.  Called by the
+// whole warp that owns environment e.
+struct PosReward {
+  float rk = 0.0f;
+  int cr = 0;
+};
+__device__ __forceinline__ PosReward reward_positions(const EnvDev& d, int a0, int A, int t0, int T) {
+  const int lane = threadIdx.x & 31;
+  PosReward q;
+  if (d.reward_type != 0 && lane < T) {
+    float dk = INFINITY;
+    for (int a = 0; a < A; ++a) {
+      const float dx = d.ax[a0 + a] - d.tx[t0 + lane], dy = d.ay[a0 + a] - d.ty[t0 + lane];
+      dk = fminf(dk, sqrtf(dx * dx + dy * dy));
+    }
+    q.rk = dk <= d.follow_dmin ? 1.0f : 0.0f;
+  }
+  for (int p = lane; p < A * A; p += 32) {
+    const int a = p / A, b = p - a * A;
+    if (b > a) {
+      const float dx = d.ax[a0 + a] - d.ax[a0 + b], dy = d.ay[a0 + a] - d.ay[a0 + b];
+      if (sqrtf(dx * dx + dy * dy) < d.d_safe) q.cr = 1;
+    }
+  }
+  q.cr = __any_sync(0xffffffffu, q.cr);
+  return q;
+}
+// The step's reward, and its sum of squared tracking errors into se, from that
+// and the errors err[0 .. nfe - 1] of the environment's filters.
+__device__ __forceinline__ float reward_errors(const EnvDev& d, const PosReward& q, int A, int T, int nfe,
+                                               const float* err, double& se) {
+  const int lane = threadIdx.x & 31;
+  float rk = q.rk;
+  if (d.reward_type == 0 && lane < T) {
+    // agent-averaged error; a shared filter's error is every agent's
+    float ek = 0.0f;
+    if (d.shared_filter) {
+      ek = err[lane];
+    } else {
+      for (int a = 0; a < A; ++a) ek += err[a * T + lane];
+      ek /= (float)A;
+    }
+    rk = tracking_reward(ek, d.eps_min, d.eps_max);
+  }
+  rk = warp_sum(rk);
+  double sq = 0.0;
+  for (int p = lane; p < nfe; p += 32) {
+    const double v = (double)err[p];
+    sq += v * v;
+  }
+  se = warp_sum_d(sq);
+  return q.cr ? -1.0f : rk / (float)T;
 }
 
 // -------------------------------------------------------------------------
@@ -237,46 +293,10 @@ __device__ __forceinline__ void obs_reward_warp(const EnvDev& d, int e, int afte
       reinterpret_cast<uint4*>(d.obs)[(long long)ia * d.NS + slot] = packed;
     }
     if (!after_reset) {
-      float rk = 0.0f;
-      if (lane < T) {
-        const int k = lane;
-        if (d.reward_type == 0) {
-          // agent-averaged error; a shared filter's error is every agent's
-          float ek = 0.0f;
-          if (d.shared_filter) {
-            ek = d.err[f0 + k];
-          } else {
-            for (int a = 0; a < A; ++a) ek += d.err[f0 + a * T + k];
-            ek /= (float)A;
-          }
-          rk = tracking_reward(ek, d.eps_min, d.eps_max);
-        } else {
-          float dk = INFINITY;
-          for (int a = 0; a < A; ++a) {
-            const float dx = d.ax[a0 + a] - d.tx[t0 + k], dy = d.ay[a0 + a] - d.ty[t0 + k];
-            dk = fminf(dk, sqrtf(dx * dx + dy * dy));
-          }
-          rk = dk <= d.follow_dmin ? 1.0f : 0.0f;
-        }
-      }
-      rk = warp_sum(rk);
-      int cr = 0;
-      for (int p = lane; p < A * A; p += 32) {
-        const int a = p / A, b = p - a * A;
-        if (b > a) {
-          const float dx = d.ax[a0 + a] - d.ax[a0 + b], dy = d.ay[a0 + a] - d.ay[a0 + b];
-          if (sqrtf(dx * dx + dy * dy) < d.d_safe) cr = 1;
-        }
-      }
-      cr = __any_sync(0xffffffffu, cr);
-      double se = 0.0;
-      const int nfe = d.filter_off[e + 1] - f0;
-      for (int p = lane; p < nfe; p += 32) {
-        const double v = (double)d.err[f0 + p];
-        se += v * v;
-      }
-      se = warp_sum_d(se);
-      const float r = cr ? -1.0f : rk / (float)T;
+      const PosReward q = reward_positions(d, a0, A, t0, T);
+      const int nfe = d.filter_off[e + 1] - f0, cr = q.cr;
+      double se;
+      const float r = reward_errors(d, q, A, T, nfe, d.err + f0, se);
       if (lane == 0) {
         d.reward[e] = r;
         d.crash[e] = cr;

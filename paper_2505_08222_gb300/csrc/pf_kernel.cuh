@@ -43,6 +43,16 @@ __device__ __forceinline__ void cp_async4(float* dst_smem, const float* src) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// Barrier of the NT threads that run the filter: the whole CTA, or (SUB) all
+// but the environment's warp in the persistent rollout.
+template <int NT, bool SUB>
+__device__ __forceinline__ void filter_bar() {
+  if constexpr (SUB)
+    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+  else
+    __syncthreads();
+}
+
 __device__ __forceinline__ float sqrt_approx(float x) {
   float y;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -79,14 +89,14 @@ __device__ __forceinline__ float warp_max_redux(float v) {
 }
 
 // Block maximum.
-template <int NT>
+template <int NT, bool SUB>
 __device__ __forceinline__ float block_max(float v, ScanScratch* sc) {
   constexpr int NW = NT / 32;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   v = warp_max_redux(v);
   if (NW == 1) return v;
   if (lane == 0) sc->max[wid] = v;
-  __syncthreads();
+  filter_bar<NT, SUB>();
   return warp_max_redux(lane < NW ? sc->max[lane] : -INFINITY);
 }
 
@@ -97,7 +107,7 @@ __device__ __forceinline__ float block_max(float v, ScanScratch* sc) {
 // 2^27, sum r^2 <= 2^42, both sides below 2^59.  One exchange through shared
 // memory; every warp reduces the warp sums itself, so the decision is the
 // same in all of them.  sc->e1 / e2 are used once per CTA.
-template <int NT>
+template <int NT, bool SUB>
 __device__ __forceinline__ bool block_ess_trigger(unsigned long long s1, unsigned long long s2, int k, int P,
                                                   ScanScratch* sc) {
   constexpr int NW = NT / 32;
@@ -112,7 +122,7 @@ __device__ __forceinline__ bool block_ess_trigger(unsigned long long s1, unsigne
       sc->e1[wid] = s1;
       sc->e2[wid] = s2;
     }
-    __syncthreads();
+    filter_bar<NT, SUB>();
     s1 = lane < NW ? sc->e1[lane] : 0ull;
     s2 = lane < NW ? sc->e2[lane] : 0ull;
 #pragma unroll
@@ -128,7 +138,7 @@ __device__ __forceinline__ bool block_ess_trigger(unsigned long long s1, unsigne
 // fused with the block sums of fx and fy (returned in place, and kept in
 // sc->fsum): one exchange through shared memory; the cross-warp scan and the
 // two sums run on three different warps.
-template <int NT>
+template <int NT, bool SUB = false>
 __device__ __forceinline__ long long block_scan_sums(long long v, float& fx, float& fy, ScanScratch* sc,
                                                      long long& W) {
   constexpr int NW = NT / 32;
@@ -155,7 +165,7 @@ __device__ __forceinline__ long long block_scan_sums(long long v, float& fx, flo
     sc->fx[wid] = fx;
     sc->fy[wid] = fy;
   }
-  __syncthreads();
+  filter_bar<NT, SUB>();
   constexpr int WX = NW >= 2 ? 1 : 0, WY = NW >= 3 ? 2 : WX;
   if (wid == 0) {
     long long t = lane < NW ? sc->tot[lane] : 0;
@@ -174,7 +184,7 @@ __device__ __forceinline__ long long block_scan_sums(long long v, float& fx, flo
     const float b = warp_sum(lane < NW ? sc->fy[lane] : 0.0f);
     if (lane == 0) sc->fsum[1] = b;
   }
-  __syncthreads();
+  filter_bar<NT, SUB>();
   W = sc->pre[NW - 1];
   fx = sc->fsum[0];
   fy = sc->fsum[1];
@@ -188,7 +198,7 @@ __device__ __forceinline__ long long block_scan_sums(long long v, float& fx, flo
 // the warp it comes from the nearest lower lane that holds one (a ballot and
 // one shuffle), across warps from the maximum of the earlier warps' last
 // markers (warp reductions).  sc->mtot is used once per CTA.
-template <int NT>
+template <int NT, bool SUB>
 __device__ __forceinline__ int block_prev_marker(int run, ScanScratch* sc) {
   constexpr int NW = NT / 32;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -198,7 +208,7 @@ __device__ __forceinline__ int block_prev_marker(int run, ScanScratch* sc) {
   if (NW == 1) return excl;
   const int last = __reduce_max_sync(0xffffffffu, run);
   if (lane == 0) sc->mtot[wid] = last;
-  __syncthreads();
+  filter_bar<NT, SUB>();
   const int prev = __reduce_max_sync(0xffffffffu, lane < wid ? sc->mtot[lane] : -1);
   return max(prev, excl);
 }
@@ -265,7 +275,7 @@ __device__ __forceinline__ int count_at(float v, float eps, const float* s_w, in
 // U0) / W (|b| <= P + 1) within 4u (P + 1); the fma rounds by u (P + 1);
 // cw replaces the floored q's by w 2^-38 2^38, which moves v by at most
 // P PPT 2^-38.  Total below (PPT + 9) u (P + 1); eps is twice that.
-template <int NT, int PPT, bool FULL>
+template <int NT, int PPT, bool FULL, bool SUB = false>
 __device__ __forceinline__ void resample_map(const float (&w)[PPT], long long excl, long long W, int base, int P,
                                              long long* s_excl, float* s_w, int* s_mark, ScanScratch* sc,
                                              int (&idx)[PPT], int* status) {
@@ -292,7 +302,7 @@ __device__ __forceinline__ void resample_map(const float (&w)[PPT], long long ex
       lo = hi;
     }
   }
-  __syncthreads();
+  filter_bar<NT, SUB>();
   int m[PPT];
   int run = -1;
 #pragma unroll
@@ -305,7 +315,7 @@ __device__ __forceinline__ void resample_map(const float (&w)[PPT], long long ex
     if (!FULL && base + q >= P) m[q] = -1;
     run = max(run, m[q]);
   }
-  int before = block_prev_marker<NT>(run, sc);
+  int before = block_prev_marker<NT, SUB>(run, sc);
 #pragma unroll
   for (int q = 0; q < PPT; ++q) {
     before = max(before, m[q]);
@@ -333,10 +343,11 @@ struct Shared {
 // (float4 streams, no slot is out of range).  ESS: weights carried across
 // steps as log-weights d.pw, resampling only when triggered.  The shared
 // memory is the kernel's: a caller that calls it again must put a block
-// barrier between the calls.
-template <int NT, int PPT, int MODE, bool ESS, bool RES>
-__device__ __forceinline__ void pf_step_body(const EnvDev& d, const int f, const uint32_t g, float (&x)[PPT],
-                                             float (&y)[PPT], float (&vx)[PPT], float (&vy)[PPT]) {
+// barrier between the calls.  SUB: the CTA has other warps beside these NT
+// threads (filter_bar).
+template <int NT, int PPT, int MODE, bool ESS, bool RES, bool SUB, typename Lists>
+__device__ __forceinline__ void pf_step_body(const EnvDev& d, const Lists& lists, const int f, const uint32_t g,
+                                             float (&x)[PPT], float (&y)[PPT], float (&vx)[PPT], float (&vy)[PPT]) {
   static_assert(PPT % 4 == 0, "PPT must be a multiple of 4");
   constexpr bool VEC = MODE >= 1, FULL = MODE == 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -366,9 +377,9 @@ __device__ __forceinline__ void pf_step_body(const EnvDev& d, const int f, const
   }
   // measurement list and the filter's header (senders are at the surface:
   // the vertical offset of every range is the target depth)
-  if (tid < d.AM) sh.meas[tid] = d.meas[(long long)f * d.AM + tid];
+  if (tid < d.AM) sh.meas[tid] = lists.meas()[(long long)f * d.AM + tid];
   if (tid == 0) {
-    const float4 hd = d.meas_hdr[f];
+    const float4 hd = lists.hdr()[f];
     sh.tgt[0] = hd.x;
     sh.tgt[1] = hd.y;
     sh.dz2 = hd.z;
@@ -436,7 +447,7 @@ __device__ __forceinline__ void pf_step_body(const EnvDev& d, const int f, const
       y[qq] = fmaf(d.dt, uy, y[qq]);
     }
   }
-  __syncthreads();  // sh.* visible
+  filter_bar<NT, SUB>();  // sh.* visible
 
   // weight (log domain); measurements outer, particles inner
   const int nm = UT_IN_BOUNDS(sh.nm >= 0 && sh.nm <= d.AM && d.AM <= kMaxAgents, d.status) ? sh.nm : 0;
@@ -486,7 +497,7 @@ __device__ __forceinline__ void pf_step_body(const EnvDev& d, const int f, const
     acc[q] = ESS ? fmaf(-acc[q], d.inv_two_s2, pwv[q]) : -acc[q] * d.inv_two_s2;
     if (FULL || base + q < P) lmax = fmaxf(lmax, acc[q]);
   }
-  lmax = block_max<NT>(lmax, &sh.scan);
+  lmax = block_max<NT, SUB>(lmax, &sh.scan);
   // max-normalised weights, their exact integer images floor(w 2^38) summed
   // per thread, and the estimate's weighted sums
   float w[PPT];
@@ -522,7 +533,7 @@ __device__ __forceinline__ void pf_step_body(const EnvDev& d, const int f, const
       s1 += r;
       s2 += r * r;
     }
-    resample = block_ess_trigger<NT>(s1, s2, d.pf_ess_num, P, &sh.scan) && nm > 0;
+    resample = block_ess_trigger<NT, SUB>(s1, s2, d.pf_ess_num, P, &sh.scan) && nm > 0;
 #pragma unroll
     for (int q = 0; q < PPT; ++q)
       if (FULL || base + q < P) d.pw[off + base + q] = resample ? 0.0f : acc[q] - lmax;
@@ -536,9 +547,9 @@ __device__ __forceinline__ void pf_step_body(const EnvDev& d, const int f, const
 #pragma unroll
     for (int q = 0; q < PPT; ++q) s_part[q * NT + tid] = make_float4(x[q], y[q], vx[q], vy[q]);
     init_markers<PPT>(s_mark, base);
-    const long long excl = block_scan_sums<NT>(qsum, swx, swy, &sh.scan, W);  // contains barriers
+    const long long excl = block_scan_sums<NT, SUB>(qsum, swx, swy, &sh.scan, W);  // contains barriers
     if (NT == 32) __syncwarp();  // single-warp blocks: order the shared-memory stores
-    resample_map<NT, PPT, FULL>(w, excl, W, base, P, s_excl, s_w, s_mark, &sh.scan, idx, d.status);
+    resample_map<NT, PPT, FULL, SUB>(w, excl, W, base, P, s_excl, s_w, s_mark, &sh.scan, idx, d.status);
 #pragma unroll
     for (int q = 0; q < PPT; ++q) {
       const int sl = slot_of<NT, PPT>(idx[q]);
@@ -549,7 +560,7 @@ __device__ __forceinline__ void pf_step_body(const EnvDev& d, const int f, const
       vy[q] = pnew.w;
     }
   } else {
-    block_scan_sums<NT>(qsum, swx, swy, &sh.scan, W);
+    block_scan_sums<NT, SUB>(qsum, swx, swy, &sh.scan, W);
     if (NT == 32) __syncwarp();
 #pragma unroll
     for (int q = 0; q < PPT; ++q) idx[q] = base + q;
@@ -611,7 +622,7 @@ __device__ __forceinline__ void pf_step_body(const EnvDev& d, const int f, const
     d.estx[f] = ex;
     d.esty[f] = ey;
     const float dx = ex - sh.tgt[0], dy = ey - sh.tgt[1];
-    d.err[f] = sqrtf(dx * dx + dy * dy);
+    lists.err()[f] = sqrtf(dx * dx + dy * dy);
   }
 }
 
@@ -687,7 +698,7 @@ template <int NT, int PPT, int MINB, int MODE, bool ESS>
 __global__ void __launch_bounds__(NT, MINB) pf_step_kernel(EnvDev d) {
   pdl_wait();  // (dependents launch as this grid's CTAs exit: no early trigger in a many-wave kernel)
   float x[PPT], y[PPT], vx[PPT], vy[PPT];
-  pf_step_body<NT, PPT, MODE, ESS, false>(d, (int)blockIdx.x, d.counters[0] + 1u, x, y, vx, vy);
+  pf_step_body<NT, PPT, MODE, ESS, false, false>(d, HandleLists{d}, (int)blockIdx.x, d.counters[0] + 1u, x, y, vx, vy);
 }
 
 // Stand-alone resample map (same device code as the fused step).
