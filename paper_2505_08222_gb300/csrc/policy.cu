@@ -212,10 +212,11 @@ __device__ __forceinline__ void pump(Loader& ld, const unsigned char* __restrict
 __device__ __forceinline__ void issue_mma(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, int N, int K,
                                           bool accumulate) {
   const uint32_t idesc = tc::idesc_bf16(128, (uint32_t)N);
+  uint64_t ad = tc::smem_desc(a_addr, 128 * 16, 128), bd = tc::smem_desc(b_addr, N * 16, 128);
   for (int k = 0; k < K / 16; ++k) {
-    const uint64_t ad = tc::smem_desc(a_addr + k * 2 * 128 * 16, 128 * 16, 128);
-    const uint64_t bd = tc::smem_desc(b_addr + k * 2 * N * 16, N * 16, 128);
     tc::mma_bf16(d_tmem, ad, bd, idesc, (accumulate || k > 0) ? 1u : 0u);
+    ad = tc::desc_advance(ad, 2 * 128 * 16);
+    bd = tc::desc_advance(bd, 2 * N * 16);
   }
 }
 
@@ -224,9 +225,10 @@ __device__ __forceinline__ void issue_mma(uint32_t d_tmem, uint32_t a_addr, uint
 __device__ __forceinline__ void issue_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_addr, int N, int K,
                                              bool accumulate) {
   const uint32_t idesc = tc::idesc_bf16(128, (uint32_t)N);
+  uint64_t bd = tc::smem_desc(b_addr, N * 16, 128);
   for (int k = 0; k < K / 16; ++k) {
-    const uint64_t bd = tc::smem_desc(b_addr + k * 2 * N * 16, N * 16, 128);
     tc::mma_bf16_ts(d_tmem, a_tmem + (uint32_t)(k * 8), bd, idesc, (accumulate || k > 0) ? 1u : 0u);
+    bd = tc::desc_advance(bd, 2 * N * 16);
   }
 }
 
@@ -1210,10 +1212,67 @@ __global__ void __launch_bounds__(Geo<D>::THREADS, D == 64 ? 2 : 1) policy_fwd_k
   }
   __syncthreads();
   const bool good = bad == 0;
-  // (kTail: four agents per warp at a time, for their independent chains)
-  constexpr int AG = MODE == kTail ? 4 : 1, NW = kThreads / 32;
 #pragma unroll 1
-  for (int sl = warp; MODE != kBody && sl < apt && good; sl += AG * NW) {
+  for (int sl = warp; MODE == kWhole && sl < p.apt && good; sl += kThreads / 32) {
+    const int lane = tid & 31, n_act = p.n_act;
+    const long long a2 = (long long)blockIdx.x * p.apt + sl;
+    if (a2 < p.NA) {  // (warp-uniform)
+      float y[D / 32];
+#pragma unroll
+      for (int i = 0; i < D / 32; ++i) y[i] = sY[sl * D + lane + 32 * i];
+      float mine = 0.0f;  // lane j: logit of action j
+      for (int j0 = 0; j0 < n_act; j0 += 8) {
+        float acc[8];
+#pragma unroll
+        for (int jj = 0; jj < 8; ++jj) {
+          acc[jj] = 0.0f;
+          if (j0 + jj < n_act) {
+            const float* w = p.head_w + (size_t)(j0 + jj) * D + lane;
+#pragma unroll
+            for (int i = 0; i < D / 32; ++i) acc[jj] = fmaf(__ldg(w + 32 * i), y[i], acc[jj]);
+          }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int jj = 0; jj < 8; ++jj) acc[jj] += __shfl_xor_sync(0xffffffffu, acc[jj], o);
+#pragma unroll
+        for (int jj = 0; jj < 8; ++jj)
+          if (lane == j0 + jj) mine = acc[jj];
+      }
+      if (lane < n_act) {
+        mine += __ldg(p.head_b + lane);
+        p.logits[a2 * n_act + lane] = mine;
+      }
+      if (p.sample) {
+        float z = -INFINITY;
+        int arg = lane;
+        if (lane < n_act) {
+          const uint32_t g = p.counters ? p.counters[0] + 1u : p.step;
+          const Rand4 r = philox(p.gid_agent + (uint32_t)a2, (uint32_t)(lane >> 2), g, TAG_GUMBEL, p.seed);
+          const int q = lane & 3;
+          const uint32_t u = q == 0 ? r.x[0] : (q == 1 ? r.x[1] : (q == 2 ? r.x[2] : r.x[3]));
+          z = mine - logf(-logf(unif_mid(u)));
+          if (!(z == z)) z = -INFINITY;  // a NaN never wins
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const float oz = __shfl_xor_sync(0xffffffffu, z, o);
+          const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
+          if (oz > z || (oz == z && oa < arg)) {
+            z = oz;
+            arg = oa;
+          }
+        }
+        if (lane == 0) p.actions[a2] = arg;
+      }
+    }
+  }
+
+  // (kTail: four agents per warp at a time, for their independent chains)
+  constexpr int AG = 4, NW = kThreads / 32;
+#pragma unroll 1
+  for (int sl = warp; MODE == kTail && sl < apt && good; sl += AG * NW) {
     const int lane = tid & 31, n_act = p.n_act;
     long long a2[AG];
     bool on[AG];  // (warp-uniform)
@@ -1222,7 +1281,7 @@ __global__ void __launch_bounds__(Geo<D>::THREADS, D == 64 ? 2 : 1) policy_fwd_k
     for (int k = 0; k < AG; ++k) {
       const int s2 = sl + k * NW;
       a2[k] = (long long)blockIdx.x * apt + s2;
-      on[k] = s2 < apt && a2[k] < p.NA && (MODE != kTail || p.ws_ok[a2[k] / p.apt] != 0);
+      on[k] = s2 < apt && a2[k] < p.NA && p.ws_ok[a2[k] / p.apt] != 0;
       mine[k] = 0.0f;
 #pragma unroll
       for (int i = 0; i < D / 32; ++i) y[k][i] = on[k] ? sY[s2 * D + lane + 32 * i] : 0.0f;
