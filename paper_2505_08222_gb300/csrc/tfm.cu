@@ -1775,26 +1775,37 @@ __global__ void pack_images_kernel(const float* __restrict__ prm, const int64_t*
 
 inline unsigned blocks_for(long long n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
+// Kinds 0 / 1 on the tensor cores.  CTAs loop over the row tiles: about as many
+// per SM per column tile as fit (three for N <= 128, two for the wider
+// products).
+template <int EPI>
+cudaError_t launch_tc_rows(const Gemm& g, cudaStream_t s) {
+  static std::atomic<unsigned long long> ready{0};
+  const cudaError_t e = smem_optin(tc_rows_kernel<EPI>, kTcRowsSmem, ready);
+  if (e != cudaSuccess) return e;
+  const size_t smem = tc_rows_smem(g.N);
+  const int per_sm = std::min(smem <= 72 * 1024 ? 3 : 2, tc_rows_ctas<EPI>());
+  const long long tiles = (g.M + 127) / 128;
+  const int n_tiles = (g.N + kTcMaxN - 1) / kTcMaxN;
+  long long ctas = (per_sm * 152 + n_tiles - 1) / n_tiles;
+  if (ctas > tiles) ctas = tiles;
+  tc_rows_kernel<EPI><<<dim3((unsigned)ctas, (unsigned)n_tiles), kTcThreads, smem, s>>>(g, g.bimg, g.status);
+  return cudaGetLastError();
+}
+
 // kind 0: forward (A row-major, B = W [N][K]); 1: input gradient (A
 // row-major, B = W [K][N]); 2: weight gradient (A and B indexed [k][.]).
 cudaError_t gemm(int kind, const Gemm& g, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0 || g.K <= 0) return cudaSuccess;
   if (kind != 2 && g.bimg && g.K % 32 == 0 && g.N % 32 == 0 && g.lda % 4 == 0 && g.ldc % 4 == 0 &&
       ((uintptr_t)g.A & 15) == 0 && ((uintptr_t)g.C & 15) == 0 && g.kchunk == g.K) {
-    static std::atomic<unsigned long long> ready{0};
-    cudaError_t e = smem_optin(tc_rows_kernel, kTcSmem, ready);
-    if (e != cudaSuccess) return e;
-    // CTAs loop over the row tiles: about as many per SM per column tile as
-    // fit (three for N <= 128, two for the wider products)
-    const size_t smem = tc_rows_smem(g.N);
-    const int per_sm = smem <= 72 * 1024 ? 3 : 2;
-    const long long tiles = (g.M + 127) / 128;
-    const int n_tiles = (g.N + kTcMaxN - 1) / kTcMaxN;
-    long long ctas = (per_sm * 152 + n_tiles - 1) / n_tiles;
-    if (ctas > tiles) ctas = tiles;
-    dim3 grid((unsigned)ctas, (unsigned)n_tiles);
-    tc_rows_kernel<<<grid, kTcThreads, smem, s>>>(g, g.bimg, g.status);
-    return cudaGetLastError();
+    switch (g.epi) {
+      case EPI_BIAS: return launch_tc_rows<EPI_BIAS>(g, s);
+      case EPI_BIAS_RES: return launch_tc_rows<EPI_BIAS_RES>(g, s);
+      case EPI_BIAS_GELU: return launch_tc_rows<EPI_BIAS_GELU>(g, s);
+      case EPI_GELU_GRAD: return launch_tc_rows<EPI_GELU_GRAD>(g, s);
+      default: return launch_tc_rows<EPI_STORE>(g, s);
+    }
   }
   const long long kc = g.kchunk > 0 ? g.kchunk : g.K;
   dim3 grid((unsigned)((g.M + 63) / 64), (unsigned)((g.N + 63) / 64), (unsigned)((g.K + kc - 1) / kc));

@@ -28,6 +28,10 @@ constexpr int kTcMaxN = 256;        // N per CTA (tensor-memory columns)
 constexpr size_t kTcStageA = (size_t)128 * kTcChunk * 2;      // 16 KB
 constexpr size_t kTcStageB = (size_t)kTcMaxN * kTcChunk * 2;  // 32 KB
 constexpr size_t kTcSmem = 2 * (kTcStageA + kTcStageB);       // 96 KB
+constexpr uint32_t kTcGrpA = 128 * 16 + 32;                   // tc_rows_kernel: bytes of 8 columns of A
+constexpr size_t kTcRowsA = (kTcChunk / 8) * (size_t)kTcGrpA; // and of its stage
+constexpr int kEpiRows = 4;                                   // rows of a thread per epilogue load
+constexpr size_t kTcRowsSmem = 2 * (kTcRowsA + kTcStageB);
 constexpr uint32_t kTcPolls = 1u << 22;
 
 // Columns of tensor memory for an N-wide accumulator (a power of two >= 32).
@@ -50,36 +54,26 @@ __host__ __device__ inline size_t img_offset(int r, int c, int R, int C) {
 __device__ __forceinline__ uint32_t pack_bf2(float lo, float hi) { return bf16x2_bits(lo, hi); }
 
 // The epilogue of four consecutive outputs (m, n .. n + 3) (float4 form of
-// epi_store; ldc, n multiples of 4).
-__device__ __forceinline__ void epi_store4(const Gemm& g, long long m, int n, float4 v) {
+// epi_store; ldc, ldr, n multiples of 4): b the bias, q what it reads beside
+// the accumulator (epi_reads: the residual or the pre-activations).
+template <int EPI>
+__device__ constexpr bool epi_reads() {
+  return EPI == EPI_BIAS_RES || EPI == EPI_GELU_GRAD;
+}
+template <int EPI>
+__device__ __forceinline__ float4 epi_load4(const Gemm& g, long long m, int n) {
+  return *reinterpret_cast<const float4*>(EPI == EPI_BIAS_RES ? g.R + m * g.ldr + n : g.aux + m * g.ldc + n);
+}
+template <int EPI>
+__device__ __forceinline__ void epi_store4(const Gemm& g, long long m, int n, float4 v, float4 b, float4 q) {
   const long long o = m * g.ldc + n;
-  float4 r;
-  switch (g.epi) {
-    case EPI_BIAS: {
-      const float4 b = *reinterpret_cast<const float4*>(g.bias + n);
-      r = make_float4(v.x + b.x, v.y + b.y, v.z + b.z, v.w + b.w);
-      break;
-    }
-    case EPI_BIAS_RES: {
-      const float4 b = *reinterpret_cast<const float4*>(g.bias + n);
-      const float4 q = *reinterpret_cast<const float4*>(g.R + m * g.ldr + n);
-      r = make_float4(v.x + b.x + q.x, v.y + b.y + q.y, v.z + b.z + q.z, v.w + b.w + q.w);
-      break;
-    }
-    case EPI_BIAS_GELU: {
-      const float4 b = *reinterpret_cast<const float4*>(g.bias + n);
-      r = make_float4(v.x + b.x, v.y + b.y, v.z + b.z, v.w + b.w);
-      *reinterpret_cast<float4*>(g.C2 + o) = make_float4(gelu_f(r.x), gelu_f(r.y), gelu_f(r.z), gelu_f(r.w));
-      break;
-    }
-    case EPI_GELU_GRAD: {
-      const float4 z = *reinterpret_cast<const float4*>(g.aux + o);
-      r = make_float4(v.x * gelu_grad_f(z.x), v.y * gelu_grad_f(z.y), v.z * gelu_grad_f(z.z), v.w * gelu_grad_f(z.w));
-      break;
-    }
-    default:
-      r = v;
-  }
+  float4 r = v;
+  if (EPI == EPI_BIAS || EPI == EPI_BIAS_GELU) r = make_float4(v.x + b.x, v.y + b.y, v.z + b.z, v.w + b.w);
+  if (EPI == EPI_BIAS_RES) r = make_float4(v.x + b.x + q.x, v.y + b.y + q.y, v.z + b.z + q.z, v.w + b.w + q.w);
+  if (EPI == EPI_GELU_GRAD)
+    r = make_float4(v.x * gelu_grad_f(q.x), v.y * gelu_grad_f(q.y), v.z * gelu_grad_f(q.z), v.w * gelu_grad_f(q.w));
+  if (EPI == EPI_BIAS_GELU)
+    *reinterpret_cast<float4*>(g.C2 + o) = make_float4(gelu_f(r.x), gelu_f(r.y), gelu_f(r.z), gelu_f(r.w));
   *reinterpret_cast<float4*>(g.C + o) = r;
 }
 
@@ -93,7 +87,7 @@ inline size_t tc_wgrad_smem(int n_i) {
 // epilogue's staging tile overlays them) and two B stages sized for
 // min(N, 256) rows; narrow products fit three CTAs per SM.
 inline size_t tc_rows_smem(int N) {
-  return 2 * kTcStageA + 2 * (size_t)std::min(kTcMaxN, N) * kTcChunk * 2;
+  return 2 * kTcRowsA + 2 * (size_t)std::min(kTcMaxN, N) * kTcChunk * 2;
 }
 
 // Kinds 0 / 1: C[m][n] = sum_k A[m][k] B(n, k) + epilogue, A FP32 row-major
@@ -105,16 +99,30 @@ inline size_t tc_rows_smem(int N) {
 // A is loaded into registers a chunk ahead (the next chunk's loads, of this
 // tile or the next, are issued as soon as the current chunk is converted,
 // so they are in flight during its MMAs and the epilogue), rounded to BF16
-// and written K-major.  The accumulator goes through a staging tile over the
-// A stages (rows of 64 floats, 16-byte chunks XOR-swizzled by row) so that
-// the epilogue reads and writes whole rows (coalesced float4 accesses).
+// and written K-major.  A warp loads two whole rows of the chunk at a time (a
+// lane per row would touch 32 lines per load); the image's groups of 8 columns
+// lie 2080 bytes apart, so its 8-byte stores hit all banks.  The accumulator
+// goes through a staging tile over the A stages (rows of 64 floats, 16-byte
+// chunks XOR-swizzled by row) so that the epilogue reads and writes whole rows
+// (coalesced float4 accesses); what it reads from memory is loaded four rows at
+// a time before any of them is stored.  Bound by HBM (FP32 activations).  The 26
+// launches of an actor step of 278,528 rows, d = 128, 3 blocks: 4720 us with a
+// lane per row and loads behind the stores, this 2963.
 __device__ __forceinline__ int epi_pos(int row, int c4) { return row * 64 + ((c4 ^ (row & 15)) << 2); }
 
-__global__ void __launch_bounds__(kTcThreads, 3) tc_rows_kernel(Gemm g, const uint16_t* __restrict__ bimg,
+// CTAs per SM that the registers allow: the GELU epilogues, in practice of
+// products too wide for three, take more of them.
+template <int EPI>
+__host__ __device__ constexpr int tc_rows_ctas() {
+  return EPI == EPI_BIAS_GELU || EPI == EPI_GELU_GRAD ? 2 : 3;
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(kTcThreads, tc_rows_ctas<EPI>()) tc_rows_kernel(Gemm g, const uint16_t* __restrict__ bimg,
                                                                 int* status) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* sA = smem;                    // [2][128 x 64] BF16
-  unsigned char* sB = smem + 2 * kTcStageA;    // [2][min(N, 256) x 64] BF16
+  unsigned char* sB = smem + 2 * kTcRowsA;     // [2][min(N, 256) x 64] BF16
   float* sE = reinterpret_cast<float*>(smem);  // epilogue staging [128][64] over the A stages
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ __align__(8) uint64_t bfull[2];
@@ -148,36 +156,25 @@ __global__ void __launch_bounds__(kTcThreads, 3) tc_rows_kernel(Gemm g, const ui
   bool ok = true;
   int q_used = 0;  // chunks committed so far (the stage ring runs across tiles)
 
-  // A of (row tile m0, chunk at k0): unit = (row, 8-column group), 2 or 4 per
-  // thread, in registers until stage_a
-  float4 xa[4][2];
+  // A of (row tile m0, chunk at k0): rows tid / 16 + 16 i, columns 4 (tid % 16)
+  // .. + 3, in registers until stage_a.  Rows past M repeat the last one (their
+  // outputs are not stored), columns past the chunk the first (not staged).
+  const int arow = tid >> 4, acol = (tid & 15) * 4;
+  float4 xa[8];
   auto load_a = [&](long long m0, int k0) {
-    const int units = 128 * (min(kTcChunk, K - k0) >> 3);
+    const float* const src = g.A + m0 * g.lda + k0 + (acol < K - k0 ? acol : 0);
+    const int last = (int)min(g.M - m0, 128LL) - 1, lda = (int)g.lda;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int u = tid + i * kTcThreads;
-      const int row = u & 127, grp = u >> 7;
-      xa[i][0] = xa[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (u < units && m0 + row < g.M) {
-        const float4* src = reinterpret_cast<const float4*>(g.A + (m0 + row) * g.lda + k0 + grp * 8);
-        xa[i][0] = __ldg(src);
-        xa[i][1] = __ldg(src + 1);
-      }
-    }
+    for (int i = 0; i < 8; ++i)
+      xa[i] = __ldg(reinterpret_cast<const float4*>(src + (long long)min(arow + 16 * i, last) * lda));
   };
-  // consecutive threads on consecutive rows of one group: conflict-free
-  // 16-byte stores
   auto stage_a = [&](unsigned char* a, int kc) {
-    const int units = 128 * (kc >> 3);
+    unsigned char* dst = a + (acol >> 3) * kTcGrpA + arow * 16 + (acol & 4) * 2;
+    if (acol < kc) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int u = tid + i * kTcThreads;
-      if (u < units) {
-        const int row = u & 127, grp = u >> 7;
-        const uint4 p = make_uint4(pack_bf2(xa[i][0].x, xa[i][0].y), pack_bf2(xa[i][0].z, xa[i][0].w),
-                                   pack_bf2(xa[i][1].x, xa[i][1].y), pack_bf2(xa[i][1].z, xa[i][1].w));
-        *reinterpret_cast<uint4*>(a + tc::kmajor_offset(row, grp * 8, 128)) = p;
-      }
+      for (int i = 0; i < 8; ++i)
+        *reinterpret_cast<uint2*>(dst + 256 * i) =
+            make_uint2(pack_bf2(xa[i].x, xa[i].y), pack_bf2(xa[i].z, xa[i].w));
     }
   };
 
@@ -192,7 +189,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) tc_rows_kernel(Gemm g, const ui
         phase ^= 1u << s;
         tc::fence_after_sync();
       }
-      unsigned char* a = sA + s * kTcStageA;
+      unsigned char* a = sA + s * kTcRowsA;
       unsigned char* b = sB + (size_t)s * b_stage;
       const bool b_new = !b_resident || q_used < 2;
       if (b_new && tid == 0) {  // the stage is free: its last MMA has completed
@@ -218,10 +215,11 @@ __global__ void __launch_bounds__(kTcThreads, 3) tc_rows_kernel(Gemm g, const ui
             ok = false, bpend |= 1u << s;
         }
         const uint32_t aa = tc::smem_addr(a), bb = tc::smem_addr(b);
+        uint64_t ad = tc::smem_desc(aa, kTcGrpA, 128), bd = tc::smem_desc(bb, Nt * 16, 128);
         for (int j = 0; j < kc / 16; ++j) {
-          const uint64_t ad = tc::smem_desc(aa + j * 2 * 128 * 16, 128 * 16, 128);
-          const uint64_t bd = tc::smem_desc(bb + j * 2 * Nt * 16, Nt * 16, 128);
           tc::mma_bf16(tmem, ad, bd, idesc, (c > 0 || j > 0) ? 1u : 0u);
+          ad = tc::desc_advance(ad, 2 * kTcGrpA);
+          bd = tc::desc_advance(bd, 2 * Nt * 16);
         }
         tc::mma_commit(&mbar[s]);
       }
@@ -257,13 +255,22 @@ __global__ void __launch_bounds__(kTcThreads, 3) tc_rows_kernel(Gemm g, const ui
       tc::fence_before_sync();
       __syncthreads();
       tc::fence_after_sync();
-      const int per_row = cw / 4;  // float4 per row: 8 or 16
-      for (int u = tid; u < 128 * per_row; u += kTcThreads) {
-        const int row = u / per_row, c4 = u - row * per_row;
-        const long long m = m0 + row;
-        if (m < g.M) {
-          const float4 v = *reinterpret_cast<const float4*>(sE + epi_pos(row, c4));
-          epi_store4(g, m, n0 + c0 + c4 * 4, v);
+      const int sh = cw == 64 ? 4 : 3;  // 16 or 8 float4 per row
+      const int c4 = tid & ((1 << sh) - 1), n = n0 + c0 + c4 * 4, step = kTcThreads >> sh;
+      const int rows = (int)min(g.M - m0, 128LL);
+      float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (EPI == EPI_BIAS || EPI == EPI_BIAS_RES || EPI == EPI_BIAS_GELU) b = __ldg(reinterpret_cast<const float4*>(g.bias + n));
+      for (int r0 = tid >> sh; r0 < rows; r0 += kEpiRows * step) {
+        float4 q[kEpiRows];
+        if constexpr (epi_reads<EPI>()) {
+#pragma unroll
+          for (int i = 0; i < kEpiRows; ++i) q[i] = epi_load4<EPI>(g, m0 + min(r0 + i * step, rows - 1), n);
+        }
+#pragma unroll
+        for (int i = 0; i < kEpiRows; ++i) {
+          const int row = r0 + i * step;
+          if (row < rows)
+            epi_store4<EPI>(g, m0 + row, n, *reinterpret_cast<const float4*>(sE + epi_pos(row, c4)), b, q[i]);
         }
       }
       __syncthreads();  // the staging tile (the A stages) is free again
@@ -337,14 +344,27 @@ __global__ void __launch_bounds__(kTcThreads, 3) tc_wgrad_kernel(Gemm g, float* 
     // their FP32 values for the bias gradient.  B (In): Ntp / 32 blocks, two
     // at a time.
     {
+      // (every load is issued, past the end from the last row or column: a
+      // load behind a condition waits for the one before it; 13 launches of a
+      // d = 128 step of 278,528 rows 2237 -> 1778 us)
       const long long mrow = m0 + warp * 8;
+      const int left = (int)min(r1 - mrow, 8LL);  // (may be negative)
+      const float* const pa = g.A + mrow * g.lda;
+      const float* const pb = g.B + mrow * g.ldb;
+      const int lda = (int)g.lda, ldb = (int)g.ldb;
       float va[4][8];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int gcol = nb0 + j * 32 + lane;
+        const int gcol = min(nb0 + j * 32 + lane, n_o - 1);
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-          va[j][i] = (mrow + i < r1 && gcol < n_o) ? __ldg(g.A + (mrow + i) * g.lda + gcol) : 0.0f;
+        for (int i = 0; i < 8; ++i) va[j][i] = __ldg(pa + min(i, left - 1) * lda + gcol);
+      }
+      if (left < 8 || nb0 + 128 > n_o) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (i >= left || nb0 + j * 32 + lane >= n_o) va[j][i] = 0.0f;
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -360,10 +380,16 @@ __global__ void __launch_bounds__(kTcThreads, 3) tc_wgrad_kernel(Gemm g, float* 
         float vb[2][8];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          const int gcol = kb0 + (j0 + h) * 32 + lane;
-          const bool on = j0 + h < Ntp / 32 && gcol < n_i;
+          const int gcol = min(kb0 + (j0 + h) * 32 + lane, n_i - 1);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) vb[h][i] = (on && mrow + i < r1) ? __ldg(g.B + (mrow + i) * g.ldb + gcol) : 0.0f;
+          for (int i = 0; i < 8; ++i) vb[h][i] = __ldg(pb + min(i, left - 1) * ldb + gcol);
+        }
+        if (left < 8 || kb0 + (j0 + 2) * 32 > n_i) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              if (i >= left || kb0 + (j0 + h) * 32 + lane >= n_i) vb[h][i] = 0.0f;
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
