@@ -743,10 +743,25 @@ __device__ __forceinline__ void mma16x16(float (&c)[2][4], const float* a, const
   }
 }
 
+// (sample, head) of item w: a 32-bit division wherever it is enough.
+struct AttItem {
+  long long s;
+  int hh;
+};
+__device__ __forceinline__ AttItem att_item(long long w, int H) {
+  if ((w >> 32) == 0) {
+    const uint32_t s = (uint32_t)w / (uint32_t)H;
+    return {(long long)s, (int)((uint32_t)w - s * (uint32_t)H)};
+  }
+  const long long s = w / H;
+  return {s, (int)(w - s * H)};
+}
+
 // Per-warp staging of one (sample, head) item: rows u = lane / 4 + 8 r
 // (r = 0, 1) of the item's 16-wide Q, K, V slices (and dO in the backward),
-// quarter lane % 4 of each row, as float4; rows u >= T are zero.  The warps
-// are persistent: the next item's slices are loaded into registers while the
+// quarter lane % 4 of each row, as float4; rows u >= T are zero (and not
+// loaded: loading a row that exists in their place was slower).  The warps are
+// persistent: the next item's slices are loaded into registers while the
 // current item is computed from shared memory.
 struct AttRows {
   float4 q[2], k[2], v[2];
@@ -770,6 +785,20 @@ __device__ __forceinline__ void att_stage(const float4 (&x)[2], float* dst, int 
   const int u0 = lane >> 2, j4 = lane & 3;
 #pragma unroll
   for (int i = 0; i < 2; ++i) *reinterpret_cast<float4*>(dst + (u0 + 8 * i) * kAttLd + 4 * j4) = x[i];
+}
+
+// A row's two accumulator tiles to memory: lanes t and t ^ 1 of a quad trade, so
+// that the even one has columns 2 t .. 2 t + 3 of the first tile and the odd one
+// columns 8 + 2 (t - 1) .. of the second: half the stores, of whole sectors
+// (655,360 items of 11 tokens: forward 504 -> 495 us, backward 872 -> 846).
+// (Every lane of the warp calls it; `row` 16 floats, 16-byte aligned.)
+__device__ __forceinline__ void att_store_row(float* row, float2 lo, float2 hi, int t, bool on) {
+  const bool odd = t & 1;
+  const float2 give = odd ? lo : hi;
+  const float gx = __shfl_xor_sync(0xffffffffu, give.x, 1), gy = __shfl_xor_sync(0xffffffffu, give.y, 1);
+  if (on)
+    *reinterpret_cast<float4*>(row + (odd ? 6 + 2 * t : 2 * t)) =
+        odd ? make_float4(gx, gy, hi.x, hi.y) : make_float4(lo.x, lo.y, gx, gy);
 }
 
 // Blocks of `threads` threads of `kernel` resident on the device at once (at
@@ -813,15 +842,16 @@ __global__ void __launch_bounds__(128, 8)
   long long w = (long long)blockIdx.x * 4 + wl;
   AttRows r;
   int ne_next = 0;
+  AttItem nx = {0, 0};
   auto fetch = [&](long long wi) {
-    const long long s = wi / H;
-    att_fetch(r, QKV, s, (int)(wi - s * H), T, d, lane);
-    ne_next = __ldg(n_ent + (sel ? (long long)__ldg(sel + s) : s));
+    nx = att_item(wi, H);
+    att_fetch(r, QKV, nx.s, nx.hh, T, d, lane);
+    ne_next = __ldg(n_ent + (sel ? (long long)__ldg(sel + nx.s) : nx.s));
   };
   if (w < items) fetch(w);
   for (; w < items; w += stride) {
-    const long long s = w / H;
-    const int hh = (int)(w - s * H);
+    const long long s = nx.s;
+    const int hh = nx.hh;
     att_stage(r.q, sQ, lane);
     att_stage(r.k, sK, lane);
     att_stage(r.v, sV, lane);
@@ -877,12 +907,8 @@ __global__ void __launch_bounds__(128, 8)
 #pragma unroll
     for (int hr = 0; hr < 2; ++hr) {
       const int row = g + 8 * hr;
-      if (row < T) {
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-          *reinterpret_cast<float2*>(O + (s * T + row) * d + hh * 16 + 8 * j + 2 * t) =
-              make_float2(o[j][2 * hr], o[j][2 * hr + 1]);
-      }
+      att_store_row(O + (s * T + row) * d + hh * 16, make_float2(o[0][2 * hr], o[0][2 * hr + 1]),
+                    make_float2(o[1][2 * hr], o[1][2 * hr + 1]), t, row < T);
     }
     __syncwarp();  // the staged tiles are read before the next item overwrites them
   }
@@ -916,25 +942,25 @@ __global__ void __launch_bounds__(128, 6)
   AttRows r;
   float4 rg[2];
   float rp[4];
+  AttItem nx = {0, 0};
   auto fetch = [&](long long wi) {
-    const long long s = wi / H;
-    const int hh = (int)(wi - s * H);
-    att_fetch(r, QKV, s, hh, T, d, lane);
+    nx = att_item(wi, H);
+    att_fetch(r, QKV, nx.s, nx.hh, T, d, lane);
     const int u0 = lane >> 2, j4 = lane & 3;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const int u = u0 + 8 * i;
-      rg[i] = u < T ? __ldg(reinterpret_cast<const float4*>(dO + (s * T + u) * d + hh * 16) + j4)
+      rg[i] = u < T ? __ldg(reinterpret_cast<const float4*>(dO + (nx.s * T + u) * d + nx.hh * 16) + j4)
                     : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    const float* Pb = P + (s * H + hh) * T * T;
+    const float* Pb = P + wi * T * T;
 #pragma unroll
     for (int i = 0; i < 4; ++i) rp[i] = pofs[i] >= 0 ? __ldg(Pb + lane + 32 * i) : 0.0f;
   };
   if (w < items) fetch(w);
   for (; w < items; w += stride) {
-    const long long s = w / H;
-    const int hh = (int)(w - s * H);
+    const long long s = nx.s;
+    const int hh = nx.hh;
     att_stage(r.q, sQ, lane);
     att_stage(r.k, sK, lane);
     att_stage(r.v, sV, lane);
@@ -983,15 +1009,13 @@ __global__ void __launch_bounds__(128, 6)
 #pragma unroll
     for (int hr = 0; hr < 2; ++hr) {
       const int row = g + 8 * hr;
-      if (row < T) {
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int c = 8 * j + 2 * t;
-          *reinterpret_cast<float2*>(out + row * ld + c) = make_float2(dq[j][2 * hr], dq[j][2 * hr + 1]);
-          *reinterpret_cast<float2*>(out + row * ld + d + c) = make_float2(dk[j][2 * hr], dk[j][2 * hr + 1]);
-          *reinterpret_cast<float2*>(out + row * ld + 2 * d + c) = make_float2(dv[j][2 * hr], dv[j][2 * hr + 1]);
-        }
-      }
+      auto store = [&](float* dst, const float (&c)[2][4]) {
+        att_store_row(dst + row * ld, make_float2(c[0][2 * hr], c[0][2 * hr + 1]),
+                      make_float2(c[1][2 * hr], c[1][2 * hr + 1]), t, row < T);
+      };
+      store(out, dq);
+      store(out + d, dk);
+      store(out + 2 * d, dv);
     }
     __syncwarp();  // the staged tiles are read before the next item overwrites them
   }
@@ -1009,7 +1033,10 @@ __global__ void __launch_bounds__(128, 6)
 // are row 0 of P and O above, by the same arithmetic.  The cost is one read
 // of K and V (and in the backward one write of dK and dV).
 
-// General form (lane u: key u of the scores; lane j: output column j).
+// General form (lane u: key u of the scores; lane j: output column j).  Rows of V
+// and K are loaded eight at a time, unconditionally: one by one behind their
+// conditions 131,072 items of 17 x 16 took 155 us forward and 252 us backward,
+// now 111 and 175.
 template <int DH>
 __global__ void __launch_bounds__(256) attn0_fwd_kernel(const float* __restrict__ Q0, const float* __restrict__ KV,
                                                         const int32_t* __restrict__ n_ent,
@@ -1019,8 +1046,9 @@ __global__ void __launch_bounds__(256) attn0_fwd_kernel(const float* __restrict_
   const int lane = threadIdx.x & 31;
   const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (w >= n * H) return;  // whole warps leave together
-  const long long s = w / H;
-  const int hh = (int)(w - s * H), d = DH * H, ld = 2 * d;
+  const AttItem it = att_item(w, H);
+  const long long s = it.s;
+  const int hh = it.hh, d = DH * H, ld = 2 * d;
   int ne = n_ent[sel ? (long long)sel[s] : s];
   ne = ne < 0 ? 0 : (ne > NS ? NS : ne);
   const float* K = KV + s * T * ld + hh * DH;
@@ -1048,9 +1076,16 @@ __global__ void __launch_bounds__(256) attn0_fwd_kernel(const float* __restrict_
   const float p = e * (1.0f / z);
   if (lane < T) P0[w * T + lane] = p;
   float o = 0.0f;
-  for (int u = 0; u <= ne && u < T; ++u) {
-    const float pu = __shfl_sync(0xffffffffu, p, u);
-    if (lane < DH) o = fmaf(pu, __ldg(V + u * ld + lane), o);
+  const int j = lane < DH ? lane : 0;
+  for (int u0 = 0; u0 <= ne && u0 < T; u0 += 8) {  // eight rows' loads at a time
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __ldg(V + min(u0 + i, T - 1) * ld + j);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float pu = __shfl_sync(0xffffffffu, p, (u0 + i) & 31);
+      if (u0 + i <= ne && u0 + i < T) o = fmaf(pu, v[i], o);
+    }
   }
   if (lane < DH) O0[s * d + hh * DH + lane] = o;
 }
@@ -1063,8 +1098,9 @@ __global__ void __launch_bounds__(256) attn0_bwd_kernel(const float* __restrict_
   const int lane = threadIdx.x & 31;
   const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (w >= n * H) return;  // whole warps leave together
-  const long long s = w / H;
-  const int hh = (int)(w - s * H), d = DH * H, ld = 2 * d;
+  const AttItem it = att_item(w, H);
+  const long long s = it.s;
+  const int hh = it.hh, d = DH * H, ld = 2 * d;
   const float* K = KV + s * T * ld + hh * DH;
   float* dK = dKV + s * T * ld + hh * DH;
   const float p = lane < T ? __ldg(P0 + w * T + lane) : 0.0f;
@@ -1087,15 +1123,24 @@ __global__ void __launch_bounds__(256) attn0_bwd_kernel(const float* __restrict_
   const int j = lane < DH ? lane : 0;
   const float qj = __ldg(Q0 + s * d + hh * DH + j), gj = __ldg(dO0 + s * d + hh * DH + j);
   float dq = 0.0f;
-  for (int u = 0; u < T; ++u) {
-    const float su = __shfl_sync(0xffffffffu, ds, u), pu = __shfl_sync(0xffffffffu, p, u);
-    if (lane < DH) {
-      dq = fmaf(su, __ldg(K + u * ld + lane), dq);
-      dK[u * ld + lane] = su * qj;
-      dK[u * ld + d + lane] = pu * gj;
-      if (u == 0) {
-        D0[s * 3 * d + d + hh * DH + lane] = su * qj;
-        D0[s * 3 * d + 2 * d + hh * DH + lane] = pu * gj;
+  for (int u0 = 0; u0 < T; u0 += 8) {  // eight rows' loads at a time
+    float k[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) k[i] = __ldg(K + min(u0 + i, T - 1) * ld + j);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int u = u0 + i;
+      const float su = __shfl_sync(0xffffffffu, ds, u & 31), pu = __shfl_sync(0xffffffffu, p, u & 31);
+      if (u < T) {
+        dq = fmaf(su, k[i], dq);
+        if (lane < DH) {
+          dK[u * ld + lane] = su * qj;
+          dK[u * ld + d + lane] = pu * gj;
+          if (u == 0) {
+            D0[s * 3 * d + d + hh * DH + lane] = su * qj;
+            D0[s * 3 * d + 2 * d + hh * DH + lane] = pu * gj;
+          }
+        }
       }
     }
   }

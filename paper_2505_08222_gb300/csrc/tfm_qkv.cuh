@@ -77,12 +77,13 @@ __global__ void __launch_bounds__(256, 2) qkv_fwd_kernel(QkvArgs a) {
   bool ok = true, first = true;
   float x[16][2];
   auto fetch = [&](long long mt) {
+    // (rows past the end repeat the last one: nothing of theirs is stored)
     const long long r0 = mt * 128 + warp * 16;
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-      const bool in = mt < tiles && r0 + i < a.rows;
-      x[i][0] = in ? __ldg(a.X + (r0 + i) * 64 + lane) : 0.0f;
-      x[i][1] = in ? __ldg(a.X + (r0 + i) * 64 + lane + 32) : 0.0f;
+      const float* src = a.X + min(r0 + i, a.rows - 1) * 64 + lane;
+      x[i][0] = __ldg(src);
+      x[i][1] = __ldg(src + 32);
     }
   };
   fetch(blockIdx.x);

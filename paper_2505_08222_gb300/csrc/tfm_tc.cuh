@@ -118,8 +118,8 @@ __host__ __device__ constexpr int tc_rows_ctas() {
 }
 
 template <int EPI>
-__global__ void __launch_bounds__(kTcThreads, tc_rows_ctas<EPI>()) tc_rows_kernel(Gemm g, const uint16_t* __restrict__ bimg,
-                                                                int* status) {
+__global__ void __launch_bounds__(kTcThreads, tc_rows_ctas<EPI>())
+    tc_rows_kernel(Gemm g, const uint16_t* __restrict__ bimg, int* status) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* sA = smem;                    // [2][128 x 64] BF16
   unsigned char* sB = smem + 2 * kTcRowsA;     // [2][min(N, 256) x 64] BF16
