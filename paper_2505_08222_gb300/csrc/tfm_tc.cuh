@@ -327,93 +327,111 @@ __global__ void __launch_bounds__(kTcThreads, 3) tc_wgrad_kernel(Gemm g, float* 
   uint32_t phase[2] = {0u, 0u};
   bool ok = true;
   float bsum[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // this thread's rows of columns nb0 + 32 j + lane of dOut
-  for (int c = 0; c < nchunks; ++c) {
+  // A chunk is staged transposed in units of 64 columns, two of dOut and then
+  // those of In: warp w takes rows 8 w .. 8 w + 7, a lane one column of each
+  // block of 32 (row loads coalesced across the warp), and packs its column's 8
+  // rows into one 16-byte core row; the lanes also sum their FP32 values of dOut
+  // for the bias gradient.  Two units are in registers: the loads run two units
+  // ahead of the staging, across chunks, so that they are in flight during the
+  // conversions, the barriers and the MMAs.  Every load is made, past the end
+  // from the last row or column (a load behind a condition waits for the one
+  // before it), and zeroed when it is staged.  13 launches of an actor step of
+  // 278,528 rows, d = 128: 2237 us with loads behind conditions, 1778 with a
+  // chunk's loads issued block by block, this 1674.
+  const int units = 2 + (Ntp / 32 + 1) / 2;
+  const int lda = (int)g.lda, ldb = (int)g.ldb;
+  auto load = [&](float (&v)[2][8], int c, int u) {
+    const long long mrow = r0 + (long long)c * kTcChunk + warp * 8;
+    const int left = (int)min(r1 - mrow, 8LL);  // (may be negative)
+    const bool in_a = u < 2;
+    const float* p = in_a ? g.A + mrow * lda : g.B + mrow * ldb;
+    const int ld = in_a ? lda : ldb;
+    const int col = (in_a ? nb0 + 64 * u : kb0 + 64 * (u - 2)) + lane, top = (in_a ? n_o : n_i) - 1;
+    const float *p0 = p + min(col, top), *p1 = p + min(col + 32, top);
+    if (left >= 8) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        v[0][i] = __ldg(p0 + i * ld);
+        v[1][i] = __ldg(p1 + i * ld);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        v[0][i] = __ldg(p0 + min(i, left - 1) * ld);
+        v[1][i] = __ldg(p1 + min(i, left - 1) * ld);
+      }
+    }
+  };
+  auto stage = [&](float (&v)[2][8], int c, int u) {
     const int s = c & 1;
-    const long long m0 = r0 + (long long)c * kTcChunk;
-    if (c >= 2) {
+    const int left = (int)min(r1 - (r0 + (long long)c * kTcChunk + warp * 8), 8LL);
+    const int base = u < 2 ? 64 * u : 64 * (u - 2);                    // first column of the tile
+    const int have = u < 2 ? n_o - nb0 - base : n_i - kb0 - base;      // columns that exist from there
+    if (left < 8 || have < 64) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (i >= left || h * 32 + lane >= have) v[h][i] = 0.0f;
+    }
+    unsigned char* dst = u < 2 ? sA + s * kTcStageA : sB + (size_t)s * b_stage;
+    const int rows = u < 2 ? 128 : Ntp;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (base + 32 * h < rows)
+        *reinterpret_cast<uint4*>(dst + tc::kmajor_offset(base + 32 * h + lane, warp * 8, rows)) =
+            make_uint4(pack_bf2(v[h][0], v[h][1]), pack_bf2(v[h][2], v[h][3]), pack_bf2(v[h][4], v[h][5]),
+                       pack_bf2(v[h][6], v[h][7]));
+    if (u < 2) {
+      float cs[2] = {0.0f, 0.0f};
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) cs[h] += v[h][i];
+      bsum[0] += u == 0 ? cs[0] : 0.0f;
+      bsum[1] += u == 0 ? cs[1] : 0.0f;
+      bsum[2] += u == 1 ? cs[0] : 0.0f;
+      bsum[3] += u == 1 ? cs[1] : 0.0f;
+    }
+  };
+  int c = 0, u = 0, lc = 0, lu = 0;  // staged next, loaded next
+  auto load_next = [&](float (&v)[2][8]) {
+    if (lc < nchunks) load(v, lc, lu);
+    if (++lu == units) lu = 0, ++lc;
+  };
+  auto step = [&](float (&v)[2][8]) {
+    const int s = c & 1;
+    if (u == 0 && c >= 2) {  // the MMAs two chunks back read this stage
       ok &= tc::mbar_wait(&mbar[s], phase[s], kTcPolls);
       phase[s] ^= 1u;
       tc::fence_after_sync();
     }
-    unsigned char* a = sA + s * kTcStageA;
-    unsigned char* b = sB + (size_t)s * b_stage;
-    // transposed staging: warp w takes rows m0 + 8 w .. + 7 of the chunk, in
-    // blocks of 32 consecutive columns (row loads coalesced across the warp);
-    // each lane packs its column's 8 rows into one 16-byte core row.  A
-    // (dOut): 4 column blocks, all 32 loads issued first; the lanes also sum
-    // their FP32 values for the bias gradient.  B (In): Ntp / 32 blocks, two
-    // at a time.
-    {
-      // (every load is issued, past the end from the last row or column: a
-      // load behind a condition waits for the one before it; 13 launches of a
-      // d = 128 step of 278,528 rows 2237 -> 1778 us)
-      const long long mrow = m0 + warp * 8;
-      const int left = (int)min(r1 - mrow, 8LL);  // (may be negative)
-      const float* const pa = g.A + mrow * g.lda;
-      const float* const pb = g.B + mrow * g.ldb;
-      const int lda = (int)g.lda, ldb = (int)g.ldb;
-      float va[4][8];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int gcol = min(nb0 + j * 32 + lane, n_o - 1);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) va[j][i] = __ldg(pa + min(i, left - 1) * lda + gcol);
-      }
-      if (left < 8 || nb0 + 128 > n_o) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            if (i >= left || nb0 + j * 32 + lane >= n_o) va[j][i] = 0.0f;
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float cs = 0.0f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) cs += va[j][i];
-        bsum[j] += cs;
-        const uint4 p = make_uint4(pack_bf2(va[j][0], va[j][1]), pack_bf2(va[j][2], va[j][3]),
-                                   pack_bf2(va[j][4], va[j][5]), pack_bf2(va[j][6], va[j][7]));
-        *reinterpret_cast<uint4*>(a + tc::kmajor_offset(j * 32 + lane, warp * 8, 128)) = p;
-      }
-      for (int j0 = 0; j0 < Ntp / 32; j0 += 2) {
-        float vb[2][8];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int gcol = min(kb0 + (j0 + h) * 32 + lane, n_i - 1);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) vb[h][i] = __ldg(pb + min(i, left - 1) * ldb + gcol);
-        }
-        if (left < 8 || kb0 + (j0 + 2) * 32 > n_i) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-              if (i >= left || kb0 + (j0 + h) * 32 + lane >= n_i) vb[h][i] = 0.0f;
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (j0 + h < Ntp / 32) {
-            const uint4 p = make_uint4(pack_bf2(vb[h][0], vb[h][1]), pack_bf2(vb[h][2], vb[h][3]),
-                                       pack_bf2(vb[h][4], vb[h][5]), pack_bf2(vb[h][6], vb[h][7]));
-            *reinterpret_cast<uint4*>(b + tc::kmajor_offset((j0 + h) * 32 + lane, warp * 8, Ntp)) = p;
-          }
-        }
-      }
-    }
+    stage(v, c, u);
+    load_next(v);
+    if (++u < units) return;
+    u = 0;
     tc::fence_async_smem();
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     if (tid == 0) {
-      const uint32_t aa = tc::smem_addr(a), bb = tc::smem_addr(b);
+      const uint32_t aa = tc::smem_addr(sA + s * kTcStageA), bb = tc::smem_addr(sB + (size_t)s * b_stage);
+      uint64_t ad = tc::smem_desc(aa, 128 * 16, 128), bd = tc::smem_desc(bb, Ntp * 16, 128);
       for (int j = 0; j < kTcChunk / 16; ++j) {
-        const uint64_t ad = tc::smem_desc(aa + j * 2 * 128 * 16, 128 * 16, 128);
-        const uint64_t bd = tc::smem_desc(bb + j * 2 * Ntp * 16, Ntp * 16, 128);
         tc::mma_bf16(tmem, ad, bd, idesc, (c > 0 || j > 0) ? 1u : 0u);
+        ad = tc::desc_advance(ad, 2 * 128 * 16);
+        bd = tc::desc_advance(bd, 2 * Ntp * 16);
       }
       tc::mma_commit(&mbar[s]);
     }
+    ++c;
+  };
+  float v0[2][8], v1[2][8];
+  load_next(v0);
+  load_next(v1);
+  while (c < nchunks) {
+    step(v0);
+    if (c < nchunks) step(v1);
   }
   for (int c = max(0, nchunks - 2); c < nchunks; ++c) {
     const int s = c & 1;
