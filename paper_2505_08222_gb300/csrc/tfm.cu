@@ -477,8 +477,9 @@ __global__ void ln_bwd_kernel(const float* __restrict__ dY, const float* __restr
 // it too, so that a block's P, one contiguous range, is read and written whole.
 // The products run on packed FP32 pairs: two keys of a score at once (staged
 // interleaved), two columns of an output at once, so each sum keeps its order.
-// Bound by issue and shared-memory loads: 131,072 items of 17 x 16 forward 274 us
-// (534 before), backward 524 (809).
+// Bound by issue and shared-memory loads: 131,072 items of 17 x 16 forward 254 us,
+// backward 500 (534 and 809 with a warp per item; 274 and 524 with the rows
+// staged one load after the other and 64-bit divisions).
 constexpr int kAttnThreads = 128;
 __host__ __device__ __forceinline__ int attn_items(int T) { return kAttnThreads / T; }
 constexpr size_t kAttnSmemMax = 112 * 1024;  // above attn_bwd_smem for every T and head width
@@ -494,28 +495,83 @@ inline size_t attn_bwd_smem(int T, int DH) {
   return ((size_t)3 * attn_rows(T) * DH + (size_t)attn_pair_rows(T) * DH + 2 * (size_t)attn_rows(T) * T + 4) * 4;
 }
 
+// (sample, head) of item w: a 32-bit division wherever it is enough.
+struct AttItem {
+  long long s;
+  int hh;
+};
+__device__ __forceinline__ AttItem att_item(long long w, int H) {
+  if ((w >> 32) == 0) {
+    const uint32_t s = (uint32_t)w / (uint32_t)H;
+    return {(long long)s, (int)((uint32_t)w - s * (uint32_t)H)};
+  }
+  const long long s = w / H;
+  return {s, (int)(w - s * H)};
+}
+
 // Column j of key u in the interleaved layout of an item's rows.
 template <int DH>
 __device__ __forceinline__ int pair_pos(int u, int j) {
   return (u >> 1) * 2 * DH + 2 * j + (u & 1);
 }
 
-// acc[u] = sum_j x[j] K[u][j] over the keys of an item (pairs), j in order.
+template <int DH>
+__device__ __forceinline__ void attn_put_pair(float* item, int u, int j, float4 v) {
+  item[pair_pos<DH>(u, j)] = v.x;
+  item[pair_pos<DH>(u, j + 1)] = v.y;
+  item[pair_pos<DH>(u, j + 2)] = v.z;
+  item[pair_pos<DH>(u, j + 3)] = v.w;
+}
+
+// Where the rows of a block's items lie: row r (item r / T from q0 on, token
+// r % T).  The divisions of r < 128 by T are products (exact: the error is below
+// 128 / 65536 < 1 / T), those by H 32-bit.
+struct AttnRows {
+  AttItem first;
+  int H, T, inv;
+  __device__ __forceinline__ AttnRows(long long q0, int h, int t) : first(att_item(q0, h)), H(h), T(t), inv(65536 / t + 1) {}
+  __device__ __forceinline__ int item(int r) const { return (r * inv) >> 16; }
+  __device__ __forceinline__ void sample(int it, long long& s, int& hh) const {
+    const unsigned h = (unsigned)(first.hh + it), ds = h / (unsigned)H;
+    s = first.s + ds;
+    hh = (int)(h - ds * (unsigned)H);
+  }
+  // float offset of its head's columns in an array of `ld` floats a token
+  __device__ __forceinline__ long long offset(int r, int ld, int dh) const {
+    const int it = item(r);
+    long long s;
+    int hh;
+    sample(it, s, hh);
+    return (s * T + r - it * T) * ld + hh * dh;
+  }
+};
+
+// acc[u] = sum_j x[j] K[u][j] over the keys u < T of an item (pairs), j in
+// order; two pairs at a time, two independent chains.
 template <int DH>
 __device__ __forceinline__ void attn_dots(const float (&x)[DH], const float* pairs, int T, float (&acc)[kMaxT + 1]) {
 #pragma unroll
-  for (int u = 0; u < kMaxT; u += 2) {
+  for (int u = 0; u < kMaxT; u += 4) {
+    constexpr int kLast = kMaxT - 1;
     acc[u] = acc[u + 1] = 0.0f;
+    if (u + 2 <= kLast) acc[u + 2] = acc[u + 3] = 0.0f;
     if (u < T) {
-      const float4* k4 = reinterpret_cast<const float4*>(pairs + (u >> 1) * 2 * DH);
-      unsigned long long s = 0ull;
+      const float4* a4 = reinterpret_cast<const float4*>(pairs + (u >> 1) * 2 * DH);
+      const float4* b4 = u + 2 < T ? a4 + DH / 2 : a4;  // (past the item: its sums are not used)
+      unsigned long long sa = 0ull, sb = 0ull;
 #pragma unroll
       for (int j = 0; j < DH; j += 2) {
-        const float4 k = k4[j / 2];  // (u, j), (u + 1, j), (u, j + 1), (u + 1, j + 1)
-        s = f2fma(f2pk(x[j], x[j]), f2pk(k.x, k.y), s);
-        s = f2fma(f2pk(x[j + 1], x[j + 1]), f2pk(k.z, k.w), s);
+        const float4 a = a4[j / 2];  // (u, j), (u + 1, j), (u, j + 1), (u + 1, j + 1)
+        sa = f2fma(f2pk(x[j], x[j]), f2pk(a.x, a.y), sa);
+        sa = f2fma(f2pk(x[j + 1], x[j + 1]), f2pk(a.z, a.w), sa);
+        if (u + 2 <= kLast) {
+          const float4 b = b4[j / 2];
+          sb = f2fma(f2pk(x[j], x[j]), f2pk(b.x, b.y), sb);
+          sb = f2fma(f2pk(x[j + 1], x[j + 1]), f2pk(b.z, b.w), sb);
+        }
       }
-      f2upk(s, acc[u], acc[u + 1]);
+      f2upk(sa, acc[u], acc[u + 1]);
+      if (u + 2 <= kLast) f2upk(sb, acc[u + 2], acc[u + 3]);
     }
   }
 }
@@ -557,30 +613,40 @@ __global__ void __launch_bounds__(kAttnThreads) attn_fwd_kernel(const float* __r
   float* sK = sV + attn_rows(T) * DH;        // [items][Tp / 2][DH][2]
   const long long q0 = (long long)blockIdx.x * ipb, nq = n * H;
   const int items = (int)(nq - q0 < ipb ? nq - q0 : ipb);
-  const int d = DH * H, ld = 3 * d;
-  for (int i = tid; i < items * T * (DH / 4); i += kAttnThreads) {
-    const int r = i / (DH / 4), c = i - r * (DH / 4), it = r / T, u = r - it * T;
-    const long long q = q0 + it, s = q / H;
-    const float* src = QKV + (s * T + u) * ld + d + (q - s * H) * DH + 4 * c;
-    const float4 k = __ldg(reinterpret_cast<const float4*>(src));
-    float* dst = sK + it * Tp * DH;
-    dst[pair_pos<DH>(u, 4 * c)] = k.x;
-    dst[pair_pos<DH>(u, 4 * c + 1)] = k.y;
-    dst[pair_pos<DH>(u, 4 * c + 2)] = k.z;
-    dst[pair_pos<DH>(u, 4 * c + 3)] = k.w;
-    reinterpret_cast<float4*>(sV)[i] = __ldg(reinterpret_cast<const float4*>(src + d));
-  }
-  const int it = tid / T, t = tid - it * T;
+  const int d = DH * H, ld = 3 * d, rows = items * T;
+  const AttnRows at(q0, H, T);
+  const int it = at.item(tid), t = tid - it * T;
   const bool on = it < items;
-  const long long q = q0 + (on ? it : 0), s = q / H;
-  const int hh = (int)(q - s * H);
-  int ne = n_ent[sel ? (long long)sel[s] : s];
+  long long s;
+  int hh;
+  at.sample(on ? it : 0, s, hh);
+  int ne = __ldg(n_ent + (sel ? (long long)__ldg(sel + s) : s));
   ne = ne < 0 ? 0 : (ne > NS ? NS : ne);
   float qv[DH];
 #pragma unroll
   for (int j = 0; j < DH; j += 4) {
     const float4 v = __ldg(reinterpret_cast<const float4*>(QKV + (s * T + (on ? t : 0)) * ld + hh * DH + j));
     qv[j] = v.x; qv[j + 1] = v.y; qv[j + 2] = v.z; qv[j + 3] = v.w;
+  }
+  constexpr int C = DH / 4, KB = C < 4 ? C : 4;
+#pragma unroll
+  for (int k0 = 0; k0 < C; k0 += KB) {
+    float4 kk[KB], vv[KB];
+#pragma unroll
+    for (int k = 0; k < KB; ++k) {
+      const int i = tid + kAttnThreads * (k0 + k);
+      const float* src = QKV + d + at.offset(min(i / C, rows - 1), ld, DH) + 4 * (i % C);
+      kk[k] = __ldg(reinterpret_cast<const float4*>(src));
+      vv[k] = __ldg(reinterpret_cast<const float4*>(src + d));
+    }
+#pragma unroll
+    for (int k = 0; k < KB; ++k) {
+      const int i = tid + kAttnThreads * (k0 + k), r = i / C;
+      if (r < rows) {
+        attn_put_pair<DH>(sK + at.item(r) * Tp * DH, r - at.item(r) * T, 4 * (i % C), kk[k]);
+        reinterpret_cast<float4*>(sV)[i] = vv[k];
+      }
+    }
   }
   __syncthreads();
   float sc[kMaxT + 1];
@@ -640,28 +706,48 @@ __global__ void __launch_bounds__(kAttnThreads) attn_bwd_kernel(const float* __r
   float* sS = sP + R * T;                  // dS
   const long long q0 = (long long)blockIdx.x * ipb, nq = n * H;
   const int items = (int)(nq - q0 < ipb ? nq - q0 : ipb);
-  const int d = DH * H, ld = 3 * d;
-  for (int i = tid; i < items * T * (DH / 4); i += kAttnThreads) {
-    const int r = i / (DH / 4), c = i - r * (DH / 4), it = r / T, u = r - it * T;
-    const long long q = q0 + it, s = q / H;
-    const long long hc = (q - s * H) * DH + 4 * c;
-    const float* src = QKV + (s * T + u) * ld + hc;
-    reinterpret_cast<float4*>(sQ)[i] = __ldg(reinterpret_cast<const float4*>(src));
-    reinterpret_cast<float4*>(sK)[i] = __ldg(reinterpret_cast<const float4*>(src + d));
-    reinterpret_cast<float4*>(sG)[i] = __ldg(reinterpret_cast<const float4*>(dO + (s * T + u) * d + hc));
-    const float4 v = __ldg(reinterpret_cast<const float4*>(src + 2 * d));
-    float* dst = sV + it * Tp * DH;
-    dst[pair_pos<DH>(u, 4 * c)] = v.x;
-    dst[pair_pos<DH>(u, 4 * c + 1)] = v.y;
-    dst[pair_pos<DH>(u, 4 * c + 2)] = v.z;
-    dst[pair_pos<DH>(u, 4 * c + 3)] = v.w;
+  const int d = DH * H, ld = 3 * d, rows = items * T, np = rows * T;
+  const AttnRows at(q0, H, T);
+  const float* const Pb = P + q0 * T * T;
+  // two 16-byte columns of each row image and eight of P's elements per turn
+  constexpr int C = DH / 4;
+  for (int b = 0; b < C / 2 || 8 * b < T; ++b) {
+    float4 x[2][4];
+    float pe[8];
+    if (b < C / 2) {
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int i = tid + kAttnThreads * (2 * b + k), r = min(i / C, rows - 1);
+        const float* src = QKV + at.offset(r, ld, DH) + 4 * (i % C);
+        x[k][0] = __ldg(reinterpret_cast<const float4*>(src));
+        x[k][1] = __ldg(reinterpret_cast<const float4*>(src + d));
+        x[k][2] = __ldg(reinterpret_cast<const float4*>(dO + at.offset(r, d, DH) + 4 * (i % C)));
+        x[k][3] = __ldg(reinterpret_cast<const float4*>(src + 2 * d));
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) pe[k] = __ldg(Pb + min(tid + kAttnThreads * (8 * b + k), np - 1));
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int i = tid + kAttnThreads * (2 * b + k), r = i / C;  // (from turn C / 2 on: past every row)
+      if (r < rows) {
+        reinterpret_cast<float4*>(sQ)[i] = x[k][0];
+        reinterpret_cast<float4*>(sK)[i] = x[k][1];
+        reinterpret_cast<float4*>(sG)[i] = x[k][2];
+        attn_put_pair<DH>(sV + at.item(r) * Tp * DH, r - at.item(r) * T, 4 * (i % C), x[k][3]);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (tid + kAttnThreads * (8 * b + k) < np) sP[tid + kAttnThreads * (8 * b + k)] = pe[k];
   }
-  for (int i = tid; i < items * T * T; i += kAttnThreads) sP[i] = __ldg(P + q0 * T * T + i);
   __syncthreads();
-  const int it = tid / T, t = tid - it * T;
+  const int it = at.item(tid), t = tid - it * T;
   const bool on = it < items;
-  const long long q = q0 + (on ? it : 0), s = q / H;
-  float* out = dQKV + (s * T + t) * ld + (q - s * H) * DH;
+  long long s;
+  int hh;
+  at.sample(on ? it : 0, s, hh);
+  float* out = dQKV + (s * T + t) * ld + hh * DH;
   unsigned long long o[DH / 2];
   if (on) {
     float g[DH], dp[kMaxT + 1];
@@ -741,20 +827,6 @@ __device__ __forceinline__ void mma16x16(float (&c)[2][4], const float* a, const
       mma_tf32(c[j], a0, a1, a2, a3, b0, b1);
     }
   }
-}
-
-// (sample, head) of item w: a 32-bit division wherever it is enough.
-struct AttItem {
-  long long s;
-  int hh;
-};
-__device__ __forceinline__ AttItem att_item(long long w, int H) {
-  if ((w >> 32) == 0) {
-    const uint32_t s = (uint32_t)w / (uint32_t)H;
-    return {(long long)s, (int)((uint32_t)w - s * (uint32_t)H)};
-  }
-  const long long s = w / H;
-  return {s, (int)(w - s * H)};
 }
 
 // Per-warp staging of one (sample, head) item: rows u = lane / 4 + 8 r
