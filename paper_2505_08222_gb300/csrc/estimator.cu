@@ -42,6 +42,38 @@ __device__ __forceinline__ void store8(unsigned char* img, int row, int k0, int 
   *reinterpret_cast<uint4*>(img + tc::kmajor_offset(row, k0, rows)) = p;
 }
 
+// x[i] += p[i] over 4 M values of read-only memory, p 16-byte aligned.
+template <int M>
+__device__ __forceinline__ void add4(float* x, const float* p) {
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    const float4 b = __ldg(reinterpret_cast<const float4*>(p) + i);
+    x[4 * i] += b.x;
+    x[4 * i + 1] += b.y;
+    x[4 * i + 2] += b.z;
+    x[4 * i + 3] += b.w;
+  }
+}
+
+// o0, o1 += the output layer's two sums over 4 M hidden units a from unit c0 on,
+// in order.
+template <int M>
+__device__ __forceinline__ void out_sums(const float* mst, int c0, const float* a, float& o0, float& o1) {
+  const float4* w4 = reinterpret_cast<const float4*>(mst + W4_OFF + c0);
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    const float4 w0 = __ldg(w4 + i), w1 = __ldg(w4 + HID / 4 + i);
+    o0 = fmaf(w0.x, a[4 * i], o0);
+    o1 = fmaf(w1.x, a[4 * i], o1);
+    o0 = fmaf(w0.y, a[4 * i + 1], o0);
+    o1 = fmaf(w1.y, a[4 * i + 1], o1);
+    o0 = fmaf(w0.z, a[4 * i + 2], o0);
+    o1 = fmaf(w1.z, a[4 * i + 2], o1);
+    o0 = fmaf(w0.w, a[4 * i + 3], o0);
+    o1 = fmaf(w1.w, a[4 * i + 3], o1);
+  }
+}
+
 // 24 consecutive features of a row from column c0 (a multiple of 8) on, as BF16
 // high parts and remainders in two operand images.
 __device__ __forceinline__ void store_features(unsigned char* hi_img, unsigned char* lo_img, int row, int c0,
@@ -259,26 +291,14 @@ __global__ void __launch_bounds__(kTE, 1) fwd_env_kernel(Net net, EnvDev d, int 
     for (int c0 = part * (HID / kParts); c0 < (part + 1) * (HID / kParts); c0 += 32) {
       float av[32];
       tc::tmem_ld32(tl + c0, av);
-      const float4* b4 = reinterpret_cast<const float4*>(bias + c0);  // (every layer's biases start at a multiple of 4)
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float4 b = __ldg(b4 + i);
-        av[4 * i] += b.x;
-        av[4 * i + 1] += b.y;
-        av[4 * i + 2] += b.z;
-        av[4 * i + 3] += b.w;
-      }
+      add4<8>(av, bias + c0);  // (every layer's biases start at a multiple of 4)
 #pragma unroll
       for (int i = 0; i < 32; i += 2) gelu2(av[i], av[i + 1]);  // erf-GELU, packed pairs
       if (l < 2) {
 #pragma unroll
         for (int i = 0; i < 32; i += 8) store8(sA, row, c0 + i, 128, av + i);
       } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          o0 = fmaf(__ldg(mst + W4_OFF + c0 + i), av[i], o0);
-          o1 = fmaf(__ldg(mst + W4_OFF + HID + c0 + i), av[i], o1);
-        }
+        out_sums<8>(mst, c0, av, o0, o1);
       }
     }
   }
@@ -410,9 +430,12 @@ __global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __res
     float x[24];
 #pragma unroll
     for (int i = 0; i < 24; i += 4) {
-      const float4 v = valid ? __ldg(reinterpret_cast<const float4*>(X + src * IN + part * 24 + i))
-                             : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float4 v = __ldg(reinterpret_cast<const float4*>(X + src * IN + part * 24 + i));
       x[i] = v.x; x[i + 1] = v.y; x[i + 2] = v.z; x[i + 3] = v.w;
+    }
+    if (!valid) {  // (row 0 of X was read)
+#pragma unroll
+      for (int i = 0; i < 24; ++i) x[i] = 0.0f;
     }
     store_features(sA, sA + 128 * IN * 2, row, part * 24, x);
     if (TRAIN) {
@@ -460,8 +483,7 @@ __global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __res
     for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
       float v[16];
       tc::tmem_ld16(tl + col + c0, v);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] += __ldg(bias + c0 + i);
+      add4<4>(v, bias + c0);
       if (TRAIN && l == 0) {
         float4* zr = reinterpret_cast<float4*>(t.z + b * HID + c0);
 #pragma unroll
@@ -490,7 +512,8 @@ __global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __res
       float v[32];
       tc::tmem_ld32(tl + c_lo + k, v);
 #pragma unroll
-      for (int i = 0; i < 32; ++i) a3[k + i] = v[i] + __ldg(mst + B3_OFF + c_lo + k + i);
+      for (int i = 0; i < 32; ++i) a3[k + i] = v[i];
+      add4<8>(a3 + k, mst + B3_OFF + c_lo + k);
     }
 #pragma unroll
     for (int i = 0; i < HID / kParts; i += 2) gelu2(a3[i], a3[i + 1]);
@@ -501,11 +524,7 @@ __global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __res
           o0 = sOut[0][row];
           o1 = sOut[1][row];
         }
-#pragma unroll
-        for (int i = 0; i < HID / kParts; ++i) {
-          o0 = fmaf(__ldg(mst + W4_OFF + c_lo + i), a3[i], o0);
-          o1 = fmaf(__ldg(mst + W4_OFF + HID + c_lo + i), a3[i], o1);
-        }
+        out_sums<HID / kParts / 4>(mst, c_lo, a3, o0, o1);
         sOut[0][row] = o0;
         sOut[1][row] = o1;
       }
@@ -566,8 +585,7 @@ __global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __res
           }
         } else {
           tc::tmem_ld16(tl + (l == 1 ? kZ2 : 0u) + c0, z);
-#pragma unroll
-          for (int i = 0; i < 16; ++i) z[i] += __ldg(bias + c0 + i);
+          add4<4>(z, bias + c0);
         }
         if (l == 2) {
           float a[16], a1[16];
@@ -576,10 +594,18 @@ __global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __res
 #pragma unroll
           for (int i = 0; i < 16; i += 2) gelu2(a[i], a[i + 1]);
 #pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 w0 = __ldg(reinterpret_cast<const float4*>(mst + W4_OFF + c0) + i);
+            const float4 w1 = __ldg(reinterpret_cast<const float4*>(mst + W4_OFF + HID + c0) + i);
+            v[4 * i] = d0 * w0.x + d1 * w1.x;
+            v[4 * i + 1] = d0 * w0.y + d1 * w1.y;
+            v[4 * i + 2] = d0 * w0.z + d1 * w1.z;
+            v[4 * i + 3] = d0 * w0.w + d1 * w1.w;
+          }
+#pragma unroll
           for (int i = 0; i < 16; ++i) {
             a1[i] = d1 * a[i];
             a[i] = d0 * a[i];
-            v[i] = d0 * __ldg(mst + W4_OFF + c0 + i) + d1 * __ldg(mst + W4_OFF + HID + c0 + i);
           }
           const float w0 = colsum16(a), w1 = colsum16(a1);
           if (lane < 16) {
