@@ -14,7 +14,7 @@
 // gradients accumulate in tensor memory over all of a CTA's tiles.  What
 // bounds both is the CUDA cores' work per hidden value (erf, and in the
 // backward the exponential of its derivative) and the chain of stages within a
-// tile.  1.97 M rows (163,840 samples' two blocks): forward 0.78 ms, backward
+// tile.  1.97 M rows (163,840 samples' two blocks): forward 0.77 ms, backward
 // 1.46 ms; the actor's gradient step 14.3 -> 10.4 ms, the critic's (32,768
 // samples) 3.24 -> 2.33.  It also serves small calls: 5 launches and 5
 // reductions become 1 and 5.
@@ -223,6 +223,10 @@ __global__ void __launch_bounds__(256, 2) ffn_fwd_kernel(FfnArgs a) {
       if (first) ok &= tc::mbar_wait(&bars[4], 0u, kTcPolls);
       ffn_mma(tmem, aY, 2048, aW1, kFfH, false);
       tc::mma_commit(&bars[0]);
+    }
+    {  // the next tile's rows into L2 meanwhile, a 128-byte line per thread (783 -> 770 us)
+      const long long nm = (mt + gridDim.x) * 128 + (tid >> 1);
+      if (nm < a.rows) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.M + nm * 64 + (tid & 1) * 32));
     }
 #pragma unroll 1
     for (int c = 0; c < 4; ++c) {

@@ -14,10 +14,10 @@
 // the K-major operand of the input gradient and, read MN-major, the operand of
 // the weight gradient, which accumulates in tensor memory over a CTA's tiles
 // (tfm_ffn.cuh).  Two CTAs per SM hide each other's stages.  The arithmetic of
-// every value is that of the separate kernels.  1.80 M rows: forward 318 us (5.8
-// TB/s; as LayerNorm and GEMM about 450), backward 0.75 ms (3.7 TB/s; as four
+// every value is that of the separate kernels.  1.80 M rows: forward 309 us (6.0
+// TB/s; as LayerNorm and GEMM about 450), backward 0.70 ms (3.9 TB/s; as four
 // kernels 1.3); what holds the backward is the latency of its staging, half of
-// a tile's 28 k cycles.
+// a tile's cycles.
 //
 // T > 0 marks the last block: dQ and Q are kept for the recurrent rows alone
 // (row s T at s), K and V as [rows][128], and the residual's gradient is zero
@@ -286,8 +286,10 @@ __global__ void __launch_bounds__(256, 2) qkv_bwd_kernel(QkvArgs a) {
       ffn_mma_rows(tmem + kDw + 64, aD + 16 * 2048, aY, !first);
       tc::mma_commit(&bars[0]);
     }
-    {  // the next tile's rows into L2 meanwhile, a 128-byte line per thread and turn
-      const long long nm = (mt + gridDim.x) * 128, w = a.T ? 128 : 192;
+    // the rows of the tile after the next into L2 meanwhile, a 128-byte line per
+    // thread and turn (two launches of 1.8 M rows: 1399 us, the next tile's 1492)
+    {
+      const long long nm = (mt + 2 * gridDim.x) * 128, w = a.T ? 128 : 192;
       const long long lines = (a.rows - nm < 128 ? a.rows - nm : 128) * w / 32;  // (none past the last tile)
       for (long long i = tid; i < lines; i += 256)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(a.dqkv + nm * w + i * 32));
