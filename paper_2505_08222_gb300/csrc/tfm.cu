@@ -20,6 +20,7 @@
 
 #include <cmath>
 #include <cstring>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -1710,24 +1711,47 @@ __global__ void __launch_bounds__(256) colsum_kernel(const float* __restrict__ A
   }
 }
 
-// out[i] = sum over p of part[p * stride + i]: block x sums columns
-// 32x .. 32x+31, thread row g the parts p = g (mod 32) in increasing p, then
-// the 32 row sums in order of g (a fixed association: deterministic).
-__global__ void __launch_bounds__(1024) reduce_kernel(const float* __restrict__ part, int nparts, long long len,
-                                                      long long stride, float* __restrict__ out) {
+// out[i] = sum over p of part[p * stride + i] for every segment of the list, the
+// partial sums that one kernel leaves: a block sums 32 columns of a segment,
+// thread row g the parts p = g (mod 32) in increasing p, then the 32 row sums in
+// order of g (a fixed association: deterministic).  One launch per list: a
+// gradient call at d = 64, 2 blocks has 8 of them where a launch per tensor made
+// 22, and small batches are bound by launches (64 samples 307 -> 259 us, 32,768
+// 1738 -> 1689).
+struct ReduceSeg {
+  const float* part;
+  long long len, stride;
+  float* out;
+};
+constexpr int kReduceSegs = 5;
+struct ReduceList {
+  ReduceSeg seg[kReduceSegs];
+  unsigned first[kReduceSegs];  // first block of each segment (past the grid: none)
+  int nparts;
+};
+__global__ void __launch_bounds__(1024) reduce_kernel(ReduceList l) {
   __shared__ float red[32][33];
   const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
-  const long long i = (long long)blockIdx.x * 32 + c;
+  ReduceSeg q = l.seg[0];
+  unsigned first = 0;
+#pragma unroll
+  for (int k = 1; k < kReduceSegs; ++k)
+    if (blockIdx.x >= l.first[k]) {
+      q = l.seg[k];
+      first = l.first[k];
+    }
+  const long long i = (long long)(blockIdx.x - first) * 32 + c;
+  const float* src = q.part + (i < q.len ? i : q.len - 1);
   float s = 0.0f;
-  if (i < len)
-    for (int p = g; p < nparts; p += 32) s += part[p * stride + i];
+#pragma unroll 4
+  for (int p = g; p < l.nparts; p += 32) s += src[p * q.stride];
   red[g][c] = s;
   __syncthreads();
-  if (g == 0 && i < len) {
+  if (g == 0 && i < q.len) {
     float t = 0.0f;
 #pragma unroll
     for (int k = 0; k < 32; ++k) t += red[k][c];
-    out[i] = t;
+    q.out[i] = t;
   }
 }
 
@@ -1963,8 +1987,21 @@ Gemm mk(const float* A, long long lda, const float* B, long long ldb, float* C, 
   return g;
 }
 
-cudaError_t reduce(const float* part, int nparts, long long len, long long stride, float* out, cudaStream_t s) {
-  reduce_kernel<<<blocks_for(len, 32), 1024, 0, s>>>(part, nparts, len, stride, out);
+cudaError_t reduce(int nparts, std::initializer_list<ReduceSeg> segs, cudaStream_t s) {
+  ReduceList l;
+  l.nparts = nparts;
+  unsigned blocks = 0;
+  int k = 0;
+  for (const ReduceSeg& q : segs) {
+    l.seg[k] = q;
+    l.first[k++] = blocks;
+    blocks += blocks_for(q.len, 32);
+  }
+  for (; k < kReduceSegs; ++k) {
+    l.seg[k] = l.seg[0];
+    l.first[k] = blocks;
+  }
+  reduce_kernel<<<blocks, 1024, 0, s>>>(l);
   return cudaGetLastError();
 }
 
@@ -1997,8 +2034,8 @@ cudaError_t wgrad(ut_tfm* t, const float* dOut, long long ldo, int n_o, const fl
     float* bias_part = t->part + splits * n_o * n_i;
     tc_wgrad_kernel<<<grid, kTcThreads, smem, s>>>(g, bias_part, t->status);
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = reduce(t->part, (int)splits, (long long)n_o * n_i, (long long)n_o * n_i, gW, s);
-    if (e == cudaSuccess) e = reduce(bias_part, (int)splits, n_o, n_o, gb, s);
+    const long long len = (long long)n_o * n_i;
+    if (e == cudaSuccess) e = reduce((int)splits, {{t->part, len, len, gW}, {bias_part, n_o, n_o, gb}}, s);
     return e;
   }
   Gemm g = mk(dOut, ldo, In, ldi, t->part, n_i, n_o, n_i, rows, EPI_PARTIAL);
@@ -2012,13 +2049,14 @@ cudaError_t wgrad(ut_tfm* t, const float* dOut, long long ldo, int n_o, const fl
   splits = (rows + kc - 1) / kc;
   g.kchunk = kc;
   cudaError_t e = gemm(2, g, s);
-  if (e == cudaSuccess) e = reduce(t->part, (int)splits, (long long)n_o * n_i, (long long)n_o * n_i, gW, s);
+  const long long len = (long long)n_o * n_i;
+  if (e == cudaSuccess) e = reduce((int)splits, {{t->part, len, len, gW}}, s);
   if (e != cudaSuccess) return e;
   long long nblk = (rows + 63) / 64;
   nblk = nblk < 1 ? 1 : (nblk > 256 ? 256 : nblk);
   colsum_kernel<<<dim3((unsigned)((n_o + 31) / 32), (unsigned)nblk), 256, 0, s>>>(dOut, ldo, rows, n_o, t->part);
   e = cudaGetLastError();
-  if (e == cudaSuccess) e = reduce(t->part, (int)nblk, n_o, n_o, gb, s);
+  if (e == cudaSuccess) e = reduce((int)nblk, {{t->part, n_o, n_o, gb}}, s);
   return e;
 }
 
@@ -2037,7 +2075,7 @@ cudaError_t ln_bwd(ut_tfm* t, const float* dY, const float* X, const float* st, 
   static const int nblk = (int)std::min<long long>(kLnBlocks, resident_blocks(ln_bwd_kernel<DJ, REC>, 256));
   ln_bwd_kernel<DJ, REC><<<nblk, 256, 0, s>>>(dY, X, st, g, base, out, t->part, rows, dY0, (unsigned)t->T);
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = reduce(t->part, nblk, 2 * 32 * DJ, 2 * 32 * DJ, grad_gb, s);
+  if (e == cudaSuccess) e = reduce(nblk, {{t->part, 2 * 32 * DJ, 2 * 32 * DJ, grad_gb}}, s);
   return e;
 }
 
@@ -2283,11 +2321,14 @@ cudaError_t backward(ut_tfm* t, const Call& c, float* grad, cudaStream_t s) {
       a.vec = t->part + 152ll * kFfSlab;
       int ctas = 0;
       e = ffn_bwd(a, &ctas, s);
-      if (e == cudaSuccess) e = reduce(a.slab, ctas, kFfH * kFfD, kFfSlab, grad + ol[T_W1], s);
-      if (e == cudaSuccess) e = reduce(a.slab + kFfH * kFfD, ctas, kFfH * kFfD, kFfSlab, grad + ol[T_W2], s);
-      if (e == cudaSuccess) e = reduce(a.vec, ctas, kFfH, kFfVec, grad + ol[T_B1], s);
-      if (e == cudaSuccess) e = reduce(a.vec + kFfH, ctas, kFfD, kFfVec, grad + ol[T_B2], s);
-      if (e == cudaSuccess) e = reduce(a.vec + kFfH + kFfD, ctas, 2 * kFfD, kFfVec, grad + ol[T_LN2G], s);
+      if (e == cudaSuccess)
+        e = reduce(ctas,
+                   {{a.slab, kFfH * kFfD, kFfSlab, grad + ol[T_W1]},
+                    {a.slab + kFfH * kFfD, kFfH * kFfD, kFfSlab, grad + ol[T_W2]},
+                    {a.vec, kFfH, kFfVec, grad + ol[T_B1]},
+                    {a.vec + kFfH, kFfD, kFfVec, grad + ol[T_B2]},
+                    {a.vec + kFfH + kFfD, 2 * kFfD, kFfVec, grad + ol[T_LN2G]}},
+                   s);
     } else {
       Gemm g = mk(t->dX, d, w + ol[T_W2], 4 * d, t->dBig, 4 * d, m, 4 * d, d, EPI_GELU_GRAD);
       g.aux = b.Z;
@@ -2319,9 +2360,12 @@ cudaError_t backward(ut_tfm* t, const Call& c, float* grad, cudaStream_t s) {
       a.vec = t->part + (long long)kQkvCtas * kQkvSlab;
       int ctas = 0;
       if (e == cudaSuccess) e = qkv_bwd(a, &ctas, s);
-      if (e == cudaSuccess) e = reduce(a.slab, ctas, kQkvSlab, kQkvSlab, grad + ol[T_WQKV], s);
-      if (e == cudaSuccess) e = reduce(a.vec, ctas, kQkvN, kQkvVec, grad + ol[T_BQKV], s);
-      if (e == cudaSuccess) e = reduce(a.vec + kQkvN, ctas, 2 * kFfD, kQkvVec, grad + ol[T_LN1G], s);
+      if (e == cudaSuccess)
+        e = reduce(ctas,
+                   {{a.slab, kQkvSlab, kQkvSlab, grad + ol[T_WQKV]},
+                    {a.vec, kQkvN, kQkvVec, grad + ol[T_BQKV]},
+                    {a.vec + kQkvN, 2 * kFfD, kQkvVec, grad + ol[T_LN1G]}},
+                   s);
       continue;
     }
     if (last) {
@@ -2350,7 +2394,7 @@ cudaError_t backward(ut_tfm* t, const Call& c, float* grad, cudaStream_t s) {
   embed_grad_kernel<TokT, DJ><<<kRowBlocks, 256, 0, s>>>((const TokT*)c.tok, c.ne, c.sel, t->dX, t->part, c.n, t->T,
                                                          t->NS);
   e = cudaGetLastError();
-  if (e == cudaSuccess) e = reduce(t->part, kRowWarps, 9 * d, 9 * d, grad + o[0], s);
+  if (e == cudaSuccess) e = reduce(kRowWarps, {{t->part, 9 * d, 9 * d, grad + o[0]}}, s);
   return e;
 }
 
@@ -2386,7 +2430,7 @@ cudaError_t run(ut_tfm* t, const Call& c, int mode, const HeadArgs& ha_in, float
   e = cudaGetLastError();
   if (e != cudaSuccess || mode == 0) return e;
   const long long plen = 2 * d + (long long)t->n_out * d + t->n_out;
-  e = reduce(t->part, kRowWarps, plen, plen, grad + o[idx], s);
+  e = reduce(kRowWarps, {{t->part, plen, plen, grad + o[idx]}}, s);
   if (e != cudaSuccess) return e;
   reduce_stats_kernel<<<1, 256, 0, s>>>(t->spart, kRowWarps, 1.0 / (double)c.n, t->stats_d);
   e = cudaGetLastError();
