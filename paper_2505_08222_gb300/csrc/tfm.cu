@@ -2295,6 +2295,11 @@ cudaError_t forward(ut_tfm* t, const Call& c, cudaStream_t s) {
   return e;
 }
 
+// Blocks of the head and embedding-gradient kernels, a warp per sample: small
+// batches start no idle warps, whose partial sums would be zeros to write and
+// add (a critic's gradient of 64 samples 264 -> 243 us).
+int row_blocks(long long n) { return (int)std::max(1ll, std::min<long long>(kRowBlocks, (n + 7) / 8)); }
+
 template <int DJ, int DH, typename TokT>
 cudaError_t backward(ut_tfm* t, const Call& c, float* grad, cudaStream_t s) {
   constexpr int d = 32 * DJ;
@@ -2391,10 +2396,10 @@ cudaError_t backward(ut_tfm* t, const Call& c, float* grad, cudaStream_t s) {
       e = ln_bwd<DJ, false>(t, t->dY, b.X, b.S1, w + ol[T_LN1G], t->dM, t->dX, grad + ol[T_LN1G], rows, s);
   }
   if (e != cudaSuccess) return e;
-  embed_grad_kernel<TokT, DJ><<<kRowBlocks, 256, 0, s>>>((const TokT*)c.tok, c.ne, c.sel, t->dX, t->part, c.n, t->T,
-                                                         t->NS);
+  const int rb = row_blocks(c.n);
+  embed_grad_kernel<TokT, DJ><<<rb, 256, 0, s>>>((const TokT*)c.tok, c.ne, c.sel, t->dX, t->part, c.n, t->T, t->NS);
   e = cudaGetLastError();
-  if (e == cudaSuccess) e = reduce(kRowWarps, {{t->part, 9 * d, 9 * d, grad + o[0]}}, s);
+  if (e == cudaSuccess) e = reduce(8 * rb, {{t->part, 9 * d, 9 * d, grad + o[0]}}, s);
   return e;
 }
 
@@ -2421,18 +2426,19 @@ cudaError_t run(ut_tfm* t, const Call& c, int mode, const HeadArgs& ha_in, float
   ha.dXL = t->dX;
   ha.part = t->part;
   ha.spart = t->spart;
+  const int rb = row_blocks(c.n);
   if (t->n_out == 1)
-    head_kernel<DJ, 1><<<kRowBlocks, 256, 0, s>>>(ha);
+    head_kernel<DJ, 1><<<rb, 256, 0, s>>>(ha);
   else if (t->n_out <= 8)
-    head_kernel<DJ, 8><<<kRowBlocks, 256, 0, s>>>(ha);
+    head_kernel<DJ, 8><<<rb, 256, 0, s>>>(ha);
   else
-    head_kernel<DJ, 16><<<kRowBlocks, 256, 0, s>>>(ha);
+    head_kernel<DJ, 16><<<rb, 256, 0, s>>>(ha);
   e = cudaGetLastError();
   if (e != cudaSuccess || mode == 0) return e;
   const long long plen = 2 * d + (long long)t->n_out * d + t->n_out;
-  e = reduce(kRowWarps, {{t->part, plen, plen, grad + o[idx]}}, s);
+  e = reduce(8 * rb, {{t->part, plen, plen, grad + o[idx]}}, s);
   if (e != cudaSuccess) return e;
-  reduce_stats_kernel<<<1, 256, 0, s>>>(t->spart, kRowWarps, 1.0 / (double)c.n, t->stats_d);
+  reduce_stats_kernel<<<1, 256, 0, s>>>(t->spart, 8 * rb, 1.0 / (double)c.n, t->stats_d);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return backward<DJ, DH, TokT>(t, c, grad, s);
