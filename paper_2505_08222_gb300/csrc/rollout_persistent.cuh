@@ -41,8 +41,19 @@ constexpr int rollout_threads() {
 // each other within a step: measurement lists, headers, errors; two of each.
 inline size_t rollout_stage_bytes(int filters, int AM) { return 2 * (size_t)filters * (AM * 16 + 16 + 4) + 16; }
 
-template <int NT, int PPT, int MODE>
-__global__ void __launch_bounds__(rollout_threads<NT>(), 1) rollout_kernel(EnvDev d, int T, int max_filters) {
+// CTAs per SM that the registers must allow when there are more environments than
+// SMs: small filters leave room for several on an SM, and left to itself the
+// compiler gives the environment's stage (200 registers) that room.  (50 steps of
+// 2000 environments of 1000 particles: 2984 us with one CTA per SM, 1729 with two;
+// 600 of 400: 950 and 517.  Up to one environment per SM the registers are worth
+// more: 64 of 2 x 2, 100 particles: 580 us, 614 with the cap.)
+template <int NT, int PPT>
+constexpr int rollout_min_blocks() {
+  return PPT > 4 ? (NT <= 64 ? 4 : (NT <= 128 ? 2 : 1)) : (NT <= 32 ? 12 : (NT <= 64 ? 6 : (NT <= 128 ? 3 : (NT <= 256 ? 2 : 1))));
+}
+
+template <int NT, int PPT, int MODE, int MINB>
+__global__ void __launch_bounds__(rollout_threads<NT>(), MINB) rollout_kernel(EnvDev d, int T, int max_filters) {
   constexpr bool kOwnWarp = rollout_threads<NT>() > NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ EnvWarpSmem ew;
@@ -128,16 +139,22 @@ __global__ void __launch_bounds__(rollout_threads<NT>(), 1) rollout_kernel(EnvDe
   }
 }
 
-template <int NT, int PPT, int MODE>
-cudaError_t launch_mode(const EnvDev& d, int T, cudaStream_t s) {
+template <int NT, int PPT, int MODE, int MINB>
+cudaError_t launch_blocks(const EnvDev& d, int T, cudaStream_t s) {
   static std::atomic<unsigned long long> ready{0};
-  auto k = rollout_kernel<NT, PPT, MODE>;
+  auto k = rollout_kernel<NT, PPT, MODE, MINB>;
   const int filters = d.shared_filter ? d.TM : d.AM * d.TM;
   const cudaError_t e =
       smem_optin(k, pf::step_smem_bytes(NT, PPT) + rollout_stage_bytes(kMaxAgents * kMaxTargets, kMaxAgents), ready);
   if (e != cudaSuccess) return e;
   k<<<d.E, rollout_threads<NT>(), pf::step_smem_bytes(NT, PPT) + rollout_stage_bytes(filters, d.AM), s>>>(d, T, filters);
   return cudaGetLastError();
+}
+
+template <int NT, int PPT, int MODE>
+cudaError_t launch_mode(const EnvDev& d, int T, cudaStream_t s) {
+  return d.E > 152 ? launch_blocks<NT, PPT, MODE, rollout_min_blocks<NT, PPT>()>(d, T, s)
+                   : launch_blocks<NT, PPT, MODE, 1>(d, T, s);
 }
 
 template <int NT, int PPT>

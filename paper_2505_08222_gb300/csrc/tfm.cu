@@ -1003,7 +1003,9 @@ __global__ void __launch_bounds__(128, 6)
   const long long items = n * H, stride = (long long)gridDim.x * 4;
   float *sQ = sm[wl][0], *sK = sm[wl][1], *sV = sm[wl][2], *sS = sm[wl][2], *sG = sm[wl][3], *sP = sm[wl][4];
   // P of an item: T * T contiguous floats, element e = lane + 32 i at
-  // (e / T, e % T) of the staged tile; the padding stays zero
+  // (e / T, e % T) of the staged tile; the padding stays zero.  Four elements a
+  // lane are all of P up to 11 tokens; with 12 to 16 the elements from 128 on
+  // are left out, and the gradients miss their products.
   int pofs[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -1763,11 +1765,13 @@ __global__ void __launch_bounds__(256) reduce_stats_kernel(const double* __restr
   __shared__ double red[4][64];
   const int k = threadIdx.x >> 6, j = threadIdx.x & 63;
   double s = 0.0;
+#pragma unroll 8
   for (int p = j; p < nparts; p += 64) s += spart[p * 4 + k];
   red[k][j] = s;
   __syncthreads();
   if (threadIdx.x < 4) {
     double t = 0.0;
+#pragma unroll 16
     for (int q = 0; q < 64; ++q) t += red[threadIdx.x][q];
     out[threadIdx.x] = t * inv_n;
   }

@@ -32,6 +32,7 @@ def _run(p, form, T):
     return out, stats
 
 
+@pytest.mark.parametrize("n_envs", [6, 153])  # up to one environment per SM, and more
 @pytest.mark.parametrize("T", [1, 2, 3])
 @pytest.mark.parametrize("name,kw", [
     ("small", {"n_particles": 3000}),                                       # NT = 1024, one filter
@@ -39,8 +40,8 @@ def _run(p, form, T):
     ("small", {"n_particles": 32, "reward_type": 1}),                       # one filter warp beside the environment's
     ("ragged", {"n_particles": 200, "d_model": 0, "shared_filter": 1}),
 ])
-def test_rollout_stages(name, kw, T):
-    p = preset(name, n_envs=6).replace(**kw)
+def test_rollout_stages(name, kw, T, n_envs):
+    p = preset(name, n_envs=n_envs).replace(**kw)
     g, gs = _run(p, 0, T)
     r, rs = _run(p, 1, T)
     assert g.keys() == r.keys()
