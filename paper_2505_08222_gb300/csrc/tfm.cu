@@ -1765,13 +1765,11 @@ __global__ void __launch_bounds__(256) reduce_stats_kernel(const double* __restr
   __shared__ double red[4][64];
   const int k = threadIdx.x >> 6, j = threadIdx.x & 63;
   double s = 0.0;
-#pragma unroll 8
   for (int p = j; p < nparts; p += 64) s += spart[p * 4 + k];
   red[k][j] = s;
   __syncthreads();
   if (threadIdx.x < 4) {
     double t = 0.0;
-#pragma unroll 16
     for (int q = 0; q < 64; ++q) t += red[threadIdx.x][q];
     out[threadIdx.x] = t * inv_n;
   }
