@@ -890,13 +890,11 @@ inline long long resident_blocks(K kernel, int threads) {
   return (long long)(b > 0 ? b : 1) * (m > 0 ? m : 152);
 }
 
-// Grid of a persistent attention kernel (4 items per block at a time): the
-// resident blocks, or fewer when there are fewer items.
-template <typename K>
-inline long long att_grid(K kernel, long long items) {
-  static const long long cap = resident_blocks(kernel, 128);  // (initialised once, thread-safe)
+// Grid of a persistent attention kernel (4 items per block at a time): its
+// resident blocks `cap`, or fewer when there are fewer items.
+inline unsigned att_grid(long long cap, long long items) {
   const long long need = (items + 3) / 4;
-  return need < cap ? need : cap;
+  return (unsigned)(need < cap ? need : cap);
 }
 
 // Attention forward on the tensor cores (tensor-core path; T <= 16, head
@@ -995,8 +993,11 @@ __global__ void __launch_bounds__(128, 8)
 // dK = dS^T Q, dV = P^T dO, as m16n8k8 TF32 MMAs over the tokens padded to
 // 16 (padded rows and columns staged as zeros), and
 // dS = P (dP - rowsum(P dP)) scale on the accumulator fragments (a row lives
-// in the 4 lanes of a quad).  dS is staged over V (V is read only by dP).
-__global__ void __launch_bounds__(128, 6)
+// in the 4 lanes of a quad).  dS is staged over V (V is read only by dP).  PE:
+// elements of P per lane, 32 PE >= T * T (att_p_per_lane).
+constexpr int att_p_per_lane(int T) { return T * T <= 128 ? 4 : 8; }
+template <int PE>
+__global__ void __launch_bounds__(128, PE == 4 ? 6 : 5)
     attn_bwd_mma_kernel(const float* __restrict__ QKV, const float* __restrict__ P, const float* __restrict__ dO,
                         float* __restrict__ dQKV, long long n, int T, int H, float scale) {
   __shared__ __align__(16) float sm[4][5][16 * kAttLd];  // Q, K, V then dS, dO, P of each warp
@@ -1005,12 +1006,10 @@ __global__ void __launch_bounds__(128, 6)
   const long long items = n * H, stride = (long long)gridDim.x * 4;
   float *sQ = sm[wl][0], *sK = sm[wl][1], *sV = sm[wl][2], *sS = sm[wl][2], *sG = sm[wl][3], *sP = sm[wl][4];
   // P of an item: T * T contiguous floats, element e = lane + 32 i at
-  // (e / T, e % T) of the staged tile; the padding stays zero.  Four elements a
-  // lane are all of P up to 11 tokens; with 12 to 16 the elements from 128 on
-  // are left out, and the gradients miss their products.
-  int pofs[4];
+  // (e / T, e % T) of the staged tile; the padding stays zero
+  int pofs[PE];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < PE; ++i) {
     const int e = lane + 32 * i;
     pofs[i] = e < T * T ? (e / T) * kAttLd + e % T : -1;
   }
@@ -1018,7 +1017,7 @@ __global__ void __launch_bounds__(128, 6)
   long long w = (long long)blockIdx.x * 4 + wl;
   AttRows r;
   float4 rg[2];
-  float rp[4];
+  float rp[PE];
   AttItem nx = {0, 0};
   auto fetch = [&](long long wi) {
     nx = att_item(wi, H);
@@ -1032,7 +1031,7 @@ __global__ void __launch_bounds__(128, 6)
     }
     const float* Pb = P + wi * T * T;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) rp[i] = pofs[i] >= 0 ? __ldg(Pb + lane + 32 * i) : 0.0f;
+    for (int i = 0; i < PE; ++i) rp[i] = pofs[i] >= 0 ? __ldg(Pb + lane + 32 * i) : 0.0f;
   };
   if (w < items) fetch(w);
   for (; w < items; w += stride) {
@@ -1043,7 +1042,7 @@ __global__ void __launch_bounds__(128, 6)
     att_stage(r.v, sV, lane);
     att_stage(rg, sG, lane);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < PE; ++i)
       if (pofs[i] >= 0) sP[pofs[i]] = rp[i];
     if (w + stride < items) fetch(w + stride);  // in flight during this item
     __syncwarp();
@@ -2088,8 +2087,8 @@ cudaError_t attn_fwd(const float* QKV, const int32_t* ne, const int32_t* sel, fl
                      int NS, int H, bool mma, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (mma && DH == 16 && T <= 16 && ((uintptr_t)QKV & 15) == 0) {
-    const long long grid = att_grid(attn_fwd_mma_kernel, n * H);
-    attn_fwd_mma_kernel<<<(unsigned)grid, 128, 0, s>>>(QKV, ne, sel, P, O, n, T, NS, H, 1.0f / sqrtf((float)DH));
+    static const long long cap = resident_blocks(attn_fwd_mma_kernel, 128);
+    attn_fwd_mma_kernel<<<att_grid(cap, n * H), 128, 0, s>>>(QKV, ne, sel, P, O, n, T, NS, H, 1.0f / sqrtf((float)DH));
     return cudaGetLastError();
   }
   static std::atomic<unsigned long long> ready{0};
@@ -2100,20 +2099,26 @@ cudaError_t attn_fwd(const float* QKV, const int32_t* ne, const int32_t* sel, fl
   return cudaGetLastError();
 }
 
+template <int PE>
+cudaError_t attn_bwd_mma(const float* QKV, const float* P, const float* dO, float* dQKV, long long n, int T, int H,
+                         cudaStream_t s) {
+  static const long long cap = resident_blocks(attn_bwd_mma_kernel<PE>, 128);
+  attn_bwd_mma_kernel<PE><<<att_grid(cap, n * H), 128, 0, s>>>(QKV, P, dO, dQKV, n, T, H, 0.25f);
+  return cudaGetLastError();
+}
+
 template <int DH>
 cudaError_t attn_bwd(const float* QKV, const float* P, const float* dO, float* dQKV, long long n, int T, int H,
                      bool mma, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (mma && DH == 16 && T <= 16 && ((uintptr_t)QKV & 15) == 0 && ((uintptr_t)dO & 15) == 0)
-    attn_bwd_mma_kernel<<<(unsigned)att_grid(attn_bwd_mma_kernel, n * H), 128, 0, s>>>(QKV, P, dO, dQKV, n, T, H,
-                                                                                       1.0f / sqrtf((float)DH));
-  else {
-    static std::atomic<unsigned long long> ready{0};
-    const cudaError_t e = smem_optin(attn_bwd_kernel<DH>, kAttnSmemMax, ready);
-    if (e != cudaSuccess) return e;
-    attn_bwd_kernel<DH><<<blocks_for(n * H, attn_items(T)), kAttnThreads, attn_bwd_smem(T, DH), s>>>(
-        QKV, P, dO, dQKV, n, T, H, 1.0f / sqrtf((float)DH));
-  }
+    return att_p_per_lane(T) == 4 ? attn_bwd_mma<4>(QKV, P, dO, dQKV, n, T, H, s)
+                                  : attn_bwd_mma<8>(QKV, P, dO, dQKV, n, T, H, s);
+  static std::atomic<unsigned long long> ready{0};
+  const cudaError_t e = smem_optin(attn_bwd_kernel<DH>, kAttnSmemMax, ready);
+  if (e != cudaSuccess) return e;
+  attn_bwd_kernel<DH><<<blocks_for(n * H, attn_items(T)), kAttnThreads, attn_bwd_smem(T, DH), s>>>(
+      QKV, P, dO, dQKV, n, T, H, 1.0f / sqrtf((float)DH));
   return cudaGetLastError();
 }
 
