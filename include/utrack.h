@@ -58,9 +58,11 @@ typedef enum {
 } ut_status;
 
 /* Caller-supplied device allocator.  alloc(bytes, stream, ctx) returns a
- * device pointer aligned to at least 256 bytes or NULL; free(ptr, stream,
- * ctx) releases it.  NULL allocator: the library uses cudaMallocAsync /
- * cudaFreeAsync on the handle's stream. */
+ * device pointer aligned to at least 256 bytes or NULL, ready for work on
+ * `stream`; free(ptr, stream, ctx) releases it, while work enqueued on that
+ * stream may still use it.  `stream` is the handle's, in policy_forward the
+ * call's.  NULL allocator: the library uses cudaMallocAsync / cudaFreeAsync on
+ * that stream. */
 typedef struct ut_allocator {
   void* (*alloc)(size_t bytes, void* stream, void* ctx);
   void (*free)(void* ptr, void* stream, void* ctx);
@@ -346,7 +348,12 @@ ut_status env_set_policy(ut_env* env, const float* params_host, int64_t n_params
  * embedding (16-byte aligned), read and replaced by the block output at the
  * recurrent token; logits_dev [n_agents][n_actions] FP32 written;
  * actions_dev [n_agents] (optional) receives Gumbel-max samples drawn at
- * global step `step`.  Errors: UT_ERR_STATE (no weights), UT_ERR_INVALID. */
+ * global step `step`.  Enqueued on cuda_stream, not synchronising.  Batches of
+ * more than three waves of tiles (912 CTAs of 128 / (1 + n_slots) agents at
+ * d_model 64, 456 at 128) take a workspace of at most 46 MB from the handle's
+ * allocator for the call, in the order of cuda_stream; in a stream capture, or
+ * where there is none to be had, the slower one-kernel form runs, with the same
+ * results bit for bit.  Errors: UT_ERR_STATE (no weights), UT_ERR_INVALID. */
 ut_status policy_forward(ut_env* env, const uint16_t* tokens_dev, const int32_t* n_ent_dev, uint16_t* h_dev,
                          float* logits_dev, int32_t* actions_dev, int64_t n_agents, int32_t n_slots, uint32_t step,
                          void* cuda_stream);

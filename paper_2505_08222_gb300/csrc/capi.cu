@@ -37,15 +37,21 @@ ut_status cuda_fail(ut_env* h, cudaError_t e, const char* where) {
 
 namespace ut {
 
+void* stream_alloc(ut_env* h, size_t bytes, cudaStream_t s) {
+  if (h->has_alloc) return h->alloc.alloc(bytes, (void*)s, h->alloc.ctx);
+  void* p = nullptr;
+  return cudaMallocAsync(&p, bytes, s) == cudaSuccess ? p : nullptr;
+}
+
+void stream_free(ut_env* h, void* p, cudaStream_t s) {
+  if (h->has_alloc) h->alloc.free(p, (void*)s, h->alloc.ctx);
+  else cudaFreeAsync(p, s);
+}
+
 void* env_alloc(ut_env* h, size_t bytes) {
   if (bytes == 0) bytes = 16;
   bytes = (bytes + 255) & ~(size_t)255;
-  void* p = nullptr;
-  if (h->has_alloc) {
-    p = h->alloc.alloc(bytes, (void*)h->stream, h->alloc.ctx);
-  } else {
-    if (cudaMallocAsync(&p, bytes, h->stream) != cudaSuccess) p = nullptr;
-  }
+  void* p = stream_alloc(h, bytes, h->stream);
   if (!p) return nullptr;
   h->allocations.push_back(p);
   if (cudaMemsetAsync(p, 0, bytes, h->stream) != cudaSuccess) return nullptr;
@@ -53,10 +59,7 @@ void* env_alloc(ut_env* h, size_t bytes) {
 }
 
 void env_free_all(ut_env* h) {
-  for (void* p : h->allocations) {
-    if (h->has_alloc) h->alloc.free(p, (void*)h->stream, h->alloc.ctx);
-    else cudaFreeAsync(p, h->stream);
-  }
+  for (void* p : h->allocations) stream_free(h, p, h->stream);
   h->allocations.clear();
 }
 

@@ -43,10 +43,7 @@ struct PolicyState {
   uint16_t* h = nullptr;
   float* logits = nullptr;
   int32_t* n_ent = nullptr;
-  // two-kernel form of large batches: the step's workspace, and the pool of
-  // policy_forward's, one per call (calls on several streams may overlap)
-  void* ws = nullptr;
-  cudaMemPool_t pool = nullptr;
+  void* ws = nullptr;  // the step's workspace of the two-kernel form (large batches)
 };
 
 namespace ut {
@@ -114,7 +111,6 @@ ut_status extension_create(ut_env* h) {
 }
 
 void extension_destroy(ut_env* h) {
-  if (h->policy && h->policy->pool) cudaMemPoolDestroy(h->policy->pool);
   delete h->policy;
   h->policy = nullptr;
   delete h->est;
@@ -177,7 +173,10 @@ extern "C" ut_status env_set_policy(ut_env* h, const float* params_host, int64_t
     ps->head = head_d;
     ps->wimg = wimg;
     // (without a workspace the step keeps the one-kernel form)
-    if (policy_split(ps->d, h->NA, 1 + h->d.NS)) ps->ws = env_alloc(h, policy_ws_bytes(ps->d, h->NA, 1 + h->d.NS));
+    if (policy_split(ps->d, h->NA, 1 + h->d.NS)) {
+      ps->ws = env_alloc(h, policy_ws_bytes(ps->d, h->NA, 1 + h->d.NS));
+      if (!ps->ws) (void)cudaGetLastError();  // (not the next launch's error)
+    }
   }
   cudaError_t e = cudaMemcpyAsync(ps->wimg, img.data(), img.size(), cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(ps->vec, vec.data(), vec.size() * 4, cudaMemcpyHostToDevice, h->stream);
@@ -193,31 +192,18 @@ extern "C" ut_status env_set_policy(ut_env* h, const float* params_host, int64_t
   return UT_OK;
 }
 
-// Workspace of one policy_forward call, stream-ordered from the handle's own
-// pool (which keeps up to 64 MB between calls and goes with the handle): NULL
-// where the one-kernel form is the faster one, in a stream capture, and when
-// there is no memory for it.
+// Workspace of one policy_forward call, from the handle's allocator in the order
+// of the call's stream and handed back after its launches (calls on several
+// streams may overlap: each has its own): NULL where the one-kernel form is the
+// faster one, in a stream capture, and when there is no memory for it.
 static void* forward_ws(ut_env* h, const PolicyDev& p, cudaStream_t s) {
   PolicyState* ps = h->policy;
   if (!policy_split(ps->d, p.NA, p.R)) return nullptr;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   void* ws = nullptr;
-  bool ok = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
-  if (ok && !ps->pool) {
-    cudaMemPoolProps props;
-    std::memset(&props, 0, sizeof(props));
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = h->device;
-    uint64_t keep = 64ull << 20;
-    ok = cudaMemPoolCreate(&ps->pool, &props) == cudaSuccess &&
-         cudaMemPoolSetAttribute(ps->pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess;
-  }
-  if (ok) ok = cudaMallocFromPoolAsync(&ws, policy_ws_bytes(ps->d, p.NA, p.R), ps->pool, s) == cudaSuccess;
-  if (!ok) {
-    (void)cudaGetLastError();
-    return nullptr;
-  }
+  if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone)
+    ws = stream_alloc(h, policy_ws_bytes(ps->d, p.NA, p.R), s);
+  if (!ws) (void)cudaGetLastError();  // (not the launch's error)
   return ws;
 }
 
@@ -256,10 +242,7 @@ extern "C" ut_status policy_forward(ut_env* h, const uint16_t* tokens_dev, const
   void* ws = forward_ws(h, p, s);
   if (ws) policy_ws_set(p, h->policy->d, ws);
   cudaError_t e = launch_policy(p, h->policy->d, s);
-  if (ws) {
-    const cudaError_t ef = cudaFreeAsync(ws, s);
-    if (e == cudaSuccess) e = ef;
-  }
+  if (ws) stream_free(h, ws, s);
   if (e != cudaSuccess) {
     h->err = std::string("policy_forward: ") + cudaGetErrorString(e);
     return UT_ERR_CUDA;

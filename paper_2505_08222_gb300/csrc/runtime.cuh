@@ -58,6 +58,11 @@ struct ut_env {
 
 namespace ut {
 
+// A buffer from the handle's allocator, ordered on stream s (NULL: none to be
+// had); env_alloc's are on the handle's stream, zeroed, and kept until
+// env_free_all.
+void* stream_alloc(ut_env* h, size_t bytes, cudaStream_t s);
+void stream_free(ut_env* h, void* p, cudaStream_t s);
 void* env_alloc(ut_env* h, size_t bytes);
 void env_free_all(ut_env* h);
 cudaError_t enqueue_step(ut_env* h, const int32_t* act, cudaStream_t s);
