@@ -380,12 +380,13 @@ __device__ __forceinline__ void train_stage(int s, size_t& off, uint32_t& bytes)
 template <bool TRAIN>
 __global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __restrict__ X,
                                                      const int32_t* __restrict__ rows, int B, float* __restrict__ out,
-                                                     TrainBufs t, int* status) {
+                                                     TrainBufs t, int* status, uint32_t test_wait_polls) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* sA = smem;          // features hi | lo, then the current A operand [128 x 256]
   unsigned char* sW = smem + 65536;  // two weight slots
   __shared__ __align__(8) uint64_t full[2];
   __shared__ __align__(8) uint64_t mbar;
+  __shared__ __align__(8) uint64_t never;  // test hook: a barrier nothing signals
   __shared__ uint32_t tbase;
   __shared__ float sOut[2][128];
   __shared__ float s_red[TRAIN ? 4 : 1][TRAIN ? NB_PART : 1];  // column sums of each 32-row quarter
@@ -405,12 +406,22 @@ __global__ void __launch_bounds__(kTE, 1) mlp_kernel(Net net, const float* __res
     tc::mbar_init(&full[0], 1);
     tc::mbar_init(&full[1], 1);
     tc::mbar_init(&mbar, 1);
+    tc::mbar_init(&never, 1);
     bad = 0;
   }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tbase;
+  if (test_wait_polls) {  // as in fwd_env_kernel
+    if (tid == 32 && !tc::mbar_wait(&never, 0u, test_wait_polls)) bad = 1;
+    __syncthreads();
+    if (bad) {
+      if (tid == 0) raise_status(status, 2);
+      if (warp == 0) tc::tmem_dealloc(tmem, kCols);
+      return;
+    }
+  }
   const uint32_t tl = tmem + ((uint32_t)quarter << 21);  // this warp's lane quarter
   const uint32_t aA = tc::smem_addr(sA), aW = tc::smem_addr(sW);
   constexpr int kStages = TRAIN ? kTrainStages : kEnvStages;
@@ -787,6 +798,7 @@ constexpr int kRedW = (int)((NW_PART / 4 + 255) / 256), kRedB = (NB_PART + 31) /
 
 __global__ void __launch_bounds__(256) grad_reduce_kernel(TrainBufs t, int splits, int n_cta) {
   const int tid = threadIdx.x;
+  if (t.result->status) return;  // (partial sums of a pass that gave up, or of an earlier one)
   if (blockIdx.x < kRedW) {
     const long long i = ((long long)blockIdx.x * 256 + tid) * 4;
     if (i >= NW_PART) return;
@@ -828,7 +840,7 @@ __global__ void __launch_bounds__(256) grad_reduce_kernel(TrainBufs t, int split
     double acc = 0.0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) acc += sl[k];
-    *t.loss = acc / t.B;
+    t.result->loss = acc / t.B;
   }
 }
 
@@ -853,9 +865,10 @@ __device__ __forceinline__ void write_images(unsigned char* img, long long i, fl
 }
 
 __global__ void adam_kernel(float* master, float* m, float* v, const float* grad, float lr, float beta1, float beta2,
-                            float eps, float c1, float c2, unsigned char* img) {
+                            float eps, float c1, float c2, unsigned char* img, EstResult* result) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= NPARAM) return;
+  if (i >= NPARAM || (result && result->status)) return;
+  if (result && i == 0) ++result->updates;
   const float g = grad[i];
   const float mi = beta1 * m[i] + (1.0f - beta1) * g;
   const float vi = beta2 * v[i] + (1.0f - beta2) * g * g;
@@ -895,12 +908,14 @@ __global__ void record_kernel(EnvDev d, float* feat, float* label) {
 
 }  // namespace
 
-cudaError_t launch_forward(const Net& net, const float* X, int B, float* out, cudaStream_t s) {
+cudaError_t launch_forward(const Net& net, const float* X, int B, float* out, int* status, uint32_t test_wait_polls,
+                           cudaStream_t s) {
   static std::atomic<unsigned long long> ready{0};
   cudaError_t e = smem_optin(mlp_kernel<false>, kEnvSmem, ready);
   if (e != cudaSuccess) return e;
   if (B <= 0) return cudaSuccess;
-  mlp_kernel<false><<<(B + kT - 1) / kT, kTE, kEnvSmem, s>>>(net, X, nullptr, B, out, TrainBufs{}, nullptr);
+  mlp_kernel<false><<<(B + kT - 1) / kT, kTE, kEnvSmem, s>>>(net, X, nullptr, B, out, TrainBufs{}, status,
+                                                              test_wait_polls);
   return cudaGetLastError();
 }
 
@@ -927,11 +942,11 @@ cudaError_t launch_loss_grad(const Net& net, const TrainBufs& t, cudaStream_t s)
   if (e != cudaSuccess) return e;
   if (t.B <= 0) return cudaSuccess;
   const int n_cta = (t.B + kT - 1) / kT;
-  mlp_kernel<true><<<n_cta, kTE, kEnvSmem, s>>>(net, t.X, t.rows, t.B, nullptr, t, nullptr);
+  mlp_kernel<true><<<n_cta, kTE, kEnvSmem, s>>>(net, t.X, t.rows, t.B, nullptr, t, &t.result->status, t.test_wait_polls);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int splits = n_cta < kWgradSplits ? n_cta : kWgradSplits;
-  wgrad_kernel<<<dim3(splits, 2, 3), kT, kWgradSmem, s>>>(t, nullptr);
+  wgrad_kernel<<<dim3(splits, 2, 3), kT, kWgradSmem, s>>>(t, &t.result->status);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   grad_reduce_kernel<<<kRedW + kRedB + 1, 256, 0, s>>>(t, splits, n_cta);
@@ -939,10 +954,10 @@ cudaError_t launch_loss_grad(const Net& net, const TrainBufs& t, cudaStream_t s)
 }
 
 cudaError_t launch_adam(float* master, float* m, float* v, const float* grad, int step, float lr, float beta1,
-                        float beta2, float eps, unsigned char* img, cudaStream_t s) {
+                        float beta2, float eps, unsigned char* img, EstResult* result, cudaStream_t s) {
   const double c1 = 1.0 - std::pow((double)beta1, step), c2 = 1.0 - std::pow((double)beta2, step);
   adam_kernel<<<(unsigned)((NPARAM + 255) / 256), 256, 0, s>>>(master, m, v, grad, lr, beta1, beta2, eps, (float)c1,
-                                                              (float)c2, img);
+                                                              (float)c2, img, result);
   return cudaGetLastError();
 }
 

@@ -54,6 +54,15 @@ struct Net {
   const float* master;       // FP32 parameters, canonical order (biases, W4)
 };
 
+// What a gradient call leaves for the host: the batch's loss, 2 once a bounded
+// wait gave up (its loss and gradient are not written then, nor is any Adam
+// update made from it on), and the Adam updates made.
+struct EstResult {
+  double loss;
+  int status;
+  int updates;
+};
+
 // Training buffers for one batch of B rows (tiles = ceil(B / 128)).  An
 // operand image holds 128 rows as [feature / 8][row][8] BF16.
 struct TrainBufs {
@@ -65,24 +74,29 @@ struct TrainBufs {
   unsigned char* a_img;   // [2][tiles] images of GELU(z1), GELU(z2)
   unsigned char* dz_img;  // [3][tiles] images of the gradients w.r.t. z
   float* grad;            // [NPARAM] FP32 gradient (every entry written)
-  double* loss;           // [1] loss of the batch
+  EstResult* result;      // loss and status of the batch
   // fixed-order partial sums (no atomics: the gradient is deterministic)
   float* part_b;          // [tiles][NB_PART] per-CTA dW4, db3, db2, db1, db4
   double* part_loss;      // [tiles] per-CTA loss sums
   float* part_w;          // [kWgradSplits][NW_PART] per-split dW1, dW2, dW3
   float huber;            // 0: squared error; > 0: Huber threshold (label units)
   int B;
+  uint32_t test_wait_polls;  // test hook, env_test_wait_timeout
 };
 
-// Outputs [B][2] of the features X [B][96].
-cudaError_t launch_forward(const Net& net, const float* X, int B, float* out, cudaStream_t s);
-// Loss and gradient of one batch (t.loss, t.grad).
+// Outputs [B][2] of the features X [B][96]; a tile of 128 rows whose wait gave
+// up is not written and raises *status.
+cudaError_t launch_forward(const Net& net, const float* X, int B, float* out, int* status, uint32_t test_wait_polls,
+                           cudaStream_t s);
+// Loss and gradient of one batch (t.result, t.grad).
 cudaError_t launch_loss_grad(const Net& net, const TrainBufs& t, cudaStream_t s);
 cudaError_t launch_forward_env(const Net& net, const EnvDev& d, int stale, uint32_t test_wait_polls,
                                cudaStream_t s);
 cudaError_t launch_record(const EnvDev& d, float* feat, float* label, cudaStream_t s);
+// result: counts the update, and holds it back once its status is set; NULL:
+// always made (a gradient from elsewhere).
 cudaError_t launch_adam(float* master, float* m, float* v, const float* grad, int step, float lr, float beta1,
-                        float beta2, float eps, unsigned char* img, cudaStream_t s);
+                        float beta2, float eps, unsigned char* img, EstResult* result, cudaStream_t s);
 cudaError_t launch_pack(const float* master, unsigned char* img, cudaStream_t s);
 cudaError_t launch_batch_rows(int32_t* rows, int B, int64_t n_rows, uint64_t seed, uint32_t step, cudaStream_t s);
 

@@ -1,6 +1,7 @@
 // Hooks through which the transformer agent (and the learned estimator) plug
 // into the environment step, and their C-ABI entry points.
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -26,7 +27,7 @@ struct EstimatorState {
   unsigned char* a_img = nullptr;
   unsigned char* dz_img = nullptr;
   int32_t* rows = nullptr;
-  double* loss = nullptr;
+  ut::est::EstResult* result = nullptr;  // (its status is 0 between calls)
   // fixed-order partial sums of the backward pass
   float* part_b = nullptr;
   double* part_loss = nullptr;
@@ -279,13 +280,13 @@ ut_status est_alloc_weights(ut_env* h) {
   float* v = (float*)env_alloc(h, est::NPARAM * 4);
   float* grad = (float*)env_alloc(h, est::NPARAM * 4);
   unsigned char* img = (unsigned char*)env_alloc(h, est::IMG_BYTES);
-  double* loss = (double*)env_alloc(h, 8);
-  if (!master || !m || !v || !grad || !img || !loss) return est_fail(h, UT_ERR_NOMEM, "estimator: allocation failed");
+  est::EstResult* result = (est::EstResult*)env_alloc(h, sizeof(est::EstResult));
+  if (!master || !m || !v || !grad || !img || !result) return est_fail(h, UT_ERR_NOMEM, "estimator: allocation failed");
   es->m = m;
   es->v = v;
   es->grad = grad;
   es->img = img;
-  es->loss = loss;
+  es->result = result;
   es->master = master;
   return UT_OK;
 }
@@ -324,7 +325,7 @@ est::Net est_net(ut_env* h) {
   return n;
 }
 
-// Loss and gradient of one batch into es->loss and grad.
+// Loss and gradient of one batch into es->result and grad.
 cudaError_t est_grad_batch(ut_env* h, const float* X, const float* Y, const int32_t* rows, int B, float huber,
                            float* grad) {
   EstimatorState* es = h->est;
@@ -337,13 +338,28 @@ cudaError_t est_grad_batch(ut_env* h, const float* X, const float* Y, const int3
   t.a_img = es->a_img;
   t.dz_img = es->dz_img;
   t.grad = grad;
-  t.loss = es->loss;
+  t.result = es->result;
   t.part_b = es->part_b;
   t.part_loss = es->part_loss;
   t.part_w = es->part_w;
   t.huber = huber;
   t.B = B;
+  t.test_wait_polls = h->test_wait_polls;
   return est::launch_loss_grad(est_net(h), t, h->stream);
+}
+
+// Waits for the call's work and reads its result; a wait that gave up is
+// reported and cleared.
+ut_status est_result(ut_env* h, est::EstResult* r, const char* what) {
+  EstimatorState* es = h->est;
+  cudaError_t e = cudaMemcpyAsync(r, es->result, sizeof(*r), cudaMemcpyDeviceToHost, h->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess && (r->status || r->updates))
+    e = cudaMemsetAsync(&es->result->status, 0, sizeof(*r) - offsetof(est::EstResult, status), h->stream);
+  if (e != cudaSuccess) return est_fail(h, UT_ERR_CUDA, cudaGetErrorString(e));
+  if (!r->status) return UT_OK;
+  h->err = std::string(what) + ": a bounded device wait gave up";
+  return UT_ERR_TIMEOUT;
 }
 
 }  // namespace
@@ -397,7 +413,8 @@ extern "C" ut_status est_forward(ut_env* h, const float* X_dev, float* out_dev, 
   if (!h || n_rows < 0 || n_rows > 0x7fffffff || (n_rows && (!X_dev || !out_dev))) return UT_ERR_INVALID;
   if (!h->est || !h->est->weights_set) return est_fail(h, UT_ERR_STATE, "est_forward: no weights");
   if (reinterpret_cast<uintptr_t>(X_dev) & 15) return est_fail(h, UT_ERR_INVALID, "est_forward: X not 16-byte aligned");
-  cudaError_t e = est::launch_forward(est_net(h), X_dev, (int)n_rows, out_dev, h->stream);
+  cudaError_t e = est::launch_forward(est_net(h), X_dev, (int)n_rows, out_dev, h->d.status, h->test_wait_polls,
+                                      h->stream);
   return e == cudaSuccess ? UT_OK : est_fail(h, UT_ERR_CUDA, cudaGetErrorString(e));
 }
 
@@ -424,13 +441,12 @@ extern "C" ut_status est_loss_grad(ut_env* h, const float* X_dev, const float* Y
     if (er != cudaSuccess) return est_fail(h, UT_ERR_CUDA, cudaGetErrorString(er));
     rows = h->est->rows;
   }
-  cudaError_t e = est_grad_batch(h, X_dev, Y_dev, rows, B, huber_delta, grad_dev);
-  double loss = 0.0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&loss, h->est->loss, 8, cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  const cudaError_t e = est_grad_batch(h, X_dev, Y_dev, rows, B, huber_delta, grad_dev);
   if (e != cudaSuccess) return est_fail(h, UT_ERR_CUDA, cudaGetErrorString(e));
-  if (loss_host) *loss_host = loss;
-  return UT_OK;
+  est::EstResult r;
+  st = est_result(h, &r, "est_loss_grad");
+  if (st == UT_OK && loss_host) *loss_host = r.loss;
+  return st;
 }
 
 extern "C" ut_status est_adam_step(ut_env* h, const float* grad_dev, float lr, float beta1, float beta2, float eps) {
@@ -441,7 +457,7 @@ extern "C" ut_status est_adam_step(ut_env* h, const float* grad_dev, float lr, f
   EstimatorState* es = h->est;
   es->adam_t += 1;
   cudaError_t e = est::launch_adam(es->master, es->m, es->v, grad_dev, es->adam_t, lr, beta1, beta2, eps, es->img,
-                                   h->stream);
+                                   nullptr, h->stream);
   return e == cudaSuccess ? UT_OK : est_fail(h, UT_ERR_CUDA, cudaGetErrorString(e));
 }
 
@@ -459,6 +475,7 @@ extern "C" ut_status est_train(ut_env* h, const float* X_dev, const float* Y_dev
   cudaEventCreate(&e1);
   cudaEventRecord(e0, h->stream);
   double first = -1.0, last = 0.0;
+  const int adam_t0 = es->adam_t;
   const bool full = (B == n_rows);  // the whole dataset as one batch, in order
   cudaError_t e = cudaSuccess;
   for (int s = 0; s < cfg->steps && e == cudaSuccess; ++s) {
@@ -474,10 +491,10 @@ extern "C" ut_status est_train(ut_env* h, const float* X_dev, const float* Y_dev
     es->adam_t += 1;
     if (e == cudaSuccess)
       e = est::launch_adam(es->master, es->m, es->v, es->grad, es->adam_t, lr, cfg->beta1, cfg->beta2, cfg->eps,
-                           es->img, h->stream);
+                           es->img, es->result, h->stream);
     if (e == cudaSuccess && (s == 0 || s == cfg->steps - 1)) {
       double l = 0.0;
-      e = cudaMemcpyAsync(&l, es->loss, 8, cudaMemcpyDeviceToHost, h->stream);
+      e = cudaMemcpyAsync(&l, &es->result->loss, 8, cudaMemcpyDeviceToHost, h->stream);
       if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
       if (s == 0) first = l;
       last = l;
@@ -490,6 +507,10 @@ extern "C" ut_status est_train(ut_env* h, const float* X_dev, const float* Y_dev
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (e != cudaSuccess) return est_fail(h, UT_ERR_CUDA, cudaGetErrorString(e));
+  est::EstResult r;
+  st = est_result(h, &r, "est_train");
+  es->adam_t = adam_t0 + r.updates;  // (all of them, unless a wait gave up)
+  if (st != UT_OK) return st;
   if (out) {
     out->loss_first = first;
     out->loss_last = last;
