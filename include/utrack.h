@@ -412,9 +412,10 @@ ut_status est_get_weights(ut_env* env, float* params_host, int64_t n_params);
  * pings or collinear senders (det A <= 1e-3 (tr A)^2 for the 2 x 2 normal
  * matrix A).  Errors: UT_ERR_INVALID (mode outside 0..4), UT_ERR_STATE. */
 ut_status est_set_mode(ut_env* env, int32_t mode);
-/* Raw network outputs out_dev [n_rows][2] of features X_dev [n_rows][96].  A
- * bounded wait that gave up leaves the outputs of its 128 rows unwritten and
- * is reported by env_metrics. */
+/* Raw network outputs out_dev [n_rows][2] of features X_dev [n_rows][96]
+ * (16-byte aligned, as in the calls below, else UT_ERR_INVALID).  A bounded wait
+ * that gave up leaves the outputs of its 128 rows unwritten and is reported by
+ * env_metrics. */
 ut_status est_forward(ut_env* env, const float* X_dev, float* out_dev, int64_t n_rows);
 /* Features [F][96] and labels [F][2] = (target - e1)/L of every filter's
  * last update (call after a step; e1, e2 = the estimates before it); needs
@@ -429,8 +430,8 @@ ut_status est_record(ut_env* env, float* feat_dev, float* label_dev);
  * L = (1/(2B)) sum over rows and both outputs of (out - y)^2; > 0: the Huber
  * loss with that threshold (label units), (1/B) sum of the per-output loss.
  * Synchronising; *loss_host (optional) receives L.
- * Errors: UT_ERR_INVALID (sizes, B > 2^22, negative threshold),
- * UT_ERR_STATE (no weights), UT_ERR_NOMEM, UT_ERR_CUDA, UT_ERR_TIMEOUT (a
+ * Errors: UT_ERR_INVALID (sizes, B > 2^22, negative threshold, X_dev not
+ * 16-byte aligned), UT_ERR_STATE (no weights), UT_ERR_NOMEM, UT_ERR_CUDA, UT_ERR_TIMEOUT (a
  * bounded wait gave up: neither the gradient nor the loss is written). */
 ut_status est_loss_grad(ut_env* env, const float* X_dev, const float* Y_dev, int64_t n_rows, int32_t B,
                         uint64_t seed, uint32_t step, float huber_delta, float* grad_dev, double* loss_host);

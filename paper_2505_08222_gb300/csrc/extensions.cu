@@ -433,6 +433,8 @@ extern "C" ut_status est_loss_grad(ut_env* h, const float* X_dev, const float* Y
       !(huber_delta >= 0.0f))
     return UT_ERR_INVALID;
   if (!h->est || !h->est->weights_set) return est_fail(h, UT_ERR_STATE, "est_loss_grad: no weights");
+  if (reinterpret_cast<uintptr_t>(X_dev) & 15)
+    return est_fail(h, UT_ERR_INVALID, "est_loss_grad: X not 16-byte aligned");
   ut_status st = est_alloc_batch(h, B);
   if (st != UT_OK) return st;
   const int32_t* rows = nullptr;
@@ -466,6 +468,7 @@ extern "C" ut_status est_train(ut_env* h, const float* X_dev, const float* Y_dev
   if (!h || !X_dev || !Y_dev || !cfg || n_rows < 1 || n_rows >= (1ll << 32)) return UT_ERR_INVALID;
   if (cfg->steps < 1 || cfg->batch < 1 || cfg->batch > (1 << 22) || !(cfg->lr > 0.0f)) return UT_ERR_INVALID;
   if (!h->est || !h->est->weights_set) return est_fail(h, UT_ERR_STATE, "est_train: no initial weights");
+  if (reinterpret_cast<uintptr_t>(X_dev) & 15) return est_fail(h, UT_ERR_INVALID, "est_train: X not 16-byte aligned");
   const int B = cfg->batch;
   ut_status st = est_alloc_batch(h, B);
   if (st != UT_OK) return st;
