@@ -168,49 +168,48 @@ __global__ void __launch_bounds__(256) sgemm_kernel(Gemm g) {
 // the host): the contiguous dimension of each operand is read in aligned
 // float4 (leading dimensions and base addresses multiples of 4 floats; M, N
 // multiples of 4 where they are contiguous), and with k-contiguous operands
-// the K range is a multiple of 32.
+// the K range is a multiple of 32.  by: the column tile.
 template <bool AK, bool BK>
-__global__ void __launch_bounds__(256) sgemm128_kernel(Gemm g) {
+__device__ __forceinline__ void sgemm128_tile(const Gemm& g, int by) {
   __shared__ __align__(16) float As[32][132];
   __shared__ __align__(16) float Bs[32][68];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const long long m0 = (long long)blockIdx.x * 128;
-  const int n0 = blockIdx.y * 64;
+  const int n0 = by * 64;
   const long long kb = (long long)blockIdx.z * g.kchunk;
   const long long ke = kb + g.kchunk < g.K ? kb + g.kchunk : g.K;
   float4 ra[4], rb[2];
-  // A slice: 128 (m) x 32 (k) as 1024 float4, four per thread.  Every load is
-  // made: past M or N from the last row or column (what it feeds is not stored),
-  // past the range of k from its last row, zeroed when it is staged.  (Behind
-  // bounds conditions each load of a partial tile waited for the one before: a
-  // forward of 64 samples at d = 128 on this path 262 us, now 221.)
+  // A slice: 128 (m) x 32 (k) as 1024 float4, four per thread; B slice: 32 (k) x
+  // 64 (n) as 512, two per thread.  Every load is made: past M or N from the last
+  // row or column (what it feeds is not stored), past the range of k from its
+  // last row, zeroed when it is staged.  (Behind bounds conditions each load of a
+  // partial tile waited for the one before: a forward of 64 samples of 4 tokens at
+  // d = 128, 2 blocks, 262 us, without them 221; with the addresses made once and
+  // the last block's pair below 215.)
+  const float *pa[4], *pb[2];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int i = tid + r * 256;
+    pa[r] = g.A + (AK ? min(m0 + (i >> 3), g.M - 1) * g.lda + (i & 7) * 4 : min(m0 + (i & 31) * 4, g.M - 4));
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int i = tid + r * 256;
+    pb[r] = g.B + (BK ? (long long)min(n0 + (i >> 3), g.N - 1) * g.ldb + (i & 7) * 4
+                      : (long long)min(n0 + (i & 15) * 4, g.N - 4));
+  }
   auto load_a = [&](long long k0) {
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      const int i = tid + r * 256;
-      if (AK) {  // (K and its split are multiples of 32)
-        const long long m = min(m0 + (i >> 3), g.M - 1), k = k0 + (i & 7) * 4;
-        ra[r] = *reinterpret_cast<const float4*>(g.A + m * g.lda + k);
-      } else {   // (M is a multiple of 4)
-        const long long k = min(k0 + (i >> 5), ke - 1), m = min(m0 + (i & 31) * 4, g.M - 4);
-        ra[r] = *reinterpret_cast<const float4*>(g.A + k * g.lda + m);
-      }
+      const long long k = k0 + ((tid + r * 256) >> 5);
+      ra[r] = *reinterpret_cast<const float4*>(pa[r] + (AK ? k0 : min(k, ke - 1) * g.lda));
     }
   };
-  // B slice: 32 (k) x 64 (n) as 512 float4, two per thread
   auto load_b = [&](long long k0) {
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-      const int i = tid + r * 256;
-      if (BK) {
-        const int n = min(n0 + (i >> 3), g.N - 1);
-        const long long k = k0 + (i & 7) * 4;
-        rb[r] = *reinterpret_cast<const float4*>(g.B + (long long)n * g.ldb + k);
-      } else {
-        const long long k = min(k0 + (i >> 4), ke - 1);
-        const int n = min(n0 + (i & 15) * 4, g.N - 4);
-        rb[r] = *reinterpret_cast<const float4*>(g.B + k * g.ldb + n);
-      }
+      const long long k = k0 + ((tid + r * 256) >> 4);
+      rb[r] = *reinterpret_cast<const float4*>(pb[r] + (BK ? k0 : min(k, ke - 1) * g.ldb));
     }
   };
   auto store = [&](long long k0) {
@@ -288,6 +287,20 @@ __global__ void __launch_bounds__(256) sgemm128_kernel(Gemm g) {
       epi_store(g, m, n, acc[i][j]);
     }
   }
+}
+
+template <bool AK, bool BK>
+__global__ void __launch_bounds__(256) sgemm128_kernel(Gemm g) {
+  sgemm128_tile<AK, BK>(g, blockIdx.y);
+}
+// Two products in one launch, column tiles 0 .. ny - 1 of a and then b's; the
+// grid covers the larger of their rows and splits.
+template <bool AK, bool BK>
+__global__ void __launch_bounds__(256) sgemm128_pair_kernel(Gemm a, Gemm b, int ny) {
+  const bool second = (int)blockIdx.y >= ny;
+  const Gemm g = second ? b : a;
+  if ((long long)blockIdx.x * 128 >= g.M || (long long)blockIdx.z * g.kchunk >= g.K) return;
+  sgemm128_tile<AK, BK>(g, (int)blockIdx.y - (second ? ny : 0));
 }
 
 // The entity tokens of one sample, 4 slots per register: lane i of v[j] holds
@@ -1692,25 +1705,34 @@ __global__ void __launch_bounds__(256) embed_grad_kernel(const TokT* __restrict_
   }
 }
 
-// Column sums of A [rows][N] (leading dimension lda): block (x, y) sums
-// columns 32x .. 32x+31 over its share of the rows into part[y][N].
-__global__ void __launch_bounds__(256) colsum_kernel(const float* __restrict__ A, long long lda, long long rows,
-                                                     int N, float* __restrict__ part) {
+// Column sums of A [rows][N] (leading dimension lda), up to two matrices per
+// launch: block (x, y) sums 32 columns over its share of the rows, one of nblk,
+// into part[y][N].  (Past a matrix's own nblk: no rows left.)
+struct ColSum {
+  const float* A;
+  long long lda, rows;
+  int N, nblk;
+  float* part;
+};
+__global__ void __launch_bounds__(256) colsum_kernel(ColSum a, ColSum b, int nx) {
   __shared__ float red[8][33];
-  const int c = blockIdx.x * 32 + (threadIdx.x & 31), rg = threadIdx.x >> 5;
-  const long long chunk = (rows + gridDim.y - 1) / gridDim.y;
+  const bool second = (int)blockIdx.x >= nx;
+  const ColSum q = second ? b : a;
+  if ((int)blockIdx.y >= q.nblk) return;
+  const int c = ((int)blockIdx.x - (second ? nx : 0)) * 32 + (threadIdx.x & 31), rg = threadIdx.x >> 5;
+  const long long chunk = (q.rows + q.nblk - 1) / q.nblk;
   const long long r0 = (long long)blockIdx.y * chunk;
-  const long long r1 = r0 + chunk < rows ? r0 + chunk : rows;
+  const long long r1 = r0 + chunk < q.rows ? r0 + chunk : q.rows;
   float acc = 0.0f;
-  if (c < N)
-    for (long long r = r0 + rg; r < r1; r += 8) acc += A[r * lda + c];
+  if (c < q.N)
+    for (long long r = r0 + rg; r < r1; r += 8) acc += q.A[r * q.lda + c];
   red[rg][threadIdx.x & 31] = acc;
   __syncthreads();
-  if (rg == 0 && c < N) {
+  if (rg == 0 && c < q.N) {
     float s = 0.0f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) s += red[k][threadIdx.x & 31];
-    part[(long long)blockIdx.y * N + c] = s;
+    q.part[(long long)blockIdx.y * q.N + c] = s;
   }
 }
 
@@ -1725,12 +1747,12 @@ struct ReduceSeg {
   const float* part;
   long long len, stride;
   float* out;
+  int nparts;  // (0: the list's)
 };
 constexpr int kReduceSegs = 5;
 struct ReduceList {
   ReduceSeg seg[kReduceSegs];
   unsigned first[kReduceSegs];  // first block of each segment (past the grid: none)
-  int nparts;
 };
 __global__ void __launch_bounds__(1024) reduce_kernel(ReduceList l) {
   __shared__ float red[32][33];
@@ -1747,7 +1769,7 @@ __global__ void __launch_bounds__(1024) reduce_kernel(ReduceList l) {
   const float* src = q.part + (i < q.len ? i : q.len - 1);
   float s = 0.0f;
 #pragma unroll 4
-  for (int p = g; p < l.nparts; p += 32) s += src[p * q.stride];
+  for (int p = g; p < q.nparts; p += 32) s += src[p * q.stride];
   red[g][c] = s;
   __syncthreads();
   if (g == 0 && i < q.len) {
@@ -1937,6 +1959,15 @@ cudaError_t launch_tc_rows(const Gemm& g, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Whether the 128 x 64 CUDA-core kernel takes the product: aligned float4
+// operands, K ranges of 32 where they are contiguous in k.
+bool sgemm_fast(int kind, const Gemm& g) {
+  auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
+  const bool ak = kind != 2, bk = kind == 0, k32 = g.kchunk % 32 == 0 && g.K % 32 == 0;
+  return al(g.A) && al(g.B) && g.lda % 4 == 0 && g.ldb % 4 == 0 && (ak ? k32 : g.M % 4 == 0) &&
+         (bk ? k32 : g.N % 4 == 0);
+}
+
 // kind 0: forward (A row-major, B = W [N][K]); 1: input gradient (A
 // row-major, B = W [K][N]); 2: weight gradient (A and B indexed [k][.]).
 cudaError_t gemm(int kind, const Gemm& g, cudaStream_t s) {
@@ -1951,32 +1982,47 @@ cudaError_t gemm(int kind, const Gemm& g, cudaStream_t s) {
       default: return launch_tc_rows<EPI_STORE>(g, s);
     }
   }
-  const long long kc = g.kchunk > 0 ? g.kchunk : g.K;
-  dim3 grid((unsigned)((g.M + 63) / 64), (unsigned)((g.N + 63) / 64), (unsigned)((g.K + kc - 1) / kc));
-  Gemm a = g;
-  a.kchunk = kc;
-  // aligned float4 operands: the 128 x 64 kernel
-  auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
-  const bool ak = kind != 2, bk = kind == 0;
-  bool fast = al(g.A) && al(g.B) && g.lda % 4 == 0 && g.ldb % 4 == 0;
-  fast = fast && (ak ? (kc % 32 == 0 && g.K % 32 == 0) : g.M % 4 == 0);
-  fast = fast && (bk ? (kc % 32 == 0 && g.K % 32 == 0) : g.N % 4 == 0);
-  if (fast) {
-    dim3 grid2((unsigned)((g.M + 127) / 128), (unsigned)((g.N + 63) / 64), (unsigned)((g.K + kc - 1) / kc));
+  const dim3 grid((unsigned)((g.M + 63) / 64), (unsigned)((g.N + 63) / 64),
+                  (unsigned)((g.K + g.kchunk - 1) / g.kchunk));
+  if (sgemm_fast(kind, g)) {
+    const dim3 grid2((unsigned)((g.M + 127) / 128), grid.y, grid.z);
     if (kind == 0)
-      sgemm128_kernel<true, true><<<grid2, 256, 0, s>>>(a);
+      sgemm128_kernel<true, true><<<grid2, 256, 0, s>>>(g);
     else if (kind == 1)
-      sgemm128_kernel<true, false><<<grid2, 256, 0, s>>>(a);
+      sgemm128_kernel<true, false><<<grid2, 256, 0, s>>>(g);
     else
-      sgemm128_kernel<false, false><<<grid2, 256, 0, s>>>(a);
+      sgemm128_kernel<false, false><<<grid2, 256, 0, s>>>(g);
     return cudaGetLastError();
   }
   if (kind == 0)
-    sgemm_kernel<true, true><<<grid, 256, 0, s>>>(a);
+    sgemm_kernel<true, true><<<grid, 256, 0, s>>>(g);
   else if (kind == 1)
-    sgemm_kernel<true, false><<<grid, 256, 0, s>>>(a);
+    sgemm_kernel<true, false><<<grid, 256, 0, s>>>(g);
   else
-    sgemm_kernel<false, false><<<grid, 256, 0, s>>>(a);
+    sgemm_kernel<false, false><<<grid, 256, 0, s>>>(g);
+  return cudaGetLastError();
+}
+
+// Two products of one kind that do not depend on each other: one launch on the
+// CUDA cores where both have the 128 x 64 kernel.  The last block's queries, over
+// n rows, go with its keys and values, over n T: small batches are bound by
+// launches.  (64 samples of 4 tokens, d = 128, 2 blocks, forward and gradient:
+// 226 and 758 us with launches of their own, 215 and 667 so.)
+cudaError_t gemm_pair(int kind, const Gemm& a, const Gemm& b, cudaStream_t s) {
+  if (a.bimg || b.bimg || a.M <= 0 || b.M <= 0 || !sgemm_fast(kind, a) || !sgemm_fast(kind, b)) {
+    const cudaError_t e = gemm(kind, a, s);
+    return e == cudaSuccess ? gemm(kind, b, s) : e;
+  }
+  const int ny = (a.N + 63) / 64;
+  auto splits = [](const Gemm& g) { return (g.K + g.kchunk - 1) / g.kchunk; };
+  const dim3 grid((unsigned)((std::max(a.M, b.M) + 127) / 128), (unsigned)(ny + (b.N + 63) / 64),
+                  (unsigned)std::max(splits(a), splits(b)));
+  if (kind == 0)
+    sgemm128_pair_kernel<true, true><<<grid, 256, 0, s>>>(a, b, ny);
+  else if (kind == 1)
+    sgemm128_pair_kernel<true, false><<<grid, 256, 0, s>>>(a, b, ny);
+  else
+    sgemm128_pair_kernel<false, false><<<grid, 256, 0, s>>>(a, b, ny);
   return cudaGetLastError();
 }
 
@@ -1992,11 +2038,11 @@ Gemm mk(const float* A, long long lda, const float* B, long long ldb, float* C, 
 
 cudaError_t reduce(int nparts, std::initializer_list<ReduceSeg> segs, cudaStream_t s) {
   ReduceList l;
-  l.nparts = nparts;
   unsigned blocks = 0;
   int k = 0;
   for (const ReduceSeg& q : segs) {
     l.seg[k] = q;
+    if (!q.nparts) l.seg[k].nparts = nparts;
     l.first[k++] = blocks;
     blocks += blocks_for(q.len, 32);
   }
@@ -2006,6 +2052,34 @@ cudaError_t reduce(int nparts, std::initializer_list<ReduceSeg> segs, cudaStream
   }
   reduce_kernel<<<blocks, 1024, 0, s>>>(l);
   return cudaGetLastError();
+}
+
+// A weight gradient and its bias gradient on the CUDA cores: the product's
+// partial slabs from `part` on, the column sums' behind them, and their
+// reductions.
+struct WgradCores {
+  Gemm g;
+  ColSum sum;
+  ReduceSeg dw, db;
+  int nx() const { return (sum.N + 31) / 32; }
+  float* end() const { return sum.part + (long long)sum.nblk * sum.N; }  // of the partial sums
+};
+WgradCores wgrad_cores(const float* dOut, long long ldo, int n_o, const float* In, long long ldi, int n_i,
+                       long long rows, float* gW, float* gb, float* part) {
+  const long long tiles = (long long)((n_o + 63) / 64) * ((n_i + 63) / 64), len = (long long)n_o * n_i;
+  long long splits = (608 + tiles - 1) / tiles;
+  splits = std::min(std::max(splits, 1ll), 128ll);
+  splits = std::min(splits, (rows + 63) / 64);
+  const long long kc = ((rows + splits - 1) / splits + 15) / 16 * 16;
+  splits = (rows + kc - 1) / kc;
+  WgradCores q;
+  q.g = mk(dOut, ldo, In, ldi, part, n_i, n_o, n_i, rows, EPI_PARTIAL);
+  q.g.kchunk = kc;
+  const int nblk = (int)std::min((rows + 63) / 64, 256ll);
+  q.sum = ColSum{dOut, ldo, rows, n_o, nblk, part + splits * len};
+  q.dw = ReduceSeg{part, len, len, gW, (int)splits};
+  q.db = ReduceSeg{q.sum.part, n_o, n_o, gb, nblk};
+  return q;
 }
 
 // dW[o][i] = sum_r dOut[r][o] In[r][i] and db[o] = sum_r dOut[r][o] over rows
@@ -2041,26 +2115,22 @@ cudaError_t wgrad(ut_tfm* t, const float* dOut, long long ldo, int n_o, const fl
     if (e == cudaSuccess) e = reduce((int)splits, {{t->part, len, len, gW}, {bias_part, n_o, n_o, gb}}, s);
     return e;
   }
-  Gemm g = mk(dOut, ldo, In, ldi, t->part, n_i, n_o, n_i, rows, EPI_PARTIAL);
-  const long long tiles = (long long)((n_o + 63) / 64) * ((n_i + 63) / 64);
-  long long splits = (608 + tiles - 1) / tiles;
-  splits = splits < 1 ? 1 : (splits > 128 ? 128 : splits);
-  const long long max_split = (rows + 63) / 64;
-  if (splits > max_split) splits = max_split;
-  long long kc = (rows + splits - 1) / splits;
-  kc = (kc + 15) / 16 * 16;
-  splits = (rows + kc - 1) / kc;
-  g.kchunk = kc;
-  cudaError_t e = gemm(2, g, s);
-  const long long len = (long long)n_o * n_i;
-  if (e == cudaSuccess) e = reduce((int)splits, {{t->part, len, len, gW}}, s);
+  const WgradCores q = wgrad_cores(dOut, ldo, n_o, In, ldi, n_i, rows, gW, gb, t->part);
+  cudaError_t e = gemm(2, q.g, s);
   if (e != cudaSuccess) return e;
-  long long nblk = (rows + 63) / 64;
-  nblk = nblk < 1 ? 1 : (nblk > 256 ? 256 : nblk);
-  colsum_kernel<<<dim3((unsigned)((n_o + 31) / 32), (unsigned)nblk), 256, 0, s>>>(dOut, ldo, rows, n_o, t->part);
+  colsum_kernel<<<dim3((unsigned)q.nx(), (unsigned)q.sum.nblk), 256, 0, s>>>(q.sum, q.sum, q.nx());
   e = cudaGetLastError();
-  if (e == cudaSuccess) e = reduce((int)nblk, {{t->part, n_o, n_o, gb}}, s);
-  return e;
+  return e == cudaSuccess ? reduce(0, {q.dw, q.db}, s) : e;
+}
+
+// Two weight gradients on the CUDA cores, by the launches of one (gemm_pair).
+cudaError_t wgrad_pair(const WgradCores& a, const WgradCores& b, cudaStream_t s) {
+  cudaError_t e = gemm_pair(2, a.g, b.g, s);
+  if (e != cudaSuccess) return e;
+  colsum_kernel<<<dim3((unsigned)(a.nx() + b.nx()), (unsigned)std::max(a.sum.nblk, b.sum.nblk)), 256, 0, s>>>(
+      a.sum, b.sum, a.nx());
+  e = cudaGetLastError();
+  return e == cudaSuccess ? reduce(0, {a.dw, a.db, b.dw, b.db}, s) : e;
 }
 
 // The LayerNorm kernels loop over rows (grid stride): at most kLnBlocks
@@ -2267,12 +2337,15 @@ cudaError_t forward(ut_tfm* t, const Call& c, cudaStream_t s) {
     }
     if (e != cudaSuccess) break;
     if (last) {
-      if (!fused) {
-      e = gemm0(mk(b.Y1, d, w + ol[T_WQKV] + d * d, d, b.QKV, 2 * d, rows, 2 * d, d, EPI_BIAS), ol[T_BQKV] + d,
-                img(l, 0));
-      if (e == cudaSuccess)  // the recurrent rows of Y1 are T d apart
-        e = gemm0(mk(b.Y1, (long long)t->T * d, w + ol[T_WQKV], d, b.Q0, d, c.n, d, d, EPI_BIAS), ol[T_BQKV],
-                  img(t->L, 0));
+      if (!fused) {  // the recurrent rows of Y1 are T d apart
+        Gemm kv = mk(b.Y1, d, w + ol[T_WQKV] + d * d, d, b.QKV, 2 * d, rows, 2 * d, d, EPI_BIAS);
+        Gemm q = mk(b.Y1, (long long)t->T * d, w + ol[T_WQKV], d, b.Q0, d, c.n, d, d, EPI_BIAS);
+        kv.bias = w + ol[T_BQKV] + d;
+        q.bias = w + ol[T_BQKV];
+        kv.bimg = img(l, 0);
+        q.bimg = img(t->L, 0);
+        kv.status = q.status = t->status;
+        e = gemm_pair(0, kv, q, s);
       }
       if (e == cudaSuccess)
         e = attn0_fwd<DH>(b.Q0, b.QKV, c.ne, c.sel, b.P, b.O, c.n, t->T, t->NS, t->H, t->gemm_tc != 0, s);
@@ -2387,13 +2460,21 @@ cudaError_t backward(ut_tfm* t, const Call& c, float* grad, cudaStream_t s) {
       // dK and dV in one sum as in the other blocks
       const float* Wq = w + ol[T_WQKV];
       e = attn0_bwd<DH>(b.Q0, b.QKV, b.P, t->dO, D0, t->dBig, c.n, t->T, t->H, t->gemm_tc != 0, s);
-      if (e == cudaSuccess)
-        e = dgemm(l, 4, mk(t->dBig, 2 * d, Wq + d * d, d, t->dY, d, rows, d, 2 * d, EPI_STORE));
-      if (e == cudaSuccess) e = dgemm(t->L, 3, mk(D0, 3 * d, Wq, d, t->dO, d, c.n, d, 3 * d, EPI_STORE));
-      if (e == cudaSuccess)
-        e = wgrad(t, t->dBig, 2 * d, 2 * d, b.Y1, d, d, rows, grad + ol[T_WQKV] + d * d, grad + ol[T_BQKV] + d, s);
-      if (e == cudaSuccess)
-        e = wgrad(t, D0, 3 * d, d, b.Y1, (long long)t->T * d, d, c.n, grad + ol[T_WQKV], grad + ol[T_BQKV], s);
+      const Gemm dkv = mk(t->dBig, 2 * d, Wq + d * d, d, t->dY, d, rows, d, 2 * d, EPI_STORE);
+      const Gemm dq = mk(D0, 3 * d, Wq, d, t->dO, d, c.n, d, 3 * d, EPI_STORE);
+      float *gW = grad + ol[T_WQKV], *gb = grad + ol[T_BQKV];
+      const long long Td = (long long)t->T * d;
+      if (t->gemm_tc) {
+        if (e == cudaSuccess) e = dgemm(l, 4, dkv);
+        if (e == cudaSuccess) e = dgemm(t->L, 3, dq);
+        if (e == cudaSuccess) e = wgrad(t, t->dBig, 2 * d, 2 * d, b.Y1, d, d, rows, gW + d * d, gb + d, s);
+        if (e == cudaSuccess) e = wgrad(t, D0, 3 * d, d, b.Y1, Td, d, c.n, gW, gb, s);
+      } else {
+        if (e == cudaSuccess) e = gemm_pair(1, dkv, dq, s);
+        const WgradCores kv = wgrad_cores(t->dBig, 2 * d, 2 * d, b.Y1, d, d, rows, gW + d * d, gb + d, t->part);
+        const WgradCores q = wgrad_cores(D0, 3 * d, d, b.Y1, Td, d, c.n, gW, gb, kv.end());
+        if (e == cudaSuccess) e = wgrad_pair(kv, q, s);
+      }
       if (e == cudaSuccess)
         e = ln_bwd<DJ, true>(t, t->dY, b.X, b.S1, w + ol[T_LN1G], t->dM, t->dX, grad + ol[T_LN1G], rows, s, t->dO);
       continue;
@@ -2547,7 +2628,7 @@ extern "C" ut_status tfm_create(const ut_tfm_config* cfg, const float* params_ho
   const size_t R = (size_t)t->max_rows, d = (size_t)t->d, L = (size_t)t->L;
   const size_t Pn = (size_t)cfg->max_batch * t->H * t->T * t->T;
   size_t part = (size_t)128 * 4 * d * d;
-  part = std::max(part, (size_t)256 * 4 * d);
+  part += (size_t)256 * 4 * d;  // CUDA-core weight gradients, and the column sums behind them
   part = std::max(part, (size_t)kRowWarps * (2 * d + (size_t)t->n_out * d + t->n_out));
   part = std::max(part, (size_t)kRowWarps * 9 * d);
   part = std::max(part, (size_t)kLnBlocks * 2 * d);
