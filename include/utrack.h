@@ -243,13 +243,14 @@ ut_status env_reset(ut_env* env, uint64_t seed);
 ut_status env_step(ut_env* env, const int32_t* actions_dev, ut_step_out* out);
 
 /* T steps with policy (or random) actions, replayed from a captured CUDA
- * graph.  Clears the device metrics first; synchronises and fills `stats`
- * (host struct) with the metrics of these T steps.  T >= 1. */
+ * graph.  The graph is captured again when T, the step's configuration or the
+ * seed of env_reset changes.  Clears the device metrics first; synchronises
+ * and fills `stats` (host struct) with the metrics of these T steps.  T >= 1. */
 ut_status rollout(ut_env* env, int32_t T, ut_rollout_stats* stats);
 
 /* Captures and instantiates (and uploads) the T-step rollout graph without
- * running it, so that a later rollout(T) starts executing at once.  Not
- * synchronising. */
+ * running it, so that a later rollout(T) under the same seed starts executing at
+ * once.  Not synchronising. */
 ut_status rollout_prepare(ut_env* env, int32_t T);
 
 /* Stage timing.  When enabled, every eager env_step records a pair of CUDA

@@ -533,7 +533,8 @@ ut_status env_metrics(ut_env* h, ut_rollout_stats* out) {
 static ut_status graph_ensure(ut_env* h, int32_t T) {
   UT_CUDA(h, ut::capture_stream_ensure(h));
   const int key = T * 16 + (h->policy_ready ? 1 : 0) + 2 * h->est_mode;  // est_mode 0..4
-  if (!h->graph_exec || h->graph_key != key || h->graph_variant != h->pf_variant) {
+  // (the captured kernels hold the seed among their arguments)
+  if (!h->graph_exec || h->graph_key != key || h->graph_variant != h->pf_variant || h->graph_seed != h->d.seed) {
     if (h->graph_exec) {
       cudaGraphExecDestroy(h->graph_exec);
       h->graph_exec = nullptr;
@@ -558,6 +559,7 @@ static ut_status graph_ensure(ut_env* h, int32_t T) {
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaGraphInstantiate");
     h->graph_key = key;
     h->graph_variant = h->pf_variant;
+    h->graph_seed = h->d.seed;
     UT_CUDA(h, cudaGraphUpload(h->graph_exec, h->cap_stream));
   }
   return UT_OK;

@@ -33,6 +33,7 @@ struct ut_env {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaGraphExec_t graph_exec = nullptr;
   int graph_key = -1, graph_variant = -1;
+  uint64_t graph_seed = 0;
   // graph-captured PPO collection (env_ppo_collect), keyed by its arguments
   cudaGraphExec_t ppo_exec = nullptr;
   std::vector<uintptr_t> ppo_key;
