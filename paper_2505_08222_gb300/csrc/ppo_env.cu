@@ -200,8 +200,8 @@ extern "C" ut_status env_ppo_collect(ut_env* h, ut_tfm* critic, int32_t T, const
   cudaError_t e = capture_stream_ensure(h);
   if (e != cudaSuccess) return cuda_fail(h, "env_ppo_collect", e);
   // the graph is rebuilt when any argument, the step's configuration or the seed changes
-  std::vector<uintptr_t> key = {(uintptr_t)critic, (uintptr_t)T, (uintptr_t)h->pf_variant, (uintptr_t)h->est_mode,
-                                (uintptr_t)h->d.seed};
+  std::vector<uintptr_t> key = {(uintptr_t)ci.id, (uintptr_t)ci.gemm_tc, (uintptr_t)T, (uintptr_t)h->pf_variant,
+                                (uintptr_t)h->est_mode, (uintptr_t)h->d.seed};
   for (const void* p : {(const void*)b->tokens, (const void*)b->n_ent, (const void*)b->h, (const void*)b->actions,
                         (const void*)b->logp, (const void*)b->reward, (const void*)b->done, (const void*)b->ctokens,
                         (const void*)b->cn_ent, (const void*)b->ch, (const void*)b->value})

@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <initializer_list>
@@ -1847,6 +1848,8 @@ __global__ void gae_agents_kernel(const float* __restrict__ adv, const int32_t* 
 #include "runtime.cuh"
 
 struct ut_tfm {
+  static std::atomic<uint64_t> created;
+  const uint64_t id = ++created;
   ut_tfm_config cfg{};
   cudaStream_t stream = nullptr;
   std::string err;
@@ -1880,6 +1883,7 @@ struct ut_tfm {
   int n_img = 0, img_max = 0;
   int* status = nullptr;
 };
+std::atomic<uint64_t> ut_tfm::created{0};
 
 namespace ut {
 namespace tfm {
@@ -2583,7 +2587,8 @@ using namespace ut::tfm;
 namespace ut {
 
 TfmInfo tfm_info(const ut_tfm* t) {
-  return TfmInfo{t->d, t->L, t->H, t->n_out, t->NS, t->cfg.tokens_bf16, (long long)t->cfg.max_batch};
+  return TfmInfo{t->d, t->L, t->H, t->n_out, t->NS, t->cfg.tokens_bf16, (long long)t->cfg.max_batch, t->id,
+                 t->gemm_tc};
 }
 
 cudaError_t tfm_forward_on(ut_tfm* t, const void* tokens, const int32_t* n_ent, const float* h, long long n,

@@ -9,10 +9,13 @@ struct ut_tfm;
 
 namespace ut {
 
-// Configuration of a handle.
+// Configuration of a handle; id: its own number among all the process's handles
+// (an address may be a later handle's again), gemm_tc: its GEMM path now.
 struct TfmInfo {
   int d, n_layers, n_heads, n_out, n_slots, tokens_bf16;
   long long max_batch;
+  uint64_t id;
+  int gemm_tc;
 };
 TfmInfo tfm_info(const ut_tfm* t);
 
