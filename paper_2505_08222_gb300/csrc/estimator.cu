@@ -942,7 +942,8 @@ cudaError_t launch_loss_grad(const Net& net, const TrainBufs& t, cudaStream_t s)
   if (e != cudaSuccess) return e;
   if (t.B <= 0) return cudaSuccess;
   const int n_cta = (t.B + kT - 1) / kT;
-  mlp_kernel<true><<<n_cta, kTE, kEnvSmem, s>>>(net, t.X, t.rows, t.B, nullptr, t, &t.result->status, t.test_wait_polls);
+  mlp_kernel<true><<<n_cta, kTE, kEnvSmem, s>>>(net, t.X, t.rows, t.B, nullptr, t, &t.result->status,
+                                                t.test_wait_polls);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int splits = n_cta < kWgradSplits ? n_cta : kWgradSplits;

@@ -44,11 +44,4 @@ __device__ __forceinline__ void gelu2(float& x0, float& x1) {
   f2upk(f2fma(f2add(X, A), f2pk(0.5f, 0.5f), f2mul(ae, q)), x0, x1);
 }
 
-// The same value for one input (identical arithmetic in lane 0).
-__device__ __forceinline__ float gelu1(float x) {
-  float y = x, unused = 0.0f;
-  gelu2(y, unused);
-  return y;
-}
-
 }  // namespace ut

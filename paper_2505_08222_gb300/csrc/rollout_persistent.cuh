@@ -43,13 +43,15 @@ inline size_t rollout_stage_bytes(int filters, int AM) { return 2 * (size_t)filt
 
 // CTAs per SM that the registers must allow when there are more environments than
 // SMs: small filters leave room for several on an SM, and left to itself the
-// compiler gives the environment's stage (200 registers) that room.  (50 steps of
+// compiler gives the environment's stage that room (202 to 216 registers at 4
+// particles per thread and up to 128 threads; 80 to 128 capped).  (50 steps of
 // 2000 environments of 1000 particles: 2984 us with one CTA per SM, 1729 with two;
 // 600 of 400: 950 and 517.  Up to one environment per SM the registers are worth
 // more: 64 of 2 x 2, 100 particles: 580 us, 614 with the cap.)
 template <int NT, int PPT>
 constexpr int rollout_min_blocks() {
-  return PPT > 4 ? (NT <= 64 ? 4 : (NT <= 128 ? 2 : 1)) : (NT <= 32 ? 12 : (NT <= 64 ? 6 : (NT <= 128 ? 3 : (NT <= 256 ? 2 : 1))));
+  if (PPT > 4) return NT <= 64 ? 4 : (NT <= 128 ? 2 : 1);
+  return NT <= 32 ? 12 : (NT <= 64 ? 6 : (NT <= 128 ? 3 : (NT <= 256 ? 2 : 1)));
 }
 
 template <int NT, int PPT, int MODE, int MINB>
@@ -147,7 +149,8 @@ cudaError_t launch_blocks(const EnvDev& d, int T, cudaStream_t s) {
   const cudaError_t e =
       smem_optin(k, pf::step_smem_bytes(NT, PPT) + rollout_stage_bytes(kMaxAgents * kMaxTargets, kMaxAgents), ready);
   if (e != cudaSuccess) return e;
-  k<<<d.E, rollout_threads<NT>(), pf::step_smem_bytes(NT, PPT) + rollout_stage_bytes(filters, d.AM), s>>>(d, T, filters);
+  const size_t smem = pf::step_smem_bytes(NT, PPT) + rollout_stage_bytes(filters, d.AM);
+  k<<<d.E, rollout_threads<NT>(), smem, s>>>(d, T, filters);
   return cudaGetLastError();
 }
 

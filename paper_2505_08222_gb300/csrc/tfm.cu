@@ -12,9 +12,11 @@
 // made for every token; its queries, attention output, feed-forward sub-block
 // and their backward run on the n recurrent rows, stored densely ([n][width]).
 //
-// The dense contractions run on CUDA cores in FP32 (a 64 x 64 register-tiled
-// GEMM); the weight gradients are split along the token rows into partial
-// slabs summed in a fixed order, so every result is deterministic.
+// The dense contractions run on the tensor cores (tfm_tc.cuh; at d = 64 most of a
+// block in four fused kernels, tfm_qkv.cuh and tfm_ffn.cuh) or, on the path chosen
+// by tfm_set_gemm_path(0), on the CUDA cores in FP32 (the register-tiled GEMMs
+// below).  The weight gradients are split along the token rows into partial slabs
+// summed in a fixed order, so every result is deterministic.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -546,7 +548,8 @@ __device__ __forceinline__ void attn_put_pair(float* item, int u, int j, float4 
 struct AttnRows {
   AttItem first;
   int H, T, inv;
-  __device__ __forceinline__ AttnRows(long long q0, int h, int t) : first(att_item(q0, h)), H(h), T(t), inv(65536 / t + 1) {}
+  __device__ __forceinline__ AttnRows(long long q0, int h, int t)
+      : first(att_item(q0, h)), H(h), T(t), inv(65536 / t + 1) {}
   __device__ __forceinline__ int item(int r) const { return (r * inv) >> 16; }
   __device__ __forceinline__ void sample(int it, long long& s, int& hh) const {
     const unsigned h = (unsigned)(first.hh + it), ds = h / (unsigned)H;
