@@ -798,7 +798,9 @@ constexpr int kRedW = (int)((NW_PART / 4 + 255) / 256), kRedB = (NB_PART + 31) /
 
 __global__ void __launch_bounds__(256) grad_reduce_kernel(TrainBufs t, int splits, int n_cta) {
   const int tid = threadIdx.x;
-  if (t.result->status) return;  // (partial sums of a pass that gave up, or of an earlier one)
+  // partial sums of a pass that gave up, or of an earlier one, go no further
+  // (looked at behind the sums: its load is in flight during theirs)
+  const int gave_up = t.result->status;
   if (blockIdx.x < kRedW) {
     const long long i = ((long long)blockIdx.x * 256 + tid) * 4;
     if (i >= NW_PART) return;
@@ -808,6 +810,7 @@ __global__ void __launch_bounds__(256) grad_reduce_kernel(TrainBufs t, int split
       const float4 v = *reinterpret_cast<const float4*>(t.part_w + (long long)p * NW_PART + i);
       s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
     }
+    if (gave_up) return;
     float* g = t.grad + part_dst(1, i);
     g[0] = s.x; g[1] = s.y; g[2] = s.z; g[3] = s.w;
     return;
@@ -822,7 +825,7 @@ __global__ void __launch_bounds__(256) grad_reduce_kernel(TrainBufs t, int split
     }
     red[g][c] = s;
     __syncthreads();
-    if (g == 0 && i < NB_PART) {
+    if (g == 0 && i < NB_PART && !gave_up) {
       float acc = 0.0f;
 #pragma unroll
       for (int k = 0; k < 8; ++k) acc += red[k][c];
@@ -836,7 +839,7 @@ __global__ void __launch_bounds__(256) grad_reduce_kernel(TrainBufs t, int split
   s = warp_sum_d(s);
   if ((tid & 31) == 0) sl[tid >> 5] = s;
   __syncthreads();
-  if (tid == 0) {
+  if (tid == 0 && !gave_up) {
     double acc = 0.0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) acc += sl[k];
@@ -867,12 +870,14 @@ __device__ __forceinline__ void write_images(unsigned char* img, long long i, fl
 __global__ void adam_kernel(float* master, float* m, float* v, const float* grad, float lr, float beta1, float beta2,
                             float eps, float c1, float c2, unsigned char* img, EstResult* result) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= NPARAM || (result && result->status)) return;
-  if (result && i == 0) ++result->updates;
+  if (i >= NPARAM) return;
+  const int gave_up = result ? result->status : 0;
   const float g = grad[i];
   const float mi = beta1 * m[i] + (1.0f - beta1) * g;
   const float vi = beta2 * v[i] + (1.0f - beta2) * g * g;
   const float th = master[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  if (gave_up) return;
+  if (result && i == 0) ++result->updates;
   m[i] = mi;
   v[i] = vi;
   master[i] = th;
