@@ -633,14 +633,15 @@ def run_ours(args):
         dist.barrier()
     agent_steps = float(shard.reduce_sums([stats["agent_steps"]])[0])
 
-    # the same timed rollout (a graph per seed, captured outside the timed
-    # region; W warm-up steps) from seeds 0..4
+    # the same timed rollout (in the graph form a graph per seed, captured
+    # outside the timed region; W warm-up steps) from seeds 0..4
     sweep, sweep_rmse = [], []
     for sd in range(5):
         env.reset(sd)
         for _ in range(W):
             env.step()
-        env.rollout_prepare(K)
+        if env.rollout_form() == 0:
+            env.rollout_prepare(K)
         torch.cuda.synchronize()
         if world > 1:
             torch.distributed.barrier()

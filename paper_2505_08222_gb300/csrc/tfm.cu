@@ -496,8 +496,8 @@ __global__ void ln_bwd_kernel(const float* __restrict__ dY, const float* __restr
 // it too, so that a block's P, one contiguous range, is read and written whole.
 // The products run on packed FP32 pairs: two keys of a score at once (staged
 // interleaved), two columns of an output at once, so each sum keeps its order.
-// Bound by issue and shared-memory loads: 131,072 items of 17 x 16 forward 254 us,
-// backward 500 (534 and 809 with a warp per item; 274 and 524 with the rows
+// Bound by the latency of its shared-memory loads (issue 28 to 36 % active):
+// 131,072 items of 17 x 16 forward 254 us, backward 500 (534 and 809 with a warp per item; 274 and 524 with the rows
 // staged one load after the other and 64-bit divisions).
 constexpr int kAttnThreads = 128;
 __host__ __device__ __forceinline__ int attn_items(int T) { return kAttnThreads / T; }
